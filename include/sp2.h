@@ -72,7 +72,12 @@ typedef enum {
  * of the tensor-core modes: (max_iter + 8) slots of P * E * ld^2 bytes (P pieces of E bytes), ld = N
  * rounded up to a multiple of 128 (256 with CTA-pair tiles); see sp2_opts.history. */
 typedef enum {
-  SP2_PREC_FP64 = 0,   /* FP64 products and FP64 everything (the plain method) */
+  SP2_PREC_FP64 = 0,   /* FP64 products and FP64 everything (the plain method).  For N >= 129 the products
+                          are formed on the tensor cores as exact integer sums of 8-bit digit products,
+                          rounded to FP64 once (56 bits per value under a power-of-two scale per row):
+                          the error of a product is below that of a chain of FP64 multiply-adds.
+                          Workspace 14 ld^2 bytes beside the two iterates (twice that with McWeeny); a
+                          handle that cannot have it multiplies on the FP64 units */
   SP2_PREC_MIXED = 1,  /* = SP2_PREC_BF16X6: each FP32 value stored exactly as three bf16
                           pieces (P = 3), products as the six piece products with a + b <= 2
                           (FP32-accurate) */
@@ -215,7 +220,8 @@ void sp2_default_opts(sp2_opts* opts);
 
 /* Create a handle for problems of size N (1 <= N <= 65536) with n_occ occupied
  * orbitals (0 <= n_occ <= N), allocating its device workspace on the current device:
- * for SP2_PREC_FP64 two N x N FP64 ping-pong buffers padded to a multiple of 64; for
+ * for SP2_PREC_FP64 two N x N FP64 ping-pong buffers padded to a multiple of 64 (and the digit
+ * buffers described there); for
  * SP2_PREC_MIXED the piece arena described at SP2_PREC_MIXED.  opts may be NULL for
  * the defaults.  On failure *out is set to NULL. */
 sp2_status sp2_create(int64_t N, int64_t n_occ, int32_t precision, const sp2_opts* opts,
@@ -361,7 +367,7 @@ sp2_status sp2_get_work_bsr(sp2_bsr h, int64_t* block_products, int64_t* needed_
  * F_dev, D_dev: N x N device buffers as in sp2_run.  info_dev: NULL or 4 device
  * int32 that receive (status, n_iter, stop_reason, hist_len) when the run ends.
  * Asynchronous on `stream`.  The workspace is one fixed device array inside the
- * library (about 4.2 MB, held on every GPU that loads the library until exit);
+ * library (about 8 MB, held on every GPU that loads the library until exit);
  * N > SP2_NOALLOC_MAX_N returns SP2_ERR_INVALID_ARG.  The first call on a device
  * looks up that array's device address and, under CUDA's default lazy module loading,
  * may load the library's device code and so allocate the array: make that first call

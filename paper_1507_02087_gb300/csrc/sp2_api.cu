@@ -24,6 +24,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "sp2_common.cuh"
+#include "sp2_f64_tc.cuh"
 #include "sp2_kernels.h"
 #include "sp2_tc.cuh"
 
@@ -593,6 +594,7 @@ struct sp2_ctx {
   int64_t pert_count = 0;
   int mcw = 0;                   // 0: SP2, 1: McWeeny, 2: McW-ACC (FP64 path)
   double* sbuf = nullptr;        // McWeeny: the shifted square S_s (ld x ld)
+  sp2::f64tc::Plan tc;           // products on the tensor cores (tc.on), or the CUDA-core kernels
   DevState* st_dev = nullptr;
   DevState* st_host = nullptr;
   cudaGraph_t graph = nullptr;
@@ -618,6 +620,10 @@ static void free_ctx(sp2_ctx* h) {
   cudaFree(h->mscr);
   cudaFree(h->lz);
   cudaFree(h->sbuf);
+  for (sp2::f64tc::Digits* d : {&h->tc.X, &h->tc.S}) {
+    cudaFree(d->dig);
+    cudaFree(d->exp);
+  }
   cudaFree(h->part_lo);
   cudaFree(h->part_hi);
   cudaFree(h->part_bad);
@@ -632,6 +638,24 @@ static void free_ctx(sp2_ctx* h) {
   delete h;
 }
 
+// Digit buffers of one ld x ld matrix, zeroed (the rows past N stay zero).
+// False (and nothing held) when the memory is not there: the CUDA-core products need none.
+static bool alloc_digits(sp2::f64tc::Digits& d, int ld) {
+  using namespace sp2::f64tc;
+  if (cudaMalloc(&d.dig, digit_bytes(ld)) == cudaSuccess && cudaMalloc(&d.exp, exp_bytes(ld)) == cudaSuccess &&
+      cudaMemset(d.dig, 0, digit_bytes(ld)) == cudaSuccess && cudaMemset(d.exp, 0, exp_bytes(ld)) == cudaSuccess)
+    return true;
+  (void)cudaGetLastError();
+  cudaFree(d.dig);
+  cudaFree(d.exp);
+  d.dig = nullptr;
+  d.exp = nullptr;
+  return false;
+}
+
+// The plan of the McWeeny step: it needs the digits of the shifted square too.
+static const sp2::f64tc::Plan* mcw_plan(const sp2_ctx* h) { return h->tc.on && h->tc.S.dig ? &h->tc : nullptr; }
+
 // The FP64 path's loop graph: a WHILE node around {square, stop test} (SP2) or {shifted
 // square, stop test, product} (McWeeny).
 static sp2_status build_f64_graph(sp2_ctx* h) {
@@ -643,11 +667,11 @@ static sp2_status build_f64_graph(sp2_ctx* h) {
   sp2_status s = add_while(h->graph, nullptr, 0, &h->cond, &node, &body);
   if (s != SP2_OK) return s;
   if (h->mcw)
-    SP2_TRY(sp2::add_mcw_loop_body(body, h->st_dev, h->buf[0], h->buf[1], h->sbuf, h->part, h->T, h->cond,
+    SP2_TRY(sp2::add_mcw_loop_body(body, h->st_dev, h->buf[0], h->buf[1], h->sbuf, h->part, h->T, h->cond, mcw_plan(h),
                                    h->mscr, h->lz, (int)h->N));
   else
-    SP2_TRY(sp2::add_f64_loop_body(body, h->st_dev, h->buf[0], h->buf[1], h->part, h->T, h->cond, h->mscr, h->lz,
-                                   (int)h->N, h->pert, h->pert_count));
+    SP2_TRY(sp2::add_f64_loop_body(body, h->st_dev, h->buf[0], h->buf[1], h->part, h->T, h->cond,
+                                   h->tc.on ? &h->tc : nullptr, h->mscr, h->lz, (int)h->N, h->pert, h->pert_count));
   SP2_TRY(cudaGraphInstantiate(&h->exec, h->graph, 0));
   return SP2_OK;
 }
@@ -658,7 +682,8 @@ static sp2_status create_f64(sp2_ctx* h) {
   h->nparts = (int)((h->N + 7) / 8 < 1024 ? (h->N + 7) / 8 : 1024);
   const size_t bytes = (size_t)h->ld * h->ld * sizeof(double);
   const size_t ntiles = (size_t)h->T * (h->T + 1) / 2;
-  bool ok = cudaMalloc(&h->part, ntiles * 2 * sizeof(double)) == cudaSuccess &&
+  const size_t part_bytes = ntiles * 2 * sp2::f64tc::RECS * sizeof(double);
+  bool ok = cudaMalloc(&h->part, part_bytes) == cudaSuccess &&
             cudaMalloc(&h->part_lo, h->nparts * sizeof(double)) == cudaSuccess &&
             cudaMalloc(&h->part_hi, h->nparts * sizeof(double)) == cudaSuccess &&
             cudaMalloc(&h->part_bad, h->nparts * sizeof(int)) == cudaSuccess &&
@@ -674,6 +699,10 @@ static sp2_status create_f64(sp2_ctx* h) {
   SP2_TRY(cudaMemcpy(h->st_dev, &init, sizeof(init), cudaMemcpyHostToDevice));
   SP2_TRY(cudaMemset(h->buf[0], 0, bytes));
   SP2_TRY(cudaMemset(h->buf[1], 0, bytes));
+  SP2_TRY(cudaMemset(h->part, 0, part_bytes));   // records below the diagonal are never written
+  h->tc.ld = h->ld;
+  h->tc.bn = sp2::f64tc::tile_width(h->ld);
+  h->tc.on = sp2::f64tc::wanted(h->N) && alloc_digits(h->tc.X, h->ld);
   *h->st_host = init;
   return build_f64_graph(h);
 }
@@ -722,11 +751,11 @@ static sp2_status enqueue_f64(sp2_ctx* h, const double* F, double* D, cudaStream
   } else {
     for (int it = 0; it <= h->opts.max_iter; ++it)
       if (h->mcw)
-        SP2_TRY(sp2::launch_mcw_step_plain(h->st_dev, h->buf[0], h->buf[1], h->sbuf, h->part, h->T, s, h->mscr,
-                                           h->lz, N));
+        SP2_TRY(sp2::launch_mcw_step_plain(h->st_dev, h->buf[0], h->buf[1], h->sbuf, h->part, h->T, s, mcw_plan(h),
+                                           h->mscr, h->lz, N));
       else
-        SP2_TRY(sp2::launch_f64_step_plain(h->st_dev, h->buf[0], h->buf[1], h->part, h->T, s, h->mscr, h->lz, N,
-                                           h->pert, h->pert_count));
+        SP2_TRY(sp2::launch_f64_step_plain(h->st_dev, h->buf[0], h->buf[1], h->part, h->T, s,
+                                           h->tc.on ? &h->tc : nullptr, h->mscr, h->lz, N, h->pert, h->pert_count));
   }
   SP2_TRY(cudaEventRecord(h->ev_loop[1], s));
   SP2_TRY(sp2::launch_copy_out(h->st_dev, h->buf[0], h->buf[1], h->ld, N, D, N, s));
@@ -888,6 +917,7 @@ extern "C" int32_t sp2_set_mcweeny(sp2_handle h, int32_t mode, double mu, double
   if (r == SP2_OK && mode > 0 && !h->sbuf) {
     const size_t bytes = (size_t)h->ld * h->ld * sizeof(double);
     if (cudaMalloc(&h->sbuf, bytes) != cudaSuccess || cudaMemset(h->sbuf, 0, bytes) != cudaSuccess) r = SP2_ERR_NOMEM;
+    else if (h->tc.on && !h->tc.S.dig) (void)alloc_digits(h->tc.S, h->ld);
   }
   if (r == SP2_OK) {
     const int32_t m = mode;

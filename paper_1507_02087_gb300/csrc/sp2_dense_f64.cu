@@ -7,6 +7,7 @@
 // The border stays zero through the iteration (0^2 = 0 and 2*0 - 0 = 0), so the
 // squaring works on whole 64 x 64 tiles with no bounds checks.
 #include "sp2_common.cuh"
+#include "sp2_f64_tc.cuh"
 #include "sp2_kernels.h"
 
 namespace sp2 {
@@ -299,9 +300,10 @@ constexpr int kFinThreads = 1024;
 // (v^2 part, ||X_{k-1}||_F^2 part, Tr[X_{k-1}] part, 0): there Tr[X_k] is taken from
 // the identity Tr[X^2] = ||X||_F^2 for symmetric X (Tr[X_k] = ||X_{k-1}||_F^2 after
 // X^2, 2 Tr[X_{k-1}] - ||X_{k-1}||_F^2 after 2X - X^2), so the polynomial choice does
-// not inherit the bias of the tensor cores' accumulation.
+// not inherit the bias of the tensor cores' accumulation.  A 64 x 64 tile has `recs` records (1, or
+// f64tc::RECS from the tensor-core products).
 __global__ void __launch_bounds__(kFinThreads)
-finalize_kernel(DevState* st, const double* __restrict__ part, int nparts, int stride,
+finalize_kernel(DevState* st, const double* __restrict__ part, int nparts, int stride, int recs,
                 cudaGraphConditionalHandle cond, double* mscr) {
   __shared__ double sm[32];
   if (st->done) {
@@ -322,7 +324,8 @@ finalize_kernel(DevState* st, const double* __restrict__ part, int nparts, int s
   if (st->norm == 1 && mscr) {                   // or m_{k-1}, the mixed norm over 64 x 64 tiles
     const int T = st->ld / kTile;
     vk = mixed_norm_cta<kFinThreads>(T, mscr, sm, [&](int I, int J) {
-      const double v2 = part[(int64_t)stride * upper_index(I, J, T)];
+      double v2 = 0.0;
+      for (int q = 0; q < recs; ++q) v2 += part[(int64_t)stride * (recs * upper_index(I, J, T) + q)];
       return I == J ? v2 : 0.5 * v2;             // off-diagonal tiles hold both mirror halves
     });
   }
@@ -365,7 +368,7 @@ __global__ void copy_out_kernel(const DevState* st, const double* __restrict__ b
 // Reduction + stop test of one FP64 square for loops driven without a CUDA graph:
 // the same rules as finalize_kernel (stride 2), ending the loop through st->done only.
 __global__ void __launch_bounds__(kFinThreads)
-finalize_plain_kernel(DevState* st, const double* __restrict__ part, int nparts, double* mscr) {
+finalize_plain_kernel(DevState* st, const double* __restrict__ part, int nparts, int recs, double* mscr) {
   __shared__ double sm[32];
   if (st->done) return;
   double a = 0.0, b = 0.0;
@@ -380,7 +383,8 @@ finalize_plain_kernel(DevState* st, const double* __restrict__ part, int nparts,
   if (st->norm == 1 && mscr) {
     const int T = st->ld / kTile;
     vk = mixed_norm_cta<kFinThreads>(T, mscr, sm, [&](int I, int J) {
-      const double v2 = part[2 * upper_index(I, J, T)];
+      double v2 = 0.0;
+      for (int q = 0; q < recs; ++q) v2 += part[2 * (recs * upper_index(I, J, T) + q)];
       return I == J ? v2 : 0.5 * v2;
     });
   }
@@ -450,26 +454,64 @@ cudaError_t launch_perturb(DevState* st, double* buf0, double* buf1, const doubl
   return cudaGetLastError();
 }
 
+// The square on the tensor cores: digits of X_{k-1}, then the product.
+static int recs_of(const f64tc::Plan* tc) { return tc ? f64tc::RECS : 1; }
+
+static cudaError_t emit_tc_square(f64tc::Sink& sink, DevState* st, double* buf0, double* buf1, double* S, double* part,
+                                  const f64tc::Plan& P, int N, f64tc::Op op) {
+  const cudaError_t e = f64tc::emit_digits(sink, st, buf0, buf1, nullptr, P, N);
+  return e != cudaSuccess ? e : f64tc::emit_product(sink, st, buf0, buf1, S, part, P, op);
+}
+
+// The McWeeny step's second product: digits of the shifted square, then S X_{k-1} (whose digits stand).
+static cudaError_t emit_tc_mcw_prod(f64tc::Sink& sink, DevState* st, double* buf0, double* buf1, double* S,
+                                    double* part, const f64tc::Plan& P, int N) {
+  const cudaError_t e = f64tc::emit_digits(sink, st, buf0, buf1, S, P, N);
+  return e != cudaSuccess ? e : f64tc::emit_product(sink, st, buf0, buf1, S, part, P, f64tc::OP_MCW_PROD);
+}
+
 cudaError_t launch_f64_step_plain(DevState* st, double* buf0, double* buf1, double* part, int T,
-                                  cudaStream_t s, double* mscr, void* lz, int N, const double* E, int64_t ecount) {
-  const int ntiles = T * (T + 1) / 2;
-  syrk_f64_kernel<<<ntiles, kSyrkThreads, 0, s>>>(st, buf0, buf1, part);
+                                  cudaStream_t s, const f64tc::Plan* tc, double* mscr, void* lz, int N, const double* E,
+                                  int64_t ecount) {
+  const int ntiles = T * (T + 1) / 2, recs = recs_of(tc), nrec = ntiles * recs;
+  if (tc) {
+    f64tc::Sink sink;
+    sink.s = s;
+    cudaError_t e = emit_tc_square(sink, st, buf0, buf1, nullptr, part, *tc, N, f64tc::OP_SP2);
+    if (e != cudaSuccess) return e;
+  } else {
+    syrk_f64_kernel<<<ntiles, kSyrkThreads, 0, s>>>(st, buf0, buf1, part);
+  }
   if (lz) {
-    cudaError_t e = launch_lanczos(st, buf0, buf1, nullptr, part, ntiles, lz, N, T * kTile, s);
+    cudaError_t e = launch_lanczos(st, buf0, buf1, nullptr, part, nrec, lz, N, T * kTile, s);
     if (e != cudaSuccess) return e;
   }
   if (E) {
     cudaError_t e = launch_perturb(st, buf0, buf1, E, ecount, N, 0, s);
     if (e != cudaSuccess) return e;
   }
-  finalize_plain_kernel<<<1, kFinThreads, 0, s>>>(st, part, ntiles, mscr);
+  finalize_plain_kernel<<<1, kFinThreads, 0, s>>>(st, part, nrec, recs, mscr);
   return cudaGetLastError();
 }
 
 cudaError_t add_mcw_loop_body(cudaGraph_t body, DevState* st, double* buf0, double* buf1, double* S, double* part,
-                              int T, cudaGraphConditionalHandle cond, double* mscr, void* lz, int N) {
-  const int ntiles = T * (T + 1) / 2;
+                              int T, cudaGraphConditionalHandle cond, const f64tc::Plan* tc, double* mscr, void* lz,
+                              int N) {
+  const int ntiles = T * (T + 1) / 2, recs = recs_of(tc);
   cudaGraphNode_t n_sq, n_fin, n_pr;
+  if (tc) {
+    f64tc::Sink sink;
+    sink.g = body;
+    cudaError_t e = emit_tc_square(sink, st, buf0, buf1, S, part, *tc, N, f64tc::OP_MCW_SQ);
+    if (e != cudaSuccess) return e;
+    if (lz && (e = add_lanczos_nodes(body, sink.last, st, buf0, buf1, S, part, ntiles * recs, lz, N, T * kTile,
+                                     &sink.last)) != cudaSuccess)
+      return e;
+    e = add_finalize_node(body, &sink.last, 1, st, part, ntiles * recs, 2, recs, cond, &n_fin, mscr);
+    if (e != cudaSuccess) return e;
+    sink.last = n_fin;
+    return emit_tc_mcw_prod(sink, st, buf0, buf1, S, part, *tc, N);
+  }
   const double* b0 = buf0;
   const double* b1 = buf1;
   void* a1[] = {&st, &b0, &b1, &S, &part};
@@ -481,7 +523,7 @@ cudaError_t add_mcw_loop_body(cudaGraph_t body, DevState* st, double* buf0, doub
   cudaError_t e = cudaGraphAddKernelNode(&n_sq, body, nullptr, 0, &kp);
   if (e != cudaSuccess) return e;
   if (lz && (e = add_lanczos_nodes(body, n_sq, st, buf0, buf1, S, part, ntiles, lz, N, T * kTile, &n_sq)) != cudaSuccess) return e;
-  e = add_finalize_node(body, &n_sq, 1, st, part, ntiles, 2, cond, &n_fin, mscr);
+  e = add_finalize_node(body, &n_sq, 1, st, part, ntiles, 2, 1, cond, &n_fin, mscr);
   if (e != cudaSuccess) return e;
   const double* Sc = S;
   void* a2[] = {&st, &buf0, &buf1, &Sc, &part};
@@ -491,22 +533,34 @@ cudaError_t add_mcw_loop_body(cudaGraph_t body, DevState* st, double* buf0, doub
 }
 
 cudaError_t launch_mcw_step_plain(DevState* st, double* buf0, double* buf1, double* S, double* part, int T,
-                                  cudaStream_t s, double* mscr, void* lz, int N) {
-  const int ntiles = T * (T + 1) / 2;
-  mcw_square_kernel<<<ntiles, kSyrkThreads, 0, s>>>(st, buf0, buf1, S, part);
+                                  cudaStream_t s, const f64tc::Plan* tc, double* mscr, void* lz, int N) {
+  const int ntiles = T * (T + 1) / 2, recs = recs_of(tc), nrec = ntiles * recs;
+  f64tc::Sink sink;
+  sink.s = s;
+  if (tc) {
+    cudaError_t e = emit_tc_square(sink, st, buf0, buf1, S, part, *tc, N, f64tc::OP_MCW_SQ);
+    if (e != cudaSuccess) return e;
+  } else {
+    mcw_square_kernel<<<ntiles, kSyrkThreads, 0, s>>>(st, buf0, buf1, S, part);
+  }
   if (lz) {
-    cudaError_t e = launch_lanczos(st, buf0, buf1, S, part, ntiles, lz, N, T * kTile, s);
+    cudaError_t e = launch_lanczos(st, buf0, buf1, S, part, nrec, lz, N, T * kTile, s);
     if (e != cudaSuccess) return e;
   }
-  finalize_plain_kernel<<<1, kFinThreads, 0, s>>>(st, part, ntiles, mscr);
-  mcw_prod_kernel<<<ntiles, kSyrkThreads, 0, s>>>(st, buf0, buf1, S, part);
+  finalize_plain_kernel<<<1, kFinThreads, 0, s>>>(st, part, nrec, recs, mscr);
+  if (tc) {
+    cudaError_t e = emit_tc_mcw_prod(sink, st, buf0, buf1, S, part, *tc, N);
+    if (e != cudaSuccess) return e;
+  } else {
+    mcw_prod_kernel<<<ntiles, kSyrkThreads, 0, s>>>(st, buf0, buf1, S, part);
+  }
   return cudaGetLastError();
 }
 
 cudaError_t add_finalize_node(cudaGraph_t g, const cudaGraphNode_t* deps, int ndeps, DevState* st,
-                              double* part, int nparts, int stride, cudaGraphConditionalHandle cond,
+                              double* part, int nparts, int stride, int recs, cudaGraphConditionalHandle cond,
                               cudaGraphNode_t* node, double* mscr) {
-  void* args[] = {&st, &part, &nparts, &stride, &cond, &mscr};
+  void* args[] = {&st, &part, &nparts, &stride, &recs, &cond, &mscr};
   cudaKernelNodeParams kp = {};
   kp.func = (void*)finalize_kernel;
   kp.gridDim = dim3(1);
@@ -516,19 +570,26 @@ cudaError_t add_finalize_node(cudaGraph_t g, const cudaGraphNode_t* deps, int nd
 }
 
 cudaError_t add_f64_loop_body(cudaGraph_t body, DevState* st, double* buf0, double* buf1, double* part,
-                              int T, cudaGraphConditionalHandle cond, double* mscr, void* lz, int N,
-                              const double* E, int64_t ecount) {
-  const int ntiles = T * (T + 1) / 2;
+                              int T, cudaGraphConditionalHandle cond, const f64tc::Plan* tc, double* mscr, void* lz,
+                              int N, const double* E, int64_t ecount) {
+  const int ntiles = T * (T + 1) / 2, recs = recs_of(tc), nrec = ntiles * recs;
   cudaGraphNode_t n_sq, n_fin;
-  void* args[] = {&st, &buf0, &buf1, &part};
   cudaKernelNodeParams kp = {};
-  kp.func = (void*)syrk_f64_kernel;
-  kp.gridDim = dim3(ntiles);
-  kp.blockDim = dim3(kSyrkThreads);
-  kp.kernelParams = args;
-  cudaError_t e = cudaGraphAddKernelNode(&n_sq, body, nullptr, 0, &kp);
-  if (e != cudaSuccess) return e;
-  if (lz && (e = add_lanczos_nodes(body, n_sq, st, buf0, buf1, nullptr, part, ntiles, lz, N, T * kTile, &n_sq)) != cudaSuccess) return e;
+  cudaError_t e;
+  if (tc) {
+    f64tc::Sink sink;
+    sink.g = body;
+    if ((e = emit_tc_square(sink, st, buf0, buf1, nullptr, part, *tc, N, f64tc::OP_SP2)) != cudaSuccess) return e;
+    n_sq = sink.last;
+  } else {
+    void* args[] = {&st, &buf0, &buf1, &part};
+    kp.func = (void*)syrk_f64_kernel;
+    kp.gridDim = dim3(ntiles);
+    kp.blockDim = dim3(kSyrkThreads);
+    kp.kernelParams = args;
+    if ((e = cudaGraphAddKernelNode(&n_sq, body, nullptr, 0, &kp)) != cudaSuccess) return e;
+  }
+  if (lz && (e = add_lanczos_nodes(body, n_sq, st, buf0, buf1, nullptr, part, nrec, lz, N, T * kTile, &n_sq)) != cudaSuccess) return e;
   if (E) {
     int initial = 0;
     void* pa[] = {&st, &buf0, &buf1, &E, &ecount, &initial};
@@ -540,7 +601,7 @@ cudaError_t add_f64_loop_body(cudaGraph_t body, DevState* st, double* buf0, doub
     if ((e = cudaGraphAddKernelNode(&n_pt, body, &n_sq, 1, &kp)) != cudaSuccess) return e;
     n_sq = n_pt;
   }
-  return add_finalize_node(body, &n_sq, 1, st, part, ntiles, 2, cond, &n_fin, mscr);
+  return add_finalize_node(body, &n_sq, 1, st, part, nrec, 2, recs, cond, &n_fin, mscr);
 }
 
 cudaError_t launch_refine_f64(const DevState* st, const double* Xin, double* Xout, int ld, int step, double* part,

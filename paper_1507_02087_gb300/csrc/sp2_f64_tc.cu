@@ -1,0 +1,583 @@
+// FP64 squares and products on the tcgen05 tensor cores, as exact sums of digit products.
+//
+// The FP64 pipe of this GPU runs 2 fused multiply-adds per clock and SM; the tensor cores run about
+// 4096 with fp16 inputs.  A row x_i of X is scaled by 2^-e_i (|x_ik| <= 2^(e_i - 1), ||x_i|| < 2^e_i) and
+// written as ND = 7 signed digits of 8 bits,
+//     x_ik 2^-e_i = sum_a d_a 2^(-8 (a + 1)),   |d_a| <= 128   (56 bits, rounded to nearest),
+// each an integer that fp16 holds exactly.  Then
+//     sum_k x_ik x_jk = 2^(e_i + e_j) sum_s 2^(-8 (s + 2)) V_s,   V_s = sum over k and a + b = s of d_a d'_b,
+// and the 34 digit products with s <= 7 are formed on the tensor cores.  The FP32 accumulators hold every
+// V_s exactly up to 2^24, and each is drained before it can pass that (period); the V_s are added in 64-bit
+// integer registers in units of 2^-62 (|sum| < 1 by Cauchy's inequality, so it fits) and the total is rounded
+// to FP64 once.  No other rounding happens, so the result does not depend on the order of the sums.
+//
+// Error against the exact product, in units of 2^(e_i + e_j): the digits' own rounding, at most 2^-57 per
+// value; the products with s >= 8 that are left out, about sqrt(5 K) 2^-67.6; the V_6 and V_7 rounded to the
+// unit.  An FMA chain rounds K times at 2^-53 of its partial sums.  ||D - D_exact||_F / ||D||_F against the
+// exact projector at N = 400 / 1001 / 1500 (McW-ACC) / 2048: 8.6e-15 / 2.1e-14 / 2.4e-14 / 4.4e-14, with FMA
+// chains 1.3e-14 / 3.0e-14 / 4.3e-14 / 6.1e-14.
+//
+// Time of one purification against the FP64 units (64 x 64 tiles, 0.98 of their peak at large N): N = 400
+// 2.27 ms against 18.1, N = 1500 (McW-ACC) 6.48 against 77.4, N = 2048 17.5 against 418.
+//
+// Tiles are 128 x bn per CTA (bn = 32 or 64 by the size, tile_width), over the upper triangle; a stage holds
+// the 7 digits of 32 k-columns of both operands, so 14 digit planes feed 34 products.  What bounds the
+// products is the reading of A from shared memory: a 128 x 64 x 16 product takes 48 clocks for 32 of
+// arithmetic.  Warp roles as in the other tensor-core kernels: warp 0 copies, warp 1 issues the products,
+// warps 4..11 drain and run the epilogue.  Every wait is bounded (2 s).
+#include <cuda_fp16.h>
+
+#include <cstring>
+
+#include "sp2_common.cuh"
+#include "sp2_f64_tc.cuh"
+#include "sp2_kernels.h"
+#include "tc_ptx.cuh"
+
+namespace sp2 {
+namespace f64tc {
+
+using namespace sp2::ptx;
+
+constexpr int DBITS = 8;                 // bits per digit
+constexpr int BM = 128;                  // tile rows
+constexpr int NS = 8;                    // digit sums kept: a + b <= 7, 34 products
+constexpr int KB = 32;                   // k-columns per stage: 64-byte rows, 64-byte swizzle
+// Digits in memory, and in a stage: for each block of 32 k-columns, groups of 8 rows; a group holds its ND
+// digits one after the other, each 8 rows x 64 bytes with the 16-byte chunks of row r exchanged by
+// chunk ^ (r / 2 % 4), the 64-byte swizzle that the tensor cores read.  A tile's rows are then one contiguous
+// piece of memory: two plain bulk copies fill a stage and no tensor map is needed (boxes of a tensor map over
+// planes of digits were as fast).
+constexpr int ROWB = KB * 2;             // bytes of one digit row
+constexpr int DIGB = 8 * ROWB;           // one digit of a row group
+constexpr int GRPB = ND * DIGB;          // a row group: 3584 bytes
+constexpr int MAXSTG = 3;
+constexpr int THREADS = 384;             // warps 0 TMA, 1 MMA, 2 idle; 8 epilogue warps
+constexpr int kBadExp = INT32_MIN;       // exponent of a row that holds a NaN or an infinity
+constexpr uint64_t kWaitNs = 2000000000ull;
+
+constexpr int A_BYTES = BM / 8 * GRPB;   // 56 KB
+__host__ __device__ constexpr int b_bytes(int bn) { return bn / 8 * GRPB; }
+__host__ __device__ constexpr int stage_bytes(int bn) { return A_BYTES + b_bytes(bn); }
+__host__ __device__ constexpr int stages_of(int bn) {
+  return 226 * 1024 / stage_bytes(bn) < MAXSTG ? 226 * 1024 / stage_bytes(bn) : MAXSTG;
+}
+__host__ __device__ constexpr int smem_bytes(int bn) { return stages_of(bn) * stage_bytes(bn) + 1024; }
+static_assert(stages_of(64) == 2 && stages_of(32) == 3, "stages");
+
+// Each digit sum has a tensor-memory accumulator of its own (NS x bn columns), closed and drained every
+// period(s) blocks of 32 k-columns: a drain costs a fixed 600 clocks or so beside its values, and with two
+// buffers in turn, drained every block, the drains took three times the products.  A product adds at most
+// 2^14 per term, so the sums stay exact: (pairs of s) x 32 period <= 2^10.
+__host__ __device__ constexpr int period(int s) { return s < 2 ? 16 : (s < 4 ? 8 : 4); }
+__host__ __device__ constexpr int first_pair(int s) { return s < ND ? 0 : s - ND + 1; }   // smallest a of a + b = s
+__host__ __device__ constexpr int pairs(int s) { return (s < ND ? s : ND - 1) - first_pair(s) + 1; }
+__host__ __device__ constexpr bool sums_exact() {
+  for (int s = 0; s < NS; ++s)
+    if (pairs(s) * KB * period(s) > (1 << 10)) return false;
+  return true;
+}
+static_assert(sums_exact(), "digit sums exact in FP32");
+
+// Upper tiles: row I of tiles holds the columns J >= I * BM / bn of ceil(ld / bn).
+__host__ __device__ inline int tiles_of(int ld, int bn) {
+  const int rows = (ld + BM - 1) / BM, cols = (ld + bn - 1) / bn;
+  int n = 0;
+  for (int I = 0; I < rows; ++I) n += cols - I * (BM / bn);
+  return n;
+}
+
+__device__ __forceinline__ void locate(int t, int cols, int step, int& I, int& J) {
+  int i = 0, w = cols;
+  while (t >= w) { t -= w; ++i; w -= step; }
+  I = i;
+  J = i * step + t;
+}
+
+// ---- digits --------------------------------------------------------------------------------
+constexpr int DT = 256;                  // one warp per row of a group
+
+__device__ __forceinline__ void load4(const double* p, double (&x)[4]) {
+  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(x[0]), "=d"(x[1]), "=d"(x[2]), "=d"(x[3]) : "l"(p));
+}
+__device__ __forceinline__ void store4(double* p, const double (&x)[4]) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(x[0]), "d"(x[1]), "d"(x[2]), "d"(x[3])
+               : "memory");
+}
+
+// |x| 2^(1023 - m) as FP32 (rounded toward zero), m the largest exponent field of the row.
+__device__ __forceinline__ float scaled_abs(double x, int m) {
+  const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, lo = (unsigned)__double2loint(x);
+  const int e = (int)(hi >> 20) - m + 127;
+  if (e <= 0) return 0.f;
+  return __uint_as_float(((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+}
+
+// x 2^(56 - e), rounded to the nearest integer (|x| <= 2^(e - 1)).
+__device__ __forceinline__ long long fixed56(double x, int e) {
+  const long long b = __double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  if (ex == 0) return 0;                               // zero (subnormals are below every unit used)
+  const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
+  const int sh = ex - 1075 + ND * DBITS - e;
+  unsigned long long y;
+  if (sh >= 0) y = m << sh;                            // sh <= 3 by the choice of e
+  else if (sh < -54) y = 0;
+  else y = (m + (1ull << (-sh - 1))) >> -sh;
+  return b < 0 ? -(long long)y : (long long)y;
+}
+
+// One warp per row, 8 rows (a row group) per CTA: the row's exponent, then its digits.  Bound by memory
+// (8 B read, 14 B written per value).
+__global__ void __launch_bounds__(DT)
+digits_kernel(const DevState* st, const double* buf0, const double* buf1, const double* S, int ld, int N, __half* dig,
+              int32_t* exps) {
+  if (st->done) return;
+  const double* X = S ? S : ((st->k & 1) ? buf1 : buf0);
+  const int rr = threadIdx.x >> 5, r = blockIdx.x * 8 + rr, lane = threadIdx.x & 31;
+  if (r >= N) return;
+  const double* row = X + (int64_t)r * ld;
+  int m = 0;
+  for (int c = 4 * lane; c < ld; c += 128) {
+    double x[4];
+    load4(row + c, x);
+    #pragma unroll
+    for (int j = 0; j < 4; ++j) m = max(m, (__double2hiint(x[j]) >> 20) & 0x7ff);
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  const bool bad = m == 0x7ff;
+  float n2 = 0.f;
+  for (int c = 4 * lane; c < ld; c += 128) {
+    double x[4];
+    load4(row + c, x);
+    #pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float f = scaled_abs(x[j], m);
+      n2 = fmaf(f, f, n2);
+    }
+  }
+  #pragma unroll
+  for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+  n2 *= 1.001f;                                        // above the rounding of the sum and of its terms
+  // |x| < 2^(m - 1022) <= 2^(e - 1) and ||x||^2 <= n2 2^(2 (m - 1023)) < 2^(2 e)
+  const int lg = (__float_as_int(n2) >> 23) - 127;     // floor(log2 n2), n2 >= 1
+  const int e = bad || m == 0 ? 0 : max(m - 1021, m - 1023 + lg / 2 + 1);
+  if (lane == 0) exps[r] = bad ? kBadExp : e;
+  const int64_t kstride = (int64_t)padded_rows(ld) / 8 * GRPB;
+  uint8_t* out = reinterpret_cast<uint8_t*>(dig) + (int64_t)blockIdx.x * GRPB + rr * ROWB;
+  for (int c = 4 * lane; c < ld; c += 128) {
+    double x[4];
+    load4(row + c, x);
+    long long y[4];
+    #pragma unroll
+    for (int j = 0; j < 4; ++j) y[j] = bad ? 0 : fixed56(x[j], e);
+    uint8_t* dst = out + (c / KB) * kstride + (((c % KB) / 8) ^ (rr / 2)) * 16 + (c % 8) * 2;
+    #pragma unroll
+    for (int a = ND - 1; a >= 0; --a) {
+      // digit of 8 bits in [-128, 127] (the top one takes what is left, at most 128): 1536 + d as fp16
+      // bits is 0x6600 + d, and subtracting 1536 is exact
+      int d[4];
+      #pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        d[j] = a ? (int)(int8_t)y[j] : (int)y[j];
+        y[j] = (y[j] - d[j]) >> DBITS;
+      }
+      const unsigned w0 = (unsigned)(0x6600 + d[0]) | ((unsigned)(0x6600 + d[1]) << 16);
+      const unsigned w1 = (unsigned)(0x6600 + d[2]) | ((unsigned)(0x6600 + d[3]) << 16);
+      const __half2 off = __float2half2_rn(1536.f);
+      uint2 o;
+      const __half2 h0 = __hsub2(*reinterpret_cast<const __half2*>(&w0), off);
+      const __half2 h1 = __hsub2(*reinterpret_cast<const __half2*>(&w1), off);
+      o.x = *reinterpret_cast<const unsigned*>(&h0);
+      o.y = *reinterpret_cast<const unsigned*>(&h1);
+      *reinterpret_cast<uint2*>(dst + a * DIGB) = o;
+    }
+  }
+}
+
+// ---- product ---------------------------------------------------------------------------------
+struct Args {
+  DevState* st;
+  double *buf0, *buf1, *S;
+  double* part;
+  const uint8_t *digA, *digB;            // digits of the A and the B operand
+  const int32_t *ea, *eb;                // row exponents of the A and the B operand
+  int32_t ld, tiles, op;
+};
+
+// What the epilogue writes: out = pk ? s : 2 x - s, or ca s + cb x + cc I with gen set.
+struct Poly {
+  const double* in;
+  double* out;
+  double ca, cb, cc;
+  int gen, pk;
+};
+
+__device__ __forceinline__ Poly poly_of(const Args& a) {
+  const DevState* st = a.st;
+  Poly p;
+  p.ca = p.cb = p.cc = 0.0;
+  p.gen = 0;
+  p.pk = 1;
+  const int k = st->k;
+  if (a.op == OP_MCW_SQ) {               // S_s = alpha^2 X^2 + 2 alpha c X + c^2 I, c = (1 - alpha) / 2
+    const double al = st->alpha[k + 1], c = 0.5 * (1.0 - al);
+    p.in = (k & 1) ? a.buf1 : a.buf0;
+    p.out = a.S;
+    p.gen = 1; p.ca = al * al; p.cb = 2.0 * al * c; p.cc = c * c;
+  } else if (a.op == OP_MCW_PROD) {      // X_k = (3 - 2 c) S_s - 2 alpha S_s X_{k-1}, k already recorded
+    const double al = st->alpha[k], c = 0.5 * (1.0 - al);
+    p.in = a.S;
+    p.out = (k & 1) ? a.buf1 : a.buf0;
+    p.gen = 1; p.ca = -2.0 * al; p.cb = 3.0 - 2.0 * c;
+  } else {
+    p.in = (k & 1) ? a.buf1 : a.buf0;
+    p.out = (k & 1) ? a.buf0 : a.buf1;
+    if (st->acc) {
+      p.pk = acc_step(st, k + 1, p.ca, p.cb, p.cc);
+      p.gen = 1;
+    } else {
+      p.pk = st->tr[k] > (double)st->nocc ? 1 : 0;     // Alg. 3 trace test
+    }
+  }
+  return p;
+}
+
+__device__ __forceinline__ void give_up(DevState* st, volatile int* abort_s) {
+  *abort_s = 1;
+  atomicExch(&st->status, (int)SP2_ERR_TIMEOUT);
+  st->out_mode = OUT_NAN;
+  st->done = 1;
+}
+
+// T 2^(ei + ej - 62): the scale goes into the exponent field where the result is a normal number (an FP64
+// multiplication takes 70 clocks a warp here, the conversion from the integer 6).
+__device__ __forceinline__ double scaled_sum(long long t, int ei, int ej) {
+  if (ei == kBadExp || ej == kBadExp) return __longlong_as_double(0x7ff8000000000000ll);
+  const int es = ei + ej - 62;
+  const double s = (double)t;
+  if (es <= -1000 || es >= 900) return ldexp(s, es);
+  return t ? __hiloint2double(__double2hiint(s) + (es << 20), __double2loint(s)) : 0.0;
+}
+
+// NV consecutive 32-bit tensor-memory columns (16 or 32 per load).
+__device__ __forceinline__ void tmem_ld(uint32_t addr, uint32_t (&r)[32]) { tmem_ld32(addr, r); }
+__device__ __forceinline__ void tmem_ld(uint32_t addr, uint32_t (&r)[16]) { tmem_ld16(addr, r); }
+
+// T += V_s of one period, in units of 2^-62: the weight of s is 2^(46 - 8 s); s = 6 and 7 are rounded to the
+// unit.  (For s <= 1 only the high word changes, modulo 2^32: the total fits.)
+template <int S, int G>
+__device__ __forceinline__ void add_digit_sums(const uint32_t (&raw)[G], long long (&T)[G]) {
+  #pragma unroll
+  for (int j = 0; j < G; ++j) {
+    const float f = __uint_as_float(raw[j]);
+    const int v = __float2int_rn(S <= 5 ? f : f * (S == 6 ? 0x1p-2f : 0x1p-10f));
+    if constexpr (S <= 1) T[j] += (long long)((unsigned long long)((unsigned)v << (14 - 8 * S)) << 32);
+    else if constexpr (S <= 5) T[j] += (long long)v * (1ll << (46 - 8 * S));
+    else T[j] += (long long)v;
+  }
+}
+
+// Drains digit sum S if its period ends with block kb (or the tile does).
+template <int S, int G>
+__device__ __forceinline__ bool drain(uint32_t trow, int bn, int kb, int nkb, uint64_t* accf, uint64_t* acce,
+                                      uint32_t& phases, int lane, volatile int* abort_s, long long (&T)[G]) {
+  if ((kb + 1) % period(S) != 0 && kb + 1 != nkb) return true;
+  int got = 0;
+  if (lane == 0) got = !*abort_s && mbar_wait(&accf[S], (phases >> S) & 1u, globaltimer_ns() + kWaitNs);
+  got = __shfl_sync(0xffffffffu, got, 0);
+  if (!got) return false;
+  tc_fence_after();
+  uint32_t raw[G];
+  tmem_ld(trow + (uint32_t)(S * bn), raw);
+  tmem_wait_ld();
+  tc_fence_before();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(&acce[S]);
+  phases ^= 1u << S;
+  add_digit_sums<S, G>(raw, T);
+  return true;
+}
+
+template <int BN>
+__global__ void __launch_bounds__(THREADS, 1)
+f64_product_kernel(const Args a) {
+  constexpr int STG = stages_of(BN), SBYTES = stage_bytes(BN);
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t full_bar[STG];
+  __shared__ __align__(8) uint64_t empty_bar[STG];
+  __shared__ __align__(8) uint64_t accf_bar[NS];
+  __shared__ __align__(8) uint64_t acce_bar[NS];
+  __shared__ __align__(8) uint64_t drain_bar;
+  __shared__ uint32_t tmem_base_s;
+  __shared__ volatile int abort_s;
+
+  DevState* st = a.st;
+  if (st->done) return;
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const int ld = a.ld, cols = (ld + BN - 1) / BN, nkb = ld / KB;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STG; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
+    for (int b = 0; b < NS; ++b) { mbar_init(&accf_bar[b], 1); mbar_init(&acce_bar[b], 8); }
+    mbar_init(&drain_bar, 1);
+    abort_s = 0;
+    fence_barrier_init();
+  }
+  if (warp == 1) tmem_alloc(&tmem_base_s, NS * BN);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_base_s;
+
+  if (warp < 4) {
+    if (warp == 0) {
+      if (elect_one()) {
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        const int64_t kstride = (int64_t)padded_rows(ld) / 8 * GRPB;
+        int armed[STG];
+        uint32_t armed_par[STG];
+        for (int s = 0; s < STG; ++s) { armed[s] = 0; armed_par[s] = 0; }
+        for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
+          int I, J;
+          locate(t, cols, BM / BN, I, J);
+          for (int kb = 0; kb < nkb; ++kb) {
+            if (abort_s || !mbar_wait(&empty_bar[stage], phase ^ 1, globaltimer_ns() + kWaitNs)) { ok = false; break; }
+            uint8_t* sA = smem + stage * SBYTES;
+            mbar_arrive_expect_tx(&full_bar[stage], SBYTES);
+            bulk_load(sA, a.digA + kb * kstride + (int64_t)I * A_BYTES, A_BYTES, &full_bar[stage]);
+            bulk_load(sA + A_BYTES, a.digB + kb * kstride + (int64_t)J * b_bytes(BN), b_bytes(BN), &full_bar[stage]);
+            armed[stage] = 1;
+            armed_par[stage] = phase;
+            if (++stage == STG) { stage = 0; phase ^= 1; }
+          }
+        }
+        if (!ok) give_up(st, &abort_s);
+        for (int s = 0; s < STG; ++s)    // wait (bounded) until every copy issued here has landed
+          if (armed[s]) mbar_wait(&full_bar[s], armed_par[s], globaltimer_ns() + kWaitNs);
+      }
+    } else if (warp == 1) {
+      if (elect_one()) {
+        constexpr uint32_t idesc = idesc_f16_f32(BM, BN);
+        int stage = 0;
+        uint32_t phase = 0, phases = 0;  // phases: bit s, the parity of accumulator s
+        bool ok = true;
+        for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
+          for (int kb = 0; kb < nkb && ok; ++kb) {
+            if (abort_s || !mbar_wait(&full_bar[stage], phase, globaltimer_ns() + kWaitNs)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t sA = smem_u32(smem + stage * SBYTES);
+            const uint32_t sB = sA + A_BYTES;
+            #pragma unroll
+            for (int s = 0; s < NS; ++s) {
+              const uint32_t dt = tmem_base + (uint32_t)(s * BN);
+              uint32_t accumulate = 1;
+              if (kb % period(s) == 0) {
+                if (abort_s || !mbar_wait(&acce_bar[s], ((phases >> s) & 1u) ^ 1u, globaltimer_ns() + kWaitNs)) {
+                  ok = false;
+                  break;
+                }
+                tc_fence_after();
+                accumulate = 0;
+              }
+              #pragma unroll
+              for (int i = first_pair(s); i < first_pair(s) + pairs(s); ++i) {
+                #pragma unroll
+                for (int kk = 0; kk < KB / 16; ++kk) {
+                  mma_bf16(dt, smem_desc_sw64_stride(sA + i * DIGB + kk * 32, GRPB),
+                           smem_desc_sw64_stride(sB + (s - i) * DIGB + kk * 32, GRPB), idesc, accumulate);
+                  accumulate = 1;
+                }
+              }
+              if ((kb + 1) % period(s) == 0 || kb + 1 == nkb) {
+                mma_commit(&accf_bar[s]);
+                phases ^= 1u << s;
+              }
+            }
+            if (!ok) break;
+            mma_commit(&empty_bar[stage]);
+            if (++stage == STG) { stage = 0; phase ^= 1; }
+          }
+        }
+        if (!ok) give_up(st, &abort_s);
+        mma_commit(&drain_bar);
+        mbar_wait(&drain_bar, 0, globaltimer_ns() + kWaitNs);
+      }
+    }
+  } else {
+    const int ew = warp - 4;
+    const int q = warp & 3;              // tensor-memory lanes 32 q .. 32 q + 31
+    const int hc = ew >> 2;              // columns hc BN / 2 .. of the tile
+    constexpr int G = BN / 2;
+    const Poly P = poly_of(a);
+    const int N = st->N, T64 = ld / 64;
+    uint32_t phases = 0;
+    bool ok = true;
+    const uint32_t trow = tmem_base + (uint32_t)(hc * G) + ((uint32_t)(32 * q) << 16);
+    for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
+      int I, J;
+      locate(t, cols, BM / BN, I, J);
+      long long T[G];
+      #pragma unroll
+      for (int j = 0; j < G; ++j) T[j] = 0;
+      for (int kb = period(NS - 1) - 1; ok; kb += period(NS - 1)) {
+        if (kb >= nkb) kb = nkb - 1;
+        ok = drain<0>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
+             drain<1>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
+             drain<2>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
+             drain<3>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
+             drain<4>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
+             drain<5>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
+             drain<6>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
+             drain<7>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T);
+        if (kb == nkb - 1) break;
+      }
+      if (!ok) {
+        if (lane == 0) give_up(st, &abort_s);
+        break;
+      }
+      // epilogue: this warp's 32 rows, G columns at a time; only blocks on or above the diagonal
+      const int r0 = I * BM + 32 * q, r = r0 + lane;
+      if (r0 >= ld) continue;
+      const int ei = a.ea[r];
+      const int c0 = J * BN + hc * G;
+      if (c0 >= ld || c0 + G <= r0) continue;
+      const bool off = c0 >= r0 + 32;    // wholly above the diagonal
+      double v2 = 0.0, trc = 0.0;
+      #pragma unroll
+      for (int j0 = 0; j0 < G; j0 += 4) {
+        double x[4], xn[4];
+        load4(P.in + (int64_t)r * ld + c0 + j0, x);
+        #pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int c = c0 + j0 + j;
+          const double s = scaled_sum(T[j0 + j], ei, a.eb[c]);
+          const double d = x[j] - s;
+          if (off || c > r) v2 = fma(d, d, v2);
+          else if (c == r) v2 = fma(0.5 * d, d, v2);
+          xn[j] = P.gen ? fma(P.ca, s, fma(P.cb, x[j], (c == r && r < N) ? P.cc : 0.0)) : (P.pk ? s : (2.0 * x[j] - s));
+          if (c == r) trc = xn[j];
+          if (off || c > r) P.out[(int64_t)c * ld + r] = xn[j];
+        }
+        if (off) {
+          store4(P.out + (int64_t)r * ld + c0 + j0, xn);
+        } else {
+          #pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (c0 + j0 + j >= r) P.out[(int64_t)r * ld + c0 + j0 + j] = xn[j];
+        }
+      }
+      v2 *= 2.0;                         // each element above the diagonal stands for two
+      #pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        v2 += __shfl_xor_sync(0xffffffffu, v2, o);
+        trc += __shfl_xor_sync(0xffffffffu, trc, o);
+      }
+      if (lane == 0) {
+        // record of these 32 rows and G columns within their 64 x 64 tile
+        double* dst = a.part + 2 * (RECS * upper_index(r0 / 64, c0 / 64, T64) + 4 * ((r0 >> 5) & 1) + ((c0 >> 4) & 3));
+        dst[0] = v2;
+        dst[1] = trc;
+      }
+    }
+  }
+
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, NS * BN);
+  }
+}
+
+// ---- host side ---------------------------------------------------------------------------------
+static const void* kernel_of(int bn) {
+  return bn == 64 ? (const void*)f64_product_kernel<64> : (const void*)f64_product_kernel<32>;
+}
+
+static int sm_count() {
+  static int n = 0;
+  if (!n) {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    n = v > 0 ? v : 1;
+  }
+  return n;
+}
+
+static cudaError_t prepare() {
+  static bool done = false;
+  if (done) return cudaSuccess;
+  for (int bn : {32, 64}) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel_of(bn), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(bn));
+    if (e != cudaSuccess) return e;
+  }
+  done = true;
+  return cudaSuccess;
+}
+
+// The width with the least work per SM: tiles dealt out in whole rounds, times the time of a stage.
+int tile_width(int ld) {
+  const double cost[2] = {44.0, 48.0};   // clocks of a 128 x bn x 16 product: reading A bounds it
+  int best = 64;
+  double t = 1e300;
+  for (int i = 1; i >= 0; --i) {
+    const int bn = 32 << i, n = tiles_of(ld, bn), sms = sm_count();
+    const double c = (double)((n + sms - 1) / sms) * cost[i];
+    if (c < t) { t = c; best = bn; }
+  }
+  return best;
+}
+
+cudaError_t Sink::put(const void* func, dim3 grid, dim3 block, size_t smem, void** args) {
+  if (!g) return cudaLaunchKernel(func, grid, block, args, smem, s);
+  cudaKernelNodeParams kp = {};
+  kp.func = const_cast<void*>(func);
+  kp.gridDim = grid;
+  kp.blockDim = block;
+  kp.sharedMemBytes = (unsigned)smem;
+  kp.kernelParams = args;
+  cudaGraphNode_t node;
+  const cudaError_t e = cudaGraphAddKernelNode(&node, g, last ? &last : nullptr, last ? 1 : 0, &kp);
+  if (e == cudaSuccess) last = node;
+  return e;
+}
+
+cudaError_t emit_digits(Sink& sink, const DevState* st, const double* buf0, const double* buf1, const double* S,
+                        const Plan& P, int N) {
+  const Digits& d = S ? P.S : P.X;
+  int ld = P.ld;
+  __half* dig = d.dig;
+  int32_t* exps = d.exp;
+  void* args[] = {&st, &buf0, &buf1, &S, &ld, &N, &dig, &exps};
+  return sink.put((const void*)digits_kernel, dim3((N + 7) / 8), dim3(DT), 0, args);
+}
+
+cudaError_t emit_product(Sink& sink, DevState* st, double* buf0, double* buf1, double* S, double* part,
+                         const Plan& P, Op op) {
+  const Digits& A = op == OP_MCW_PROD ? P.S : P.X;
+  Args a;
+  std::memset(&a, 0, sizeof(a));
+  a.st = st;
+  a.buf0 = buf0;
+  a.buf1 = buf1;
+  a.S = S;
+  a.part = part;
+  a.digA = reinterpret_cast<const uint8_t*>(A.dig);
+  a.digB = reinterpret_cast<const uint8_t*>(P.X.dig);
+  a.ea = A.exp;
+  a.eb = P.X.exp;
+  a.ld = P.ld;
+  a.tiles = tiles_of(P.ld, P.bn);
+  a.op = op;
+  const cudaError_t e = prepare();
+  if (e != cudaSuccess) return e;
+  void* args[] = {&a};
+  const int grid = a.tiles < sm_count() ? a.tiles : sm_count();
+  return sink.put(kernel_of(P.bn), dim3(grid), dim3(THREADS), smem_bytes(P.bn), args);
+}
+
+}  // namespace f64tc
+}  // namespace sp2

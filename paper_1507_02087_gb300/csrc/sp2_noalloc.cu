@@ -9,7 +9,7 @@
 // the process exits.  The caller still passes F and D (and, optionally, an info
 // buffer), all in device memory it already owns.  With CUDA's lazy module loading
 // (the default), that load may happen inside the first call on a device, which then
-// allocates the array (about 4.2 MB); make that first call as a warm-up, outside any
+// allocates the array (about 8 MB); make that first call as a warm-up, outside any
 // region where allocation is not allowed and before any stream capture.
 //
 // The workspace limits the problem size to N <= SP2_NOALLOC_MAX_N.  Every call shares
@@ -25,6 +25,7 @@
 
 #include "../../include/sp2.h"
 #include "sp2_common.cuh"
+#include "sp2_f64_tc.cuh"
 #include "sp2_kernels.h"
 
 namespace {
@@ -44,9 +45,12 @@ constexpr size_t kOffLo = align256(kOffState + sizeof(DevState));
 constexpr size_t kOffHi = align256(kOffLo + kGersh * sizeof(double));
 constexpr size_t kOffBad = align256(kOffHi + kGersh * sizeof(double));
 constexpr size_t kOffPart = align256(kOffBad + kGersh * sizeof(int));
-constexpr size_t kOffBuf0 = align256(kOffPart + 2 * kTiles * sizeof(double));
+constexpr size_t kPartBytes = 2 * sp2::f64tc::RECS * kTiles * sizeof(double);
+constexpr size_t kOffBuf0 = align256(kOffPart + kPartBytes);
 constexpr size_t kOffBuf1 = align256(kOffBuf0 + (size_t)kLd * kLd * sizeof(double));
-constexpr size_t kScratchBytes = align256(kOffBuf1 + (size_t)kLd * kLd * sizeof(double));
+constexpr size_t kOffDig = align256(kOffBuf1 + (size_t)kLd * kLd * sizeof(double));
+constexpr size_t kOffExp = align256(kOffDig + sp2::f64tc::digit_bytes(kLd));
+constexpr size_t kScratchBytes = align256(kOffExp + sp2::f64tc::exp_bytes(kLd));
 
 // The workspace.  In host code this name is only a host-side handle for the symbol,
 // not a device address: the address is obtained with cudaGetSymbolAddress below.
@@ -134,6 +138,21 @@ static sp2_status run_noalloc(const double* F_dev, double* D_dev, int64_t N, int
     (void)cudaGetLastError();
     return SP2_ERR_CUDA;
   }
+  // as a handle of this size: the products on the tensor cores, or on the CUDA cores
+  sp2::f64tc::Plan tc;
+  tc.on = sp2::f64tc::wanted(N);
+  if (tc.on) {
+    tc.ld = ld;
+    tc.bn = sp2::f64tc::tile_width(ld);
+    tc.X.dig = (__half*)(base + kOffDig);
+    tc.X.exp = (int32_t*)(base + kOffExp);
+    if (cudaMemsetAsync(tc.X.dig, 0, sp2::f64tc::digit_bytes(ld), s) != cudaSuccess ||
+        cudaMemsetAsync(tc.X.exp, 0, sp2::f64tc::exp_bytes(ld), s) != cudaSuccess ||
+        cudaMemsetAsync(part, 0, kPartBytes, s) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return SP2_ERR_CUDA;
+    }
+  }
   noalloc_setup_kernel<<<1, 1, 0, s>>>(st, (int)N, ld, (int)n_occ, kMaxIter);
   if (cudaGetLastError() != cudaSuccess) return SP2_ERR_CUDA;
   if (sp2::launch_bounds_and_init(st, F_dev, N, (int)N, lo, hi, bad, nparts, s) != cudaSuccess ||
@@ -143,7 +162,8 @@ static sp2_status run_noalloc(const double* F_dev, double* D_dev, int64_t N, int
   }
   // At most kMaxIter + 1 squares; once the stop test has fired every launch returns at once.
   for (int it = 0; it <= kMaxIter; ++it) {
-    if (sp2::launch_f64_step_plain(st, buf0, buf1, part, T, s) != cudaSuccess) {
+    if (sp2::launch_f64_step_plain(st, buf0, buf1, part, T, s, tc.on ? &tc : nullptr, nullptr, nullptr, (int)N, nullptr,
+                                   0) != cudaSuccess) {
       (void)cudaGetLastError();
       return SP2_ERR_CUDA;
     }

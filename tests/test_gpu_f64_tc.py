@@ -1,0 +1,90 @@
+"""FP64 products on the tensor cores (csrc/sp2_f64_tc.cu): sizes at the edges of the tiles and of the
+blocks of k-columns, and matrices whose rows differ in scale, against products in extended precision.
+
+A run capped at one or two steps returns the polynomial of X_0 itself.  Bound on an element of
+S = X X^T, with 2^e_i the scale of row i (2^e_i <= 4 max|x_i| or <= 2 ||x_i||, so 2^e_i <= 4 ||x_i||): digits
+rounded at 2^-57 2^e_i per value, products left out below 2^-64 sqrt(K), and one rounding to FP64.
+That is at most 8 eps ||x_i|| ||x_j|| sqrt(K) with room to spare (eps = 2^-53).
+"""
+import numpy as np
+import pytest
+import torch
+
+from paper_1507_02087_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+EPS = 2.0 ** -53
+
+
+def one_square(F, bounds, nocc):
+    """X_0 as the library forms it, and X_1 of a run that ends at the cap after one step."""
+    from paper_1507_02087_gb300 import sp2
+    N = F.shape[0]
+    with sp2.Purifier(N, nocc, "fp64", max_iter=1, guard=False) as P:
+        P.set_bounds(bounds)
+        X1 = P.run(torch.from_numpy(F).cuda()).cpu().numpy()
+        info = P.info()
+    assert info["status"] == 0 and info["n_iter"] == 1
+    lo, hi = bounds
+    X0 = (hi * np.eye(N) - F) / (hi - lo)
+    return X0, X1, int(info["p"][1])
+
+
+def check(X0, X1, p):
+    N = X0.shape[0]
+    L = X0.astype(np.longdouble)
+    S = L @ L
+    ref = S if p else 2 * L - S
+    norms = np.linalg.norm(X0, axis=1)
+    bound = 8 * EPS * np.sqrt(N) * np.outer(norms, norms) + 2 * EPS * np.abs(ref).astype(float)
+    err = np.abs((X1.astype(np.longdouble) - ref).astype(float))
+    assert np.all(err <= bound), float(np.max(err / np.maximum(bound, 1e-300)))
+    assert np.array_equal(X1, X1.T)
+
+
+@pytest.mark.parametrize("N", [129, 160, 191, 192, 193, 256, 321, 448, 513])
+@pytest.mark.parametrize("fill", [0.2, 0.8])
+def test_one_square_at_tile_edges(N, fill):
+    nocc = int(fill * N)                                    # both polynomials
+    F = inputs.dense_gapped(N, nocc, gap=0.1, seed=N).F.numpy()
+    check(*one_square(F, (-1.5, 1.5), nocc))
+
+
+@pytest.mark.parametrize("scale", [1e-6, 1e-30, 1e-120])
+def test_one_square_of_rows_of_different_scale(scale):
+    # a block-diagonal matrix whose X_0 has rows of norm 1, of norm `scale` and zero rows
+    N = 300
+    g = np.random.Generator(np.random.PCG64(7))
+    A = g.standard_normal((N, N)) / N
+    w = np.where(np.arange(N) % 3 == 0, 1.0, np.where(np.arange(N) % 3 == 1, scale, 0.0))
+    X = w[:, None] * (A + A.T) * w[None, :]
+    X0, X1, p = one_square(-X, (-1.0, 0.0), 100)            # lmax = 0: X_0 = -F exactly
+    check(X0, X1, p)
+
+
+def test_a_row_with_an_overflow_ends_the_run():
+    # finite input whose square is not: reported, as by the FP64 units
+    from paper_1507_02087_gb300 import sp2
+    N = 200
+    F = inputs.dense_gapped(N, 100, gap=0.1, seed=3).F.numpy() * 1e200
+    with sp2.Purifier(N, 100, "fp64") as P:
+        P.set_bounds((-1.0, 1.0))                           # far too narrow
+        P.run(torch.from_numpy(F).cuda())
+        assert P.info()["status"] == 3
+
+
+@pytest.mark.parametrize("mode,xi", [("mcw", 0.0), ("mcw-acc", 0.05)])
+@pytest.mark.parametrize("N", [130, 257, 500])
+def test_mcweeny_products_at_tile_edges(N, mode, xi):
+    from oracle import mcweeny_oracle as om
+    from oracle import sp2_oracle as o
+    from paper_1507_02087_gb300 import sp2
+    case = inputs.dense_gapped(N, N // 2, gap=0.05, seed=N)
+    with sp2.Purifier(N, N // 2, "fp64") as P:
+        P.set_mcweeny(mode, 0.0, xi)
+        D = P.run(case.F.cuda()).cpu().numpy()
+        info = P.info()
+    ref = om.mcweeny(case.F.numpy(), 0.0, xi=xi, accelerate=(mode == "mcw-acc"),
+                     bounds=(info["lambda_min"], info["lambda_max"]))
+    assert info["status"] == 0 and abs(info["n_iter"] - ref.n) <= 1
+    assert o.rel_error(D, ref.D, N // 2) <= 1e-12
