@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
   DevState* st = a.st;
   if (!st->iter_active) return;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int ntiles = *a.r.tnnz;
   const Mat& X = a.X;
   const int nb = a.nb, W = a.W;
@@ -172,15 +172,15 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
     } else if (warp == 1) {
       // ---------------- MMA issuer ----------------
       constexpr uint32_t idesc = idesc_f16_f32(TTR * B, TN);
-      int stage = 0, buf = 0;
-      uint32_t phase = 0, bphase = 0;
-      bool ok = true;
-      unsigned long long kblocks = 0ull, needed = 0ull;
-      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        const int nk = a.r.meta[(int64_t)t * TMETA];
-        kblocks += (unsigned long long)nk;
-        needed += (unsigned long long)a.r.meta[(int64_t)t * TMETA + 65];
-        if (lane == 0) {
+      if (elect_one()) {
+        int stage = 0, buf = 0;
+        uint32_t phase = 0, bphase = 0;
+        bool ok = true;
+        unsigned long long kblocks = 0ull, needed = 0ull;
+        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+          const int nk = a.r.meta[(int64_t)t * TMETA];
+          kblocks += (unsigned long long)nk;
+          needed += (unsigned long long)a.r.meta[(int64_t)t * TMETA + 65];
           for (int k0 = 0; k0 < nk && ok; k0 += TCHK) {
             if (abort_s || !mbar_wait(&acce_bar[buf], bphase ^ 1, globaltimer_ns() + kTcWaitNs)) { ok = false; break; }
             tc_fence_after();
@@ -212,9 +212,6 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
             if (++buf == 2) { buf = 0; bphase ^= 1; }
           }
         }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      }
-      if (lane == 0) {
         // executed 32 x 32 x 32 block products: the tile's 32 block pairs times its K blocks
         atomicAdd(&st->bprod, kblocks * (unsigned long long)(TTR * TTC));
         atomicAdd(&st->uprod, needed);   // the tiles' needed products (tile metadata)
