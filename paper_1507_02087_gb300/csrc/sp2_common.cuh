@@ -111,12 +111,26 @@ __host__ __device__ __forceinline__ bool corrects_run(const DevState* st) {
   return st->status == SP2_OK && st->out_mode == OUT_COPY && st->reason != SP2_STOP_CAP;
 }
 
+// log2 of a positive normal number in FP32 arithmetic (NaN for anything else).
+__device__ __forceinline__ float log2_rough(double x) {
+  const int hi = __double2hiint(x);
+  const int ex = hi >> 20;                       // sign and exponent field
+  if (ex < 1 || ex >= 0x7ff) return __int_as_float(0x7fc00000);
+  const float m = __uint_as_float(0x3f800000u | ((unsigned)(hi & 0xfffff) << 3) | ((unsigned)__double2loint(x) >> 29));
+  return (float)(ex - 1023) + log2f(m);
+}
+
 // The paper's convergence-order test (Alg. 3; §2 relaxed order qtilde), only
 // evaluated when v_{i-2} < 1, and in its logarithmic form.
 __device__ __forceinline__ bool order_test_stops(double v_i, double v_im2, double qtilde, double C = kC2sp) {
   if (v_im2 == 0.0) return true;
   if (!(v_im2 < 1.0)) return false;
   if (v_i == 0.0) return false;
+  // For 0 < v_im2 < 1 this is log2(v_i / C) > qtilde log2(v_im2).  FP64 logarithms take several
+  // microseconds on one thread, so FP32 ones decide wherever they leave no doubt: each is within 2^-20 of
+  // its value (relative to max(1, |log2|), below 1100), far below the margin.
+  const double m = log2_rough(v_i) - (double)log2f((float)C) - qtilde * (double)log2_rough(v_im2);
+  if (isfinite(m) && fabs(m) > 0.01 * fmax(1.0, qtilde)) return m > 0.0;
   return log(v_i / C) / log(v_im2) < qtilde;
 }
 
@@ -301,6 +315,55 @@ __device__ __forceinline__ double block_sum(double x, double* smem) {
   return t;
 }
 
+// Three such sums at once, of values that only the first n threads hold (the others hold +0): the same
+// shuffle tree and order of warps, so the same bits, but the warps past n are left out and the three
+// serial sums run side by side (an FP64 addition waits about 70 clocks for the one before).  smem: 96 doubles.
+template <int NT>
+__device__ __forceinline__ void block_sum3(double& a, double& b, double& c, int n, double* smem) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nw = n >= NT ? NT / 32 : (n + 31) / 32;
+  if (warp < nw) {
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      b += __shfl_xor_sync(0xffffffffu, b, o);
+      c += __shfl_xor_sync(0xffffffffu, c, o);
+    }
+    if (lane == 0) { smem[warp] = a; smem[32 + warp] = b; smem[64 + warp] = c; }
+  }
+  __syncthreads();
+  if (warp < 3 && lane == 0) {
+    double t = 0.0;
+    for (int w = 0; w < nw; ++w) t += smem[32 * warp + w];
+    smem[32 * warp] = t;
+  }
+  __syncthreads();
+  a = smem[0];
+  b = smem[32];
+  c = smem[64];
+  __syncthreads();
+}
+
+// Brings the lines of the state that record_and_test reads next (the header, and the histories around
+// square k + 1) into this SM's L1, one line per thread, so that the single thread that runs the test does not
+// wait for them one after the other.
+__device__ __forceinline__ void touch_state(const DevState* st, int k) {
+  const char* p = nullptr;
+  const int i = threadIdx.x;
+  if (i < 4) p = reinterpret_cast<const char*>(st) + 128 * i;
+  else if (i == 4) p = reinterpret_cast<const char*>(&st->v[k < 2 ? 0 : k - 2]);
+  else if (i == 5) p = reinterpret_cast<const char*>(&st->v[k]);
+  else if (i == 6) p = reinterpret_cast<const char*>(&st->tr[k]);
+  else if (i == 7) p = reinterpret_cast<const char*>(&st->p[k]);
+  else if (i == 8) p = reinterpret_cast<const char*>(&st->alpha[k + 1]);
+  else if (i == 9) p = reinterpret_cast<const char*>(&st->psched[k + 1]);
+  else if (i == 10) p = reinterpret_cast<const char*>(&st->mcw);
+  if (p) {
+    int v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(reinterpret_cast<uintptr_t>(p) & ~uintptr_t(3)));
+  }
+}
+
 // Index of upper tile (I, J), I <= J, in a T x T grid whose upper tiles are numbered by rows.
 __host__ __device__ __forceinline__ int64_t upper_index(int I, int J, int T) {
   return (int64_t)I * T - (int64_t)I * (I - 1) / 2 + (J - I);
@@ -310,7 +373,7 @@ __host__ __device__ __forceinline__ int64_t upper_index(int I, int J, int T) {
 // `block_n2(I, J)` = ||block (I, J)||_F^2 for I <= J (the matrix is symmetric).  One CTA of
 // NT threads: the matrix goes to `scr` (nb^2 doubles, then two vectors of nb), and its
 // largest eigenvalue comes from kMixedIters power steps from the all-ones vector, the last
-// one as a Rayleigh quotient; every sum in a fixed order.
+// one as a Rayleigh quotient; every sum in a fixed order.  `sm`: 96 doubles.
 constexpr int kMixedIters = 200;
 
 template <int NT, class BlockN2>
@@ -332,19 +395,23 @@ __device__ double mixed_norm_cta(int nb, double* scr, double* sm, BlockN2 block_
       for (int j = 0; j < nb; ++j) acc += M[(int64_t)i * nb + j] * x[j];
       y[i] = acc;
     }
-    __syncthreads();
-    double ss = 0.0, xy = 0.0;
+    double ss = 0.0, xy = 0.0, none = 0.0;
     for (int i = tid; i < nb; i += NT) {
       ss += y[i] * y[i];
       xy += x[i] * y[i];
     }
-    ss = block_sum<NT>(ss, sm);
-    xy = block_sum<NT>(xy, sm);
+    block_sum3<NT>(ss, xy, none, nb, sm);
     lam = xy;                                  // x has unit norm: Rayleigh quotient
     if (!(ss > 0.0)) { lam = 0.0; break; }
     const double inv = 1.0 / sqrt(ss);
-    for (int i = tid; i < nb; i += NT) x[i] = y[i] * inv;
-    __syncthreads();
+    bool same = true;
+    for (int i = tid; i < nb; i += NT) {
+      const double xn = y[i] * inv;
+      same = same && xn == x[i];
+      x[i] = xn;
+    }
+    // a fixed point: every further step would give the same vector and quotient
+    if (__syncthreads_and(same)) break;
   }
   return lam;
 }

@@ -305,20 +305,19 @@ constexpr int kFinThreads = 1024;
 __global__ void __launch_bounds__(kFinThreads)
 finalize_kernel(DevState* st, const double* __restrict__ part, int nparts, int stride, int recs,
                 cudaGraphConditionalHandle cond, double* mscr) {
-  __shared__ double sm[32];
+  __shared__ double sm[96];
   if (st->done) {
     if (threadIdx.x == 0) cudaGraphSetConditional(cond, 0);
     return;
   }
+  touch_state(st, st->k);
   double a = 0.0, b = 0.0, c = 0.0;
   for (int t = threadIdx.x; t < nparts; t += kFinThreads) {
     a += part[(int64_t)stride * t];
     b += part[(int64_t)stride * t + 1];
     if (stride > 2) c += part[(int64_t)stride * t + 2];
   }
-  a = block_sum<kFinThreads>(a, sm);
-  b = block_sum<kFinThreads>(b, sm);
-  c = block_sum<kFinThreads>(c, sm);
+  block_sum3<kFinThreads>(a, b, c, nparts, sm);
   double vk = sqrt(a);                           // v_{k-1} = ||X_{k-1} - X_{k-1}^2||_F
   if (st->norm == 2) vk = st->spec_e;            // or e_{k-1}, the Lanczos estimate of the 2-norm
   if (st->norm == 1 && mscr) {                   // or m_{k-1}, the mixed norm over 64 x 64 tiles
@@ -369,15 +368,15 @@ __global__ void copy_out_kernel(const DevState* st, const double* __restrict__ b
 // the same rules as finalize_kernel (stride 2), ending the loop through st->done only.
 __global__ void __launch_bounds__(kFinThreads)
 finalize_plain_kernel(DevState* st, const double* __restrict__ part, int nparts, int recs, double* mscr) {
-  __shared__ double sm[32];
+  __shared__ double sm[96];
   if (st->done) return;
-  double a = 0.0, b = 0.0;
+  touch_state(st, st->k);
+  double a = 0.0, b = 0.0, c = 0.0;
   for (int t = threadIdx.x; t < nparts; t += kFinThreads) {
     a += part[2 * (int64_t)t];
     b += part[2 * (int64_t)t + 1];
   }
-  a = block_sum<kFinThreads>(a, sm);
-  b = block_sum<kFinThreads>(b, sm);
+  block_sum3<kFinThreads>(a, b, c, nparts, sm);
   double vk = sqrt(a);
   if (st->norm == 2) vk = st->spec_e;
   if (st->norm == 1 && mscr) {

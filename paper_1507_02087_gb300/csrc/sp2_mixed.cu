@@ -171,12 +171,13 @@ constexpr int kFT = 1024;
 // 2 Tr[X_{k-1}] - ||X_{k-1}||_F^2 after 2X - X^2, so the polynomial choice does not
 // inherit the bias of the tensor cores' accumulation.
 __global__ void __launch_bounds__(kFT) batch_finalize_kernel(const Instance* inst, int count) {
-  __shared__ double sm[32];
+  __shared__ double sm[96];
   const int i = blockIdx.x;
   if (i >= count) return;
   const Instance& In = inst[i];
   DevState* st = In.st;
   if (st->done) return;
+  touch_state(st, st->k);
   const int nparts = In.nparts;
   double a = 0.0, b = 0.0, c = 0.0;
   for (int t = threadIdx.x; t < nparts; t += kFT) {
@@ -184,9 +185,7 @@ __global__ void __launch_bounds__(kFT) batch_finalize_kernel(const Instance* ins
     b += In.part[4 * (int64_t)t + 1];
     c += In.part[4 * (int64_t)t + 2];
   }
-  a = block_sum<kFT>(a, sm);
-  b = block_sum<kFT>(b, sm);
-  c = block_sum<kFT>(c, sm);
+  block_sum3<kFT>(a, b, c, nparts, sm);
   double vk = sqrt(a);
   if (st->norm == 2) vk = st->spec_e;   // e_{k-1}, the Lanczos estimate of the 2-norm (one problem)
   if (st->norm == 1 && In.mscr) {
