@@ -239,65 +239,87 @@ __device__ __forceinline__ int locate(const Job& job, int t, int& I, int& J) {
   return i;
 }
 
-// 8 consecutive values (16-byte aligned) from / to the planes of a slot.
+// 16 consecutive values of a row (32-byte aligned) as they lie in the planes of a slot: W words of 32 bytes
+// per plane.  A thread of the epilogue owns a row, so a warp's access touches 32 rows whatever its width; 32
+// bytes fill the sector.
 template <int FMT>
-__device__ __forceinline__ void load8(const __nv_bfloat16* slot, int64_t plane, int64_t off, float (&x)[8]) {
-  if constexpr (FMT == FMT_TF32X2) {   // 32-byte aligned: off is a multiple of 8 values
-    const float4* hi = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(slot) + off);
-    const float4* lo = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(slot) + plane + off);
-    const float4 h0 = hi[0], h1 = hi[1], l0 = lo[0], l1 = lo[1];
-    x[0] = h0.x + l0.x; x[1] = h0.y + l0.y; x[2] = h0.z + l0.z; x[3] = h0.w + l0.w;
-    x[4] = h1.x + l1.x; x[5] = h1.y + l1.y; x[6] = h1.z + l1.z; x[7] = h1.w + l1.w;
-  } else if constexpr (FMT == FMT_FP16X2) {
-    const uint4 a = *reinterpret_cast<const uint4*>(slot + off);
-    const uint4 b = *reinterpret_cast<const uint4*>(slot + plane + off);
-    const __half* pa = reinterpret_cast<const __half*>(&a);
-    const __half* pb = reinterpret_cast<const __half*>(&b);
+struct Row16 {
+  static constexpr int W = FMT == FMT_TF32X2 ? 2 : 1;
+  uint32_t v[np_of(FMT)][W][8];
+};
+
+template <int FMT>
+__device__ __forceinline__ void load_row16(const __nv_bfloat16* slot, int64_t plane, int64_t off, Row16<FMT>& x) {
+  const char* p = reinterpret_cast<const char*>(slot) + off * esize_of(FMT);
+  #pragma unroll
+  for (int a = 0; a < np_of(FMT); ++a)
     #pragma unroll
-    for (int e = 0; e < 8; ++e) x[e] = (__half2float(pa[e]) + __half2float(pb[e])) * kF16InvScale;
-  } else {
-    const uint4 a = *reinterpret_cast<const uint4*>(slot + off);
-    const uint4 b = *reinterpret_cast<const uint4*>(slot + plane + off);
-    const uint4 c = *reinterpret_cast<const uint4*>(slot + 2 * plane + off);
-    const __nv_bfloat16* pa = reinterpret_cast<const __nv_bfloat16*>(&a);
-    const __nv_bfloat16* pb = reinterpret_cast<const __nv_bfloat16*>(&b);
-    const __nv_bfloat16* pc = reinterpret_cast<const __nv_bfloat16*>(&c);
-    #pragma unroll
-    for (int e = 0; e < 8; ++e)
-      x[e] = (__bfloat162float(pa[e]) + __bfloat162float(pb[e])) + __bfloat162float(pc[e]);
-  }
+    for (int w = 0; w < Row16<FMT>::W; ++w) ldg32(p + a * plane * esize_of(FMT) + 32 * w, x.v[a][w]);
 }
 
 template <int FMT>
-__device__ __forceinline__ void store8(__nv_bfloat16* slot, int64_t plane, int64_t off, const float (&x)[8]) {
+__device__ __forceinline__ void store_row16(__nv_bfloat16* slot, int64_t plane, int64_t off, const Row16<FMT>& x) {
+  char* p = reinterpret_cast<char*>(slot) + off * esize_of(FMT);
+  #pragma unroll
+  for (int a = 0; a < np_of(FMT); ++a)
+    #pragma unroll
+    for (int w = 0; w < Row16<FMT>::W; ++w) stg32(p + a * plane * esize_of(FMT) + 32 * w, x.v[a][w]);
+}
+
+// Value e (0..15).
+template <int FMT>
+__device__ __forceinline__ float value_of(const Row16<FMT>& row, int e) {
   if constexpr (FMT == FMT_TF32X2) {
-    float h[8], l[8];
-    #pragma unroll
-    for (int e = 0; e < 8; ++e) split_tf32x2(x[e], h[e], l[e]);
-    float4* hi = reinterpret_cast<float4*>(reinterpret_cast<float*>(slot) + off);
-    float4* lo = reinterpret_cast<float4*>(reinterpret_cast<float*>(slot) + plane + off);
-    hi[0] = make_float4(h[0], h[1], h[2], h[3]);
-    hi[1] = make_float4(h[4], h[5], h[6], h[7]);
-    lo[0] = make_float4(l[0], l[1], l[2], l[3]);
-    lo[1] = make_float4(l[4], l[5], l[6], l[7]);
-  } else if constexpr (FMT == FMT_FP16X2) {
-    uint4 a, b;
-    __half* pa = reinterpret_cast<__half*>(&a);
-    __half* pb = reinterpret_cast<__half*>(&b);
-    #pragma unroll
-    for (int e = 0; e < 8; ++e) split_fp16x2(x[e], pa[e], pb[e]);
-    *reinterpret_cast<uint4*>(slot + off) = a;
-    *reinterpret_cast<uint4*>(slot + plane + off) = b;
+    return __uint_as_float(row.v[0][e >> 3][e & 7]) + __uint_as_float(row.v[1][e >> 3][e & 7]);
   } else {
-    uint4 a, b, c;
-    __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(&a);
-    __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(&b);
-    __nv_bfloat16* pc = reinterpret_cast<__nv_bfloat16*>(&c);
+    const int i = e >> 1, sh = 16 * (e & 1);
+    const unsigned short u0 = (unsigned short)(row.v[0][0][i] >> sh), u1 = (unsigned short)(row.v[1][0][i] >> sh);
+    if constexpr (FMT == FMT_FP16X2) {
+      return (__half2float(__ushort_as_half(u0)) + __half2float(__ushort_as_half(u1))) * kF16InvScale;
+    } else {
+      const unsigned short u2 = (unsigned short)(row.v[2][0][i] >> sh);
+      return (__bfloat162float(__ushort_as_bfloat16(u0)) + __bfloat162float(__ushort_as_bfloat16(u1))) +
+             __bfloat162float(__ushort_as_bfloat16(u2));
+    }
+  }
+}
+
+// Values e and e + 1 (e even) as pieces.
+template <int FMT>
+__device__ __forceinline__ void set_values(Row16<FMT>& row, int e, float x0, float x1) {
+  if constexpr (FMT == FMT_TF32X2) {
+    float h0, l0, h1, l1;
+    split_tf32x2(x0, h0, l0);
+    split_tf32x2(x1, h1, l1);
+    row.v[0][e >> 3][e & 7] = __float_as_uint(h0);
+    row.v[1][e >> 3][e & 7] = __float_as_uint(l0);
+    row.v[0][e >> 3][(e & 7) + 1] = __float_as_uint(h1);
+    row.v[1][e >> 3][(e & 7) + 1] = __float_as_uint(l1);
+  } else if constexpr (FMT == FMT_FP16X2) {
+    __half a0, a1, b0, b1;
+    split_fp16x2(x0, a0, a1);
+    split_fp16x2(x1, b0, b1);
+    row.v[0][0][e >> 1] = __half_as_ushort(a0) | ((uint32_t)__half_as_ushort(b0) << 16);
+    row.v[1][0][e >> 1] = __half_as_ushort(a1) | ((uint32_t)__half_as_ushort(b1) << 16);
+  } else {
+    __nv_bfloat16 a[3], b[3];
+    split_bf16x3(x0, a[0], a[1], a[2]);
+    split_bf16x3(x1, b[0], b[1], b[2]);
     #pragma unroll
-    for (int e = 0; e < 8; ++e) split_bf16x3(x[e], pa[e], pb[e], pc[e]);
-    *reinterpret_cast<uint4*>(slot + off) = a;
-    *reinterpret_cast<uint4*>(slot + plane + off) = b;
-    *reinterpret_cast<uint4*>(slot + 2 * plane + off) = c;
+    for (int p = 0; p < 3; ++p)
+      row.v[p][0][e >> 1] = __bfloat16_as_ushort(a[p]) | ((uint32_t)__bfloat16_as_ushort(b[p]) << 16);
+  }
+}
+
+// The pieces of value e into the planes at `off`.
+template <int FMT>
+__device__ __forceinline__ void store_value(__nv_bfloat16* slot, int64_t plane, int64_t off, const Row16<FMT>& row, int e) {
+  #pragma unroll
+  for (int p = 0; p < np_of(FMT); ++p) {
+    if constexpr (FMT == FMT_TF32X2)
+      reinterpret_cast<uint32_t*>(slot)[p * plane + off] = row.v[p][e >> 3][e & 7];
+    else
+      reinterpret_cast<unsigned short*>(slot)[p * plane + off] = (unsigned short)(row.v[p][0][e >> 1] >> (16 * (e & 1)));
   }
 }
 
@@ -307,97 +329,105 @@ struct Partials {
   double trd;   // sum of the diagonal x
 };
 
-// Epilogue for row r, columns c0 .. c0+31 of the tile, with the accumulated product s
-// (FMT_FP16X2: S^2 times the product, removed here); worked in groups of 8 columns (one
-// 16-byte access per plane).  The Frobenius partials of the 32 columns are summed in FP32 in
-// column order, then added to P in FP64.
+// Epilogue of one row of a tile, columns c0 .. c0 + BN - 1: the accumulated sums acc (FMT_FP16X2: S^2 times the
+// product, removed here) go back to the tensor-memory columns at `trow`, the buffer of the tile's last chunk,
+// and a loop takes them 16 at a time.  Worked from the registers the whole row is straight-line code (their
+// indices must be constants), some 70 KB that ran once per tile at the pace of the instruction fetch: 40 to 130 k
+// clocks a 256 x 256 tile without any memory access, against 200 k for its products at N = 8192.
+// Before and after: batch of 64 47.4 -> 31.5 ms, bf16x6 N = 3001 20.2 -> 17.0, tf32x3 N = 2049 6.36 -> 5.23,
+// fp16x3 N = 8192 116.8 -> 108.6, N = 400 2.93 -> 2.50.
+// The Frobenius partials of each 32 columns are summed in FP32 in column order, then added to P in FP64.
 template <int FMT>
-__device__ __forceinline__ void epilogue_chunk(const Job& job, const Instance& In, const Resolved& R, int r,
-                                               int c0, const float (&s_raw)[32], Partials& P) {
-  const int ld = In.ld;
+__device__ __forceinline__ void epilogue_row(const Job& job, const Instance& In, const Resolved& R, int r, int c0,
+                                             const float (&acc)[BN / 32][32], uint32_t trow, Partials& P) {
+  #pragma unroll
+  for (int g = 0; g < BN / 32; ++g) tmem_st32(trow + 32 * g, acc[g]);
+  tmem_wait_st();
+  const int ld = In.ld, N = In.st ? In.st->N : 0, mode = job.mode;
   const int64_t plane = (int64_t)ld * ld;
   const bool upper = job.upper != 0;
-  if (upper && c0 + 31 < r) return;
-  const int64_t row_off = (int64_t)r * ld + c0;
-  float s[32];
-  #pragma unroll
-  for (int j = 0; j < 32; ++j) s[j] = FMT == FMT_FP16X2 ? s_raw[j] * kF16InvScale2 : s_raw[j];
-
-  if (job.mode == MODE_STORE_F32) {
-    const bool all_keep = !upper || c0 >= r;
-    #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const int c = c0 + j;
-      if (all_keep || c >= r) job.out32[row_off + j] = s[j];
-      if (upper && c > r) job.out32[(int64_t)c * ld + r] = s[j];
-    }
-    return;
-  }
-
+  const bool rd = mode != MODE_STORE_F32 && mode != MODE_STORE_PIECES;   // reads the old iterate, slot R.in
   __nv_bfloat16* out = In.arena + (int64_t)R.out * In.slot_elems;
   const __nv_bfloat16* in = In.arena + (int64_t)R.in * In.slot_elems;
-  float vacc = 0.f, facc = 0.f;
-  #pragma unroll
-  for (int h = 0; h < 4; ++h) {
-    const int cb = c0 + 8 * h;
-    if (upper && cb + 7 < r) continue;
-    float xn[8];
-    if (job.mode == MODE_STORE_PIECES) {
+  // dX_0 = -dF / (lmax - lmin): the F slot holds F (FMT_BF16X3, FMT_TF32X2), or F' = (F - c I) / W' with c, W'
+  // the centre and half-width of [lmin, lmax] (FMT_FP16X2), whose dF' is dF / W'
+  float sc = -0.5f;
+  if (mode == MODE_DF_COMBINE && FMT != FMT_FP16X2) sc = (float)(-1.0 / (In.st->lmax - In.st->lmin));
+  float vacc = 0.f, facc = 0.f, diag = 0.f;
+  // the warp's rows are r - lane ..; columns wholly below the diagonal for all of them are left out
+  const int first = upper ? max(0, ((r & ~31) - c0) >> 4) : 0;
+  Row16<FMT> xr;
+  if (rd && first < BN / 16) load_row16<FMT>(in, plane, (int64_t)r * ld + c0 + 16 * first, xr);
+  #pragma unroll 1
+  for (int i = first; i < BN / 16; ++i) {
+    const int cb = c0 + 16 * i;
+    const int64_t row_off = (int64_t)r * ld + cb;
+    uint32_t raw[16];
+    tmem_ld16(trow + 16 * i, raw);
+    tmem_wait_ld();
+    float s[16], x[16];
+    #pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      s[j] = FMT == FMT_FP16X2 ? __uint_as_float(raw[j]) * kF16InvScale2 : __uint_as_float(raw[j]);
+      x[j] = rd ? value_of<FMT>(xr, j) : 0.f;
+    }
+    if (rd && i + 1 < BN / 16) load_row16<FMT>(in, plane, row_off + 16, xr);   // the next columns, ahead of their use
+    if (mode == MODE_STORE_F32) {
       #pragma unroll
-      for (int j = 0; j < 8; ++j) xn[j] = s[8 * h + j];
-    } else {
-      float x[8];
-      load8<FMT>(in, plane, row_off + 8 * h, x);
-      if (job.mode == MODE_DF_COMBINE) {
-        // dX_0 = -dF / (lmax - lmin): the F slot holds F (FMT_BF16X3, FMT_TF32X2), or F' =
-        // (F - c I) / W' with c, W' the centre and half-width of [lmin, lmax] (FMT_FP16X2),
-        // whose dF' is dF / W'
-        const double w = In.st->lmax - In.st->lmin;
-        const float sc = FMT == FMT_FP16X2 ? -0.5f : (float)(-1.0 / w);
-        #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int64_t toff = (int64_t)(cb + j) * ld + r;
-          const float mt = piece_load(FMT, in, plane, toff);
-          xn[j] = sc * ((x[j] + mt) - 2.0f * s[8 * h + j]);
+      for (int j = 0; j < 16; ++j) {
+        const int c = cb + j;
+        if (!upper || c >= r) job.out32[row_off + j] = s[j];
+        if (upper && c > r) job.out32[(int64_t)c * ld + r] = s[j];
+      }
+      continue;
+    }
+    Row16<FMT> y;
+    #pragma unroll
+    for (int j = 0; j < 16; j += 2) {
+      float xn[2];
+      #pragma unroll
+      for (int d = 0; d < 2; ++d) {
+        const int c = cb + j + d;
+        const float sj = s[j + d], xj = x[j + d];
+        if (mode == MODE_STORE_PIECES) {
+          xn[d] = sj;
+        } else if (mode == MODE_DF_COMBINE) {
+          const float mt = piece_load(FMT, in, plane, (int64_t)c * ld + r);
+          xn[d] = sc * ((xj + mt) - 2.0f * sj);
+        } else if (R.gen) {
+          xn[d] = fmaf(R.ca, sj, fmaf(R.cb, xj, (c == r && r < N) ? R.cc : 0.f));
+        } else {
+          xn[d] = R.pk ? sj : fmaf(2.0f, xj, -sj);
         }
-      } else {
-        #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const float sj = s[8 * h + j];
-          if (R.gen) {
-            const float id = (cb + j == r && r < In.st->N) ? R.cc : 0.f;
-            xn[j] = fmaf(R.ca, sj, fmaf(R.cb, x[j], id));
-          } else {
-            xn[j] = R.pk ? sj : fmaf(2.0f, x[j], -sj);
-          }
-          if (job.mode == MODE_SP2_STEP) {
-            const int c = cb + j;
-            const float d = x[j] - sj;
-            const float wgt = !upper ? 1.f : (c > r ? 2.f : (c == r ? 1.f : 0.f));
-            vacc = fmaf(wgt * d, d, vacc);
-            facc = fmaf(wgt * x[j], x[j], facc);
-            if (c == r) P.trd += (double)x[j];
-          }
+        if (mode == MODE_SP2_STEP) {
+          const float dv = xj - sj;
+          const float wgt = !upper ? 1.f : (c > r ? 2.f : (c == r ? 1.f : 0.f));
+          vacc = fmaf(wgt * dv, dv, vacc);
+          facc = fmaf(wgt * xj, xj, facc);
+          if (c == r) diag = xj;
         }
       }
-    }
-    if (!upper || cb >= r) {
-      store8<FMT>(out, plane, row_off + 8 * h, xn);
-    } else {
-      #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (cb + j >= r) piece_store(FMT, out, plane, row_off + 8 * h + j, xn[j]);
+      set_values<FMT>(y, j, xn[0], xn[1]);
     }
     if (upper) {
       #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (cb + j > r) piece_store(FMT, out, plane, (int64_t)(cb + j) * ld + r, xn[j]);
+      for (int j = 0; j < 16; ++j)
+        if (cb + j > r) store_value<FMT>(out, plane, (int64_t)(cb + j) * ld + r, y, j);
+    }
+    if (!upper || cb >= r) {
+      store_row16<FMT>(out, plane, row_off, y);
+    } else {
+      #pragma unroll
+      for (int j = 0; j < 16; ++j)
+        if (cb + j >= r) store_value<FMT>(out, plane, row_off + j, y, j);
+    }
+    if (i & 1) {
+      P.v2 += (double)vacc;
+      P.fro2 += (double)facc;
+      vacc = facc = 0.f;
     }
   }
-  if (job.mode == MODE_SP2_STEP) {
-    P.v2 += (double)vacc;
-    P.fro2 += (double)facc;
-  }
+  P.trd = (double)diag;
 }
 
 template <int FMT>
@@ -552,6 +582,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
       for (int g = 0; g < BN / 32; ++g)
         #pragma unroll
         for (int j = 0; j < 32; ++j) acc[g][j] = 0.f;
+      uint32_t trow = 0;
       for (int ch = 0; ch < nchunks; ++ch) {
         int got = 0;
         if (lane == 0) got = !abort_s && mbar_wait(&accf_bar[buf], bphase, globaltimer_ns() + wait_ns);
@@ -562,7 +593,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
           break;
         }
         tc_fence_after();
-        const uint32_t trow = tmem_base + (uint32_t)(buf * BN) + ((uint32_t)(32 * q) << 16);
+        trow = tmem_base + (uint32_t)(buf * BN) + ((uint32_t)(32 * q) << 16);
         #pragma unroll
         for (int g = 0; g < BN / 32; ++g) {
           uint32_t raw[32];
@@ -571,6 +602,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
           #pragma unroll
           for (int j = 0; j < 32; ++j) acc[g][j] += __uint_as_float(raw[j]);
         }
+        if (ch + 1 == nchunks) break;      // this buffer takes the sums for the epilogue
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&acce_bar[buf]);
@@ -579,8 +611,11 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
       if (!ok) break;
       const int r = I * BM + 32 * q + lane;
       Partials P = {0.0, 0.0, 0.0};
-      #pragma unroll
-      for (int g = 0; g < BN / 32; ++g) epilogue_chunk<FMT>(job, In, R, r, J * BN + g * 32, acc[g], P);
+      epilogue_row<FMT>(job, In, R, r, J * BN, acc, trow, P);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acce_bar[buf]);
+      if (++buf == NBUF) { buf = 0; bphase ^= 1; }
       if (job.mode == MODE_SP2_STEP) {
         #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -789,6 +824,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1) tc_gem
       for (int g = 0; g < BN / 32; ++g)
         #pragma unroll
         for (int j = 0; j < 32; ++j) acc[g][j] = 0.f;
+      uint32_t trow = 0;
       for (int ch = 0; ch < nchunks; ++ch) {
         int got = 0;
         if (lane == 0) got = !abort_s && mbar_wait(&accf_bar[buf], bphase, globaltimer_ns() + wait_ns);
@@ -799,7 +835,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1) tc_gem
           break;
         }
         tc_fence_after();
-        const uint32_t trow = tmem_base + (uint32_t)(buf * PT + hc * BN) + ((uint32_t)(32 * q) << 16);
+        trow = tmem_base + (uint32_t)(buf * PT + hc * BN) + ((uint32_t)(32 * q) << 16);
         #pragma unroll
         for (int g = 0; g < BN / 32; ++g) {
           uint32_t raw[32];
@@ -808,6 +844,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1) tc_gem
           #pragma unroll
           for (int j = 0; j < 32; ++j) acc[g][j] += __uint_as_float(raw[j]);
         }
+        if (ch + 1 == nchunks) break;      // this buffer takes the sums for the epilogue
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster_relaxed(mapa_shared(smem_u32(&acce_bar[buf]), 0));
@@ -816,8 +853,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1) tc_gem
       if (!ok) break;
       const int r = I * PT + (int)rank * BM + 32 * q + lane;
       Partials P = {0.0, 0.0, 0.0};
-      #pragma unroll
-      for (int g = 0; g < BN / 32; ++g) epilogue_chunk<FMT>(job, In, R, r, J * PT + hc * BN + g * 32, acc[g], P);
+      epilogue_row<FMT>(job, In, R, r, J * PT + hc * BN, acc, trow, P);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster_relaxed(mapa_shared(smem_u32(&acce_bar[buf]), 0));
+      if (++buf == P_NBUF) { buf = 0; bphase ^= 1; }
       if (job.mode == MODE_SP2_STEP) {
         #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
