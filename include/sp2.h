@@ -131,7 +131,9 @@ typedef struct {
                            the handle's problems is timed with each choice on scratch memory and
                            the faster one is kept (when the scratch would exceed 2 GiB, a model
                            of the two kernels' measured rates decides instead); the choice is
-                           reported in sp2_info.tile */
+                           reported in sp2_info.tile.  Small problems, whose tiles leave most SMs
+                           idle, take 128 x 64 or 128 x 32 tiles instead, without a timing
+                           (reported as 1) */
   int32_t norm;         /* error measure of the stop test: 0 = Frobenius v_i = ||X_i - X_i^2||_F
                            (default); 1 = the mixed norm m_i of §2, the spectral norm of the
                            matrix of Frobenius norms of the square kernel's tiles (64 x 64 on the
@@ -168,7 +170,7 @@ typedef struct {
   const double*  v;        /* v[i] = ||X_i - X_i^2||_F, i < hist_len (host memory owned by the handle) */
   const double*  trace;    /* trace[i] = Tr[X_i], i <= n_iter */
   const uint8_t* p;        /* p[i] in {0,1} for 1 <= i <= n_iter: 1 = X^2, 0 = 2X - X^2 */
-  int32_t tile;            /* SP2_PREC_MIXED: tensor-core tiles in use, 1 = 128 x 128 per SM,
+  int32_t tile;            /* SP2_PREC_MIXED: tensor-core tiles in use, 1 = 128 x 128 (or narrower) per SM,
                               2 = 256 x 256 per SM pair (as chosen by sp2_opts.tile or its
                               tuner); 0 on the other paths */
 } sp2_info;

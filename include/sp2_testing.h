@@ -23,7 +23,8 @@ extern "C" {
  * arena_dev 16-byte aligned.  With upper = 1 only C's upper triangle is computed and
  * mirrored (meaningful when A B^T is symmetric); with upper = 0 every element is.
  * tile: 1 = 128 x 128 tiles, one per SM; 2 = 256 x 256 tiles, one per pair of SMs
- * (ld a multiple of 256); 0 = 2 when ld is a multiple of 256, else 1.
+ * (ld a multiple of 256); 3, 4 = 128 x 64 and 128 x 32 tiles, one per SM; 0 = 2 when ld is a
+ * multiple of 256, else 1.
  * out_dev: ld x ld FP32, row-major.  Synchronises `stream`; returns an sp2_status
  * (SP2_ERR_INVALID_ARG for bad arguments, SP2_ERR_TIMEOUT if a device-side wait gave up). */
 int32_t sp2_test_tc_gemm(const void* arena_dev, int32_t ld, int32_t nslots, int32_t a_slot, int32_t b_slot,

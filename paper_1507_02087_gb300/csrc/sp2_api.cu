@@ -165,8 +165,8 @@ static int tune_tiles(const std::vector<int64_t>& N, int fmt, int lowprec) {
       I.nslots = 2;
       I.slot_elems = sp2::tc::slot_units_of(fmt, ld);
       I.tile_off_upper = I.tile_off_upper2 = tiles;
-      tiles += sp2::tc_tiles(ld, 1, pair);
-      ok = sp2::tc_make_maps(arena, ld, 2, fmt, &I.mapA, &I.mapB) == cudaSuccess;
+      tiles += sp2::tc_tiles(ld, 1, pair, 128);
+      ok = sp2::tc_make_maps(arena, ld, 2, fmt, &I) == cudaSuccess;
     }
     if (!ok) break;
     Job j;
@@ -180,6 +180,7 @@ static int tune_tiles(const std::vector<int64_t>& N, int fmt, int lowprec) {
     j.inst = dinst;
     j.out_slot = 1;
     j.pair = pair;
+    j.tn = 128;
     j.fmt = fmt;
     j.lowprec = lowprec;
     j.err = err;
@@ -233,7 +234,8 @@ struct MixedEngine {
   double* part_hi = nullptr;
   int* part_bad = nullptr;
   int pb = 1, sb = 1;
-  int pair = 0;                    // tensor-core tiles: 1 = 256 x 256 per SM pair, 0 = 128 x 128 per SM
+  int pair = 0;                    // tensor-core tiles: 1 = 256 x 256 per SM pair, 0 = 128 x tn per SM
+  int tn = 128;
   int total_upper = 0, total_full = 0;   // tiles of one launch, in the unit above
   int32_t* err_dev = nullptr;
   int32_t* err_host = nullptr;
@@ -277,6 +279,7 @@ struct MixedEngine {
     j.rule = rule;
     j.count = count;
     j.pair = pair;
+    j.tn = tn;
     j.total_tiles = upper ? total_upper : total_full;
     j.inst = inst_dev;
     j.err = err_dev;
@@ -334,7 +337,12 @@ struct MixedEngine {
     arenas.assign(count, nullptr);
     parts.assign(count, nullptr);
     const int H = o.max_iter + 2;
-    pair = (o.tile == 0 ? tune_tiles(N, fmt, lp_main) : o.tile) == 2 ? 1 : 0;
+    if (o.tile == 0) {   // narrow single tiles where they fit in one round, else the faster kind
+      std::vector<int> lds;
+      for (int64_t n : N) lds.push_back(round_up(n, LD_ALIGN));
+      tn = sp2::tc_tile_width(lds.data(), count);
+    }
+    pair = tn == 128 && (o.tile == 0 ? tune_tiles(N, fmt, lp_main) : o.tile) == 2 ? 1 : 0;
     const int align = pair ? PT : LD_ALIGN;
     auto ld_of = [&](int64_t n) { return round_up(n, align); };
     // Keep every iterate (full history) or recompute them in the derivative pass; without
@@ -373,10 +381,11 @@ struct MixedEngine {
       I.st = st_dev + k;
       I.tile_off_upper = I.tile_off_upper2 = off_u;
       I.tile_off_full = I.tile_off_full2 = off_f;
-      off_u += pair ? pair_tiles_of(ld, 1) : tiles_of(ld, 1);
-      off_f += pair ? pair_tiles_of(ld, 0) : tiles_of(ld, 0);
-      I.nparts = nparts_of(ld, pair);
+      off_u += sp2::tc_tiles(ld, 1, pair, tn);
+      off_f += sp2::tc_tiles(ld, 0, pair, tn);
+      I.nparts = nparts_of(ld, pair, tn);
       I.rec_pair = pair;
+      I.rec_block = epi_warps(tn) * (BM / tn);
       const size_t abytes = (size_t)nslots * I.slot_elems * 2;
       if (cudaMalloc(&arenas[k], abytes) != cudaSuccess ||
           cudaMalloc(&parts[k], sizeof(double) * 4 * I.nparts) != cudaSuccess) {
@@ -397,7 +406,7 @@ struct MixedEngine {
         mscrs.push_back(ms);
         I.mscr = ms;
       }
-      SP2_TRY(sp2::tc_make_maps(arenas[k], ld, nslots, fmt, &I.mapA, &I.mapB));
+      SP2_TRY(sp2::tc_make_maps(arenas[k], ld, nslots, fmt, &I));
       if (o.norm == 2) {   // spectral-norm stop: single problems only (one Lanczos scratch)
         if (count != 1) return SP2_ERR_UNSUPPORTED;
         if (cudaMalloc(&lz, sp2::lanczos_scratch_bytes(ld)) != cudaSuccess) {

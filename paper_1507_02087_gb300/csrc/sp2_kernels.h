@@ -100,9 +100,11 @@ cudaError_t launch_copy_f64(const DevState* st, const double* X, int ld, int N, 
 
 // ---- tensor-core path ------------------------------------------------------------------------
 // TMA tensor maps over a piece arena of `nslots` ld x ld matrices in piece format `fmt`
-// (tc::Fmt; boxes of 128 rows).
-cudaError_t tc_make_maps(void* arena, int ld, int nslots, int fmt, CUtensorMap* mapA, CUtensorMap* mapB);
-int tc_tiles(int ld, int upper, int pair);
+// (tc::Fmt), into the instance record.
+cudaError_t tc_make_maps(void* arena, int ld, int nslots, int fmt, tc::Instance* inst);
+int tc_tiles(int ld, int upper, int pair, int tn);
+// Columns of the single-CTA tiles for problems with the given leading dimensions (see sp2_tc_gemm.cu).
+int tc_tile_width(const int* ld, int count);
 int tc_grid_for(int total_tiles, int pair);
 cudaError_t tc_launch(const tc::Job& job, cudaStream_t s);
 cudaError_t tc_add_node(cudaGraph_t g, const cudaGraphNode_t* deps, int ndeps, const tc::Job& job,

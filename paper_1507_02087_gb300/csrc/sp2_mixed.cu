@@ -189,8 +189,8 @@ __global__ void __launch_bounds__(kFT) batch_finalize_kernel(const Instance* ins
   double vk = sqrt(a);
   if (st->norm == 2) vk = st->spec_e;   // e_{k-1}, the Lanczos estimate of the 2-norm (one problem)
   if (st->norm == 1 && In.mscr) {
-    // mixed norm over 128 x 128 blocks: a 128 x 128 tile holds 4 records (one per epilogue
-    // warp, 32 rows each); a 256 x 256 pair tile holds 16, record 8 rank + 4 hc + q covering
+    // mixed norm over 128 x 128 blocks: single-CTA tiles give rec_block records per block (one per
+    // epilogue warp); a 256 x 256 pair tile holds 16, record 8 rank + 4 hc + q covering
     // rows 128 rank + 32 q .., columns 128 hc ..; off-diagonal blocks are counted twice
     const int nb = In.ld / tc::BM;
     const double* pt = In.part;
@@ -198,9 +198,10 @@ __global__ void __launch_bounds__(kFT) batch_finalize_kernel(const Instance* ins
     vk = mixed_norm_cta<kFT>(nb, In.mscr, sm, [&](int I, int J) {
       int64_t r0;
       if (pair) r0 = 16 * upper_index(I / 2, J / 2, nb / 2) + 8 * (I & 1) + 4 * (J & 1);
-      else r0 = 4 * upper_index(I, J, nb);
+      else r0 = In.rec_block * upper_index(I, J, nb);
       double v2 = 0.0;
-      for (int q = 0; q < 4; ++q) v2 += pt[4 * (r0 + q)];
+      const int n = pair ? 4 : In.rec_block;
+      for (int q = 0; q < n; ++q) v2 += pt[4 * (r0 + q)];
       return I == J ? v2 : 0.5 * v2;
     });
   }

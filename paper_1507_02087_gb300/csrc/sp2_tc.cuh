@@ -45,7 +45,7 @@ constexpr float kF16InvScale = 1.f / 16384.f;
 constexpr float kF16InvScale2 = 1.f / (16384.f * 16384.f);
 
 constexpr int BM = 128;          // tile rows (MMA M)
-constexpr int BN = 128;          // tile cols (MMA N)
+constexpr int BN = 128;          // tile cols (MMA N) of the CTA's share of a pair tile, and the widest single tile
 constexpr int BK = 64;           // k-block of the 16-bit formats: 64 values = 128 B rows, 128-byte swizzle
 constexpr int ROW_BYTES = 128;   // one k-block row of any format (FMT_TF32X2: 32 values)
 constexpr int KSTEPS = 4;        // MMAs per k-block row and product: 32 B each (16 16-bit or 8 tf32 values)
@@ -81,14 +81,21 @@ static_assert(stages_of(FMT_FP16X2) * stage_bytes_of(FMT_FP16X2) == STAGES * STA
 // as fit in its bytes, up to MAX_STAGES (full products: 2 bf16 or 3 fp16 / tf32 stages; one-piece
 // low-precision products: 6).
 constexpr int MAX_STAGES = 6;
-__host__ __device__ constexpr int ring_stage_bytes(int npl) { return npl * (A_PIECE_BYTES + B_PIECE_BYTES); }
-__host__ __device__ constexpr int ring_stages(int npl) {
-  return STAGES * STAGE_BYTES / ring_stage_bytes(npl) < MAX_STAGES ? STAGES * STAGE_BYTES / ring_stage_bytes(npl)
-                                                                   : MAX_STAGES;
+__host__ __device__ constexpr int ring_stage_bytes(int npl, int tn = BN) { return npl * (A_PIECE_BYTES + tn * ROW_BYTES); }
+__host__ __device__ constexpr int ring_stages(int npl, int tn = BN) {
+  return STAGES * STAGE_BYTES / ring_stage_bytes(npl, tn) < MAX_STAGES
+             ? STAGES * STAGE_BYTES / ring_stage_bytes(npl, tn)
+             : MAX_STAGES;
 }
 static_assert(ring_stages(1) == MAX_STAGES && ring_stages(2) == 3 && ring_stages(3) == 2, "ring geometry");
-constexpr int THREADS = 192;     // warp 0: TMA, warp 1: MMA, warps 2-5: epilogue
-constexpr int TMEM_COLS = NBUF * BN;   // four 128 x 128 fp32 chunk accumulators
+// Single-CTA tiles are 128 x tn, tn = 128, 64 or 32.  The narrow ones serve problems whose 128 x 128 tiles leave
+// most SMs idle: what a small square takes is the latency of one tile, above all its epilogue.
+// Epilogue warps: two per tensor-memory lane quadrant with half the columns each, but at least the 32
+// columns whose Frobenius partials are summed together.
+__host__ __device__ constexpr int epi_cols(int tn) { return tn == 32 ? 32 : tn / 2; }
+__host__ __device__ constexpr int epi_warps(int tn) { return 4 * (tn / epi_cols(tn)); }
+__host__ __device__ constexpr int threads_of(int tn) { return 64 + 32 * epi_warps(tn); }   // warp 0: TMA, warp 1: MMA
+constexpr int BOX_N = 32;        // rows of a B box of the single-CTA kernel
 constexpr int LD_ALIGN = 128;    // ld is a multiple of the tile size
 constexpr int MAX_BATCH = 256;   // instances per batch
 
@@ -149,7 +156,8 @@ __host__ __device__ __forceinline__ int rslot(int lowmem, int hist0, int j) {
 // keep the alignment CUtensorMap requires).
 struct Instance {
   CUtensorMap mapA;     // box 64 x 128 (A operand; k innermost)
-  CUtensorMap mapB;     // box 64 x 128 (B operand)
+  CUtensorMap mapB;     // box 64 x 128 (B operand of the CTA pair)
+  CUtensorMap mapN;     // box 64 x BOX_N (B operand of single-CTA tiles)
   __nv_bfloat16* arena;
   int64_t slot_elems;   // 3 * ld * ld
   DevState* st;
@@ -163,6 +171,7 @@ struct Instance {
   int32_t tile_off_full2;   // first global pair-tile index (full schedule)
   int32_t nparts;           // forward-square partial records (4 doubles each) per launch
   int32_t rec_pair;         // 1: the records come from CTA-pair tiles (16 per 256 x 256 tile)
+  int32_t rec_block;        // otherwise: records per 128 x 128 block (a block's tiles follow one another)
   double* mscr;             // mixed-norm scratch ((ld/128)^2 + 2 ld/128 doubles), or null
   int32_t fmt;              // Fmt of the arena
   int32_t np;               // pieces (planes) per slot: np_of(fmt)
@@ -180,6 +189,7 @@ struct Job {
   int32_t a_slot[2], b_slot[2];   // SLOTS_FIXED operands; SLOTS_REFINE step in a_slot[0]
   int32_t out_slot;
   int32_t pair;         // 1: 256 x 256 CTA-pair tiles (every instance's ld a multiple of 256)
+  int32_t tn;           // single-CTA tiles: columns of a tile (128, 64 or 32)
   int32_t lowprec;      // 1: the low-precision product of the format (FMT_BF16X3: pieces 0 and 1,
                         // the three products with a + b <= 1, about 16 bits; FMT_FP16X2: p0 q0,
                         // 11 bits); the derivative pass, and every product of SP2_PREC_BF16X3
@@ -256,9 +266,9 @@ __device__ __forceinline__ void piece_store(int fmt, __nv_bfloat16* slot, int64_
   slot[2 * plane + off] = c;
 }
 
-__host__ __device__ __forceinline__ int tiles_of(int ld, int upper) {
+__host__ __device__ __forceinline__ int tiles_of(int ld, int upper, int tn) {
   const int R = ld / BM;
-  return upper ? R * (R + 1) / 2 : R * R;
+  return (BM / tn) * (upper ? R * (R + 1) / 2 : R * R);
 }
 
 __host__ __device__ __forceinline__ int pair_tiles_of(int ld, int upper) {
@@ -267,8 +277,8 @@ __host__ __device__ __forceinline__ int pair_tiles_of(int ld, int upper) {
 }
 
 // Partial records one forward square writes: one per (tile, epilogue warp).
-__host__ __device__ __forceinline__ int nparts_of(int ld, int pair) {
-  return pair ? 2 * P_EPI_WARPS * pair_tiles_of(ld, 1) : 4 * tiles_of(ld, 1);
+__host__ __device__ __forceinline__ int nparts_of(int ld, int pair, int tn) {
+  return pair ? 2 * P_EPI_WARPS * pair_tiles_of(ld, 1) : epi_warps(tn) * tiles_of(ld, 1, tn);
 }
 
 }  // namespace tc

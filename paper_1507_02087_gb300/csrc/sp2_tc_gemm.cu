@@ -23,6 +23,7 @@
 #include <cudaTypedefs.h>
 
 #include <cstring>
+#include <type_traits>
 
 #include "../../include/sp2_testing.h"
 #include "sp2_kernels.h"
@@ -136,8 +137,8 @@ __device__ __forceinline__ Resolved resolve(const Job& j, const Instance& I, int
 #endif
   Resolved r = resolve_slots(j, I);
 #if SP2_DEVICE_CHECKS
-  const int ns = I.nslots, T = j.pair ? PT : BM;
-  bool ok = ti >= 0 && tj >= 0 && (ti + 1) * T <= I.ld && (tj + 1) * T <= I.ld;
+  const int ns = I.nslots, T = j.pair ? PT : BM, TJ = j.pair ? PT : j.tn;
+  bool ok = ti >= 0 && tj >= 0 && (ti + 1) * T <= I.ld && (tj + 1) * TJ <= I.ld;
   for (int t = 0; t < j.nterms; ++t) ok = ok && r.a[t] >= 0 && r.a[t] < ns && r.b[t] >= 0 && r.b[t] < ns;
   if (j.mode != MODE_STORE_F32) ok = ok && r.out >= 0 && r.out < ns;
   if (j.mode == MODE_SP2_STEP || j.mode == MODE_DERIV_STEP || j.mode == MODE_DF_COMBINE)
@@ -216,7 +217,7 @@ __device__ __forceinline__ int tile_off(const Job& job, const Instance& in) {
 }
 
 // Global tile t -> (instance, tile row I, tile column J), in units of the launch's tile
-// (128 x 128, or 256 x 256 for CTA pairs): row-major within an instance, over the upper
+// (128 x tn, or 256 x 256 for CTA pairs): row-major within an instance, over the upper
 // triangle (J >= I) or all tiles.  A banded walk (column by column within bands of 2..16 tile
 // rows, so that co-resident CTAs share B panels in L2) was measured slower at N = 8192
 // (1.84-1.93 ms against 1.81 ms per forward square) and is not used.
@@ -226,15 +227,15 @@ __device__ __forceinline__ int locate(const Job& job, int t, int& I, int& J) {
     if (t < tile_off(job, job.inst[i + 1])) break;
   const Instance& in = job.inst[i];
   t -= tile_off(job, in);
-  const int R = in.ld / (job.pair ? PT : BM);
+  const int R = in.ld / (job.pair ? PT : BM), f = job.pair ? 1 : BM / job.tn;   // f tiles across a square one
   if (!job.upper) {
-    I = t / R;
-    J = t % R;
+    I = t / (R * f);
+    J = t % (R * f);
   } else {
     int r = 0;
-    while (t >= R - r) { t -= R - r; ++r; }
+    while (t >= (R - r) * f) { t -= (R - r) * f; ++r; }
     I = r;
-    J = r + t;
+    J = r * f + t;
   }
   return i;
 }
@@ -296,18 +297,23 @@ __device__ __forceinline__ void set_values(Row16<FMT>& row, int e, float x0, flo
     row.v[0][e >> 3][(e & 7) + 1] = __float_as_uint(h1);
     row.v[1][e >> 3][(e & 7) + 1] = __float_as_uint(l1);
   } else if constexpr (FMT == FMT_FP16X2) {
-    __half a0, a1, b0, b1;
-    split_fp16x2(x0, a0, a1);
-    split_fp16x2(x1, b0, b1);
-    row.v[0][0][e >> 1] = __half_as_ushort(a0) | ((uint32_t)__half_as_ushort(b0) << 16);
-    row.v[1][0][e >> 1] = __half_as_ushort(a1) | ((uint32_t)__half_as_ushort(b1) << 16);
+    // split_fp16x2 of both values, in paired conversions
+    const float y0 = x0 * kF16Scale, y1 = x1 * kF16Scale;
+    const __half2 p0 = __floats2half2_rn(y0, y1);
+    const float2 f = __half22float2(p0);
+    const __half2 p1 = __floats2half2_rn(y0 - f.x, y1 - f.y);
+    row.v[0][0][e >> 1] = *reinterpret_cast<const uint32_t*>(&p0);
+    row.v[1][0][e >> 1] = *reinterpret_cast<const uint32_t*>(&p1);
   } else {
-    __nv_bfloat16 a[3], b[3];
-    split_bf16x3(x0, a[0], a[1], a[2]);
-    split_bf16x3(x1, b[0], b[1], b[2]);
+    // split_bf16x3 of both values
     #pragma unroll
-    for (int p = 0; p < 3; ++p)
-      row.v[p][0][e >> 1] = __bfloat16_as_ushort(a[p]) | ((uint32_t)__bfloat16_as_ushort(b[p]) << 16);
+    for (int p = 0; p < 3; ++p) {
+      const __nv_bfloat162 q = __floats2bfloat162_rn(x0, x1);
+      const float2 f = __bfloat1622float2(q);
+      x0 -= f.x;
+      x1 -= f.y;
+      row.v[p][0][e >> 1] = *reinterpret_cast<const uint32_t*>(&q);
+    }
   }
 }
 
@@ -329,7 +335,7 @@ struct Partials {
   double trd;   // sum of the diagonal x
 };
 
-// Epilogue of one row of a tile, columns c0 .. c0 + BN - 1: the accumulated sums acc (FMT_FP16X2: S^2 times the
+// Epilogue of one row of a tile, columns c0 .. c0 + COLS - 1: the accumulated sums acc (FMT_FP16X2: S^2 times the
 // product, removed here) go back to the tensor-memory columns at `trow`, the buffer of the tile's last chunk,
 // and a loop takes them 16 at a time.  Worked from the registers the whole row is straight-line code (their
 // indices must be constants), some 70 KB that ran once per tile at the pace of the instruction fetch: 40 to 130 k
@@ -337,11 +343,11 @@ struct Partials {
 // Before and after: batch of 64 47.4 -> 31.5 ms, bf16x6 N = 3001 20.2 -> 17.0, tf32x3 N = 2049 6.36 -> 5.23,
 // fp16x3 N = 8192 116.8 -> 108.6, N = 400 2.93 -> 2.50.
 // The Frobenius partials of each 32 columns are summed in FP32 in column order, then added to P in FP64.
-template <int FMT>
+template <int FMT, int COLS>
 __device__ __forceinline__ void epilogue_row(const Job& job, const Instance& In, const Resolved& R, int r, int c0,
-                                             const float (&acc)[BN / 32][32], uint32_t trow, Partials& P) {
+                                             const float (&acc)[COLS / 32][32], uint32_t trow, Partials& P) {
   #pragma unroll
-  for (int g = 0; g < BN / 32; ++g) tmem_st32(trow + 32 * g, acc[g]);
+  for (int g = 0; g < COLS / 32; ++g) tmem_st32(trow + 32 * g, acc[g]);
   tmem_wait_st();
   const int ld = In.ld, N = In.st ? In.st->N : 0, mode = job.mode;
   const int64_t plane = (int64_t)ld * ld;
@@ -354,32 +360,19 @@ __device__ __forceinline__ void epilogue_row(const Job& job, const Instance& In,
   float sc = -0.5f;
   if (mode == MODE_DF_COMBINE && FMT != FMT_FP16X2) sc = (float)(-1.0 / (In.st->lmax - In.st->lmin));
   float vacc = 0.f, facc = 0.f, diag = 0.f;
-  // the warp's rows are r - lane ..; columns wholly below the diagonal for all of them are left out
-  const int first = upper ? max(0, ((r & ~31) - c0) >> 4) : 0;
-  Row16<FMT> xr;
-  if (rd && first < BN / 16) load_row16<FMT>(in, plane, (int64_t)r * ld + c0 + 16 * first, xr);
-  #pragma unroll 1
-  for (int i = first; i < BN / 16; ++i) {
-    const int cb = c0 + 16 * i;
+  // 16 columns from cb; KIND 0: every element is written at its place only (not `upper`), 1: all of the warp's
+  // elements lie above the diagonal, 2: some lie on it or below
+  auto columns = [&](auto kind_c, int cb, const float (&s)[16], const float (&x)[16]) {
+    constexpr int KIND = decltype(kind_c)::value;
     const int64_t row_off = (int64_t)r * ld + cb;
-    uint32_t raw[16];
-    tmem_ld16(trow + 16 * i, raw);
-    tmem_wait_ld();
-    float s[16], x[16];
-    #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      s[j] = FMT == FMT_FP16X2 ? __uint_as_float(raw[j]) * kF16InvScale2 : __uint_as_float(raw[j]);
-      x[j] = rd ? value_of<FMT>(xr, j) : 0.f;
-    }
-    if (rd && i + 1 < BN / 16) load_row16<FMT>(in, plane, row_off + 16, xr);   // the next columns, ahead of their use
     if (mode == MODE_STORE_F32) {
       #pragma unroll
       for (int j = 0; j < 16; ++j) {
         const int c = cb + j;
-        if (!upper || c >= r) job.out32[row_off + j] = s[j];
-        if (upper && c > r) job.out32[(int64_t)c * ld + r] = s[j];
+        if (KIND < 2 || c >= r) job.out32[row_off + j] = s[j];
+        if (KIND == 1 || (KIND == 2 && c > r)) job.out32[(int64_t)c * ld + r] = s[j];
       }
-      continue;
+      return;
     }
     Row16<FMT> y;
     #pragma unroll
@@ -395,33 +388,55 @@ __device__ __forceinline__ void epilogue_row(const Job& job, const Instance& In,
           const float mt = piece_load(FMT, in, plane, (int64_t)c * ld + r);
           xn[d] = sc * ((xj + mt) - 2.0f * sj);
         } else if (R.gen) {
-          xn[d] = fmaf(R.ca, sj, fmaf(R.cb, xj, (c == r && r < N) ? R.cc : 0.f));
+          xn[d] = fmaf(R.ca, sj, fmaf(R.cb, xj, (KIND != 1 && c == r && r < N) ? R.cc : 0.f));
         } else {
           xn[d] = R.pk ? sj : fmaf(2.0f, xj, -sj);
         }
         if (mode == MODE_SP2_STEP) {
           const float dv = xj - sj;
-          const float wgt = !upper ? 1.f : (c > r ? 2.f : (c == r ? 1.f : 0.f));
+          const float wgt = KIND == 0 ? 1.f : (KIND == 1 || c > r ? 2.f : (c == r ? 1.f : 0.f));
           vacc = fmaf(wgt * dv, dv, vacc);
           facc = fmaf(wgt * xj, xj, facc);
-          if (c == r) diag = xj;
+          if (KIND != 1 && c == r) diag = xj;
         }
       }
       set_values<FMT>(y, j, xn[0], xn[1]);
     }
-    if (upper) {
+    if (KIND > 0) {
       #pragma unroll
       for (int j = 0; j < 16; ++j)
-        if (cb + j > r) store_value<FMT>(out, plane, (int64_t)(cb + j) * ld + r, y, j);
+        if (KIND == 1 || cb + j > r) store_value<FMT>(out, plane, (int64_t)(cb + j) * ld + r, y, j);
     }
-    if (!upper || cb >= r) {
+    if (KIND < 2 || cb >= r) {
       store_row16<FMT>(out, plane, row_off, y);
     } else {
       #pragma unroll
       for (int j = 0; j < 16; ++j)
         if (cb + j >= r) store_value<FMT>(out, plane, row_off + j, y, j);
     }
-    if (i & 1) {
+  };
+  // the warp's rows are r0 ..; columns wholly below the diagonal for all of them are left out
+  const int r0 = r & ~31;
+  const int first = upper ? max(0, (r0 - c0) >> 4) : 0;
+  Row16<FMT> xr;
+  if (rd && first < COLS / 16) load_row16<FMT>(in, plane, (int64_t)r * ld + c0 + 16 * first, xr);
+  #pragma unroll 1
+  for (int i = first; i < COLS / 16; ++i) {
+    const int cb = c0 + 16 * i;
+    uint32_t raw[16];
+    tmem_ld16(trow + 16 * i, raw);
+    tmem_wait_ld();
+    float s[16], x[16];
+    #pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      s[j] = FMT == FMT_FP16X2 ? __uint_as_float(raw[j]) * kF16InvScale2 : __uint_as_float(raw[j]);
+      x[j] = rd ? value_of<FMT>(xr, j) : 0.f;
+    }
+    if (rd && i + 1 < COLS / 16) load_row16<FMT>(in, plane, (int64_t)r * ld + cb + 16, xr);   // ahead of their use
+    if (!upper) columns(std::integral_constant<int, 0>(), cb, s, x);
+    else if (cb >= r0 + 32) columns(std::integral_constant<int, 1>(), cb, s, x);
+    else columns(std::integral_constant<int, 2>(), cb, s, x);
+    if ((i & 1) && mode == MODE_SP2_STEP) {
       P.v2 += (double)vacc;
       P.fro2 += (double)facc;
       vacc = facc = 0.f;
@@ -430,11 +445,12 @@ __device__ __forceinline__ void epilogue_row(const Job& job, const Instance& In,
   P.trd = (double)diag;
 }
 
-template <int FMT>
-__global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
+template <int FMT, int TN>
+__global__ void __launch_bounds__(threads_of(TN), 1) tc_gemm_kernel(const Job job) {
   // the job's ring: stages of the pieces it loads (ring_stages in sp2_tc.cuh)
   const int npl = pieces_loaded<FMT>(job);
-  const int stg = ring_stages(npl), sbytes = ring_stage_bytes(npl);
+  const int stg = ring_stages(npl, TN), sbytes = ring_stage_bytes(npl, TN);
+  constexpr int COLS = epi_cols(TN), EW = epi_warps(TN), BP = TN * ROW_BYTES;   // BP: bytes of one piece of B
   using PR = Products<FMT>;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[MAX_STAGES];
@@ -450,12 +466,12 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
   const uint64_t wait_ns = job.wait_ms > 0 ? (uint64_t)job.wait_ms * 1000000ull : kWaitNs;
   if (threadIdx.x == 0) {
     for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-    for (int a = 0; a < NBUF; ++a) { mbar_init(&accf_bar[a], 1); mbar_init(&acce_bar[a], 4); }
+    for (int a = 0; a < NBUF; ++a) { mbar_init(&accf_bar[a], 1); mbar_init(&acce_bar[a], EW); }
     mbar_init(&drain_bar, 1);
     abort_s = 0;
     fence_barrier_init();
   }
-  if (warp == 1) tmem_alloc(&tmem_base_s, TMEM_COLS);
+  if (warp == 1) tmem_alloc(&tmem_base_s, NBUF * TN);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -479,7 +495,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
         const Resolved R = resolve(job, In, I, J);
         if (!R.active) continue;
         const CUtensorMap* mA = &In.mapA;
-        const CUtensorMap* mB = &In.mapB;
+        const CUtensorMap* mB = &In.mapN;
         const int nkb = In.ld / bk_of(FMT);
         for (int term = 0; term < job.nterms && ok; ++term) {
           for (int kb = 0; kb < nkb; ++kb) {
@@ -495,11 +511,14 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
             }
             uint8_t* sA = smem + stage * sbytes;
             uint8_t* sB = sA + npl * A_PIECE_BYTES;
-            mbar_arrive_expect_tx(&full_bar[stage], npl * (A_PIECE_BYTES + B_PIECE_BYTES));
+            mbar_arrive_expect_tx(&full_bar[stage], npl * (A_PIECE_BYTES + BP));
             for (int p = 0; p < npl; ++p)
               tma_load_4d(sA + p * A_PIECE_BYTES, mA, kb * bk_of(FMT), I * BM, p, R.a[term], &full_bar[stage]);
             for (int p = 0; p < npl; ++p)
-              tma_load_4d(sB + p * B_PIECE_BYTES, mB, kb * bk_of(FMT), J * BN, p, R.b[term], &full_bar[stage]);
+              #pragma unroll
+              for (int b = 0; b < TN / BOX_N; ++b)
+                tma_load_4d(sB + p * BP + b * BOX_N * ROW_BYTES, mB, kb * bk_of(FMT), J * TN + b * BOX_N, p, R.b[term],
+                            &full_bar[stage]);
             armed[stage] = 1;
             armed_par[stage] = phase;
             if (++stage == stg) { stage = 0; phase ^= 1; }
@@ -514,7 +533,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     if (elect_one()) {
-      constexpr uint32_t idesc = idesc_of<FMT>(BM, BN);
+      constexpr uint32_t idesc = idesc_of<FMT>(BM, TN);
       // the format's piece products, smallest first; low-precision jobs take the tail
       const int q0 = job.lowprec ? PR::lp_first : 0;
       int stage = 0, buf = 0;
@@ -527,7 +546,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
         if (!resolve(job, In, I, J).active) continue;
         const int nchunks = job.nterms * (In.ld / bk_of(FMT)) / chunk_kb(job, In.ld);
         for (int ch = 0; ch < nchunks && ok; ++ch) {
-          const uint32_t dt = tmem_base + (uint32_t)(buf * BN);
+          const uint32_t dt = tmem_base + (uint32_t)(buf * TN);
           uint32_t accumulate = 0;
           for (int kc = 0; kc < chunk_kb(job, In.ld); ++kc) {
             // the ring stage first, then (on the chunk's first stage) the free chunk buffer, as in
@@ -546,7 +565,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
                 for (int q = 0; q < PR::n; ++q) {
                   if (q < q0 || (q == PR::n - 1) != (pass == 1)) continue;
                   const uint64_t ad = smem_desc_sw128(sA + PR::a(q) * A_PIECE_BYTES + kk * 32);
-                  const uint64_t bd = smem_desc_sw128(sB + PR::b(q) * B_PIECE_BYTES + kk * 32);
+                  const uint64_t bd = smem_desc_sw128(sB + PR::b(q) * BP + kk * 32);
                   mma_fmt<FMT, false>(dt, ad, bd, idesc, accumulate);
                   accumulate = 1;
                 }
@@ -565,8 +584,10 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
       mbar_wait(&drain_bar, 0, globaltimer_ns() + wait_ns);
     }
   } else {
-    // ---------------- chunk draining + epilogue (warps 2..5) ----------------
+    // ---------------- chunk draining + epilogue (warps 2 ..) ----------------
+    const int ew = warp - 2;
     const int q = warp & 3;      // TMEM lanes 32q .. 32q+31
+    const int hc = ew >> 2;      // columns hc COLS .. of the tile
     int buf = 0;
     uint32_t bphase = 0;
     bool ok = true;
@@ -577,9 +598,9 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
       const Resolved R = resolve(job, In, I, J);
       if (!R.active) continue;
       const int nchunks = job.nterms * (In.ld / bk_of(FMT)) / chunk_kb(job, In.ld);
-      float acc[BN / 32][32];
+      float acc[COLS / 32][32];
       #pragma unroll
-      for (int g = 0; g < BN / 32; ++g)
+      for (int g = 0; g < COLS / 32; ++g)
         #pragma unroll
         for (int j = 0; j < 32; ++j) acc[g][j] = 0.f;
       uint32_t trow = 0;
@@ -593,9 +614,9 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
           break;
         }
         tc_fence_after();
-        trow = tmem_base + (uint32_t)(buf * BN) + ((uint32_t)(32 * q) << 16);
+        trow = tmem_base + (uint32_t)(buf * TN + hc * COLS) + ((uint32_t)(32 * q) << 16);
         #pragma unroll
-        for (int g = 0; g < BN / 32; ++g) {
+        for (int g = 0; g < COLS / 32; ++g) {
           uint32_t raw[32];
           tmem_ld32(trow + g * 32, raw);
           tmem_wait_ld();
@@ -611,7 +632,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
       if (!ok) break;
       const int r = I * BM + 32 * q + lane;
       Partials P = {0.0, 0.0, 0.0};
-      epilogue_row<FMT>(job, In, R, r, J * BN, acc, trow, P);
+      epilogue_row<FMT, COLS>(job, In, R, r, J * TN + hc * COLS, acc, trow, P);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&acce_bar[buf]);
@@ -625,7 +646,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
         }
         if (lane == 0) {
           const int lt = t - In.tile_off_upper;        // tile index within the instance
-          double* dst = In.part + 4 * (4 * (int64_t)lt + q);
+          double* dst = In.part + 4 * (EW * (int64_t)lt + ew);
           dst[0] = P.v2;
           dst[1] = P.fro2;
           dst[2] = P.trd;
@@ -638,7 +659,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(const Job job) {
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, TMEM_COLS);
+    tmem_dealloc(tmem_base, NBUF * TN);
   }
 }
 
@@ -853,7 +874,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1) tc_gem
       if (!ok) break;
       const int r = I * PT + (int)rank * BM + 32 * q + lane;
       Partials P = {0.0, 0.0, 0.0};
-      epilogue_row<FMT>(job, In, R, r, J * PT + hc * BN, acc, trow, P);
+      epilogue_row<FMT, BN>(job, In, R, r, J * PT + hc * BN, acc, trow, P);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster_relaxed(mapa_shared(smem_u32(&acce_bar[buf]), 0));
@@ -904,7 +925,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
   return fn;
 }
 
-cudaError_t tc_make_maps(void* arena, int ld, int nslots, int fmt, CUtensorMap* mapA, CUtensorMap* mapB) {
+cudaError_t tc_make_maps(void* arena, int ld, int nslots, int fmt, tc::Instance* inst) {
   auto enc = get_encode();
   if (!enc) return cudaErrorNotSupported;
   if (ld % tc::LD_ALIGN != 0 || (reinterpret_cast<uintptr_t>(arena) & 15) != 0) return cudaErrorInvalidValue;
@@ -917,13 +938,15 @@ cudaError_t tc_make_maps(void* arena, int ld, int nslots, int fmt, CUtensorMap* 
   cuuint64_t strides[3] = {(cuuint64_t)ld * es, (cuuint64_t)ld * ld * es, (cuuint64_t)np * ld * ld * es};
   cuuint32_t estr[4] = {1, 1, 1, 1};
   const cuuint32_t bk = (cuuint32_t)tc::bk_of(fmt);   // 128-byte rows in every format
-  cuuint32_t boxA[4] = {bk, (cuuint32_t)tc::BM, 1, 1};
-  cuuint32_t boxB[4] = {bk, (cuuint32_t)tc::BN, 1, 1};
-  CUresult r1 = enc(mapA, dt, 4, arena, dims, strides, boxA, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  CUresult r2 = enc(mapB, dt, 4, arena, dims, strides, boxB, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return (r1 == CUDA_SUCCESS && r2 == CUDA_SUCCESS) ? cudaSuccess : cudaErrorInvalidValue;
+  CUtensorMap* maps[3] = {&inst->mapA, &inst->mapB, &inst->mapN};
+  const cuuint32_t rows[3] = {(cuuint32_t)tc::BM, (cuuint32_t)tc::BN, (cuuint32_t)tc::BOX_N};
+  for (int m = 0; m < 3; ++m) {
+    cuuint32_t box[4] = {bk, rows[m], 1, 1};
+    if (enc(maps[m], dt, 4, arena, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return cudaErrorInvalidValue;
+  }
+  return cudaSuccess;
 }
 
 static int sm_count() {
@@ -937,24 +960,28 @@ static int sm_count() {
   return n;
 }
 
-// The kernel instance for a job: tile kind x piece format.
-static void* kernel_of(int pair, int fmt) {
-  if (pair) return fmt == tc::FMT_TF32X2   ? (void*)tc::tc_gemm_pair_kernel<tc::FMT_TF32X2>
-                   : fmt == tc::FMT_FP16X2 ? (void*)tc::tc_gemm_pair_kernel<tc::FMT_FP16X2>
-                                           : (void*)tc::tc_gemm_pair_kernel<tc::FMT_BF16X3>;
-  return fmt == tc::FMT_TF32X2   ? (void*)tc::tc_gemm_kernel<tc::FMT_TF32X2>
-         : fmt == tc::FMT_FP16X2 ? (void*)tc::tc_gemm_kernel<tc::FMT_FP16X2>
-                                 : (void*)tc::tc_gemm_kernel<tc::FMT_BF16X3>;
+// The kernel instance for a job: tile kind (and width) x piece format.
+template <int FMT>
+static void* kernel_of_fmt(int pair, int tn) {
+  return pair        ? (void*)tc::tc_gemm_pair_kernel<FMT>
+         : tn == 128 ? (void*)tc::tc_gemm_kernel<FMT, 128>
+         : tn == 64  ? (void*)tc::tc_gemm_kernel<FMT, 64>
+                     : (void*)tc::tc_gemm_kernel<FMT, 32>;
+}
+static void* kernel_of(int pair, int tn, int fmt) {
+  return fmt == tc::FMT_TF32X2   ? kernel_of_fmt<tc::FMT_TF32X2>(pair, tn)
+         : fmt == tc::FMT_FP16X2 ? kernel_of_fmt<tc::FMT_FP16X2>(pair, tn)
+                                 : kernel_of_fmt<tc::FMT_BF16X3>(pair, tn);
 }
 
 static cudaError_t tc_prepare() {
   static bool done = false;
   if (done) return cudaSuccess;
   cudaError_t e = cudaSuccess;
-  for (int pair = 0; pair < 2 && e == cudaSuccess; ++pair)
+  for (int kind = 0; kind < 4 && e == cudaSuccess; ++kind)   // pair, then the single widths
     for (int fmt = 0; fmt < 3 && e == cudaSuccess; ++fmt)
-      e = cudaFuncSetAttribute(kernel_of(pair, fmt), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               pair ? tc::P_SMEM_BYTES : tc::SMEM_BYTES);
+      e = cudaFuncSetAttribute(kernel_of(kind == 0, 16 << kind, fmt), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               kind == 0 ? tc::P_SMEM_BYTES : tc::SMEM_BYTES);
   if (e == cudaSuccess) done = true;
   return e;
 }
@@ -969,7 +996,7 @@ static int pair_slots() {
     cfg.blockDim = dim3(tc::P_THREADS);
     cfg.dynamicSmemBytes = tc::P_SMEM_BYTES;
     int c = 0;
-    if (cudaOccupancyMaxActiveClusters(&c, kernel_of(1, tc::FMT_BF16X3), &cfg) != cudaSuccess || c <= 0) {
+    if (cudaOccupancyMaxActiveClusters(&c, kernel_of(1, 128, tc::FMT_BF16X3), &cfg) != cudaSuccess || c <= 0) {
       (void)cudaGetLastError();
       c = sm_count() / 2;
     }
@@ -989,23 +1016,33 @@ int tc_grid_for(int total_tiles, int pair) {
   return t < s ? t : s;
 }
 
-int tc_tiles(int ld, int upper, int pair) { return pair ? tc::pair_tiles_of(ld, upper) : tc::tiles_of(ld, upper); }
+int tc_tiles(int ld, int upper, int pair, int tn) {
+  return pair ? tc::pair_tiles_of(ld, upper) : tc::tiles_of(ld, upper, tn);
+}
+
+// The narrowest width whose upper tiles all run at once, or 128 (then 128 x 128 and pair tiles compete): a launch
+// that leaves SMs idle takes the time of one tile, and a narrower tile is shorter, in its epilogue above all
+// (16 columns of it take about 3 k clocks). fp16x3 at N = 400, 10 tiles of 128 columns against 40 of 32 on 152 SMs:
+// 2.50 -> 1.73 ms a purification.
+int tc_tile_width(const int* ld, int count) {
+  for (int tn : {32, 64}) {
+    int64_t n = 0;
+    for (int i = 0; i < count; ++i) n += tc::tiles_of(ld[i], 1, tn);
+    if (n <= sm_count()) return tn;
+  }
+  return 128;
+}
+
+static dim3 tc_block(const tc::Job& job) { return dim3(job.pair ? tc::P_THREADS : tc::threads_of(job.tn)); }
+static int tc_smem(const tc::Job& job) { return job.pair ? tc::P_SMEM_BYTES : tc::SMEM_BYTES; }
 
 cudaError_t tc_launch(const tc::Job& job, cudaStream_t s) {
   cudaError_t e = tc_prepare();
   if (e != cudaSuccess) return e;
-  if (job.pair) {
-    const dim3 g(tc_grid_for(job.total_tiles, 1));
-    if (job.fmt == tc::FMT_TF32X2) tc::tc_gemm_pair_kernel<tc::FMT_TF32X2><<<g, tc::P_THREADS, tc::P_SMEM_BYTES, s>>>(job);
-    else if (job.fmt == tc::FMT_FP16X2) tc::tc_gemm_pair_kernel<tc::FMT_FP16X2><<<g, tc::P_THREADS, tc::P_SMEM_BYTES, s>>>(job);
-    else tc::tc_gemm_pair_kernel<tc::FMT_BF16X3><<<g, tc::P_THREADS, tc::P_SMEM_BYTES, s>>>(job);
-  } else {
-    const dim3 g(tc_grid_for(job.total_tiles, 0));
-    if (job.fmt == tc::FMT_TF32X2) tc::tc_gemm_kernel<tc::FMT_TF32X2><<<g, tc::THREADS, tc::SMEM_BYTES, s>>>(job);
-    else if (job.fmt == tc::FMT_FP16X2) tc::tc_gemm_kernel<tc::FMT_FP16X2><<<g, tc::THREADS, tc::SMEM_BYTES, s>>>(job);
-    else tc::tc_gemm_kernel<tc::FMT_BF16X3><<<g, tc::THREADS, tc::SMEM_BYTES, s>>>(job);
-  }
-  return cudaGetLastError();
+  tc::Job j = job;
+  void* args[] = {&j};
+  return cudaLaunchKernel(kernel_of(job.pair, job.tn, job.fmt), dim3(tc_grid_for(job.total_tiles, job.pair)),
+                          tc_block(job), args, tc_smem(job), s);
 }
 
 cudaError_t tc_add_node(cudaGraph_t g, const cudaGraphNode_t* deps, int ndeps, const tc::Job& job,
@@ -1015,10 +1052,10 @@ cudaError_t tc_add_node(cudaGraph_t g, const cudaGraphNode_t* deps, int ndeps, c
   tc::Job j = job;
   void* args[] = {&j};
   cudaKernelNodeParams kp = {};
-  kp.func = kernel_of(job.pair, job.fmt);
+  kp.func = kernel_of(job.pair, job.tn, job.fmt);
   kp.gridDim = dim3(tc_grid_for(job.total_tiles, job.pair));
-  kp.blockDim = dim3(job.pair ? tc::P_THREADS : tc::THREADS);
-  kp.sharedMemBytes = job.pair ? tc::P_SMEM_BYTES : tc::SMEM_BYTES;
+  kp.blockDim = tc_block(job);
+  kp.sharedMemBytes = (unsigned)tc_smem(job);
   kp.kernelParams = args;
   return cudaGraphAddKernelNode(node, g, deps, ndeps, &kp);
 }
@@ -1032,14 +1069,14 @@ extern "C" int32_t sp2_test_tc_gemm(const void* arena_dev, int32_t ld, int32_t n
 
 // Shared by the product test entries: one launch of the product of slots a and b, status back.
 static int32_t run_test_product(const void* arena_dev, int32_t ld, int32_t nslots, int32_t a_slot, int32_t b_slot,
-                                int32_t upper, int pair, int32_t fmt, int32_t lowprec, int32_t wait_ms,
+                                int32_t upper, int pair, int tn, int32_t fmt, int32_t lowprec, int32_t wait_ms,
                                 int32_t test_skip, float* out_dev, cudaStream_t s);
 
 extern "C" int32_t sp2_test_tc_timeout(const void* arena_dev, int32_t ld, int32_t wait_ms, float* out_dev,
                                        void* stream) {
   if (!arena_dev || !out_dev || ld <= 0 || ld % sp2::tc::LD_ALIGN != 0 || wait_ms < 1 || wait_ms > 2000)
     return SP2_ERR_INVALID_ARG;
-  return run_test_product(arena_dev, ld, 1, 0, 0, 0, 0, 0, 0, wait_ms, 1, out_dev, (cudaStream_t)stream);
+  return run_test_product(arena_dev, ld, 1, 0, 0, 0, 0, 128, 0, 0, wait_ms, 1, out_dev, (cudaStream_t)stream);
 }
 
 extern "C" int32_t sp2_build_device_checks(void) { return SP2_DEVICE_CHECKS ? 1 : 0; }
@@ -1050,27 +1087,28 @@ extern "C" int32_t sp2_test_tc_bounds(const void* arena_dev, int32_t ld, int32_t
       bad_slot >= nslots + 1024)
     return SP2_ERR_INVALID_ARG;
   if (!SP2_DEVICE_CHECKS) return SP2_ERR_UNSUPPORTED;
-  return run_test_product(arena_dev, ld, nslots, bad_slot, 0, 0, 0, 0, 0, 0, 0, out_dev, (cudaStream_t)stream);
+  return run_test_product(arena_dev, ld, nslots, bad_slot, 0, 0, 0, 128, 0, 0, 0, 0, out_dev, (cudaStream_t)stream);
 }
 
 extern "C" int32_t sp2_test_tc_gemm_ex(const void* arena_dev, int32_t ld, int32_t nslots, int32_t a_slot,
                                        int32_t b_slot, int32_t upper, int32_t tile, int32_t fmt, int32_t lowprec,
                                        float* out_dev, void* stream) {
   if (!arena_dev || !out_dev || ld <= 0 || ld % sp2::tc::LD_ALIGN != 0 || nslots <= 0 || a_slot < 0 ||
-      b_slot < 0 || a_slot >= nslots || b_slot >= nslots || (upper != 0 && upper != 1) || tile < 0 || tile > 2 ||
+      b_slot < 0 || a_slot >= nslots || b_slot >= nslots || (upper != 0 && upper != 1) || tile < 0 || tile > 4 ||
       (tile == 2 && ld % sp2::tc::PT != 0) || fmt < 0 || fmt > 2 || (lowprec != 0 && lowprec != 1))
     return SP2_ERR_INVALID_ARG;
   const int pair = tile == 2 || (tile == 0 && ld % sp2::tc::PT == 0);
-  return run_test_product(arena_dev, ld, nslots, a_slot, b_slot, upper, pair, fmt, lowprec, 0, 0, out_dev,
+  const int tn = tile == 3 ? 64 : (tile == 4 ? 32 : 128);
+  return run_test_product(arena_dev, ld, nslots, a_slot, b_slot, upper, pair, tn, fmt, lowprec, 0, 0, out_dev,
                           (cudaStream_t)stream);
 }
 
 static int32_t run_test_product(const void* arena_dev, int32_t ld, int32_t nslots, int32_t a_slot, int32_t b_slot,
-                                int32_t upper, int pair, int32_t fmt, int32_t lowprec, int32_t wait_ms,
+                                int32_t upper, int pair, int tn, int32_t fmt, int32_t lowprec, int32_t wait_ms,
                                 int32_t test_skip, float* out_dev, cudaStream_t s) {
   sp2::tc::Instance hinst;
   std::memset(&hinst, 0, sizeof(hinst));
-  if (sp2::tc_make_maps(const_cast<void*>(arena_dev), ld, nslots, fmt, &hinst.mapA, &hinst.mapB) != cudaSuccess) {
+  if (sp2::tc_make_maps(const_cast<void*>(arena_dev), ld, nslots, fmt, &hinst) != cudaSuccess) {
     (void)cudaGetLastError();
     return SP2_ERR_CUDA;
   }
@@ -1097,11 +1135,12 @@ static int32_t run_test_product(const void* arena_dev, int32_t ld, int32_t nslot
   j.rule = sp2::tc::SLOTS_FIXED;
   j.count = 1;
   j.pair = pair;
+  j.tn = tn;
   j.fmt = fmt;
   j.lowprec = lowprec;
   j.wait_ms = wait_ms;
   j.test_skip = test_skip;
-  j.total_tiles = sp2::tc_tiles(ld, upper, pair);
+  j.total_tiles = sp2::tc_tiles(ld, upper, pair, tn);
   j.inst = dinst;
   j.a_slot[0] = a_slot;
   j.b_slot[0] = b_slot;

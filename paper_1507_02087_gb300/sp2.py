@@ -257,11 +257,11 @@ def _info_dict(info) -> dict:
 def sp2_test_tc_gemm(arena, ld: int, nslots: int, a_slot: int, b_slot: int, upper: bool, out,
                      stream=None, tile: str = "auto", fmt: str = "bf16", lowprec: bool = False) -> None:
     """Tensor-core product C = A B^T over a piece arena (see include/sp2_testing.h).
-    tile: "128" (128 x 128 per SM), "pair" (256 x 256 per SM pair) or "auto"; fmt "bf16"
+    tile: "128", "64", "32" (128 rows x so many columns per SM), "pair" (256 x 256 per SM pair) or "auto"; fmt "bf16"
     (three bf16 planes per slot), "fp16" (two fp16 planes of 2^14 x) or "tf32" (two FP32 planes
     holding tf32 values); lowprec: the format's low-precision product."""
     _check(lib().sp2_test_tc_gemm_ex(arena.data_ptr(), ld, nslots, a_slot, b_slot, 1 if upper else 0,
-                                     TILES[tile], {"bf16": 0, "fp16": 1, "tf32": 2}[fmt], 1 if lowprec else 0,
+                                     {**TILES, "64": 3, "32": 4}[tile], {"bf16": 0, "fp16": 1, "tf32": 2}[fmt], 1 if lowprec else 0,
                                      out.data_ptr(), _stream_ptr(stream)), "sp2_test_tc_gemm_ex")
 
 
