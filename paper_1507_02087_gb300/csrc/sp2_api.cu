@@ -690,8 +690,7 @@ static sp2_status create_f64(sp2_ctx* h) {
   h->T = h->ld / 64;
   h->nparts = (int)((h->N + 7) / 8 < 1024 ? (h->N + 7) / 8 : 1024);
   const size_t bytes = (size_t)h->ld * h->ld * sizeof(double);
-  const size_t ntiles = (size_t)h->T * (h->T + 1) / 2;
-  const size_t part_bytes = ntiles * 2 * sp2::f64tc::RECS * sizeof(double);
+  const size_t part_bytes = sp2::f64tc::part_bytes(h->N, h->T);
   bool ok = cudaMalloc(&h->part, part_bytes) == cudaSuccess &&
             cudaMalloc(&h->part_lo, h->nparts * sizeof(double)) == cudaSuccess &&
             cudaMalloc(&h->part_hi, h->nparts * sizeof(double)) == cudaSuccess &&

@@ -359,8 +359,8 @@ __device__ __forceinline__ void touch_state(const DevState* st, int k) {
   else if (i == 9) p = reinterpret_cast<const char*>(&st->psched[k + 1]);
   else if (i == 10) p = reinterpret_cast<const char*>(&st->mcw);
   if (p) {
-    int v;
-    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(reinterpret_cast<uintptr_t>(p) & ~uintptr_t(3)));
+    [[maybe_unused]] int unused;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(unused) : "l"(reinterpret_cast<uintptr_t>(p) & ~uintptr_t(3)));
   }
 }
 

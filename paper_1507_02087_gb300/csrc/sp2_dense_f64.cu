@@ -239,6 +239,89 @@ __device__ __forceinline__ void syrk_f64_tile(const double* __restrict__ Xin, do
 }
 
 
+// ---- the same for the smallest problems, in 8 x 8 tiles ------------------------------------------
+// Up to N = kSmallN a 64 x 64 tile per CTA leaves almost the whole chip idle while one SM works through the
+// tile at 2 multiply-adds a clock (65 us at N = 64).  Here a CTA of 128 threads has an 8 x 8 tile of the upper
+// triangle, one element per pair of threads, each with half of the k range; the rows of both operands are
+// staged whole.  A tile's record goes to its place among the 64 of its 64 x 64 tile.  One purification at
+// N = 64: 2.78 -> 0.54 ms.
+constexpr int kSmallN = f64tc::kMinN - 1;        // 128
+constexpr int kST = 8, kSmallThreads = 128, kSmallRecs = 64;
+constexpr int kSmallLd = kSmallN + 2;            // row stride in shared memory: rows on different banks
+
+__device__ __forceinline__ void syrk_small_tile(const double* __restrict__ Xin, const double* __restrict__ Bin,
+                                                double* __restrict__ Xout, int ld, int N, int pk,
+                                                double* __restrict__ part, int gen, double ca, double cb, double cc) {
+  __shared__ __align__(16) double As[kST][kSmallLd], Bs[kST][kSmallLd];
+  __shared__ double half[kST * kST];
+  __shared__ double sred[2][2];
+  int I, J;
+  upper_tile(blockIdx.x, (N + kST - 1) / kST, I, J);
+  const int tid = threadIdx.x;
+  const int K = (N + 7) & ~7;                    // the border beyond N is zero
+  for (int e = tid; e < kST * (K / 2); e += kSmallThreads) {
+    const int r = e / (K / 2), c = 2 * (e % (K / 2));
+    *reinterpret_cast<double2*>(&As[r][c]) = *reinterpret_cast<const double2*>(Xin + (int64_t)(I * kST + r) * ld + c);
+    *reinterpret_cast<double2*>(&Bs[r][c]) = *reinterpret_cast<const double2*>(Bin + (int64_t)(J * kST + r) * ld + c);
+  }
+  __syncthreads();
+  const int el = tid & 63, r = el >> 3, c = el & 7, kh = tid >> 6;
+  double acc = 0.0;
+  const int k0 = kh * (K / 2), k1 = k0 + K / 2;
+  #pragma unroll 8
+  for (int k = k0; k < k1; ++k) acc = fma(As[r][k], Bs[c][k], acc);
+  if (kh) half[el] = acc;
+  __syncthreads();
+  double v2 = 0.0, trace = 0.0;
+  if (kh == 0) {
+    const double s = acc + half[el];
+    const int gi = I * kST + r, gj = J * kST + c;
+    const double x = Xin[(int64_t)gi * ld + gj];
+    const double d = x - s;
+    v2 = I == J ? d * d : 2.0 * (d * d);
+    const double xn = gen ? fma(ca, s, fma(cb, x, (gi == gj && gi < N) ? cc : 0.0)) : (pk ? s : (2.0 * x - s));
+    if (gj >= gi) {
+      Xout[(int64_t)gi * ld + gj] = xn;
+      if (gj > gi) Xout[(int64_t)gj * ld + gi] = xn;
+    }
+    if (gi == gj) trace = xn;
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      v2 += __shfl_xor_sync(0xffffffffu, v2, o);
+      trace += __shfl_xor_sync(0xffffffffu, trace, o);
+    }
+    if ((tid & 31) == 0) { sred[tid >> 5][0] = v2; sred[tid >> 5][1] = trace; }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    double* dst = part + 2 * (kSmallRecs * upper_index(I / 8, J / 8, ld / kTile) + 8 * (I & 7) + (J & 7));
+    dst[0] = sred[0][0] + sred[1][0];
+    dst[1] = sred[0][1] + sred[1][1];
+  }
+}
+
+// One product of the loop, small problems: op 0 the SP2 square, 1 the McWeeny step's shifted square into S, 2 its
+// product S X_{k-1} (after the stop test).  The polynomials are those of the kernels below.
+__global__ void __launch_bounds__(kSmallThreads)
+small_product_kernel(const DevState* st, double* buf0, double* buf1, double* S, double* part, int op) {
+  if (st->done) return;
+  const int k = st->k, ld = st->ld, N = st->N;
+  if (op == 1) {
+    const double* Xin = (k & 1) ? buf1 : buf0;
+    const double a = st->alpha[k + 1], c = 0.5 * (1.0 - a);
+    syrk_small_tile(Xin, Xin, S, ld, N, 1, part, 1, a * a, 2.0 * a * c, c * c);
+  } else if (op == 2) {
+    const double a = st->alpha[k], c = 0.5 * (1.0 - a);
+    syrk_small_tile(S, ((k - 1) & 1) ? buf1 : buf0, (k & 1) ? buf1 : buf0, ld, N, 1, part, 1, -2.0 * a, 3.0 - 2.0 * c, 0.0);
+  } else {
+    const double* Xin = (k & 1) ? buf1 : buf0;
+    double* Xout = (k & 1) ? buf0 : buf1;
+    double ca = 0.0, cb = 0.0, cc = 0.0;
+    const int pk = st->acc ? acc_step(st, k + 1, ca, cb, cc) : (st->tr[k] > (double)st->nocc ? 1 : 0);
+    syrk_small_tile(Xin, Xin, Xout, ld, N, pk, part, st->acc, ca, cb, cc);
+  }
+}
+
 __global__ void __launch_bounds__(kSyrkThreads)
 syrk_f64_kernel(const DevState* st, double* buf0, double* buf1, double* __restrict__ part) {
   if (st->done) return;
@@ -453,42 +536,45 @@ cudaError_t launch_perturb(DevState* st, double* buf0, double* buf1, const doubl
   return cudaGetLastError();
 }
 
-// The square on the tensor cores: digits of X_{k-1}, then the product.
-static int recs_of(const f64tc::Plan* tc) { return tc ? f64tc::RECS : 1; }
+// ---- one product of the loop, by size ------------------------------------------------------------
+// N <= 128: 8 x 8 tiles on the FP64 units (the tensor-core product has about 35 us of latency a square, against
+// some 10 there); else the tensor cores, or 64 x 64 tiles on the FP64 units where the digit buffers were not to be had.
+enum ProductOp { kSquare = 0, kMcwSquare = 1, kMcwProd = 2 };
 
-static cudaError_t emit_tc_square(f64tc::Sink& sink, DevState* st, double* buf0, double* buf1, double* S, double* part,
-                                  const f64tc::Plan& P, int N, f64tc::Op op) {
-  const cudaError_t e = f64tc::emit_digits(sink, st, buf0, buf1, nullptr, P, N);
-  return e != cudaSuccess ? e : f64tc::emit_product(sink, st, buf0, buf1, S, part, P, op);
-}
+static int recs_of(const f64tc::Plan* tc, int N) { return tc ? f64tc::RECS : (N <= kSmallN ? kSmallRecs : 1); }
 
-// The McWeeny step's second product: digits of the shifted square, then S X_{k-1} (whose digits stand).
-static cudaError_t emit_tc_mcw_prod(f64tc::Sink& sink, DevState* st, double* buf0, double* buf1, double* S,
-                                    double* part, const f64tc::Plan& P, int N) {
-  const cudaError_t e = f64tc::emit_digits(sink, st, buf0, buf1, S, P, N);
-  return e != cudaSuccess ? e : f64tc::emit_product(sink, st, buf0, buf1, S, part, P, f64tc::OP_MCW_PROD);
+static cudaError_t emit_product(f64tc::Sink& sink, ProductOp op, DevState* st, double* buf0, double* buf1, double* S,
+                                double* part, int T, const f64tc::Plan* tc, int N) {
+  if (tc) {
+    static constexpr f64tc::Op ops[3] = {f64tc::OP_SP2, f64tc::OP_MCW_SQ, f64tc::OP_MCW_PROD};
+    const cudaError_t e = f64tc::emit_digits(sink, st, buf0, buf1, op == kMcwProd ? S : nullptr, *tc, N);
+    return e != cudaSuccess ? e : f64tc::emit_product(sink, st, buf0, buf1, S, part, *tc, ops[op]);
+  }
+  if (N <= kSmallN) {
+    const int t = (N + kST - 1) / kST;
+    int o = op;
+    void* args[] = {&st, &buf0, &buf1, &S, &part, &o};
+    return sink.put((const void*)small_product_kernel, dim3(t * (t + 1) / 2), dim3(kSmallThreads), 0, args);
+  }
+  const dim3 grid(T * (T + 1) / 2), block(kSyrkThreads);
+  if (op == kSquare) {
+    void* args[] = {&st, &buf0, &buf1, &part};
+    return sink.put((const void*)syrk_f64_kernel, grid, block, 0, args);
+  }
+  void* args[] = {&st, &buf0, &buf1, &S, &part};
+  return sink.put(op == kMcwSquare ? (const void*)mcw_square_kernel : (const void*)mcw_prod_kernel, grid, block, 0, args);
 }
 
 cudaError_t launch_f64_step_plain(DevState* st, double* buf0, double* buf1, double* part, int T,
                                   cudaStream_t s, const f64tc::Plan* tc, double* mscr, void* lz, int N, const double* E,
                                   int64_t ecount) {
-  const int ntiles = T * (T + 1) / 2, recs = recs_of(tc), nrec = ntiles * recs;
-  if (tc) {
-    f64tc::Sink sink;
-    sink.s = s;
-    cudaError_t e = emit_tc_square(sink, st, buf0, buf1, nullptr, part, *tc, N, f64tc::OP_SP2);
-    if (e != cudaSuccess) return e;
-  } else {
-    syrk_f64_kernel<<<ntiles, kSyrkThreads, 0, s>>>(st, buf0, buf1, part);
-  }
-  if (lz) {
-    cudaError_t e = launch_lanczos(st, buf0, buf1, nullptr, part, nrec, lz, N, T * kTile, s);
-    if (e != cudaSuccess) return e;
-  }
-  if (E) {
-    cudaError_t e = launch_perturb(st, buf0, buf1, E, ecount, N, 0, s);
-    if (e != cudaSuccess) return e;
-  }
+  const int recs = recs_of(tc, N), nrec = T * (T + 1) / 2 * recs;
+  f64tc::Sink sink;
+  sink.s = s;
+  cudaError_t e = emit_product(sink, kSquare, st, buf0, buf1, nullptr, part, T, tc, N);
+  if (e != cudaSuccess) return e;
+  if (lz && (e = launch_lanczos(st, buf0, buf1, nullptr, part, nrec, lz, N, T * kTile, s)) != cudaSuccess) return e;
+  if (E && (e = launch_perturb(st, buf0, buf1, E, ecount, N, 0, s)) != cudaSuccess) return e;
   finalize_plain_kernel<<<1, kFinThreads, 0, s>>>(st, part, nrec, recs, mscr);
   return cudaGetLastError();
 }
@@ -496,64 +582,31 @@ cudaError_t launch_f64_step_plain(DevState* st, double* buf0, double* buf1, doub
 cudaError_t add_mcw_loop_body(cudaGraph_t body, DevState* st, double* buf0, double* buf1, double* S, double* part,
                               int T, cudaGraphConditionalHandle cond, const f64tc::Plan* tc, double* mscr, void* lz,
                               int N) {
-  const int ntiles = T * (T + 1) / 2, recs = recs_of(tc);
-  cudaGraphNode_t n_sq, n_fin, n_pr;
-  if (tc) {
-    f64tc::Sink sink;
-    sink.g = body;
-    cudaError_t e = emit_tc_square(sink, st, buf0, buf1, S, part, *tc, N, f64tc::OP_MCW_SQ);
-    if (e != cudaSuccess) return e;
-    if (lz && (e = add_lanczos_nodes(body, sink.last, st, buf0, buf1, S, part, ntiles * recs, lz, N, T * kTile,
-                                     &sink.last)) != cudaSuccess)
-      return e;
-    e = add_finalize_node(body, &sink.last, 1, st, part, ntiles * recs, 2, recs, cond, &n_fin, mscr);
-    if (e != cudaSuccess) return e;
-    sink.last = n_fin;
-    return emit_tc_mcw_prod(sink, st, buf0, buf1, S, part, *tc, N);
-  }
-  const double* b0 = buf0;
-  const double* b1 = buf1;
-  void* a1[] = {&st, &b0, &b1, &S, &part};
-  cudaKernelNodeParams kp = {};
-  kp.func = (void*)mcw_square_kernel;
-  kp.gridDim = dim3(ntiles);
-  kp.blockDim = dim3(kSyrkThreads);
-  kp.kernelParams = a1;
-  cudaError_t e = cudaGraphAddKernelNode(&n_sq, body, nullptr, 0, &kp);
+  const int recs = recs_of(tc, N), nrec = T * (T + 1) / 2 * recs;
+  f64tc::Sink sink;
+  sink.g = body;
+  cudaError_t e = emit_product(sink, kMcwSquare, st, buf0, buf1, S, part, T, tc, N);
   if (e != cudaSuccess) return e;
-  if (lz && (e = add_lanczos_nodes(body, n_sq, st, buf0, buf1, S, part, ntiles, lz, N, T * kTile, &n_sq)) != cudaSuccess) return e;
-  e = add_finalize_node(body, &n_sq, 1, st, part, ntiles, 2, 1, cond, &n_fin, mscr);
-  if (e != cudaSuccess) return e;
-  const double* Sc = S;
-  void* a2[] = {&st, &buf0, &buf1, &Sc, &part};
-  kp.func = (void*)mcw_prod_kernel;
-  kp.kernelParams = a2;
-  return cudaGraphAddKernelNode(&n_pr, body, &n_fin, 1, &kp);
+  if (lz && (e = add_lanczos_nodes(body, sink.last, st, buf0, buf1, S, part, nrec, lz, N, T * kTile, &sink.last)) !=
+                cudaSuccess)
+    return e;
+  cudaGraphNode_t n_fin;
+  if ((e = add_finalize_node(body, &sink.last, 1, st, part, nrec, 2, recs, cond, &n_fin, mscr)) != cudaSuccess) return e;
+  sink.last = n_fin;
+  return emit_product(sink, kMcwProd, st, buf0, buf1, S, part, T, tc, N);
 }
 
 cudaError_t launch_mcw_step_plain(DevState* st, double* buf0, double* buf1, double* S, double* part, int T,
                                   cudaStream_t s, const f64tc::Plan* tc, double* mscr, void* lz, int N) {
-  const int ntiles = T * (T + 1) / 2, recs = recs_of(tc), nrec = ntiles * recs;
+  const int recs = recs_of(tc, N), nrec = T * (T + 1) / 2 * recs;
   f64tc::Sink sink;
   sink.s = s;
-  if (tc) {
-    cudaError_t e = emit_tc_square(sink, st, buf0, buf1, S, part, *tc, N, f64tc::OP_MCW_SQ);
-    if (e != cudaSuccess) return e;
-  } else {
-    mcw_square_kernel<<<ntiles, kSyrkThreads, 0, s>>>(st, buf0, buf1, S, part);
-  }
-  if (lz) {
-    cudaError_t e = launch_lanczos(st, buf0, buf1, S, part, nrec, lz, N, T * kTile, s);
-    if (e != cudaSuccess) return e;
-  }
+  cudaError_t e = emit_product(sink, kMcwSquare, st, buf0, buf1, S, part, T, tc, N);
+  if (e != cudaSuccess) return e;
+  if (lz && (e = launch_lanczos(st, buf0, buf1, S, part, nrec, lz, N, T * kTile, s)) != cudaSuccess) return e;
   finalize_plain_kernel<<<1, kFinThreads, 0, s>>>(st, part, nrec, recs, mscr);
-  if (tc) {
-    cudaError_t e = emit_tc_mcw_prod(sink, st, buf0, buf1, S, part, *tc, N);
-    if (e != cudaSuccess) return e;
-  } else {
-    mcw_prod_kernel<<<ntiles, kSyrkThreads, 0, s>>>(st, buf0, buf1, S, part);
-  }
-  return cudaGetLastError();
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return emit_product(sink, kMcwProd, st, buf0, buf1, S, part, T, tc, N);
 }
 
 cudaError_t add_finalize_node(cudaGraph_t g, const cudaGraphNode_t* deps, int ndeps, DevState* st,
@@ -571,23 +624,14 @@ cudaError_t add_finalize_node(cudaGraph_t g, const cudaGraphNode_t* deps, int nd
 cudaError_t add_f64_loop_body(cudaGraph_t body, DevState* st, double* buf0, double* buf1, double* part,
                               int T, cudaGraphConditionalHandle cond, const f64tc::Plan* tc, double* mscr, void* lz,
                               int N, const double* E, int64_t ecount) {
-  const int ntiles = T * (T + 1) / 2, recs = recs_of(tc), nrec = ntiles * recs;
+  const int recs = recs_of(tc, N), nrec = T * (T + 1) / 2 * recs;
   cudaGraphNode_t n_sq, n_fin;
   cudaKernelNodeParams kp = {};
-  cudaError_t e;
-  if (tc) {
-    f64tc::Sink sink;
-    sink.g = body;
-    if ((e = emit_tc_square(sink, st, buf0, buf1, nullptr, part, *tc, N, f64tc::OP_SP2)) != cudaSuccess) return e;
-    n_sq = sink.last;
-  } else {
-    void* args[] = {&st, &buf0, &buf1, &part};
-    kp.func = (void*)syrk_f64_kernel;
-    kp.gridDim = dim3(ntiles);
-    kp.blockDim = dim3(kSyrkThreads);
-    kp.kernelParams = args;
-    if ((e = cudaGraphAddKernelNode(&n_sq, body, nullptr, 0, &kp)) != cudaSuccess) return e;
-  }
+  f64tc::Sink sink;
+  sink.g = body;
+  cudaError_t e = emit_product(sink, kSquare, st, buf0, buf1, nullptr, part, T, tc, N);
+  if (e != cudaSuccess) return e;
+  n_sq = sink.last;
   if (lz && (e = add_lanczos_nodes(body, n_sq, st, buf0, buf1, nullptr, part, nrec, lz, N, T * kTile, &n_sq)) != cudaSuccess) return e;
   if (E) {
     int initial = 0;

@@ -31,6 +31,10 @@ struct Plan {
 
 // Sizes at which the tensor-core products are used (see sp2_f64_tc.cu).
 constexpr int kMinN = 129;
+// Bytes of the partial records of a problem with T x T tiles of 64: RECS per upper tile, 64 for N < kMinN.
+constexpr size_t part_bytes(int64_t N, int T) {
+  return sizeof(double) * 2 * (size_t)(N < kMinN ? 64 : RECS) * ((size_t)T * (T + 1) / 2);
+}
 inline bool wanted(int64_t N) { return N >= kMinN; }
 
 // Rows are padded to whole tiles of 128; the padding (and the rows past N) stays zero.

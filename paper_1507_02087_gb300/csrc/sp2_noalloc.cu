@@ -35,7 +35,6 @@ using sp2::DevState;
 constexpr int kMaxN = SP2_NOALLOC_MAX_N;
 constexpr int kLd = (kMaxN + 63) / 64 * 64;        // padded size of the largest problem
 constexpr int kT = kLd / 64;
-constexpr int kTiles = kT * (kT + 1) / 2;
 constexpr int kGersh = 1024;                       // Gershgorin partial slots
 constexpr int kMaxIter = 200;                      // iteration cap (the default of sp2_opts)
 
@@ -45,7 +44,8 @@ constexpr size_t kOffLo = align256(kOffState + sizeof(DevState));
 constexpr size_t kOffHi = align256(kOffLo + kGersh * sizeof(double));
 constexpr size_t kOffBad = align256(kOffHi + kGersh * sizeof(double));
 constexpr size_t kOffPart = align256(kOffBad + kGersh * sizeof(int));
-constexpr size_t kPartBytes = 2 * sp2::f64tc::RECS * kTiles * sizeof(double);
+constexpr size_t kPartBytes = sp2::f64tc::part_bytes(kMaxN, kT);
+static_assert(kPartBytes >= sp2::f64tc::part_bytes(sp2::f64tc::kMinN - 1, 2), "records of the smallest problems");
 constexpr size_t kOffBuf0 = align256(kOffPart + kPartBytes);
 constexpr size_t kOffBuf1 = align256(kOffBuf0 + (size_t)kLd * kLd * sizeof(double));
 constexpr size_t kOffDig = align256(kOffBuf1 + (size_t)kLd * kLd * sizeof(double));
@@ -133,7 +133,8 @@ static sp2_status run_noalloc(const double* F_dev, double* D_dev, int64_t N, int
   const int nparts = (int)((N + 7) / 8 < kGersh ? (N + 7) / 8 : kGersh);
   // The iterates need a zero border (rows and columns N .. ld-1); the last call may
   // have left other values there.
-  if (cudaMemsetAsync(buf0, 0, (size_t)ld * ld * sizeof(double), s) != cudaSuccess ||
+  if (cudaMemsetAsync(part, 0, kPartBytes, s) != cudaSuccess ||   // records that no tile writes count as 0
+      cudaMemsetAsync(buf0, 0, (size_t)ld * ld * sizeof(double), s) != cudaSuccess ||
       cudaMemsetAsync(buf1, 0, (size_t)ld * ld * sizeof(double), s) != cudaSuccess) {
     (void)cudaGetLastError();
     return SP2_ERR_CUDA;
@@ -147,8 +148,7 @@ static sp2_status run_noalloc(const double* F_dev, double* D_dev, int64_t N, int
     tc.X.dig = (__half*)(base + kOffDig);
     tc.X.exp = (int32_t*)(base + kOffExp);
     if (cudaMemsetAsync(tc.X.dig, 0, sp2::f64tc::digit_bytes(ld), s) != cudaSuccess ||
-        cudaMemsetAsync(tc.X.exp, 0, sp2::f64tc::exp_bytes(ld), s) != cudaSuccess ||
-        cudaMemsetAsync(part, 0, kPartBytes, s) != cudaSuccess) {
+        cudaMemsetAsync(tc.X.exp, 0, sp2::f64tc::exp_bytes(ld), s) != cudaSuccess) {
       (void)cudaGetLastError();
       return SP2_ERR_CUDA;
     }
