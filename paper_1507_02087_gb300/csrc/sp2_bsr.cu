@@ -1174,6 +1174,7 @@ static sp2_status build_graph(sp2_bsr_ctx* h) {
   (void)numeric_grid();
   (void)meta_sms();
   tc_prepare();
+  if (h->lz) BSR_TRY(lanczos_prepare());
   cudaStream_t cs;
   BSR_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
   cudaError_t e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);

@@ -63,6 +63,8 @@ cudaError_t launch_mcw_step_plain(DevState* st, double* buf0, double* buf1, doub
 // McWeeny step's shifted square (null for SP2 / SP2-ACC); part / ntiles are the square's
 // (v^2, trace) partial records, whose v^2 sum sets the FP32 scaling of X - X^2.
 size_t lanczos_scratch_bytes(int ld);
+// Kernel attributes of the estimate (before any stream capture).
+cudaError_t lanczos_prepare();
 cudaError_t add_lanczos_nodes(cudaGraph_t g, cudaGraphNode_t dep, DevState* st, const double* buf0,
                               const double* buf1, const double* S, const double* part, int ntiles, void* lz,
                               int N, int ld, cudaGraphNode_t* last);

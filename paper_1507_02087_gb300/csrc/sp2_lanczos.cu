@@ -16,13 +16,17 @@
 // Per estimate: start (1 CTA: coefficients, start vector, a power-of-two scale 2^-s with 2^s near
 // v_{k-1} from the square's Frobenius partials), form (A 2^-s rounded to FP32 once: the ld x ld
 // FP32 matrix, half the bytes of one FP64 iterate, is then read kLzSteps times, from L2 where it
-// fits), kLzSteps x step (w = A q_j, one warp per row, FP32 products summed in FP32 per lane and
-// FP64 across lanes; the last CTA to finish, found by an atomic ticket after a fence, runs the
-// FP64 three-term update, so no CTA waits on another), eig (1 warp).  The FP32 rounding of A and
+// fits), kLzSteps x step, eig (1 CTA).  Step j first finishes step j - 1: every CTA sums the partials of
+// alpha_{j-1}, forms r = w - alpha q_{j-1} - beta q_{j-2}, ||r|| and q_j = r / ||r|| for all N entries by itself
+// (FP64; 2 N clocks of the SM's FP64 units), then multiplies its rows: w = A q_j, one warp per row, FP32 products
+// summed in FP32 per lane and FP64 across lanes.  The steps thus have one launch between them and no CTA that
+// the others wait for: with the last CTA to finish doing the update alone, a step took 15 us at N = 1001, most of
+// it in that CTA's serial FP64 sums.  The FP32 rounding of A and
 // of the products perturbs A by about 1e-7 of its norm, far below the Lanczos truncation error.
 #include <math.h>
 
 #include "sp2_common.cuh"
+#include "sp2_f64_tc.cuh"
 #include "sp2_kernels.h"
 #include "sp2_tc.cuh"
 
@@ -31,21 +35,22 @@ namespace {
 
 constexpr int kLzSteps = 32;          // Lanczos steps per estimate
 constexpr int kLzThreads = 1024;      // start: one CTA
-constexpr int kLzMvThreads = 512;     // step: 16 warps, one row per warp at a time
-constexpr int kLzMvBlocks = 152 * 2;  // step grid cap = number of partial sums
-constexpr int kSturmRounds = 6;       // 33^6 > 2^30: below FP32 resolution of the interval
+constexpr int kLzMvBlocks = 152;      // step grid cap (one CTA per SM) = number of partial sums
+constexpr int kLzMvThreads = 1024;    // threads of a step: 512 while the grid cap is not reached, else 1024
+constexpr int kLzSmemN = 16384;       // q_j in shared memory up to this size
+constexpr int kSturmThreads = 1024;   // 512 points per side
+constexpr int kSturmRounds = 3;       // 513^3 > 2^27: below FP32 resolution of the interval
 
 struct LzScratch {
   double scale;               // 2^-s applied before rounding A to FP32
-  int32_t m;                  // completed steps
+  int32_t m;                  // finished steps (alpha[0 .. m-1])
   int32_t live;               // 0 once the Krylov space is invariant (beta = 0) or not finite
-  uint32_t ticket;            // CTAs of the current step that have finished their rows
-  int32_t _pad;
   double alpha[kLzSteps];     // diagonal of the tridiagonal matrix
   double beta[kLzSteps + 1];  // beta[j] couples q_{j-1} and q_j; beta[0] = 0
-  double part[kLzMvBlocks];   // per-CTA partials of q_j . A q_j
+  double part[2][kLzMvBlocks];  // per-CTA partials of q_j . A q_j, by the parity of j
 };
-// followed by q_{j-1}, q_j, w (FP64, ld each), q_j in FP32 (ld) and A 2^-s in FP32 (ld x ld)
+// followed by three vectors q (q_j in j % 3) and two w (w_j in j % 2), FP64, ld each, q_j in FP32 (ld; used for
+// N > kLzSmemN) and A 2^-s in FP32 (ld x ld)
 
 constexpr size_t kVecOff = (sizeof(LzScratch) + 255) / 256 * 256;
 
@@ -53,7 +58,7 @@ __device__ __forceinline__ double* lz_vec(LzScratch* lz, int ld, int which) {
   return reinterpret_cast<double*>(reinterpret_cast<char*>(lz) + kVecOff) + (size_t)which * ld;
 }
 __device__ __forceinline__ float* lz_q32(LzScratch* lz, int ld) {
-  return reinterpret_cast<float*>(lz_vec(lz, ld, 3));
+  return reinterpret_cast<float*>(lz_vec(lz, ld, 5));
 }
 __device__ __forceinline__ float* lz_a32(LzScratch* lz, int ld) { return lz_q32(lz, ld) + ld; }
 
@@ -92,15 +97,16 @@ __device__ __forceinline__ void lz_operands(const DevState* st, const double* bu
 __global__ void __launch_bounds__(kLzThreads)
 lz_start_kernel(const DevState* st, const double* __restrict__ part, int ntiles, const int* ntiles_dev, int rec,
                 LzScratch* lz, int N, int ld) {
-  __shared__ double sm[32];
+  __shared__ double sm[96];
   if (st->done) return;
   const int cnt = ntiles_dev ? *ntiles_dev : ntiles;
-  double v2 = 0.0;                               // v_{k-1}^2 from the square's partials
+  double v2 = 0.0, ss = 0.0, none = 0.0;         // v_{k-1}^2 from the square's partials
   for (int t = threadIdx.x; t < cnt; t += kLzThreads) v2 += part[rec * (int64_t)t];
-  v2 = block_sum<kLzThreads>(v2, sm);
-  double* qp = lz_vec(lz, ld, 0);
-  double* q = lz_vec(lz, ld, 1);
-  float* q32 = lz_q32(lz, ld);
+  for (int i = threadIdx.x; i < N; i += kLzThreads) {
+    const double u = start_entry(i);
+    ss = fma(u, u, ss);
+  }
+  block_sum3<kLzThreads>(v2, ss, none, kLzThreads, sm);
   if (threadIdx.x == 0) {
     const double v = sqrt(v2);
     int e = (v > 0.0 && isfinite(v)) ? ilogb(v) : 0;
@@ -108,23 +114,11 @@ lz_start_kernel(const DevState* st, const double* __restrict__ part, int ntiles,
     lz->scale = ldexp(1.0, -e);
     lz->m = 0;
     lz->live = 1;
-    lz->ticket = 0;
     lz->beta[0] = 0.0;
   }
-  double ss = 0.0;
-  for (int i = threadIdx.x; i < ld; i += kLzThreads) {
-    const double u = i < N ? start_entry(i) : 0.0;
-    q[i] = u;
-    qp[i] = 0.0;
-    ss = fma(u, u, ss);
-  }
-  ss = block_sum<kLzThreads>(ss, sm);
+  double* q = lz_vec(lz, ld, 0);
   const double inv = 1.0 / sqrt(ss);
-  for (int i = threadIdx.x; i < ld; i += kLzThreads) {
-    const double u = q[i] * inv;
-    q[i] = u;
-    q32[i] = (float)u;
-  }
+  for (int i = threadIdx.x; i < N; i += kLzThreads) q[i] = start_entry(i) * inv;
 }
 
 // A 2^-s = ((a + b) X_{k-1} - Y + c I) (2^-s / a), rounded to FP32, over the whole ld x ld
@@ -184,23 +178,94 @@ __global__ void lz_form_tc_kernel(const DevState* st, const tc::Instance* inst, 
   }
 }
 
-// One Lanczos step: w = A q_j (one warp per row, FP32 products, 16-byte loads) and the CTA's
-// share of q_j . w; the last CTA to finish its rows then computes alpha_j = q_j . w,
-// r = w - alpha_j q_j - beta_j q_{j-1}, beta_{j+1} = ||r|| and q_{j+1} = r / beta_{j+1} in FP64.
+// Sum over the CTA (fixed order), the result in every thread; sm: 33 doubles.
+__device__ __forceinline__ double cta_sum(double x, double* sm) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  #pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  if (lane == 0) sm[warp] = x;
+  __syncthreads();
+  if (warp == 0) {
+    double t = lane < nw ? sm[lane] : 0.0;
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) sm[32] = t;
+  }
+  __syncthreads();
+  return sm[32];
+}
+
+// Step j of the recurrence (see the header): q_j for all entries, then w_j and the CTA's share of alpha_j for its
+// rows.  Vectors alternate, so no CTA writes what another may still read.
 __global__ void __launch_bounds__(kLzMvThreads)
 lz_step_kernel(const DevState* st, LzScratch* lz, int j, int N, int ld) {
-  __shared__ double sm[32];
-  __shared__ int s_last;
+  extern __shared__ __align__(16) float lz_smem[];
+  __shared__ double sm[2][33];
+  __shared__ double s_alpha;
   if (st->done || !lz->live) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  float* q32 = N <= kLzSmemN ? lz_smem : lz_q32(lz, ld);   // past it every CTA writes the same values
+  double* q = lz_vec(lz, ld, j % 3);
+  const int per = nw;                                       // rows of a CTA per sweep: one per warp
+  auto mine = [&](int i) { return (i / per) % (int)gridDim.x == (int)blockIdx.x; };
+  if (j == 0) {
+    for (int i = threadIdx.x; i < ld; i += blockDim.x) q32[i] = i < N ? (float)q[i] : 0.f;
+  } else {
+    const double* q1 = lz_vec(lz, ld, (j + 2) % 3);         // q_{j-1}
+    const double* q2 = lz_vec(lz, ld, (j + 1) % 3);         // q_{j-2}
+    const double* w1 = lz_vec(lz, ld, 3 + ((j - 1) & 1));
+    if (warp == 0) {
+      double a = 0.0;
+      for (int t = lane; t < (int)gridDim.x; t += 32) a += lz->part[(j - 1) & 1][t];
+      #pragma unroll
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (lane == 0) s_alpha = a;
+    }
+    __syncthreads();
+    const double a = s_alpha, bj = lz->beta[j - 1];
+    double ss = 0.0;
+    auto residual = [&](int i) { return w1[i] - a * q1[i] - (j > 1 ? bj * q2[i] : 0.0); };
+    double keep[4];                                         // this thread's first entries, kept for the second pass
+    #pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      const int i = threadIdx.x + n * blockDim.x;
+      keep[n] = i < N ? residual(i) : 0.0;
+      ss = fma(keep[n], keep[n], ss);
+    }
+    for (int i = threadIdx.x + 4 * blockDim.x; i < N; i += blockDim.x) {
+      const double r = residual(i);
+      ss = fma(r, r, ss);
+    }
+    ss = cta_sum(ss, sm[0]);
+    const double b = sqrt(ss);
+    const bool finite = isfinite(a) && isfinite(b);
+    const bool more = finite && b > 1e-300;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      lz->alpha[j - 1] = finite ? a : __longlong_as_double(0x7ff8000000000000ll);
+      lz->m = j;
+      lz->beta[j] = b;
+      if (!more) lz->live = 0;
+    }
+    if (!more) return;
+    const double ib = 1.0 / b;
+    auto put = [&](int i, double u) {
+      q32[i] = (float)u;
+      if (i < N && mine(i)) q[i] = u;
+    };
+    #pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      const int i = threadIdx.x + n * blockDim.x;
+      if (i < ld) put(i, keep[n] * ib);
+    }
+    for (int i = threadIdx.x + 4 * blockDim.x; i < ld; i += blockDim.x) put(i, i < N ? residual(i) * ib : 0.0);
+  }
+  __syncthreads();
   const float4* __restrict__ A = reinterpret_cast<const float4*>(lz_a32(lz, ld));
-  const float4* __restrict__ q4 = reinterpret_cast<const float4*>(lz_q32(lz, ld));
-  double* qp = lz_vec(lz, ld, 0);
-  double* q = lz_vec(lz, ld, 1);
-  double* w = lz_vec(lz, ld, 2);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float4* q4 = reinterpret_cast<const float4*>(q32);
+  double* w = lz_vec(lz, ld, 3 + (j & 1));
   const int h = ld / 4;
   double pa = 0.0;
-  for (int r = blockIdx.x * (kLzMvThreads / 32) + warp; r < N; r += gridDim.x * (kLzMvThreads / 32)) {
+  for (int r = blockIdx.x * per + warp; r < N; r += gridDim.x * per) {
     const float4* ar = A + (int64_t)r * h;
     float s0 = 0.f, s1 = 0.f;
     int i = lane;
@@ -221,48 +286,8 @@ lz_step_kernel(const DevState* st, LzScratch* lz, int j, int N, int ld) {
       pa = fma(q[r], s, pa);
     }
   }
-  if (lane == 0) __threadfence();                // this warp's w rows, before the ticket
-  pa = block_sum<kLzMvThreads>(pa, sm);
-  if (threadIdx.x == 0) {
-    lz->part[blockIdx.x] = pa;
-    __threadfence();
-    s_last = atomicAdd(&lz->ticket, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-
-  // the last CTA: every row of w and every partial is written
-  double a = 0.0;
-  for (int t = threadIdx.x; t < (int)gridDim.x; t += kLzMvThreads) a += __ldcg(&lz->part[t]);
-  a = block_sum<kLzMvThreads>(a, sm);
-  const double bj = lz->beta[j];
-  double ss = 0.0;
-  for (int i = threadIdx.x; i < N; i += kLzMvThreads) {
-    const double r = __ldcg(&w[i]) - a * q[i] - bj * qp[i];
-    w[i] = r;
-    ss = fma(r, r, ss);
-  }
-  ss = block_sum<kLzMvThreads>(ss, sm);
-  const double b = sqrt(ss);
-  const bool finite = isfinite(a) && isfinite(b);
-  const bool more = j + 1 < kLzSteps && finite && b > 1e-300;
-  if (threadIdx.x == 0) {
-    lz->alpha[j] = finite ? a : __longlong_as_double(0x7ff8000000000000ll);
-    lz->m = j + 1;
-    if (j + 1 < kLzSteps) lz->beta[j + 1] = b;
-    if (!more) lz->live = 0;
-    lz->ticket = 0;
-  }
-  if (!more) return;
-  const double ib = 1.0 / b;
-  float* q32 = lz_q32(lz, ld);
-  for (int i = threadIdx.x; i < N; i += kLzMvThreads) {
-    const double u = w[i] * ib;
-    qp[i] = q[i];
-    q[i] = u;
-    q32[i] = (float)u;
-  }
+  pa = cta_sum(pa, sm[1]);
+  if (threadIdx.x == 0) lz->part[j & 1][blockIdx.x] = pa;
 }
 
 // Number of eigenvalues of the m x m tridiagonal (alpha, beta) below x: the count of negative
@@ -280,54 +305,75 @@ __device__ __forceinline__ int sturm_count(const float* al, const float* be2, in
   return cnt;
 }
 
-__global__ void __launch_bounds__(32)
-lz_eig_kernel(DevState* st, const LzScratch* lz) {
+// Closes the last step (alpha from its partials, `blocks` of them) and takes the extreme eigenvalues of the
+// tridiagonal matrix: 512 threads per side, each a point of the bracket.
+__global__ void __launch_bounds__(kSturmThreads)
+lz_eig_kernel(DevState* st, const LzScratch* lz, int blocks) {
   __shared__ float al[kLzSteps], be2[kLzSteps];
+  __shared__ int s_bad, s_cnt[2];
+  __shared__ float s_lo[2], s_hi[2];
   if (st->done) return;
-  const int lane = threadIdx.x;
-  const int m = lz->m;
-  bool bad = m < 1;
-  if (lane < m) {
-    const double a = lz->alpha[lane], b = lane ? lz->beta[lane] : 0.0;
-    bad = bad || !isfinite(a) || !isfinite(b) || fabs(a) > 1e30 || fabs(b) > 1e15;
-    al[lane] = (float)a;
-    be2[lane] = (float)(b * b);
+  const int tid = threadIdx.x, lane = tid & 31, side = tid >> 9, pt = tid & 511;
+  const int done = lz->m;                        // finished in the steps; a live run has one more to close
+  const int m = done + (lz->live ? 1 : 0);
+  if (tid < 32) {
+    double last = 0.0;
+    for (int t = lane; t < blocks; t += 32) last += lz->part[(m - 1) & 1][t];
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) last += __shfl_xor_sync(0xffffffffu, last, o);
+    bool bad = m < 1;
+    if (lane < m) {
+      const double a = lane < done ? lz->alpha[lane] : last, b = lane ? lz->beta[lane] : 0.0;
+      bad = bad || !isfinite(a) || !isfinite(b) || fabs(a) > 1e30 || fabs(b) > 1e15;
+      al[lane] = (float)a;
+      be2[lane] = (float)(b * b);
+    }
+    bad = __any_sync(0xffffffffu, bad);
+    __syncwarp();
+    if (lane == 0) s_bad = bad;
+    // Gershgorin interval of T
+    float lo = INFINITY, hi = -INFINITY;
+    if (!bad && lane < m) {
+      const float rad = sqrtf(be2[lane]) + (lane + 1 < m ? sqrtf(be2[lane + 1]) : 0.0f);
+      lo = al[lane] - rad;
+      hi = al[lane] + rad;
+    }
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    if (lane == 0) {
+      const float pad = 1e-30f + 0x1p-20f * fmaxf(fabsf(lo), fabsf(hi));
+      s_lo[0] = s_lo[1] = lo - pad;              // brackets of the largest (side 0) and the smallest (side 1)
+      s_hi[0] = s_hi[1] = hi + pad;
+    }
   }
-  bad = __any_sync(0xffffffffu, bad);
-  __syncwarp();
-  if (bad) {
-    if (lane == 0) st->spec_e = __longlong_as_double(0x7ff8000000000000ll);
+  __syncthreads();
+  if (s_bad) {
+    if (tid == 0) st->spec_e = __longlong_as_double(0x7ff8000000000000ll);
     return;
   }
-  float lo = INFINITY, hi = -INFINITY;
-  for (int i = 0; i < m; ++i) {                  // Gershgorin interval of T
-    const float rad = sqrtf(be2[i]) + (i + 1 < m ? sqrtf(be2[i + 1]) : 0.0f);
-    lo = fminf(lo, al[i] - rad);
-    hi = fmaxf(hi, al[i] + rad);
-  }
-  const float pad = 1e-30f + 0x1p-20f * fmaxf(fabsf(lo), fabsf(hi));
-  lo -= pad;
-  hi += pad;
-  float lo1 = lo, hi1 = hi, lo2 = lo, hi2 = hi;  // brackets of the largest and the smallest
   for (int round = 0; round < kSturmRounds; ++round) {
-    const float f = (float)(lane + 1) / 33.0f;
-    const float x1 = lo1 + (hi1 - lo1) * f;
-    const float x2 = lo2 + (hi2 - lo2) * f;
-    // largest: the points with fewer than m eigenvalues below them form a prefix
-    const int L = __popc(__ballot_sync(0xffffffffu, sturm_count(al, be2, m, x1) <= m - 1));
-    // smallest: the points with no eigenvalue below them form a prefix
-    const int S = __popc(__ballot_sync(0xffffffffu, sturm_count(al, be2, m, x2) == 0));
-    const float xl1 = __shfl_sync(0xffffffffu, x1, L > 0 ? L - 1 : 0);
-    const float xh1 = __shfl_sync(0xffffffffu, x1, L < 32 ? L : 31);
-    const float xl2 = __shfl_sync(0xffffffffu, x2, S > 0 ? S - 1 : 0);
-    const float xh2 = __shfl_sync(0xffffffffu, x2, S < 32 ? S : 31);
-    if (L > 0) lo1 = xl1;
-    if (L < 32) hi1 = xh1;
-    if (S > 0) lo2 = xl2;
-    if (S < 32) hi2 = xh2;
+    if (tid < 2) s_cnt[tid] = 0;
+    __syncthreads();
+    const float lo = s_lo[side], hi = s_hi[side];
+    auto point = [&](int i) { return lo + (hi - lo) * ((float)(i + 1) / 513.0f); };
+    const int c = sturm_count(al, be2, m, point(pt));
+    // largest: the points with fewer than m eigenvalues below them form a prefix; smallest: those with none
+    const unsigned v = __ballot_sync(0xffffffffu, side == 0 ? c <= m - 1 : c == 0);
+    if (lane == 0) atomicAdd(&s_cnt[side], __popc(v));
+    __syncthreads();
+    const int n = s_cnt[side];
+    __syncthreads();
+    if (pt == 0) {
+      if (n > 0) s_lo[side] = point(n - 1);
+      if (n < 512) s_hi[side] = point(n);
+    }
+    __syncthreads();
   }
-  if (lane == 0) {
-    const double top = 0.5 * ((double)lo1 + (double)hi1), bot = 0.5 * ((double)lo2 + (double)hi2);
+  if (tid == 0) {
+    const double top = 0.5 * ((double)s_lo[0] + (double)s_hi[0]), bot = 0.5 * ((double)s_lo[1] + (double)s_hi[1]);
     st->spec_e = fmax(fabs(top), fabs(bot)) / lz->scale;
   }
 }
@@ -358,10 +404,13 @@ __global__ void lz_form_pairs_kernel(const DevState* st, const int* __restrict__
   }
 }
 
+// Step launch: a row per warp, 16 warps a CTA up to the grid cap, then 32.
+int step_threads(int N) { return N <= 16 * kLzMvBlocks ? 512 : kLzMvThreads; }
 int step_blocks(int N) {
-  const int b = (N + kLzMvThreads / 32 - 1) / (kLzMvThreads / 32);
+  const int per = step_threads(N) / 32, b = (N + per - 1) / per;
   return b < kLzMvBlocks ? (b < 1 ? 1 : b) : kLzMvBlocks;
 }
+int step_smem(int N, int ld) { return N <= kLzSmemN ? 4 * ld : 0; }
 
 int form_blocks(int ld) {
   const int64_t b = ((int64_t)ld * (ld / 2) + 255) / 256;
@@ -370,63 +419,73 @@ int form_blocks(int ld) {
 
 }  // namespace
 
+cudaError_t lanczos_prepare() {
+  static bool done = false;
+  if (done) return cudaSuccess;
+  const cudaError_t e =
+      cudaFuncSetAttribute(lz_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kLzSmemN + 4096);
+  done = e == cudaSuccess;
+  return e;
+}
+
 size_t lanczos_scratch_bytes(int ld) {
-  return kVecOff + 3 * sizeof(double) * (size_t)ld + sizeof(float) * ((size_t)ld + (size_t)ld * ld);
+  return kVecOff + 5 * sizeof(double) * (size_t)ld + sizeof(float) * ((size_t)ld + (size_t)ld * ld);
+}
+
+// start, form (the caller's kernel and arguments), the steps and eig, on a stream or as a chain of graph nodes.
+static cudaError_t emit(f64tc::Sink& sink, DevState* st, const double* part, int ntiles, const int* ntiles_dev, int rec,
+                        LzScratch* lz, int N, int ld, const void* form, void** form_args, const void* fill = nullptr,
+                        void** fill_args = nullptr) {
+  cudaError_t e = lanczos_prepare();
+  if (e != cudaSuccess) return e;
+  const DevState* cst = st;
+  const LzScratch* clz = lz;
+  void* a0[] = {&cst, &part, &ntiles, &ntiles_dev, &rec, &lz, &N, &ld};
+  if ((e = sink.put((const void*)lz_start_kernel, dim3(1), dim3(kLzThreads), 0, a0)) != cudaSuccess) return e;
+  if (fill && (e = sink.put(fill, dim3(form_blocks(ld)), dim3(256), 0, fill_args)) != cudaSuccess) return e;
+  if ((e = sink.put(form, dim3(form_blocks(ld)), dim3(256), 0, form_args)) != cudaSuccess) return e;
+  for (int j = 0; j < kLzSteps; ++j) {
+    void* a[] = {&cst, &lz, &j, &N, &ld};
+    e = sink.put((const void*)lz_step_kernel, dim3(step_blocks(N)), dim3(step_threads(N)), step_smem(N, ld), a);
+    if (e != cudaSuccess) return e;
+  }
+  int blocks = step_blocks(N);
+  void* a1[] = {&st, &clz, &blocks};
+  return sink.put((const void*)lz_eig_kernel, dim3(1), dim3(kSturmThreads), 0, a1);
+}
+
+static cudaError_t emit_f64(f64tc::Sink& sink, DevState* st, const double* buf0, const double* buf1, const double* S,
+                            const double* part, int ntiles, void* scratch, int N, int ld) {
+  LzScratch* lz = static_cast<LzScratch*>(scratch);
+  const DevState* cst = st;
+  void* form[] = {&cst, &buf0, &buf1, &S, &lz};
+  return emit(sink, st, part, ntiles, nullptr, 2, lz, N, ld, (const void*)lz_form_kernel, form);
+}
+
+static cudaError_t emit_tc(f64tc::Sink& sink, DevState* st, const tc::Instance* inst, const double* part, int nparts,
+                           void* scratch, int N, int ld) {
+  LzScratch* lz = static_cast<LzScratch*>(scratch);
+  const DevState* cst = st;
+  void* form[] = {&cst, &inst, &lz};
+  return emit(sink, st, part, nparts, nullptr, 4, lz, N, ld, (const void*)lz_form_tc_kernel, form);
 }
 
 cudaError_t add_lanczos_nodes(cudaGraph_t g, cudaGraphNode_t dep, DevState* st, const double* buf0,
                               const double* buf1, const double* S, const double* part, int ntiles, void* scratch,
                               int N, int ld, cudaGraphNode_t* last) {
-  LzScratch* lz = static_cast<LzScratch*>(scratch);
-  const DevState* cst = st;
-  cudaKernelNodeParams kp = {};
-  cudaGraphNode_t prev = dep, node;
-  const int* no_count = nullptr;
-  int rec = 2;
-  void* a0[] = {&cst, &part, &ntiles, &no_count, &rec, &lz, &N, &ld};
-  kp.func = (void*)lz_start_kernel;
-  kp.gridDim = dim3(1);
-  kp.blockDim = dim3(kLzThreads);
-  kp.kernelParams = a0;
-  cudaError_t e = cudaGraphAddKernelNode(&node, g, &prev, 1, &kp);
-  if (e != cudaSuccess) return e;
-  prev = node;
-  void* a1[] = {&cst, &buf0, &buf1, &S, &lz};
-  kp.func = (void*)lz_form_kernel;
-  kp.gridDim = dim3(form_blocks(ld));
-  kp.blockDim = dim3(256);
-  kp.kernelParams = a1;
-  if ((e = cudaGraphAddKernelNode(&node, g, &prev, 1, &kp)) != cudaSuccess) return e;
-  prev = node;
-  for (int j = 0; j < kLzSteps; ++j) {
-    int jj = j;
-    void* a2[] = {&cst, &lz, &jj, &N, &ld};
-    kp.func = (void*)lz_step_kernel;
-    kp.gridDim = dim3(step_blocks(N));
-    kp.blockDim = dim3(kLzMvThreads);
-    kp.kernelParams = a2;
-    if ((e = cudaGraphAddKernelNode(&node, g, &prev, 1, &kp)) != cudaSuccess) return e;
-    prev = node;
-  }
-  const LzScratch* clz = lz;
-  void* a3[] = {&st, &clz};
-  kp.func = (void*)lz_eig_kernel;
-  kp.gridDim = dim3(1);
-  kp.blockDim = dim3(32);
-  kp.kernelParams = a3;
-  e = cudaGraphAddKernelNode(&node, g, &prev, 1, &kp);
-  *last = node;
+  f64tc::Sink sink;
+  sink.g = g;
+  sink.last = dep;
+  const cudaError_t e = emit_f64(sink, st, buf0, buf1, S, part, ntiles, scratch, N, ld);
+  *last = sink.last;
   return e;
 }
 
 cudaError_t launch_lanczos(DevState* st, const double* buf0, const double* buf1, const double* S,
                            const double* part, int ntiles, void* scratch, int N, int ld, cudaStream_t s) {
-  LzScratch* lz = static_cast<LzScratch*>(scratch);
-  lz_start_kernel<<<1, kLzThreads, 0, s>>>(st, part, ntiles, nullptr, 2, lz, N, ld);
-  lz_form_kernel<<<form_blocks(ld), 256, 0, s>>>(st, buf0, buf1, S, lz);
-  for (int j = 0; j < kLzSteps; ++j) lz_step_kernel<<<step_blocks(N), kLzMvThreads, 0, s>>>(st, lz, j, N, ld);
-  lz_eig_kernel<<<1, 32, 0, s>>>(st, lz);
-  return cudaGetLastError();
+  f64tc::Sink sink;
+  sink.s = s;
+  return emit_f64(sink, st, buf0, buf1, S, part, ntiles, scratch, N, ld);
 }
 
 // Tensor-core path, one problem: the estimate for the square just written into `inst`'s arena;
@@ -434,67 +493,31 @@ cudaError_t launch_lanczos(DevState* st, const double* buf0, const double* buf1,
 cudaError_t add_lanczos_tc_nodes(cudaGraph_t g, cudaGraphNode_t dep, DevState* st, const tc::Instance* inst,
                                  const double* part, int nparts, void* scratch, int N, int ld,
                                  cudaGraphNode_t* last) {
-  LzScratch* lz = static_cast<LzScratch*>(scratch);
-  const DevState* cst = st;
-  cudaKernelNodeParams kp = {};
-  cudaGraphNode_t prev = dep, node;
-  const int* no_count = nullptr;
-  int rec = 4;
-  void* a0[] = {&cst, &part, &nparts, &no_count, &rec, &lz, &N, &ld};
-  kp.func = (void*)lz_start_kernel;
-  kp.gridDim = dim3(1);
-  kp.blockDim = dim3(kLzThreads);
-  kp.kernelParams = a0;
-  cudaError_t e = cudaGraphAddKernelNode(&node, g, &prev, 1, &kp);
-  if (e != cudaSuccess) return e;
-  prev = node;
-  void* a1[] = {&cst, &inst, &lz};
-  kp.func = (void*)lz_form_tc_kernel;
-  kp.gridDim = dim3(form_blocks(ld));
-  kp.blockDim = dim3(256);
-  kp.kernelParams = a1;
-  if ((e = cudaGraphAddKernelNode(&node, g, &prev, 1, &kp)) != cudaSuccess) return e;
-  prev = node;
-  for (int j = 0; j < kLzSteps; ++j) {
-    int jj = j;
-    void* a2[] = {&cst, &lz, &jj, &N, &ld};
-    kp.func = (void*)lz_step_kernel;
-    kp.gridDim = dim3(step_blocks(N));
-    kp.blockDim = dim3(kLzMvThreads);
-    kp.kernelParams = a2;
-    if ((e = cudaGraphAddKernelNode(&node, g, &prev, 1, &kp)) != cudaSuccess) return e;
-    prev = node;
-  }
-  const LzScratch* clz = lz;
-  void* a3[] = {&st, &clz};
-  kp.func = (void*)lz_eig_kernel;
-  kp.gridDim = dim3(1);
-  kp.blockDim = dim3(32);
-  kp.kernelParams = a3;
-  e = cudaGraphAddKernelNode(&node, g, &prev, 1, &kp);
-  *last = node;
+  f64tc::Sink sink;
+  sink.g = g;
+  sink.last = dep;
+  const cudaError_t e = emit_tc(sink, st, inst, part, nparts, scratch, N, ld);
+  *last = sink.last;
   return e;
 }
 
 cudaError_t launch_lanczos_tc(DevState* st, const tc::Instance* inst, const double* part, int nparts, void* scratch,
                               int N, int ld, cudaStream_t s) {
-  LzScratch* lz = static_cast<LzScratch*>(scratch);
-  lz_start_kernel<<<1, kLzThreads, 0, s>>>(st, part, nparts, nullptr, 4, lz, N, ld);
-  lz_form_tc_kernel<<<form_blocks(ld), 256, 0, s>>>(st, inst, lz);
-  for (int j = 0; j < kLzSteps; ++j) lz_step_kernel<<<step_blocks(N), kLzMvThreads, 0, s>>>(st, lz, j, N, ld);
-  lz_eig_kernel<<<1, 32, 0, s>>>(st, lz);
-  return cudaGetLastError();
+  f64tc::Sink sink;
+  sink.s = s;
+  return emit_tc(sink, st, inst, part, nparts, scratch, N, ld);
 }
 
 cudaError_t launch_lanczos_pairs(DevState* st, const int* row, const int* col, const int* nnz_p, const double* part,
                                  void* scratch, int nb, int ld, cudaStream_t s) {
   LzScratch* lz = static_cast<LzScratch*>(scratch);
-  lz_start_kernel<<<1, kLzThreads, 0, s>>>(st, part, 0, nnz_p, 2, lz, nb, ld);
-  lz_zero_kernel<<<form_blocks(ld), 256, 0, s>>>(st, lz, ld);
-  lz_form_pairs_kernel<<<form_blocks(ld), 256, 0, s>>>(st, row, col, nnz_p, part, lz, ld);
-  for (int j = 0; j < kLzSteps; ++j) lz_step_kernel<<<step_blocks(nb), kLzMvThreads, 0, s>>>(st, lz, j, nb, ld);
-  lz_eig_kernel<<<1, 32, 0, s>>>(st, lz);
-  return cudaGetLastError();
+  const DevState* cst = st;
+  f64tc::Sink sink;
+  sink.s = s;
+  void* fill[] = {&cst, &lz, &ld};
+  void* form[] = {&cst, &row, &col, &nnz_p, &part, &lz, &ld};
+  return emit(sink, st, part, 0, nnz_p, 2, lz, nb, ld, (const void*)lz_form_pairs_kernel, form,
+              (const void*)lz_zero_kernel, fill);
 }
 
 }  // namespace sp2
