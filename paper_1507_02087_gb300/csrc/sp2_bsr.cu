@@ -816,11 +816,34 @@ __global__ void set_kept_bits_kernel(const DevState* st, Pairs P, const uint8_t*
   }
 }
 
-// kept upper block q -> row I at the rank of J, its transpose -> row J at the rank of I
+// kept upper block q -> row I at the rank of J, its transpose -> row J at the rank of I.  Each thread has 4 values
+// of a row; the transpose goes through shared memory, so that every store is 8 or 16 bytes of a row (as single
+// values with a stride of a row they bounded the kernel: 0.84 ms a square on the 32 x 24 x 24 lattice, 0.15 now).
+// Bound by memory: 4 KB read and, with pieces, 16 KB written per pair.
 __global__ void __launch_bounds__(NT)
 fill_next_kernel(const DevState* st, Pairs P, const uint8_t* skeep, const float* svals, Mat Y, int W) {
+  __shared__ float t[B][B + 1];
   if (st && !st->iter_active) return;
   const int nnz = *P.nnz;
+  const int r = threadIdx.x >> 3, c = 4 * (threadIdx.x & 7);
+  auto put = [&](int pos, float4 v) {
+    *reinterpret_cast<float4*>(Y.vals + (int64_t)pos * BE + r * B + c) = v;
+    if (Y.pvals) {   // the fp16 pieces of 2^14 v, the tensor-core operands
+      __half p[2][4];
+      tc::split_fp16x2(v.x, p[0][0], p[1][0]);
+      tc::split_fp16x2(v.y, p[0][1], p[1][1]);
+      tc::split_fp16x2(v.z, p[0][2], p[1][2]);
+      tc::split_fp16x2(v.w, p[0][3], p[1][3]);
+      char* dst = reinterpret_cast<char*>(Y.pvals) + (int64_t)pos * 4 * BE + 2 * (c & 7);
+      #pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        uint2 o;
+        o.x = __half_as_ushort(p[a][0]) | ((uint32_t)__half_as_ushort(p[a][1]) << 16);
+        o.y = __half_as_ushort(p[a][2]) | ((uint32_t)__half_as_ushort(p[a][3]) << 16);
+        *reinterpret_cast<uint2*>(dst + piece_offset(a, r, c & ~7)) = o;
+      }
+    }
+  };
   for (int q = blockIdx.x; q < nnz; q += gridDim.x) {
     if (!skeep[q]) continue;
     const int I = P.row[q], J = P.col[q];
@@ -830,22 +853,13 @@ fill_next_kernel(const DevState* st, Pairs P, const uint8_t* skeep, const float*
       Y.ci[pij] = J;
       Y.ci[pji] = I;
     }
-    const float* src = svals + (int64_t)q * BE;
-    for (int e = threadIdx.x; e < BE; e += NT) {
-      const float v = src[e];
-      const int64_t et = (e % B) * B + e / B;
-      Y.vals[(int64_t)pij * BE + e] = v;
-      if (I != J) Y.vals[(int64_t)pji * BE + et] = v;
-      if (Y.pvals) {   // the fp16 pieces of 2^14 v, the tensor-core operands
-        __half p0, p1;
-        tc::split_fp16x2(v, p0, p1);
-        Y.pvals[(int64_t)pij * 2 * BE + e] = p0;
-        Y.pvals[(int64_t)pij * 2 * BE + BE + e] = p1;
-        if (I != J) {
-          Y.pvals[(int64_t)pji * 2 * BE + et] = p0;
-          Y.pvals[(int64_t)pji * 2 * BE + BE + et] = p1;
-        }
-      }
+    const float4 v = *reinterpret_cast<const float4*>(svals + (int64_t)q * BE + r * B + c);
+    put(pij, v);
+    if (I != J) {
+      t[r][c] = v.x; t[r][c + 1] = v.y; t[r][c + 2] = v.z; t[r][c + 3] = v.w;
+      __syncthreads();
+      put(pji, make_float4(t[c][r], t[c + 1][r], t[c + 2][r], t[c + 3][r]));
+      __syncthreads();
     }
   }
 }
@@ -1022,7 +1036,6 @@ struct sp2_bsr_ctx {
   bool ran = false;
   // tensor-core block products (opts.bsr_cuda_cores == 0)
   bool tc = false;
-  TcMaps* maps_dev = nullptr;    // TMA maps over X[0].pvals and X[1].pvals
   int* tiles = nullptr;          // [ceil(nb/4) * ceil(nb/8)]
   int* tptr = nullptr;           // [ceil(nb/4) + 1]
   int* tnnz = nullptr;
@@ -1049,7 +1062,7 @@ static void bsr_free(sp2_bsr_ctx* h) {
     cudaFree(h->X[p].rp); cudaFree(h->X[p].ci); cudaFree(h->X[p].vals); cudaFree(h->X[p].bits);
     cudaFree(h->X[p].rank); cudaFree(h->X[p].pvals);
   }
-  cudaFree(h->maps_dev); cudaFree(h->tiles); cudaFree(h->tptr); cudaFree(h->tnnz); cudaFree(h->meta);
+  cudaFree(h->tiles); cudaFree(h->tptr); cudaFree(h->tnnz); cudaFree(h->meta);
   cudaFree(h->S.ptr); cudaFree(h->S.col); cudaFree(h->S.row); cudaFree(h->S.nnz);
   cudaFree(h->FP.ptr); cudaFree(h->FP.col); cudaFree(h->FP.row); cudaFree(h->FP.nnz);
   cudaFree(h->sbits); cudaFree(h->svals); cudaFree(h->skeep); cudaFree(h->spart); cudaFree(h->sn2);
@@ -1135,7 +1148,7 @@ static cudaError_t add_round(sp2_bsr_ctx* h, cudaGraph_t g, cudaStream_t s, int 
     r.tiles = h->tiles;
     r.tnnz = h->tnnz;
     r.meta = h->meta;
-    tc_numeric_launch(st, Xc, h->maps_dev, parity, nb, W, r, s);
+    tc_numeric_launch(st, Xc, nb, W, r, s);
   } else {
     bsr_numeric_kernel<<<numeric_grid(), NUM_THREADS, NUM_SMEM, s>>>(st, Xc, W, h->S, h->svals, h->skeep,
                                                                     h->spart, h->sn2, tau2);
@@ -1154,7 +1167,7 @@ static cudaError_t add_round(sp2_bsr_ctx* h, cudaGraph_t g, cudaStream_t s, int 
   rank_kernel<<<nb, 32, 0, s>>>(Xn.bits, nb, W, Xn.rank, st);
   row_counts_kernel<<<nb, 64, 0, s>>>(Xn.bits, nb, W, 0, h->counts, st);
   scan_kernel<<<1, 1024, 0, s>>>(h->counts, nb, Xn.rp, nullptr, st);
-  fill_next_kernel<<<grid_persistent(), NT, 0, s>>>(st, h->S, h->skeep, h->svals, Xn, W);
+  fill_next_kernel<<<2 * grid_persistent(), NT, 0, s>>>(st, h->S, h->skeep, h->svals, Xn, W);
   return cudaGetLastError();
 }
 
@@ -1256,18 +1269,10 @@ extern "C" sp2_status sp2_create_bsr_ex(int64_t N, int64_t n_occ, double tau, in
     for (int p = 0; p < 2 && ok; ++p)
       ok = cudaMalloc(&h->X[p].pvals, pbytes) == cudaSuccess &&
            cudaMemset(h->X[p].pvals, 0, pbytes) == cudaSuccess;   // block `cap` stays zero
-    ok = ok && cudaMalloc(&h->maps_dev, sizeof(TcMaps)) == cudaSuccess &&
-         cudaMalloc(&h->tiles, sizeof(int) * (size_t)ng * ncg) == cudaSuccess &&
+    ok = ok && cudaMalloc(&h->tiles, sizeof(int) * (size_t)ng * ncg) == cudaSuccess &&
          cudaMalloc(&h->tptr, sizeof(int) * (ng + 1)) == cudaSuccess &&
          cudaMalloc(&h->tnnz, sizeof(int)) == cudaSuccess &&
          cudaMalloc(&h->meta, sizeof(int) * TMETA * (size_t)ng * ncg) == cudaSuccess;
-    if (ok) {
-      TcMaps m;
-      std::memset(&m, 0, sizeof(m));
-      ok = tc_piece_map(h->X[0].pvals, h->cap, &m.map[0]) == cudaSuccess &&
-           tc_piece_map(h->X[1].pvals, h->cap, &m.map[1]) == cudaSuccess &&
-           cudaMemcpy(h->maps_dev, &m, sizeof(m), cudaMemcpyHostToDevice) == cudaSuccess;
-    }
   }
   if (ok && rule == SP2_TRUNC_MIXED) ok = cudaMalloc(&h->mixscr, mixctl_scratch_bytes(nb)) == cudaSuccess;
   if (ok && o.norm == 1) {
@@ -1372,7 +1377,7 @@ extern "C" sp2_status sp2_run_bsr(sp2_bsr h, const int32_t* row_ptr_dev, const i
   rank_kernel<<<nb, 32, 0, s>>>(X0.bits, nb, W, X0.rank, nullptr);
   row_counts_kernel<<<nb, 64, 0, s>>>(X0.bits, nb, W, 0, h->counts, nullptr);
   scan_kernel<<<1, 1024, 0, s>>>(h->counts, nb, X0.rp, nullptr, nullptr);
-  fill_next_kernel<<<grid_persistent(), NT, 0, s>>>(nullptr, h->FP, h->skeep, h->svals, X0, W);
+  fill_next_kernel<<<2 * grid_persistent(), NT, 0, s>>>(nullptr, h->FP, h->skeep, h->svals, X0, W);
   BSR_TRY(cudaGetLastError());
   // the loop: rounds in pairs (X[0] -> X[1] -> X[0]) until the device-side stop
   BSR_TRY(cudaEventRecord(h->ev[0], s));

@@ -3,7 +3,6 @@
 // block products).
 #pragma once
 
-#include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -24,9 +23,16 @@ struct Mat {          // one block-sparse iterate
   float* vals;        // [cap][32][32]
   uint32_t* bits;     // [nb][W]
   int* rank;          // [nb][W]: set bits of the row in words before w
-  __half* pvals;      // [cap + 1][2][32][32]: each block as two fp16 pieces of 2^14 x (the operands of
-                      // the tensor-core products); block `cap` is all zero and stands for absent blocks
+  __half* pvals;      // [cap + 1] blocks of 4 KB: each block as two fp16 pieces of 2^14 x (the operands of
+                      // the tensor-core products) in the order of the shared-memory stages (piece_offset);
+                      // block `cap` is all zero and stands for absent blocks
 };
+
+// Byte offset of piece p of columns c .. c + 7 (c a multiple of 8) of row r in a block of pvals: groups of 8 rows,
+// in each the two pieces, 8 rows x 64 bytes with the 16-byte chunks exchanged as the 64-byte swizzle wants.
+__host__ __device__ constexpr int piece_offset(int p, int r, int c) {
+  return (r >> 3) * 1024 + p * 512 + (r & 7) * 64 + (((c >> 3) ^ ((r >> 1) & 3)) * 16);
+}
 
 struct Pairs {        // upper (I, J >= I) block pairs of a pattern
   int* ptr;           // [nb + 1]
@@ -48,10 +54,6 @@ __device__ __forceinline__ int find_block(const Mat& m, int W, int I, int K) {
 // per round in row-major tile order.
 constexpr int TTR = 4;             // block rows per tile
 constexpr int TTC = 8;             // block columns per tile
-
-struct TcMaps {                    // TMA maps over the piece planes of the two ping-pong iterates
-  CUtensorMap map[2];
-};
 
 // The inputs of one round's tensor-core square besides the iterate: the square's pattern bits
 // (upper part, one row per block row), its pair list, and the per-pair outputs the truncation and
@@ -79,12 +81,9 @@ cudaError_t tc_tiles_launch(const DevState* st, const Mat& X, const Pairs& P, co
                             int* counts, int* tptr, int* tnnz, int* tiles, int* meta, cudaStream_t s);
 // The numeric square of the round on the tensor cores: X_k = p_k(X~_{k-1}) for every upper pair
 // of the square's pattern, with the per-pair partials, block norms and keep flags.
-cudaError_t tc_numeric_launch(DevState* st, const Mat& X, const TcMaps* maps, int parity, int nb, int W,
-                              const TcRound& r, cudaStream_t s);
+cudaError_t tc_numeric_launch(DevState* st, const Mat& X, int nb, int W, const TcRound& r, cudaStream_t s);
 // Device queries and kernel attributes of the tensor-core square (before any stream capture).
 void tc_prepare();
-// TMA map over the piece planes of an iterate with `cap` blocks (+ the zero block).
-cudaError_t tc_piece_map(const __half* pvals, int64_t cap, CUtensorMap* map);
 
 }  // namespace bsr
 }  // namespace sp2

@@ -8,8 +8,9 @@
 // S[I0.., J0..] = sum over K of X[I0.., K] X[J0.., K]^T (X symmetric), the sum over the K blocks
 // that one of the tile's 4 rows and one of its 8 columns both hold; a block a row lacks is the
 // all-zero block.  Each iterate keeps, beside its FP32 blocks, every block as two fp16 pieces of
-// 2^14 x (the FMT_FP16X2 format of the dense path), so a K block is 12 TMA boxes of 32 x 32 per
-// piece into one ring stage, and a tile's product is the three piece products p0 q0 + p0 q1 +
+// 2^14 x (the FMT_FP16X2 format of the dense path) in the order of a ring stage, so a K block is 12 contiguous
+// copies of 4 KB (as 24 tensor-map boxes of 32 rows x 64 bytes they bounded the kernel: 6.2 ms a square on the
+// 32 x 24 x 24 lattice, 2.9 now, with the epilogue's loop and its halved FP64 work), and a tile's product is the three piece products p0 q0 + p0 q1 +
 // p1 q0 per 16-wide k-step, accumulated in tensor memory in chunks of 4 K blocks (24 truncating
 // FP32 additions, as on the dense path) and added into registers with round-to-nearest additions.
 //
@@ -19,8 +20,6 @@
 // warps per tensor-memory lane quadrant = block row, 128 columns = 4 blocks each) and run the
 // epilogue of the tile's pairs.  Every wait is bounded (2 s); a wait that gives up records
 // SP2_ERR_TIMEOUT in the run's state, ends the run and winds the kernel down.
-#include <cudaTypedefs.h>
-
 #include <cstring>
 
 #include "../../include/sp2.h"
@@ -34,10 +33,10 @@ namespace bsr {
 using namespace sp2::ptx;
 
 constexpr int TSTG = 4;                            // ring stages, one K block each
-constexpr int PIECE_BYTES = B * B * 2;             // one 32 x 32 fp16 piece
-constexpr int A_PLANE = TTR * PIECE_BYTES;         // the 128 rows of one piece of A
-constexpr int B_PLANE = TTC * PIECE_BYTES;         // the 256 rows of one piece of B
-constexpr int TSTAGE = 2 * (A_PLANE + B_PLANE);    // 48 KB
+constexpr int BLK = 4 * BE;                        // a block's two pieces
+constexpr int GRP = BLK / 4;                       // its 8-row groups, both pieces
+constexpr int A_BYTES = TTR * BLK;                 // the 128 rows of A
+constexpr int TSTAGE = (TTR + TTC) * BLK;          // 48 KB
 constexpr int TSMEM = TSTG * TSTAGE + 1024;        // + alignment slack
 constexpr int TCHK = 4;                            // K blocks per tensor-memory chunk
 constexpr int TN = TTC * B;                        // 256 accumulator columns per chunk buffer
@@ -59,8 +58,6 @@ constexpr int TMAXW = 64;                          // bitmap words per row (nb <
 struct TcArgs {
   DevState* st;
   Mat X;
-  const TcMaps* maps;
-  int parity;
   int nb, W, ncg;                                  // ncg: column groups of 8 blocks
   int zero_blk;                                    // index of the all-zero block
   int64_t pair_cap;                                // capacity of the square's pair arrays
@@ -103,7 +100,6 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
     setmaxnreg_dec<T_REG_CTRL>();
     if (warp == 0) {
       // ---------------- K-block discovery + TMA producer ----------------
-      const CUtensorMap* map = &a.maps->map[a.parity];
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -145,21 +141,17 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
               ok = false;
               break;
             }
-            // lane j < 12 copies its own block's two pieces: row j of A (j < 4) or row j - 4 of B;
-            // the expected bytes are armed first, so no copy can complete the phase early
+            // lane j < 12 copies its own block: row j of A (j < 4) or row j - 4 of B; the expected bytes are
+            // armed first, so no copy can complete the phase early
             if (lane == 0) {
               mbar_arrive_expect_tx(&full_bar[stage], TSTAGE);
               armed[stage] = 1;
               armed_par[stage] = phase;
             }
             __syncwarp();
-            if (lane < TTR + TTC) {
-              uint8_t* dst = smem + stage * TSTAGE +
-                             (lane < TTR ? lane * PIECE_BYTES : 2 * A_PLANE + (lane - TTR) * PIECE_BYTES);
-              const int plane = lane < TTR ? A_PLANE : B_PLANE;
-              tma_load_3d(dst, map, 0, 0, 2 * posj, &full_bar[stage]);
-              tma_load_3d(dst + plane, map, 0, 0, 2 * posj + 1, &full_bar[stage]);
-            }
+            if (lane < TTR + TTC)
+              bulk_load(smem + stage * TSTAGE + lane * BLK, reinterpret_cast<const char*>(X.pvals) + (int64_t)posj * BLK, BLK,
+                        &full_bar[stage]);
             if (++stage == TSTG) { stage = 0; phase ^= 1; }
           }
         }
@@ -191,19 +183,18 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
               if (abort_s || !mbar_wait(&full_bar[stage], phase, globaltimer_ns() + kTcWaitNs)) { ok = false; break; }
               tc_fence_after();
               const uint32_t sA = smem_u32(smem + stage * TSTAGE);
-              const uint32_t sB = sA + 2 * A_PLANE;
+              const uint32_t sB = sA + A_BYTES;
+              auto piece = [](uint32_t base, int p, int kk) { return smem_desc_sw64_stride(base + p * (GRP / 2) + kk * 32, GRP); };
               #pragma unroll
               for (int kk = 0; kk < B / 16; ++kk) {
                 // p1 q0 and p0 q1 of the whole K block first, then p0 q0: the small products are
                 // added while the accumulator is still small
-                mma_bf16(dt, smem_desc_sw64(sA + 1 * A_PLANE + kk * 32), smem_desc_sw64(sB + kk * 32), idesc,
-                         accumulate);
+                mma_bf16(dt, piece(sA, 1, kk), piece(sB, 0, kk), idesc, accumulate);
                 accumulate = 1;
-                mma_bf16(dt, smem_desc_sw64(sA + kk * 32), smem_desc_sw64(sB + 1 * B_PLANE + kk * 32), idesc, 1);
+                mma_bf16(dt, piece(sA, 0, kk), piece(sB, 1, kk), idesc, 1);
               }
               #pragma unroll
-              for (int kk = 0; kk < B / 16; ++kk)
-                mma_bf16(dt, smem_desc_sw64(sA + kk * 32), smem_desc_sw64(sB + kk * 32), idesc, 1);
+              for (int kk = 0; kk < B / 16; ++kk) mma_bf16(dt, piece(sA, 0, kk), piece(sB, 0, kk), idesc, 1);
               mma_commit(&empty_bar[stage]);
               if (++stage == TSTG) { stage = 0; phase ^= 1; }
             }
@@ -239,17 +230,12 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
       const int I0 = (code / a.ncg) * TTR, J0 = (code % a.ncg) * TTC;
       const int* meta = a.r.meta + (int64_t)t * TMETA;
       const int nk = meta[0];
-      int qis[4], pos[4];
-      #pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        qis[g] = meta[1 + TTC * q + 4 * hc + g];
-        pos[g] = meta[33 + TTC * q + 4 * hc + g];
-      }
       float acc[4][32];
       #pragma unroll
       for (int g = 0; g < 4; ++g)
         #pragma unroll
         for (int j = 0; j < 32; ++j) acc[g][j] = 0.f;
+      uint32_t trow = 0;
       for (int k0 = 0; k0 < nk; k0 += TCHK) {
         int got = 0;
         if (lane == 0) got = !abort_s && mbar_wait(&accf_bar[buf], bphase, globaltimer_ns() + kTcWaitNs);
@@ -260,7 +246,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
           break;
         }
         tc_fence_after();
-        const uint32_t trow = tmem_base + (uint32_t)(buf * TN + hc * 128) + ((uint32_t)(32 * q) << 16);
+        trow = tmem_base + (uint32_t)(buf * TN + hc * 128) + ((uint32_t)(32 * q) << 16);
         #pragma unroll
         for (int g = 0; g < 4; ++g) {
           uint32_t raw[32];
@@ -269,20 +255,27 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
           #pragma unroll
           for (int j = 0; j < 32; ++j) acc[g][j] += __uint_as_float(raw[j]);
         }
+        if (k0 + TCHK >= nk) break;          // this buffer takes the sums for the epilogue
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&acce_bar[buf]);
         if (++buf == 2) { buf = 0; bphase ^= 1; }
       }
       if (!ok) break;
-      // epilogue of the tile's upper pairs in this warp's four blocks; lane = row of the block
+      if (nk > 0) {
+        #pragma unroll
+        for (int g = 0; g < 4; ++g) tmem_st32(trow + 32 * g, acc[g]);
+        tmem_wait_st();
+      }
+      // epilogue of the tile's upper pairs in this warp's four blocks; lane = row of the block.  A loop over the
+      // blocks, their sums taken back from tensor memory: four copies of its code are bound by the instruction fetch
       const int I = I0 + q;
-      #pragma unroll
+      #pragma unroll 1
       for (int g = 0; g < 4; ++g) {
         const int J = J0 + 4 * hc + g;
-        const int qi = qis[g];               // -1: not an upper pair of the square's pattern
+        const int qi = meta[1 + TTC * q + 4 * hc + g];   // -1: not an upper pair of the square's pattern
         if (qi < 0 || !dcheck(qi < a.pair_cap, &st->status)) continue;
-        int po = pos[g];
+        int po = meta[33 + TTC * q + 4 * hc + g];
         if (po >= 0 && !dcheck(po < a.zero_blk, &st->status)) po = -1;
         float old[32];
         if (po >= 0) {
@@ -297,8 +290,18 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
           for (int j = 0; j < 32; ++j) old[j] = 0.f;
         }
         float sv32[32];
-        #pragma unroll
-        for (int j = 0; j < 32; ++j) sv32[j] = acc[g][j] * tc::kF16InvScale2;
+        {
+          uint32_t raw[32];
+          if (nk > 0) {
+            tmem_ld32(trow + 32 * g, raw);
+            tmem_wait_ld();
+          } else {
+            #pragma unroll
+            for (int j = 0; j < 32; ++j) raw[j] = 0u;
+          }
+          #pragma unroll
+          for (int j = 0; j < 32; ++j) sv32[j] = __uint_as_float(raw[j]) * tc::kF16InvScale2;
+        }
         float4* dst = reinterpret_cast<float4*>(a.r.svals + (int64_t)qi * BE + lane * B);
         if (I == J) {
           // a diagonal block of the square: the tensor cores sum (r, c) and (c, r) in different
@@ -313,7 +316,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
             if (j < lane) sv32[j] = blk[j * B + lane];
           __syncwarp();
         }
-        float vloc = 0.f;
+        float vloc = 0.f, diag = 0.f;
         double trloc = 0.0, rs = 0.0;
         float nwv[32];
         #pragma unroll
@@ -323,18 +326,20 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
                        : (pk ? sv : fmaf(2.0f, old[j], -sv));
           const float d = old[j] - sv;
           vloc = fmaf(d, d, vloc);
-          if (I == J && lane == j) trloc += (double)nwv[j];
+          if (lane == j) diag = nwv[j];
           const double x = (double)nwv[j];
-          rs = __dadd_rn(rs, __dmul_rn(x, x));          // row `lane`, left to right
+          rs = __fma_rn(x, x, rs);                      // row `lane`, left to right (the square is exact)
         }
         #pragma unroll
         for (int v = 0; v < 8; ++v) dst[v] = make_float4(nwv[4 * v], nwv[4 * v + 1], nwv[4 * v + 2], nwv[4 * v + 3]);
         double n2 = 0.0;                                  // then the rows top to bottom
         for (int rr = 0; rr < 32; ++rr) n2 = __dadd_rn(n2, __shfl_sync(0xffffffffu, rs, rr));
         #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          vloc += __shfl_xor_sync(0xffffffffu, vloc, o);
-          trloc += __shfl_xor_sync(0xffffffffu, trloc, o);
+        for (int o = 16; o > 0; o >>= 1) vloc += __shfl_xor_sync(0xffffffffu, vloc, o);
+        if (I == J) {
+          trloc = (double)diag;
+          #pragma unroll
+          for (int o = 16; o > 0; o >>= 1) trloc += __shfl_xor_sync(0xffffffffu, trloc, o);
         }
         if (lane == 0) {
           a.r.spart[2 * (int64_t)qi] = (I == J ? 1.0 : 2.0) * (double)vloc;
@@ -342,6 +347,12 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
           a.r.skeep[qi] = (I == J || n2 >= a.r.tau2) ? 1 : 0;
           a.r.sn2[qi] = n2;
         }
+      }
+      if (nk > 0) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acce_bar[buf]);
+        if (++buf == 2) { buf = 0; bphase ^= 1; }
       }
     }
   }
@@ -351,34 +362,6 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
     tc_fence_after();
     tmem_dealloc(tmem_base, 2 * TN);
   }
-}
-
-static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  if (!fn) {
-    cudaDriverEntryPointQueryResult q;
-    void* p = nullptr;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  }
-  return fn;
-}
-
-cudaError_t tc_piece_map(const __half* pvals, int64_t cap, CUtensorMap* map) {
-  auto enc = encode_fn();
-  if (!enc) return cudaErrorNotSupported;
-  if ((reinterpret_cast<uintptr_t>(pvals) & 15) != 0) return cudaErrorInvalidValue;
-  // (column, row, piece block): piece p of block q is plane 2 q + p
-  cuuint64_t dims[3] = {(cuuint64_t)B, (cuuint64_t)B, (cuuint64_t)(2 * (cap + 1))};
-  cuuint64_t strides[2] = {(cuuint64_t)B * 2, (cuuint64_t)B * B * 2};
-  cuuint32_t box[3] = {(cuuint32_t)B, (cuuint32_t)B, 1};
-  cuuint32_t estr[3] = {1, 1, 1};
-  const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half*>(pvals), dims, strides, box,
-                         estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
-                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 static int tc_grid() {
@@ -396,14 +379,11 @@ static int tc_grid() {
 
 void tc_prepare() { (void)tc_grid(); }
 
-cudaError_t tc_numeric_launch(DevState* st, const Mat& X, const TcMaps* maps, int parity, int nb, int W,
-                              const TcRound& r, cudaStream_t s) {
+cudaError_t tc_numeric_launch(DevState* st, const Mat& X, int nb, int W, const TcRound& r, cudaStream_t s) {
   TcArgs a;
   std::memset(&a, 0, sizeof(a));
   a.st = st;
   a.X = X;
-  a.maps = maps;
-  a.parity = parity;
   a.nb = nb;
   a.W = W;
   a.ncg = (nb + TTC - 1) / TTC;
