@@ -690,7 +690,8 @@ static sp2_status create_f64(sp2_ctx* h) {
   h->T = h->ld / 64;
   h->nparts = (int)((h->N + 7) / 8 < 1024 ? (h->N + 7) / 8 : 1024);
   const size_t bytes = (size_t)h->ld * h->ld * sizeof(double);
-  const size_t part_bytes = sp2::f64tc::part_bytes(h->N, h->T);
+  sp2::f64tc::choose_tiles(h->tc, h->ld);
+  const size_t part_bytes = sp2::f64tc::part_bytes(h->N, h->T, h->tc.recs > 0 ? h->tc.recs : 1);
   bool ok = cudaMalloc(&h->part, part_bytes) == cudaSuccess &&
             cudaMalloc(&h->part_lo, h->nparts * sizeof(double)) == cudaSuccess &&
             cudaMalloc(&h->part_hi, h->nparts * sizeof(double)) == cudaSuccess &&
@@ -708,9 +709,7 @@ static sp2_status create_f64(sp2_ctx* h) {
   SP2_TRY(cudaMemset(h->buf[0], 0, bytes));
   SP2_TRY(cudaMemset(h->buf[1], 0, bytes));
   SP2_TRY(cudaMemset(h->part, 0, part_bytes));   // records below the diagonal are never written
-  h->tc.ld = h->ld;
-  h->tc.bn = sp2::f64tc::tile_width(h->ld);
-  h->tc.on = sp2::f64tc::wanted(h->N) && alloc_digits(h->tc.X, h->ld);
+  h->tc.on = sp2::f64tc::wanted(h->N) && h->tc.bn > 0 && alloc_digits(h->tc.X, h->ld);
   *h->st_host = init;
   return build_f64_graph(h);
 }
@@ -753,6 +752,8 @@ static sp2_status enqueue_f64(sp2_ctx* h, const double* F, double* D, cudaStream
   SP2_TRY(sp2::launch_bounds_and_init(h->st_dev, F, N, N, h->part_lo, h->part_hi, h->part_bad, h->nparts, s));
   SP2_TRY(sp2::launch_scale_f64(h->st_dev, F, N, N, h->buf[0], h->ld, s));
   if (h->pert) SP2_TRY(sp2::launch_perturb(h->st_dev, h->buf[0], h->buf[1], h->pert, h->pert_count, N, 1, s));
+  if (h->mcw ? mcw_plan(h) != nullptr : h->tc.on)
+    SP2_TRY(sp2::launch_f64_digits(h->st_dev, h->buf[0], h->buf[1], h->tc, N, s));
   SP2_TRY(cudaEventRecord(h->ev_loop[0], s));
   if (h->opts.launch_mode == 0) {
     SP2_TRY(cudaGraphLaunch(h->exec, s));

@@ -79,7 +79,7 @@ struct DevState {
   double spec_e;       // norm = 2: the Lanczos estimate of ||X_{k-1} - X_{k-1}^2||_2 of the last square
   double tr_shift;     // Tr[E_k] of a prescribed perturbation added to the square just written
   int32_t ubounds;     // 1: the caller's outer bounds (ub_lo, ub_hi) replace the Gershgorin bounds
-  int32_t _pad4;
+  int32_t wrote;       // FP64 path: the ping-pong buffer that holds the newest iterate
   double ub_lo, ub_hi;
   // SP2-ACC (Alg. 4 / Alg. 5): set by sp2_set_homo_lumo, schedule filled by the init kernel
   int32_t acc;         // 1: homo/lumo-based accelerated expansion

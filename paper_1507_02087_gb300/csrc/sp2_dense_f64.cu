@@ -104,6 +104,7 @@ init_kernel(DevState* st, const double* __restrict__ F, int64_t ldf, const doubl
     st->scale_a = sa; st->scale_w = sw;
     st->dk = 0;
     st->tr_shift = 0.0;
+    st->wrote = 0;
     st->k = 0; st->done = 0; st->n_out = 0; st->reason = SP2_STOP_EXACT;
     st->status = SP2_OK; st->out_buf = 0; st->out_mode = OUT_COPY; st->hist_len = 0;
     st->tr[0] = 0.0; st->p[0] = 0;
@@ -383,8 +384,8 @@ constexpr int kFinThreads = 1024;
 // (v^2 part, ||X_{k-1}||_F^2 part, Tr[X_{k-1}] part, 0): there Tr[X_k] is taken from
 // the identity Tr[X^2] = ||X||_F^2 for symmetric X (Tr[X_k] = ||X_{k-1}||_F^2 after
 // X^2, 2 Tr[X_{k-1}] - ||X_{k-1}||_F^2 after 2X - X^2), so the polynomial choice does
-// not inherit the bias of the tensor cores' accumulation.  A 64 x 64 tile has `recs` records (1, or
-// f64tc::RECS from the tensor-core products).
+// not inherit the bias of the tensor cores' accumulation.  A 64 x 64 tile has `recs` records (see
+// recs_of).
 __global__ void __launch_bounds__(kFinThreads)
 finalize_kernel(DevState* st, const double* __restrict__ part, int nparts, int stride, int recs,
                 cudaGraphConditionalHandle cond, double* mscr) {
@@ -537,18 +538,19 @@ cudaError_t launch_perturb(DevState* st, double* buf0, double* buf1, const doubl
 }
 
 // ---- one product of the loop, by size ------------------------------------------------------------
+// The digits a tensor-core product needs are made before the loop (X_0, launch_f64_digits) and after each product:
+// of the new iterate, beside the stop test (which only that needs), and of the McWeeny step's square.
 // N <= 128: 8 x 8 tiles on the FP64 units (the tensor-core product has about 35 us of latency a square, against
 // some 10 there); else the tensor cores, or 64 x 64 tiles on the FP64 units where the digit buffers were not to be had.
 enum ProductOp { kSquare = 0, kMcwSquare = 1, kMcwProd = 2 };
 
-static int recs_of(const f64tc::Plan* tc, int N) { return tc ? f64tc::RECS : (N <= kSmallN ? kSmallRecs : 1); }
+static int recs_of(const f64tc::Plan* tc, int N) { return tc ? tc->recs : (N <= kSmallN ? kSmallRecs : 1); }
 
 static cudaError_t emit_product(f64tc::Sink& sink, ProductOp op, DevState* st, double* buf0, double* buf1, double* S,
                                 double* part, int T, const f64tc::Plan* tc, int N) {
   if (tc) {
     static constexpr f64tc::Op ops[3] = {f64tc::OP_SP2, f64tc::OP_MCW_SQ, f64tc::OP_MCW_PROD};
-    const cudaError_t e = f64tc::emit_digits(sink, st, buf0, buf1, op == kMcwProd ? S : nullptr, *tc, N);
-    return e != cudaSuccess ? e : f64tc::emit_product(sink, st, buf0, buf1, S, part, *tc, ops[op]);
+    return f64tc::emit_product(sink, st, buf0, buf1, S, part, *tc, ops[op]);
   }
   if (N <= kSmallN) {
     const int t = (N + kST - 1) / kST;
@@ -576,7 +578,15 @@ cudaError_t launch_f64_step_plain(DevState* st, double* buf0, double* buf1, doub
   if (lz && (e = launch_lanczos(st, buf0, buf1, nullptr, part, nrec, lz, N, T * kTile, s)) != cudaSuccess) return e;
   if (E && (e = launch_perturb(st, buf0, buf1, E, ecount, N, 0, s)) != cudaSuccess) return e;
   finalize_plain_kernel<<<1, kFinThreads, 0, s>>>(st, part, nrec, recs, mscr);
-  return cudaGetLastError();
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return tc ? f64tc::emit_digits(sink, st, buf0, buf1, nullptr, *tc, N) : cudaSuccess;
+}
+
+cudaError_t launch_f64_digits(const DevState* st, const double* buf0, const double* buf1, const f64tc::Plan& P, int N,
+                              cudaStream_t s) {
+  f64tc::Sink sink;
+  sink.s = s;
+  return f64tc::emit_digits(sink, st, buf0, buf1, nullptr, P, N);
 }
 
 cudaError_t add_mcw_loop_body(cudaGraph_t body, DevState* st, double* buf0, double* buf1, double* S, double* part,
@@ -587,13 +597,26 @@ cudaError_t add_mcw_loop_body(cudaGraph_t body, DevState* st, double* buf0, doub
   sink.g = body;
   cudaError_t e = emit_product(sink, kMcwSquare, st, buf0, buf1, S, part, T, tc, N);
   if (e != cudaSuccess) return e;
+  cudaGraphNode_t before[2] = {sink.last, sink.last};          // what the product waits for
+  if (tc) {                                                    // digits of S beside the estimate and the test
+    f64tc::Sink side;
+    side.g = body;
+    side.last = sink.last;
+    if ((e = f64tc::emit_digits(side, st, buf0, buf1, S, *tc, N)) != cudaSuccess) return e;
+    before[1] = side.last;
+  }
   if (lz && (e = add_lanczos_nodes(body, sink.last, st, buf0, buf1, S, part, nrec, lz, N, T * kTile, &sink.last)) !=
                 cudaSuccess)
     return e;
-  cudaGraphNode_t n_fin;
-  if ((e = add_finalize_node(body, &sink.last, 1, st, part, nrec, 2, recs, cond, &n_fin, mscr)) != cudaSuccess) return e;
-  sink.last = n_fin;
-  return emit_product(sink, kMcwProd, st, buf0, buf1, S, part, T, tc, N);
+  if ((e = add_finalize_node(body, &sink.last, 1, st, part, nrec, 2, recs, cond, &before[0], mscr)) != cudaSuccess)
+    return e;
+  if (tc) {
+    if ((e = cudaGraphAddEmptyNode(&sink.last, body, before, 2)) != cudaSuccess) return e;
+  } else {
+    sink.last = before[0];
+  }
+  if ((e = emit_product(sink, kMcwProd, st, buf0, buf1, S, part, T, tc, N)) != cudaSuccess) return e;
+  return tc ? f64tc::emit_digits(sink, st, buf0, buf1, nullptr, *tc, N) : cudaSuccess;
 }
 
 cudaError_t launch_mcw_step_plain(DevState* st, double* buf0, double* buf1, double* S, double* part, int T,
@@ -603,10 +626,12 @@ cudaError_t launch_mcw_step_plain(DevState* st, double* buf0, double* buf1, doub
   sink.s = s;
   cudaError_t e = emit_product(sink, kMcwSquare, st, buf0, buf1, S, part, T, tc, N);
   if (e != cudaSuccess) return e;
+  if (tc && (e = f64tc::emit_digits(sink, st, buf0, buf1, S, *tc, N)) != cudaSuccess) return e;
   if (lz && (e = launch_lanczos(st, buf0, buf1, S, part, nrec, lz, N, T * kTile, s)) != cudaSuccess) return e;
   finalize_plain_kernel<<<1, kFinThreads, 0, s>>>(st, part, nrec, recs, mscr);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  return emit_product(sink, kMcwProd, st, buf0, buf1, S, part, T, tc, N);
+  if ((e = emit_product(sink, kMcwProd, st, buf0, buf1, S, part, T, tc, N)) != cudaSuccess) return e;
+  return tc ? f64tc::emit_digits(sink, st, buf0, buf1, nullptr, *tc, N) : cudaSuccess;
 }
 
 cudaError_t add_finalize_node(cudaGraph_t g, const cudaGraphNode_t* deps, int ndeps, DevState* st,
@@ -643,7 +668,10 @@ cudaError_t add_f64_loop_body(cudaGraph_t body, DevState* st, double* buf0, doub
     cudaGraphNode_t n_pt;
     if ((e = cudaGraphAddKernelNode(&n_pt, body, &n_sq, 1, &kp)) != cudaSuccess) return e;
     n_sq = n_pt;
+    sink.last = n_pt;
   }
+  // digits of the new iterate, beside the estimate and the stop test
+  if (tc && (e = f64tc::emit_digits(sink, st, buf0, buf1, nullptr, *tc, N)) != cudaSuccess) return e;
   return add_finalize_node(body, &n_sq, 1, st, part, nrec, 2, recs, cond, &n_fin, mscr);
 }
 

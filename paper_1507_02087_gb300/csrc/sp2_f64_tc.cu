@@ -18,9 +18,12 @@
 // chains 1.3e-14 / 3.0e-14 / 4.3e-14 / 6.1e-14.
 //
 // Time of one purification against the FP64 units (64 x 64 tiles, 0.98 of their peak at large N): N = 400
-// 2.27 ms against 18.1, N = 1500 (McW-ACC) 6.48 against 77.4, N = 2048 17.5 against 418.
+// 1.37 ms against 18.1, N = 1500 (McW-ACC) 5.38 against 77.4, N = 2048 16.5 against 418.
 //
-// Tiles are 128 x bn per CTA (bn = 32 or 64 by the size, tile_width), over the upper triangle; a stage holds
+// Tiles are 128 x bn (bn = 32 or 64), over the upper triangle; where they are fewer than the SMs, or fill the
+// last round badly, a cluster of ks CTAs shares a tile's k range (choose_tiles): each sums its part, then gives
+// each of the others its columns through distributed shared memory, and every CTA finishes 64 / ks columns.  The
+// sums are integers, so the split changes no bit.  A stage holds
 // the 7 digits of 32 k-columns of both operands, so 14 digit planes feed 34 products.  What bounds the
 // products is the reading of A from shared memory: a 128 x 64 x 16 product takes 48 clocks for 32 of
 // arithmetic.  Warp roles as in the other tensor-core kernels: warp 0 copies, warp 1 issues the products,
@@ -62,14 +65,30 @@ __host__ __device__ constexpr int stage_bytes(int bn) { return A_BYTES + b_bytes
 __host__ __device__ constexpr int stages_of(int bn) {
   return 226 * 1024 / stage_bytes(bn) < MAXSTG ? 226 * 1024 / stage_bytes(bn) : MAXSTG;
 }
-__host__ __device__ constexpr int smem_bytes(int bn) { return stages_of(bn) * stage_bytes(bn) + 1024; }
+// Exchange buffer of a split tile: from each of the other CTAs, the sums of this CTA's columns.
+__host__ __device__ constexpr int exchange_bytes(int ks) { return (ks - 1) * (BM * 64 * 8 / ks); }
+__host__ __device__ constexpr int smem_bytes(int bn, int ks) {
+  return stages_of(bn) * stage_bytes(bn) + exchange_bytes(ks) + 1024;
+}
+static_assert(smem_bytes(64, 8) <= 227 * 1024 - 512, "shared memory");
 static_assert(stages_of(64) == 2 && stages_of(32) == 3, "stages");
 
-// Each digit sum has a tensor-memory accumulator of its own (NS x bn columns), closed and drained every
-// period(s) blocks of 32 k-columns: a drain costs a fixed 600 clocks or so beside its values, and with two
-// buffers in turn, drained every block, the drains took three times the products.  A product adds at most
-// 2^14 per term, so the sums stay exact: (pairs of s) x 32 period <= 2^10.
+// Each digit sum has a tensor-memory accumulator of its own (NS x bn columns), closed and drained once in
+// period(s) blocks of 32 k-columns, at phase(s), and at the end of the tile: a drain costs a warp about 1.2 k clocks,
+// and with two buffers in turn, drained every block, the drains took three times the products.  The phases spread
+// the drains over the blocks, two at most in one, so that a block's products (3 k clocks) hide them: a sum's next
+// product comes a block after it was closed.  A product adds at most 2^14 per term, so the sums stay exact:
+// (pairs of s) x 32 period <= 2^10.
 __host__ __device__ constexpr int period(int s) { return s < 2 ? 16 : (s < 4 ? 8 : 4); }
+__host__ __device__ constexpr int phase(int s) { return (int)((0x210315b7u >> (4 * s)) & 15u); }   // 7 11 5 1 3 0 1 2
+__host__ __device__ constexpr bool closes(int kb, int s) { return (kb & (period(s) - 1)) == phase(s); }
+// The sums that close at blocks kb = 8 h .. 8 h + 7 (mod 16), a byte of bits each.
+__host__ __device__ constexpr uint64_t closing(int h) {
+  uint64_t m = 0;
+  for (int kb = 0; kb < 8; ++kb)
+    for (int s = 0; s < NS; ++s) m |= (uint64_t)(closes(8 * h + kb, s) ? 1 : 0) << (8 * kb + s);
+  return m;
+}
 __host__ __device__ constexpr int first_pair(int s) { return s < ND ? 0 : s - ND + 1; }   // smallest a of a + b = s
 __host__ __device__ constexpr int pairs(int s) { return (s < ND ? s : ND - 1) - first_pair(s) + 1; }
 __host__ __device__ constexpr bool sums_exact() {
@@ -133,7 +152,7 @@ __global__ void __launch_bounds__(DT)
 digits_kernel(const DevState* st, const double* buf0, const double* buf1, const double* S, int ld, int N, __half* dig,
               int32_t* exps) {
   if (st->done) return;
-  const double* X = S ? S : ((st->k & 1) ? buf1 : buf0);
+  const double* X = S ? S : (st->wrote ? buf1 : buf0);
   const int rr = threadIdx.x >> 5, r = blockIdx.x * 8 + rr, lane = threadIdx.x & 31;
   if (r >= N) return;
   const double* row = X + (int64_t)r * ld;
@@ -250,58 +269,58 @@ __device__ __forceinline__ void give_up(DevState* st, volatile int* abort_s) {
   st->done = 1;
 }
 
-// T 2^(ei + ej - 62): the scale goes into the exponent field where the result is a normal number (an FP64
-// multiplication takes 70 clocks a warp here, the conversion from the integer 6).
-__device__ __forceinline__ double scaled_sum(long long t, int ei, int ej) {
-  if (ei == kBadExp || ej == kBadExp) return __longlong_as_double(0x7ff8000000000000ll);
-  const int es = ei + ej - 62;
-  const double s = (double)t;
-  if (es <= -1000 || es >= 900) return ldexp(s, es);
-  return t ? __hiloint2double(__double2hiint(s) + (es << 20), __double2loint(s)) : 0.0;
-}
-
-// NV consecutive 32-bit tensor-memory columns (16 or 32 per load).
+// 16 or 32 consecutive 32-bit tensor-memory columns.
 __device__ __forceinline__ void tmem_ld(uint32_t addr, uint32_t (&r)[32]) { tmem_ld32(addr, r); }
 __device__ __forceinline__ void tmem_ld(uint32_t addr, uint32_t (&r)[16]) { tmem_ld16(addr, r); }
 
-// T += V_s of one period, in units of 2^-62: the weight of s is 2^(46 - 8 s); s = 6 and 7 are rounded to the
-// unit.  (For s <= 1 only the high word changes, modulo 2^32: the total fits.)
-template <int S, int G>
-__device__ __forceinline__ void add_digit_sums(const uint32_t (&raw)[G], long long (&T)[G]) {
-  #pragma unroll
-  for (int j = 0; j < G; ++j) {
-    const float f = __uint_as_float(raw[j]);
-    const int v = __float2int_rn(S <= 5 ? f : f * (S == 6 ? 0x1p-2f : 0x1p-10f));
-    if constexpr (S <= 1) T[j] += (long long)((unsigned long long)((unsigned)v << (14 - 8 * S)) << 32);
-    else if constexpr (S <= 5) T[j] += (long long)v * (1ll << (46 - 8 * S));
-    else T[j] += (long long)v;
-  }
-}
-
-// Drains digit sum S if its period ends with block kb (or the tile does).
-template <int S, int G>
-__device__ __forceinline__ bool drain(uint32_t trow, int bn, int kb, int nkb, uint64_t* accf, uint64_t* acce,
-                                      uint32_t& phases, int lane, volatile int* abort_s, long long (&T)[G]) {
-  if ((kb + 1) % period(S) != 0 && kb + 1 != nkb) return true;
-  int got = 0;
-  if (lane == 0) got = !*abort_s && mbar_wait(&accf[S], (phases >> S) & 1u, globaltimer_ns() + kWaitNs);
-  got = __shfl_sync(0xffffffffu, got, 0);
-  if (!got) return false;
-  tc_fence_after();
-  uint32_t raw[G];
-  tmem_ld(trow + (uint32_t)(S * bn), raw);
+// Four 64-bit sums whose low and high words lie in two tensor-memory areas.
+__device__ __forceinline__ void load_sums(uint32_t lo, uint32_t hi, long long (&t)[4]) {
+  uint32_t a[4], b[4];
+  tmem_ld4(lo, a);
+  tmem_ld4(hi, b);
   tmem_wait_ld();
-  tc_fence_before();
-  __syncwarp();
-  if (lane == 0) mbar_arrive(&acce[S]);
-  phases ^= 1u << S;
-  add_digit_sums<S, G>(raw, T);
-  return true;
+  #pragma unroll
+  for (int j = 0; j < 4; ++j) t[j] = (long long)(((unsigned long long)b[j] << 32) | a[j]);
 }
 
-template <int BN>
-__global__ void __launch_bounds__(THREADS, 1)
+// T += V_s of one period, in units of 2^-62: the weight of s is 2^(46 - 8 s), for s <= 1
+// in the high word alone (modulo 2^32: the total fits); s = 6 and 7 are rounded to the unit.  One piece of code for every s: as
+// straight-line code for each of them the drains were bound by the instruction fetch (2 k clocks a drain; the integer
+// conversions, 8.5 clocks a warp each, take 550).
+template <int G>
+__device__ __forceinline__ void add_digit_sums(int s, const uint32_t (&raw)[G], long long (&T)[G]) {
+  if (s <= 1) {                          // only the high word changes
+    const int m = 1 << (14 - 8 * s);
+    #pragma unroll
+    for (int j = 0; j < G; ++j)
+      T[j] += (long long)((unsigned long long)((unsigned)__float2int_rn(__uint_as_float(raw[j])) * (unsigned)m) << 32);
+    return;
+  }
+  const float scale = s <= 5 ? 1.f : (s == 6 ? 0x1p-2f : 0x1p-10f);
+  const int m = s <= 5 ? 1 << (46 - 8 * s) : 1;
+  #pragma unroll
+  for (int j = 0; j < G; ++j) T[j] += (long long)__float2int_rn(__uint_as_float(raw[j]) * scale) * m;
+}
+
+// T 2^(ei + ej - 62) where the result is no normal number.
+__device__ __noinline__ double scaled_sum_rare(long long t, int ei, int ej) {
+  if (ei == kBadExp || ej == kBadExp) return __longlong_as_double(0x7ff8000000000000ll);
+  return ldexp((double)t, ei + ej - 62);
+}
+
+// T 2^(ei + ej - 62): the scale goes into the exponent field where the result is a normal number (an FP64
+// multiplication takes 70 clocks a warp here, the conversion from the integer 6).
+__device__ __forceinline__ double scaled_sum(long long t, int ei, int ej) {
+  const int es = ei + ej - 62;
+  if (ei == kBadExp || ej == kBadExp || es <= -1000 || es >= 900) return scaled_sum_rare(t, ei, ej);
+  const double s = (double)t;
+  return t ? __hiloint2double(__double2hiint(s) + (es << 20), __double2loint(s)) : 0.0;
+}
+
+template <int BN, int KS>
+__global__ void __cluster_dims__(KS, 1, 1) __launch_bounds__(THREADS, 1)
 f64_product_kernel(const Args a) {
+  static_assert(KS == 1 || BN == 64, "split tiles are 64 wide");
   constexpr int STG = stages_of(BN), SBYTES = stage_bytes(BN);
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[STG];
@@ -309,6 +328,8 @@ f64_product_kernel(const Args a) {
   __shared__ __align__(8) uint64_t accf_bar[NS];
   __shared__ __align__(8) uint64_t acce_bar[NS];
   __shared__ __align__(8) uint64_t drain_bar;
+  __shared__ __align__(8) uint64_t xfull_bar[8];     // split tiles, per epilogue warp: the others' sums are here,
+  __shared__ __align__(8) uint64_t xempty_bar[8];    // and the others have taken this CTA's
   __shared__ uint32_t tmem_base_s;
   __shared__ volatile int abort_s;
 
@@ -316,8 +337,13 @@ f64_product_kernel(const Args a) {
   if (st->done) return;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-  const int ld = a.ld, cols = (ld + BN - 1) / BN, nkb = ld / KB;
+  const int ld = a.ld, cols = (ld + BN - 1) / BN;
+  const int rank = KS > 1 ? (int)cluster_ctarank() : 0;
+  const int unit = blockIdx.x / KS, units = gridDim.x / KS;       // clusters
+  const int kb0 = (ld / KB) * rank / KS, nkb = (ld / KB) * (rank + 1) / KS - kb0;   // this CTA's k-blocks
+  if (blockIdx.x == 0 && threadIdx.x == 0 && a.op != OP_MCW_SQ) st->wrote = (st->k + (a.op == OP_SP2 ? 1 : 0)) & 1;
   if (threadIdx.x == 0) {
+    for (int w = 0; w < 8; ++w) { mbar_init(&xfull_bar[w], KS > 1 ? KS - 1 : 1); mbar_init(&xempty_bar[w], KS > 1 ? KS - 1 : 1); }
     for (int s = 0; s < STG; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
     for (int b = 0; b < NS; ++b) { mbar_init(&accf_bar[b], 1); mbar_init(&acce_bar[b], 8); }
     mbar_init(&drain_bar, 1);
@@ -326,7 +352,8 @@ f64_product_kernel(const Args a) {
   }
   if (warp == 1) tmem_alloc(&tmem_base_s, NS * BN);
   tc_fence_before();
-  __syncthreads();
+  if (KS > 1) cluster_sync();            // the barriers of every CTA are initialised
+  else __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
 
@@ -340,15 +367,15 @@ f64_product_kernel(const Args a) {
         int armed[STG];
         uint32_t armed_par[STG];
         for (int s = 0; s < STG; ++s) { armed[s] = 0; armed_par[s] = 0; }
-        for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
+        for (int t = unit; t < a.tiles && ok; t += units) {
           int I, J;
           locate(t, cols, BM / BN, I, J);
           for (int kb = 0; kb < nkb; ++kb) {
             if (abort_s || !mbar_wait(&empty_bar[stage], phase ^ 1, globaltimer_ns() + kWaitNs)) { ok = false; break; }
             uint8_t* sA = smem + stage * SBYTES;
             mbar_arrive_expect_tx(&full_bar[stage], SBYTES);
-            bulk_load(sA, a.digA + kb * kstride + (int64_t)I * A_BYTES, A_BYTES, &full_bar[stage]);
-            bulk_load(sA + A_BYTES, a.digB + kb * kstride + (int64_t)J * b_bytes(BN), b_bytes(BN), &full_bar[stage]);
+            bulk_load(sA, a.digA + (kb0 + kb) * kstride + (int64_t)I * A_BYTES, A_BYTES, &full_bar[stage]);
+            bulk_load(sA + A_BYTES, a.digB + (kb0 + kb) * kstride + (int64_t)J * b_bytes(BN), b_bytes(BN), &full_bar[stage]);
             armed[stage] = 1;
             armed_par[stage] = phase;
             if (++stage == STG) { stage = 0; phase ^= 1; }
@@ -364,7 +391,7 @@ f64_product_kernel(const Args a) {
         int stage = 0;
         uint32_t phase = 0, phases = 0;  // phases: bit s, the parity of accumulator s
         bool ok = true;
-        for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
+        for (int t = unit; t < a.tiles && ok; t += units) {
           for (int kb = 0; kb < nkb && ok; ++kb) {
             if (abort_s || !mbar_wait(&full_bar[stage], phase, globaltimer_ns() + kWaitNs)) { ok = false; break; }
             tc_fence_after();
@@ -374,7 +401,7 @@ f64_product_kernel(const Args a) {
             for (int s = 0; s < NS; ++s) {
               const uint32_t dt = tmem_base + (uint32_t)(s * BN);
               uint32_t accumulate = 1;
-              if (kb % period(s) == 0) {
+              if (kb == 0 || closes(kb - 1, s)) {
                 if (abort_s || !mbar_wait(&acce_bar[s], ((phases >> s) & 1u) ^ 1u, globaltimer_ns() + kWaitNs)) {
                   ok = false;
                   break;
@@ -391,7 +418,7 @@ f64_product_kernel(const Args a) {
                   accumulate = 1;
                 }
               }
-              if ((kb + 1) % period(s) == 0 || kb + 1 == nkb) {
+              if (closes(kb, s) || kb + 1 == nkb) {
                 mma_commit(&accf_bar[s]);
                 phases ^= 1u << s;
               }
@@ -410,50 +437,148 @@ f64_product_kernel(const Args a) {
     const int ew = warp - 4;
     const int q = warp & 3;              // tensor-memory lanes 32 q .. 32 q + 31
     const int hc = ew >> 2;              // columns hc BN / 2 .. of the tile
-    constexpr int G = BN / 2;
+    constexpr int G = BN / 2, C = G / KS;       // columns a warp sums, and finishes
+    uint32_t xphase = 0;
     const Poly P = poly_of(a);
     const int N = st->N, T64 = ld / 64;
     uint32_t phases = 0;
     bool ok = true;
     const uint32_t trow = tmem_base + (uint32_t)(hc * G) + ((uint32_t)(32 * q) << 16);
-    for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
+    for (int t = unit; t < a.tiles && ok; t += units) {
       int I, J;
       locate(t, cols, BM / BN, I, J);
       long long T[G];
       #pragma unroll
       for (int j = 0; j < G; ++j) T[j] = 0;
-      for (int kb = period(NS - 1) - 1; ok; kb += period(NS - 1)) {
-        if (kb >= nkb) kb = nkb - 1;
-        ok = drain<0>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
-             drain<1>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
-             drain<2>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
-             drain<3>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
-             drain<4>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
-             drain<5>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
-             drain<6>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T) &&
-             drain<7>(trow, BN, kb, nkb, accf_bar, acce_bar, phases, lane, &abort_s, T);
-        if (kb == nkb - 1) break;
+      uint32_t held = 0;                 // accumulators 6 and 7 stay with this warp until its tile is finished
+      for (int kb = 0; ok && kb < nkb; ++kb) {
+        const bool last = kb == nkb - 1;
+        constexpr uint64_t c0 = closing(0), c1 = closing(1);
+        uint32_t todo = last ? 255u : (uint32_t)(((kb & 8) ? c1 : c0) >> (8 * (kb & 7))) & 255u;
+        while (todo) {
+          const int s = __ffs(todo) - 1;
+          todo &= todo - 1u;
+          int got = 0;
+          if (lane == 0) got = !abort_s && mbar_wait(&accf_bar[s], (phases >> s) & 1u, globaltimer_ns() + kWaitNs);
+          got = __shfl_sync(0xffffffffu, got, 0);
+          if (!got) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          uint32_t raw[G];
+          tmem_ld(trow + (uint32_t)(s * BN), raw);
+          tmem_wait_ld();
+          phases ^= 1u << s;
+          if (last && s >= 6) {
+            held |= 1u << s;
+          } else {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acce_bar[s]);
+          }
+          add_digit_sums(s, raw, T);
+        }
       }
+      // the sums go to the columns of accumulators 6 (low words) and 7 (high words), from which the rest takes
+      // them four at a time in loops
+      const uint32_t lo = trow + 6 * BN, hi = trow + 7 * BN;
+      if (nkb > 0 && ok) {
+        uint32_t wlo[G], whi[G];
+        #pragma unroll
+        for (int j = 0; j < G; ++j) {
+          wlo[j] = (uint32_t)(unsigned long long)T[j];
+          whi[j] = (uint32_t)((unsigned long long)T[j] >> 32);
+        }
+        #pragma unroll
+        for (int j = 0; j < G; j += 16) {
+          tmem_st16(lo + j, wlo + j);
+          tmem_st16(hi + j, whi + j);
+        }
+        tmem_wait_st();
+      }
+      if constexpr (KS > 1) {
+        // to every other CTA its columns, from every other CTA this one's; the slot of sender p is p, less
+        // one past the receiver
+        const uint32_t slots = smem_u32(smem + STG * SBYTES);
+        const uint64_t until = globaltimer_ns() + kWaitNs;
+        int go = ok;
+        if (lane == 0) go = ok && !abort_s && mbar_wait_cluster(&xempty_bar[ew], xphase ^ 1, until);
+        go = __shfl_sync(0xffffffffu, go, 0);
+        if (go) {
+          #pragma unroll 1
+          for (int j = 0; j < G; j += 4) {
+            const int o = j / C;
+            if (o == rank) continue;
+            long long t[4] = {0, 0, 0, 0};
+            if (nkb > 0) load_sums(lo + j, hi + j, t);
+            const uint32_t dst = mapa_shared(slots, o) +
+                                 (uint32_t)((((rank < o ? rank : rank - 1) * 8 + ew) * C + j % C) * 256 + lane * 8);
+            #pragma unroll
+            for (int d = 0; d < 4; ++d) st_cluster_u64(dst + d * 256, (unsigned long long)t[d]);
+          }
+          __syncwarp();
+          if (lane == 0) {
+            #pragma unroll 1
+            for (int o = 0; o < KS; ++o)
+              if (o != rank) mbar_arrive_cluster(mapa_shared(smem_u32(&xfull_bar[ew]), o));
+            go = mbar_wait_cluster(&xfull_bar[ew], xphase, until);
+          }
+          go = __shfl_sync(0xffffffffu, go, 0);
+        }
+        if (!go) ok = false;
+      }
+      // after the tile: the others may overwrite the exchanged sums, the products the held accumulators
+      auto release = [&]() {
+        if (KS > 1) {
+          __syncwarp();
+          if (lane == 0) {
+            #pragma unroll 1
+            for (int o = 0; o < KS; ++o)
+              if (o != rank) mbar_arrive_cluster(mapa_shared(smem_u32(&xempty_bar[ew]), o));
+          }
+          xphase ^= 1;
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          if (held & 64u) mbar_arrive(&acce_bar[6]);
+          if (held & 128u) mbar_arrive(&acce_bar[7]);
+        }
+      };
       if (!ok) {
         if (lane == 0) give_up(st, &abort_s);
         break;
       }
-      // epilogue: this warp's 32 rows, G columns at a time; only blocks on or above the diagonal
+      // epilogue: this warp's 32 rows, C columns; only blocks on or above the diagonal
       const int r0 = I * BM + 32 * q, r = r0 + lane;
-      if (r0 >= ld) continue;
+      const int c0 = J * BN + hc * G + rank * C;
+      if (r0 >= ld || c0 >= ld || c0 + C <= r0) {
+        release();
+        continue;
+      }
       const int ei = a.ea[r];
-      const int c0 = J * BN + hc * G;
-      if (c0 >= ld || c0 + G <= r0) continue;
       const bool off = c0 >= r0 + 32;    // wholly above the diagonal
       double v2 = 0.0, trc = 0.0;
-      #pragma unroll
-      for (int j0 = 0; j0 < G; j0 += 4) {
-        double x[4], xn[4];
-        load4(P.in + (int64_t)r * ld + c0 + j0, x);
+      double xl[4];                      // the old values, loaded a step ahead
+      load4(P.in + (int64_t)r * ld + c0, xl);
+      #pragma unroll 1
+      for (int j0 = 0; j0 < C; j0 += 4) {
+        double x[4] = {xl[0], xl[1], xl[2], xl[3]}, xn[4];
+        if (j0 + 4 < C) load4(P.in + (int64_t)r * ld + c0 + j0 + 4, xl);
+        long long F[4] = {0, 0, 0, 0};
+        if (nkb > 0) load_sums(lo + rank * C + j0, hi + rank * C + j0, F);
+        if constexpr (KS > 1) {
+          const unsigned long long* src = reinterpret_cast<const unsigned long long*>(smem + STG * SBYTES);
+          #pragma unroll
+          for (int p = 0; p < KS - 1; ++p)
+            #pragma unroll
+            for (int j = 0; j < 4; ++j) F[j] += (long long)src[((p * 8 + ew) * C + j0 + j) * 32 + lane];
+        }
         #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const int c = c0 + j0 + j;
-          const double s = scaled_sum(T[j0 + j], ei, a.eb[c]);
+          const double s = scaled_sum(F[j], ei, a.eb[c]);
           const double d = x[j] - s;
           if (off || c > r) v2 = fma(d, d, v2);
           else if (c == r) v2 = fma(0.5 * d, d, v2);
@@ -469,6 +594,7 @@ f64_product_kernel(const Args a) {
             if (c0 + j0 + j >= r) P.out[(int64_t)r * ld + c0 + j0 + j] = xn[j];
         }
       }
+      release();
       v2 *= 2.0;                         // each element above the diagonal stands for two
       #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
@@ -476,15 +602,21 @@ f64_product_kernel(const Args a) {
         trc += __shfl_xor_sync(0xffffffffu, trc, o);
       }
       if (lane == 0) {
-        // record of these 32 rows and G columns within their 64 x 64 tile
-        double* dst = a.part + 2 * (RECS * upper_index(r0 / 64, c0 / 64, T64) + 4 * ((r0 >> 5) & 1) + ((c0 >> 4) & 3));
+        // record of these 32 rows and C columns within their 64 x 64 tile
+        constexpr int half = 64 / C;     // records of 32 rows
+        double* dst = a.part + 2 * (2 * half * upper_index(r0 / 64, c0 / 64, T64) + half * ((r0 >> 5) & 1) + (c0 & 63) / C);
         dst[0] = v2;
         dst[1] = trc;
       }
     }
   }
 
-  __syncthreads();
+  if (KS > 1) {                          // the others' accesses to this CTA's shared memory are over
+    __syncwarp();
+    cluster_sync();
+  } else {
+    __syncthreads();
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, NS * BN);
@@ -492,8 +624,12 @@ f64_product_kernel(const Args a) {
 }
 
 // ---- host side ---------------------------------------------------------------------------------
-static const void* kernel_of(int bn) {
-  return bn == 64 ? (const void*)f64_product_kernel<64> : (const void*)f64_product_kernel<32>;
+static const void* kernel_of(int bn, int ks) {
+  if (bn == 32) return (const void*)f64_product_kernel<32, 1>;
+  return ks == 8   ? (const void*)f64_product_kernel<64, 8>
+         : ks == 4 ? (const void*)f64_product_kernel<64, 4>
+         : ks == 2 ? (const void*)f64_product_kernel<64, 2>
+                   : (const void*)f64_product_kernel<64, 1>;
 }
 
 static int sm_count() {
@@ -507,28 +643,60 @@ static int sm_count() {
   return n;
 }
 
-static cudaError_t prepare() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  for (int bn : {32, 64}) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel_of(bn), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(bn));
-    if (e != cudaSuccess) return e;
+// Tiles that run at once: SMs, or the clusters of ks that the GPU holds.  Sets the kernels' attributes first; 0 if
+// that fails.
+static int slots_of(int bn, int ks) {
+  static int cached[2][4] = {};
+  int& n = cached[bn == 64][ks == 8 ? 3 : ks / 2];
+  if (n) return n;
+  if (cudaFuncSetAttribute(kernel_of(bn, ks), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(bn, ks)) !=
+      cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
   }
-  done = true;
-  return cudaSuccess;
+  int v = sm_count();
+  if (ks > 1) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ks * (sm_count() / ks));
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = smem_bytes(bn, ks);
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = ks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&v, kernel_of(bn, ks), &cfg) != cudaSuccess || v < 1) {
+      (void)cudaGetLastError();
+      return 0;
+    }
+  }
+  n = v;
+  return n;
 }
 
-// The width with the least work per SM: tiles dealt out in whole rounds, times the time of a stage.
-int tile_width(int ld) {
-  const double cost[2] = {44.0, 48.0};   // clocks of a 128 x bn x 16 product: reading A bounds it
-  int best = 64;
-  double t = 1e300;
-  for (int i = 1; i >= 0; --i) {
-    const int bn = 32 << i, n = tiles_of(ld, bn), sms = sm_count();
-    const double c = (double)((n + sms - 1) / sms) * cost[i];
-    if (c < t) { t = c; best = bn; }
+// The shape with the least time in this model: rounds of tiles, each its k-blocks (68 products of 48 clocks, 44 at
+// width 32: reading A bounds them) and about 12 k clocks for filling the pipe, the last drains and the epilogue,
+// less with fewer columns to finish.  One iteration of a run, unsplit and split: N = 400 54 -> 37 us (16 tiles, 152 SMs),
+// N = 700 76 -> 45, N = 1500 (156 tiles) 260 -> 213; N = 2048 stays unsplit.
+void choose_tiles(Plan& P, int ld) {
+  P.ld = ld;
+  double best = 1e300;
+  for (int i = 0; i < 5; ++i) {
+    const int bn = i == 4 ? 32 : 64, ks = i == 4 ? 1 : 1 << i;
+    const int slots = slots_of(bn, ks);
+    if (slots < 1) continue;
+    const int n = tiles_of(ld, bn), kb = (ld / KB + ks - 1) / ks;
+    const double tile = kb * 2.0 * 34.0 * (bn == 64 ? 48.0 : 44.0) + 6000.0 + (bn == 64 ? 8000.0 / ks : 4000.0) +
+                        (ks > 1 ? 2000.0 : 0.0);
+    const double t = (double)((n + slots - 1) / slots) * tile;
+    if (t < best) {
+      best = t;
+      P.bn = bn;
+      P.ks = ks;
+      P.recs = 2 * 64 / (bn / 2 / ks);
+    }
   }
-  return best;
 }
 
 cudaError_t Sink::put(const void* func, dim3 grid, dim3 block, size_t smem, void** args) {
@@ -572,11 +740,11 @@ cudaError_t emit_product(Sink& sink, DevState* st, double* buf0, double* buf1, d
   a.ld = P.ld;
   a.tiles = tiles_of(P.ld, P.bn);
   a.op = op;
-  const cudaError_t e = prepare();
-  if (e != cudaSuccess) return e;
+  const int slots = slots_of(P.bn, P.ks);
+  if (slots < 1) return cudaErrorNotSupported;
   void* args[] = {&a};
-  const int grid = a.tiles < sm_count() ? a.tiles : sm_count();
-  return sink.put(kernel_of(P.bn), dim3(grid), dim3(THREADS), smem_bytes(P.bn), args);
+  const int units = a.tiles < slots ? a.tiles : slots;
+  return sink.put(kernel_of(P.bn, P.ks), dim3(units * P.ks), dim3(THREADS), smem_bytes(P.bn, P.ks), args);
 }
 
 }  // namespace f64tc

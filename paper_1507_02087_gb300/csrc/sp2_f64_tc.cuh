@@ -14,7 +14,7 @@ struct DevState;
 namespace f64tc {
 
 constexpr int ND = 7;              // digits per value
-constexpr int RECS = 8;            // partial records (2 doubles) per upper 64 x 64 tile
+constexpr int MAX_RECS = 32;       // partial records (2 doubles) per upper 64 x 64 tile, at most (Plan::recs)
 
 // The digits of one ld x ld matrix, in the order of the shared-memory stages (see sp2_f64_tc.cu), and one
 // power-of-two exponent per row.
@@ -25,15 +25,18 @@ struct Digits {
 
 struct Plan {
   Digits X, S;                     // of the iterate; of the McWeeny step's shifted square (dig null: none)
-  int ld = 0, bn = 0;              // bn: columns of an output tile (32, 64 or 128)
+  int ld = 0;
+  int bn = 0, ks = 0;              // columns of an output tile (32 or 64); CTAs that share its k range (1, 2, 4, 8)
+  int recs = 0;                    // records per 64 x 64 tile: 32 rows x the columns one warp finishes
   bool on = false;
 };
 
 // Sizes at which the tensor-core products are used (see sp2_f64_tc.cu).
 constexpr int kMinN = 129;
-// Bytes of the partial records of a problem with T x T tiles of 64: RECS per upper tile, 64 for N < kMinN.
-constexpr size_t part_bytes(int64_t N, int T) {
-  return sizeof(double) * 2 * (size_t)(N < kMinN ? 64 : RECS) * ((size_t)T * (T + 1) / 2);
+// Bytes of the partial records of a problem with T x T tiles of 64 and `recs` records per upper tile (64 for
+// N < kMinN).
+constexpr size_t part_bytes(int64_t N, int T, int recs) {
+  return sizeof(double) * 2 * (size_t)(N < kMinN ? 64 : recs) * ((size_t)T * (T + 1) / 2);
 }
 inline bool wanted(int64_t N) { return N >= kMinN; }
 
@@ -41,8 +44,8 @@ inline bool wanted(int64_t N) { return N >= kMinN; }
 constexpr int padded_rows(int ld) { return (ld + 127) / 128 * 128; }
 constexpr size_t digit_bytes(int ld) { return (size_t)ND * ld * padded_rows(ld) * sizeof(__half); }
 constexpr size_t exp_bytes(int ld) { return (size_t)ld * sizeof(int32_t); }
-// Tile width for matrices with leading dimension ld.
-int tile_width(int ld);
+// Tile shape for matrices with leading dimension ld (bn, ks, recs and ld of the plan).
+void choose_tiles(Plan& P, int ld);
 // What one product writes.
 enum Op : int32_t {
   OP_SP2 = 0,      // X_k from X_{k-1} (Alg. 3, or the scheduled polynomial of Alg. 5)
@@ -58,7 +61,7 @@ struct Sink {
   cudaError_t put(const void* func, dim3 grid, dim3 block, size_t smem, void** args);
 };
 
-// Digits of X_{k-1} (buf0 / buf1 by the state's square count), or of S when `S` is given.
+// Digits of the newest iterate (buf0 or buf1, st->wrote), or of S when `S` is given.
 cudaError_t emit_digits(Sink& sink, const DevState* st, const double* buf0, const double* buf1, const double* S,
                         const Plan& P, int N);
 // The product `op` over the upper tiles, with the partial records of the stop test.

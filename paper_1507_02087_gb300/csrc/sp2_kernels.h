@@ -43,10 +43,14 @@ cudaError_t launch_scale_f64(const DevState* st, const double* F, int64_t ldf, i
 // finalize), added to `body` as kernel nodes.  `mscr` (T^2 + 2T doubles, or null) is the
 // scratch of the mixed-norm stop, used when the state asks for it; `lz` (lanczos_scratch_bytes,
 // or null) adds the Lanczos estimate of the spectral norm between the square and the finalize; `tc`
-// (or null) forms the products on the tensor cores, `part` then holding f64tc::RECS records a tile.
+// (or null) forms the products on the tensor cores, `part` then holding the plan's records per tile and the digits of X_0 made before
+// (launch_f64_digits).
 cudaError_t add_f64_loop_body(cudaGraph_t body, DevState* st, double* buf0, double* buf1, double* part,
                               int T, cudaGraphConditionalHandle cond, const f64tc::Plan* tc, double* mscr, void* lz,
                               int N, const double* E, int64_t ecount);
+// Digits of X_0 for the first product of a run (once it is scaled and perturbed).
+cudaError_t launch_f64_digits(const DevState* st, const double* buf0, const double* buf1, const f64tc::Plan& P, int N,
+                              cudaStream_t s);
 // Alg. 1's prescribed perturbation: E_i (i < count, N x N row-major each) added to X_0 (initial)
 // or to the square just written; in the loop bodies it follows the Lanczos nodes.
 cudaError_t launch_perturb(DevState* st, double* buf0, double* buf1, const double* E, int64_t count, int N,

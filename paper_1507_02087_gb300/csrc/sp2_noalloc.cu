@@ -44,8 +44,8 @@ constexpr size_t kOffLo = align256(kOffState + sizeof(DevState));
 constexpr size_t kOffHi = align256(kOffLo + kGersh * sizeof(double));
 constexpr size_t kOffBad = align256(kOffHi + kGersh * sizeof(double));
 constexpr size_t kOffPart = align256(kOffBad + kGersh * sizeof(int));
-constexpr size_t kPartBytes = sp2::f64tc::part_bytes(kMaxN, kT);
-static_assert(kPartBytes >= sp2::f64tc::part_bytes(sp2::f64tc::kMinN - 1, 2), "records of the smallest problems");
+constexpr size_t kPartBytes = sp2::f64tc::part_bytes(kMaxN, kT, sp2::f64tc::MAX_RECS);
+static_assert(kPartBytes >= sp2::f64tc::part_bytes(sp2::f64tc::kMinN - 1, 2, 1), "records of the smallest problems");
 constexpr size_t kOffBuf0 = align256(kOffPart + kPartBytes);
 constexpr size_t kOffBuf1 = align256(kOffBuf0 + (size_t)kLd * kLd * sizeof(double));
 constexpr size_t kOffDig = align256(kOffBuf1 + (size_t)kLd * kLd * sizeof(double));
@@ -143,8 +143,8 @@ static sp2_status run_noalloc(const double* F_dev, double* D_dev, int64_t N, int
   sp2::f64tc::Plan tc;
   tc.on = sp2::f64tc::wanted(N);
   if (tc.on) {
-    tc.ld = ld;
-    tc.bn = sp2::f64tc::tile_width(ld);
+    sp2::f64tc::choose_tiles(tc, ld);
+    if (tc.bn <= 0) return SP2_ERR_CUDA;
     tc.X.dig = (__half*)(base + kOffDig);
     tc.X.exp = (int32_t*)(base + kOffExp);
     if (cudaMemsetAsync(tc.X.dig, 0, sp2::f64tc::digit_bytes(ld), s) != cudaSuccess ||
@@ -156,7 +156,8 @@ static sp2_status run_noalloc(const double* F_dev, double* D_dev, int64_t N, int
   noalloc_setup_kernel<<<1, 1, 0, s>>>(st, (int)N, ld, (int)n_occ, kMaxIter);
   if (cudaGetLastError() != cudaSuccess) return SP2_ERR_CUDA;
   if (sp2::launch_bounds_and_init(st, F_dev, N, (int)N, lo, hi, bad, nparts, s) != cudaSuccess ||
-      sp2::launch_scale_f64(st, F_dev, N, (int)N, buf0, ld, s) != cudaSuccess) {
+      sp2::launch_scale_f64(st, F_dev, N, (int)N, buf0, ld, s) != cudaSuccess ||
+      (tc.on && sp2::launch_f64_digits(st, buf0, buf1, tc, (int)N, s) != cudaSuccess)) {
     (void)cudaGetLastError();
     return SP2_ERR_CUDA;
   }

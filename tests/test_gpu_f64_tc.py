@@ -50,6 +50,27 @@ def test_one_square_at_tile_edges(N, fill):
     check(*one_square(F, (-1.5, 1.5), nocc))
 
 
+@pytest.mark.parametrize("N", [700, 1001, 1500, 2049, 3000])     # k ranges split over 4, 2, 4, 1 and 1 CTAs, or so
+def test_one_square_against_fp64_matmul(N):
+    F = torch.randn(N, N, dtype=torch.float64, generator=torch.Generator().manual_seed(N)).cuda()
+    F = (F + F.T) / (4 * N ** 0.5)
+    nocc = N // 3
+    from paper_1507_02087_gb300 import sp2
+    with sp2.Purifier(N, nocc, "fp64", max_iter=1, guard=False) as P:
+        P.set_bounds((-1.5, 1.5))
+        X1 = P.run(F)
+        info = P.info()
+    X0 = (1.5 * torch.eye(N, dtype=torch.float64, device="cuda") - F) / 3.0
+    S = X0 @ X0                                              # its own error is within the same bound
+    ref = S if info["p"][1] else 2 * X0 - S
+    norms = torch.linalg.norm(X0, dim=1)
+    bound = 16 * EPS * N ** 0.5 * torch.outer(norms, norms) + 2 * EPS * ref.abs()
+    assert bool(((X1 - ref).abs() <= bound).all()) and torch.equal(X1, X1.T)
+    v = float(torch.linalg.norm(X0 - S))
+    assert info["v"][0] == pytest.approx(v, rel=1e-12)
+    assert info["trace"][1] == pytest.approx(float(torch.trace(ref)), rel=1e-12)
+
+
 @pytest.mark.parametrize("scale", [1e-6, 1e-30, 1e-120])
 def test_one_square_of_rows_of_different_scale(scale):
     # a block-diagonal matrix whose X_0 has rows of norm 1, of norm `scale` and zero rows
