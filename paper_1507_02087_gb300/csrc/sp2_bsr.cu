@@ -192,10 +192,22 @@ bsr_init_kernel(DevState* st, const int* rp, const int* ci, const double* vals, 
   __shared__ double sm[32];
   __shared__ double s_lmin, s_lmax;
   __shared__ int s_bad;
+  // bounds over the block rows: per thread, then over the warps
+  __shared__ double w_lo[32], w_hi[32];
+  double tlo = INFINITY, thi = -INFINITY;
+  int tbad = 0;
+  for (int I = threadIdx.x; I < nb; I += kIT) { tlo = fmin(tlo, lo_in[I]); thi = fmax(thi, hi_in[I]); tbad |= bad_in[I]; }
+  #pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    tlo = fmin(tlo, __shfl_xor_sync(0xffffffffu, tlo, o));
+    thi = fmax(thi, __shfl_xor_sync(0xffffffffu, thi, o));
+  }
+  if ((threadIdx.x & 31) == 0) { w_lo[threadIdx.x >> 5] = tlo; w_hi[threadIdx.x >> 5] = thi; }
+  tbad = __syncthreads_or(tbad);
   if (threadIdx.x == 0) {
     double lo = INFINITY, hi = -INFINITY;
-    int bad = 0;
-    for (int I = 0; I < nb; ++I) { lo = fmin(lo, lo_in[I]); hi = fmax(hi, hi_in[I]); bad |= bad_in[I]; }
+    int bad = tbad ? 1 : 0;
+    for (int w = 0; w < kIT / 32; ++w) { lo = fmin(lo, w_lo[w]); hi = fmax(hi, w_hi[w]); }
     if (!isfinite(lo) || !isfinite(hi)) bad = 1;
     if (st->ubounds) {                           // the caller's outer bounds (§3: any serve)
       lo = st->ub_lo;
@@ -497,14 +509,26 @@ bsr_numeric_kernel(DevState* st, Mat X, int W, Pairs P, float* svals, uint8_t* s
 // u_q = floor(2 n2_q / 2^(e-40)) units (2^e <= tau^2 < 2^(e+1)), the budget is
 // floor(tau^2 / 2^(e-40)).  The pairs with key (n2 bits, q) <= K* are dropped, K* the
 // largest key whose prefix sum is within the budget.  Integer sums do not depend on the
-// summation order, so one CTA finds K* by a radix select: eight passes over the bytes of
+// summation order, so K* comes from a radix select over the whole GPU: six passes over 11 bits each of
 // the n2 bit pattern (non-negative doubles order like their bit patterns), each a
-// 256-bucket histogram of units over the candidates that share the digits chosen so far,
+// histogram of units over the candidates that share the digits chosen so far, one launch per pass,
 // find the value G whose candidates no longer all fit; they all weigh u(G), so the first
 // m = (budget - units below G) / u(G) of them in q order are dropped.  The pair list is
 // in (I, J) order, so q breaks ties as (I, J) does.  `cbits` (nnz entries of scratch)
-// caches each pair's candidate bits (~0 if none).
-constexpr int kEC = 512;
+// caches each pair's candidate bits (~0 if none).  Nine launches of about 3 us; as one CTA with eight passes
+// it took 115 us for 5.9 k pairs, and its time grew with them.
+constexpr int kEC = 256, kECBins = 2048, kECPasses = 6;
+
+struct EcStep { unsigned long long prefix, below; };
+struct EcScratch {
+  unsigned long long total;                       // units of all candidates
+  EcStep step[kECPasses + 1];                     // digits chosen and units below them after so many passes
+  unsigned long long hist[kECPasses][kECBins];
+  int ties[1];                                    // per CTA: pairs with the key's bits (grid entries)
+};
+
+__host__ __device__ constexpr int ec_shift(int pass) { return pass < 5 ? 53 - 11 * pass : 0; }   // 53 42 31 20 9 0
+__host__ __device__ constexpr int ec_bits(int pass) { return pass < 5 ? 11 : 9; }
 
 __device__ __forceinline__ uint64_t ec_units(uint64_t bits, int e) {
   return (uint64_t)floor(ldexp(__longlong_as_double((long long)bits), 41 - e));
@@ -516,107 +540,214 @@ __device__ __forceinline__ uint64_t warp_sum_u64(uint64_t v) {
   return v;
 }
 
-__global__ void __launch_bounds__(kEC)
-bsr_errctl_kernel(const DevState* st, const double* n2, const int* row, const int* col, const int* nnz_p,
-                  uint64_t* cbits, uint8_t* keep, double tau2) {
-  __shared__ unsigned long long hist[256];
-  __shared__ unsigned long long s_u64[2];
-  __shared__ int s_int[kEC + 1];
-  if (st && !st->iter_active) return;
-  const int nnz = *nnz_p;
-  const int tid = threadIdx.x, lane = tid & 31;
-  constexpr uint64_t kNone = ~0ull;
-  if (!(tau2 > 0.0)) {
-    for (int q = tid; q < nnz; q += kEC) keep[q] = 1;
-    return;
+// The digit of pass `pass` from its histogram: the first bin whose units no longer fit (the last one if all do).
+// Every CTA computes it, one of them writes it down.  sm: kEC + 2 values.
+__device__ __forceinline__ EcStep ec_choose(EcScratch* S, int pass, uint64_t budget, unsigned long long* sm) {
+  const EcStep prev = S->step[pass];
+  const int nb = 1 << ec_bits(pass), per = (nb + kEC - 1) / kEC, tid = threadIdx.x;
+  unsigned long long loc = 0ull;
+  for (int i = 0; i < per; ++i) {
+    const int d = tid * per + i;
+    if (d < nb) loc += S->hist[pass][d];
   }
-  const int e = ilogb(tau2);     // 2^e <= tau^2 < 2^(e+1)
-  const uint64_t budget = (uint64_t)floor(ldexp(tau2, 40 - e));
-  // candidate bits and the total of their units
-  if (tid == 0) s_u64[0] = 0ull;
+  sm[tid] = loc;
+  if (tid == 0) { sm[kEC] = prev.below; sm[kEC + 1] = 0ull; }
   __syncthreads();
+  // exclusive prefix over the threads' sums
+  unsigned long long run = prev.below;
+  for (int o = 1; o < kEC; o <<= 1) {
+    const unsigned long long t = tid >= o ? sm[tid - o] : 0ull;
+    __syncthreads();
+    sm[tid] += t;
+    __syncthreads();
+  }
+  run += tid ? sm[tid - 1] : 0ull;
+  __syncthreads();
+  // the first bin d with run + hist[d] > budget; bins are scanned in order, so the smallest such d wins
+  __shared__ int s_d;
+  if (tid == 0) s_d = nb - 1;
+  __syncthreads();
+  for (int i = 0; i < per; ++i) {
+    const int d = tid * per + i;
+    if (d >= nb - 1) break;
+    const unsigned long long h = S->hist[pass][d];
+    if (run + h > budget) { atomicMin(&s_d, d); break; }
+    run += h;
+  }
+  __syncthreads();
+  const int d = s_d;
+  // units below bin d
+  if (d / per == tid) {
+    unsigned long long below = prev.below + (tid ? sm[tid - 1] : 0ull);
+    for (int k = tid * per; k < d; ++k) below += S->hist[pass][k];
+    sm[kEC] = below;
+  }
+  __syncthreads();
+  EcStep r;
+  r.prefix = prev.prefix | ((unsigned long long)d << ec_shift(pass));
+  r.below = sm[kEC];
+  __syncthreads();
+  return r;
+}
+
+__device__ __forceinline__ uint64_t ec_budget(double tau2, int& e) {
+  e = ilogb(tau2);                                // 2^e <= tau^2 < 2^(e+1)
+  return (uint64_t)floor(ldexp(tau2, 40 - e));
+}
+
+// candidate bits and the total of their units (total zeroed before), the histograms cleared
+__global__ void __launch_bounds__(kEC)
+ec_candidates_kernel(const DevState* st, const double* n2, const int* row, const int* col, const int* nnz_p,
+                     uint64_t* cbits, double tau2, EcScratch* S) {
+  if (st && !st->iter_active) return;
+  const int nnz = *nnz_p, lane = threadIdx.x & 31;
+  int e;
+  (void)ec_budget(tau2, e);
+  const int first = blockIdx.x * kEC + threadIdx.x, all = gridDim.x * kEC;
+  for (int i = first; i < kECPasses * kECBins; i += all) (&S->hist[0][0])[i] = 0ull;
+  if (first == 0) S->step[0] = EcStep{0ull, 0ull};
   uint64_t acc = 0;
-  for (int q = tid; q < nnz; q += kEC) {
+  for (int q = first; q < nnz; q += all) {
     const double v = n2[q];
     const bool c = row[q] != col[q] && 2.0 * v <= tau2;
-    const uint64_t b = c ? (uint64_t)__double_as_longlong(v) : kNone;
+    const uint64_t b = c ? (uint64_t)__double_as_longlong(v) : ~0ull;
     cbits[q] = b;
     if (c) acc += ec_units(b, e);
   }
   acc = warp_sum_u64(acc);
-  if (lane == 0) atomicAdd(&s_u64[0], (unsigned long long)acc);
+  if (lane == 0 && acc) atomicAdd(&S->total, (unsigned long long)acc);
+}
+
+__global__ void __launch_bounds__(kEC)
+ec_pass_kernel(const DevState* st, const int* nnz_p, const uint64_t* cbits, double tau2, EcScratch* S, int pass) {
+  __shared__ unsigned long long hist[kECBins];
+  __shared__ unsigned long long sm[kEC + 2];
+  if (st && !st->iter_active) return;
+  int e;
+  const uint64_t budget = ec_budget(tau2, e);
+  if (S->total <= budget) return;                 // everything fits
+  const int tid = threadIdx.x, lane = tid & 31, nnz = *nnz_p;
+  uint64_t prefix = 0, pmask = 0;
+  if (pass > 0) {
+    const EcStep c = ec_choose(S, pass - 1, budget, sm);
+    if (blockIdx.x == 0 && tid == 0) S->step[pass] = c;
+    prefix = c.prefix;
+    pmask = ~0ull << ec_shift(pass - 1);
+  }
+  const int shift = ec_shift(pass), bins = 1 << ec_bits(pass);
+  for (int d = tid; d < bins; d += kEC) hist[d] = 0ull;
   __syncthreads();
-  const uint64_t total = s_u64[0];
-  uint64_t gbits = kNone;   // candidates with bits < gbits are dropped ...
-  int qstar = -1;           // ... and those with bits == gbits and q <= qstar
-  if (total > budget) {
-    uint64_t prefix = 0, pmask = 0, below = 0;
-    for (int shift = 56; shift >= 0; shift -= 8) {
-      for (int d = tid; d < 256; d += kEC) hist[d] = 0ull;
-      __syncthreads();
-      for (int q0 = 0; q0 < nnz; q0 += kEC) {
-        const int q = q0 + tid;
-        const uint64_t b = q < nnz ? cbits[q] : kNone;
-        const bool in = b != kNone && (b & pmask) == prefix;
-        const int dig = in ? (int)((b >> shift) & 255u) : -1;
-        const uint64_t u = in ? ec_units(b, e) : 0ull;
-        const unsigned vm = __ballot_sync(0xffffffffu, in);
-        if (!vm) continue;
-        const int d0 = __shfl_sync(0xffffffffu, dig, __ffs(vm) - 1);
-        if (__all_sync(0xffffffffu, !in || dig == d0)) {
-          const uint64_t sum = warp_sum_u64(u);     // one atomic for the warp's common digit
-          if (lane == 0) atomicAdd(&hist[d0], (unsigned long long)sum);
-        } else if (in) {
-          atomicAdd(&hist[dig], (unsigned long long)u);
-        }
-      }
-      __syncthreads();
-      if (tid == 0) {
-        uint64_t run = below;
-        int d = 0;
-        for (; d < 255; ++d) {
-          if (run + hist[d] > budget) break;
-          run += hist[d];
-        }
-        s_u64[0] = run;
-        s_u64[1] = (uint64_t)d;
-      }
-      __syncthreads();
-      below = s_u64[0];
-      prefix |= s_u64[1] << shift;
-      pmask |= 255ull << shift;
-      __syncthreads();
+  for (int q0 = blockIdx.x * kEC; q0 < nnz; q0 += gridDim.x * kEC) {
+    const int q = q0 + tid;
+    const uint64_t b = q < nnz ? cbits[q] : ~0ull;
+    const bool in = b != ~0ull && (b & pmask) == prefix;
+    const int dig = in ? (int)((b >> shift) & (uint64_t)(bins - 1)) : -1;
+    const uint64_t u = in ? ec_units(b, e) : 0ull;
+    const unsigned vm = __ballot_sync(0xffffffffu, in);
+    if (!vm) continue;
+    const int d0 = __shfl_sync(0xffffffffu, dig, __ffs(vm) - 1);
+    if (__all_sync(0xffffffffu, !in || dig == d0)) {
+      const uint64_t sum = warp_sum_u64(u);       // one atomic for the warp's common digit
+      if (lane == 0) atomicAdd(&hist[d0], (unsigned long long)sum);
+    } else if (in) {
+      atomicAdd(&hist[dig], (unsigned long long)u);
     }
-    gbits = prefix;
-    // every candidate with bits == gbits weighs u(gbits) > 0; m of them fit
-    const uint64_t ug = ec_units(gbits, e);
-    const uint64_t m = (budget - below) / ug;
-    // the m-th member in q order: counts over contiguous q ranges, then a scan
-    const int chunk = (nnz + kEC - 1) / kEC;
-    const int lo = tid * chunk, hi = min(nnz, lo + chunk);
-    int c = 0;
-    for (int q = lo; q < hi; ++q) c += cbits[q] == gbits ? 1 : 0;
-    s_int[tid + 1] = c;
-    if (tid == 0) s_int[0] = 0;
-    __syncthreads();
-    if (tid == 0) {
-      for (int t = 1; t <= kEC; ++t) s_int[t] += s_int[t - 1];
-      s_u64[0] = ~0ull;
-    }
-    __syncthreads();
-    if (m > 0 && (uint64_t)s_int[tid] < m && m <= (uint64_t)s_int[tid + 1]) {
-      int seen = s_int[tid];
-      for (int q = lo; q < hi; ++q)
-        if (cbits[q] == gbits && (uint64_t)(++seen) == m) { s_u64[0] = (unsigned long long)q; break; }
-    }
-    __syncthreads();
-    qstar = m > 0 ? (int)s_u64[0] : -1;
   }
-  for (int q = tid; q < nnz; q += kEC) {
-    const uint64_t b = cbits[q];
-    const bool drop = b != kNone && (b < gbits || (b == gbits && q <= qstar));
-    keep[q] = drop ? 0 : 1;
+  __syncthreads();
+  for (int d = tid; d < bins; d += kEC)
+    if (hist[d]) atomicAdd(&S->hist[pass][d], hist[d]);
+}
+
+// The key's bits G and how many pairs weigh them before each CTA's range of q.
+__global__ void __launch_bounds__(kEC)
+ec_ties_kernel(const DevState* st, const int* nnz_p, const uint64_t* cbits, double tau2, EcScratch* S) {
+  __shared__ unsigned long long sm[kEC + 2];
+  __shared__ int s_n;
+  if (st && !st->iter_active) return;
+  int e;
+  const uint64_t budget = ec_budget(tau2, e);
+  if (S->total <= budget) return;
+  const EcStep c = ec_choose(S, kECPasses - 1, budget, sm);
+  if (blockIdx.x == 0 && threadIdx.x == 0) S->step[kECPasses] = c;
+  if (threadIdx.x == 0) s_n = 0;
+  __syncthreads();
+  const int nnz = *nnz_p, chunk = (nnz + gridDim.x - 1) / gridDim.x;
+  const int lo = blockIdx.x * chunk, hi = min(nnz, lo + chunk);
+  int n = 0;
+  for (int q = lo + threadIdx.x; q < hi; q += kEC) n += cbits[q] == c.prefix ? 1 : 0;
+  if (n) atomicAdd(&s_n, n);
+  __syncthreads();
+  if (threadIdx.x == 0) S->ties[blockIdx.x] = s_n;
+}
+
+__global__ void __launch_bounds__(kEC)
+ec_keep_kernel(const DevState* st, const int* nnz_p, const uint64_t* cbits, double tau2, EcScratch* S, uint8_t* keep) {
+  __shared__ int s_warp[kEC / 32];
+  __shared__ int s_before;
+  if (st && !st->iter_active) return;
+  int e;
+  const uint64_t budget = ec_budget(tau2, e);
+  const int nnz = *nnz_p, chunk = (nnz + gridDim.x - 1) / gridDim.x, tid = threadIdx.x, lane = tid & 31;
+  const int lo = blockIdx.x * chunk, hi = min(nnz, lo + chunk);
+  if (S->total <= budget) {
+    for (int q = lo + tid; q < hi; q += kEC) keep[q] = cbits[q] == ~0ull ? 1 : 0;
+    return;
   }
+  const EcStep c = S->step[kECPasses];
+  const uint64_t gbits = c.prefix;
+  // every candidate with bits == gbits weighs u(gbits) > 0; the first m of them fit
+  const uint64_t m = (budget - c.below) / ec_units(gbits, e);
+  if (tid == 0) s_before = 0;
+  __syncthreads();
+  int b4 = 0;
+  for (int t = tid; t < (int)blockIdx.x; t += kEC) b4 += S->ties[t];
+  if (b4) atomicAdd(&s_before, b4);
+  __syncthreads();
+  uint64_t before = (uint64_t)s_before;
+  const bool any = S->ties[blockIdx.x] > 0;
+  for (int q0 = lo; q0 < hi; q0 += kEC) {
+    const int q = q0 + tid;
+    const uint64_t b = q < hi ? cbits[q] : ~0ull;
+    const bool tie = b == gbits;
+    uint64_t rank = 0;                             // ties at smaller q
+    if (any) {
+      const unsigned v = __ballot_sync(0xffffffffu, tie);
+      if (lane == 0) s_warp[tid >> 5] = __popc(v);
+      __syncthreads();
+      int pre = 0, all = 0;
+      for (int w = 0; w < kEC / 32; ++w) {
+        if (w < (tid >> 5)) pre += s_warp[w];
+        all += s_warp[w];
+      }
+      rank = before + (uint64_t)(pre + __popc(v & ((1u << lane) - 1u)));
+      before += (uint64_t)all;
+      __syncthreads();
+    }
+    if (q < hi) keep[q] = b != ~0ull && (b < gbits || (tie && rank < m)) ? 0 : 1;
+  }
+}
+
+__global__ void ec_all_kernel(const DevState* st, const int* nnz_p, uint8_t* keep) {   // tau = 0 drops nothing
+  if (st && !st->iter_active) return;
+  const int nnz = *nnz_p;
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nnz; q += gridDim.x * blockDim.x) keep[q] = 1;
+}
+
+size_t errctl_scratch_bytes(int grid) { return sizeof(EcScratch) + sizeof(int) * grid; }
+
+// scratch: errctl_scratch_bytes(grid)
+void launch_errctl(const DevState* st, const double* n2, const int* row, const int* col, const int* nnz_p, uint64_t* cbits,
+                   uint8_t* keep, double tau2, void* scratch, int grid, cudaStream_t s) {
+  if (!(tau2 > 0.0)) {
+    ec_all_kernel<<<grid, kEC, 0, s>>>(st, nnz_p, keep);
+    return;
+  }
+  EcScratch* S = static_cast<EcScratch*>(scratch);
+  cudaMemsetAsync(&S->total, 0, sizeof(S->total), s);
+  ec_candidates_kernel<<<grid, kEC, 0, s>>>(st, n2, row, col, nnz_p, cbits, tau2, S);
+  for (int p = 0; p < kECPasses; ++p) ec_pass_kernel<<<grid, kEC, 0, s>>>(st, nnz_p, cbits, tau2, S, p);
+  ec_ties_kernel<<<grid, kEC, 0, s>>>(st, nnz_p, cbits, tau2, S);
+  ec_keep_kernel<<<grid, kEC, 0, s>>>(st, nnz_p, cbits, tau2, S, keep);
 }
 
 // ---- mixed-norm truncation (rule 2) ------------------------------------------------------
@@ -779,20 +910,43 @@ void launch_mixctl(const DevState* st, const double* n2, const int* ptr, const i
   mix_keep_kernel<<<grid, 256, 0, s>>>(st, n2, row, col, nnz_p, tau, cut, keep);
 }
 
-// per-round reduction over the pairs and the stop test (stored-diagonal trace)
-__global__ void __launch_bounds__(1024)
-bsr_finalize_kernel(DevState* st, const double* spart, const int* nnz_p, cudaGraphConditionalHandle cond,
-                    int use_cond) {
+// The pairs' partials (v^2, trace) summed over the GPU into kFinParts records: FP64 additions run at two a clock and
+// SM, so one CTA took 64 us for the 128 k pairs of a 32 x 24 x 24 lattice, in each kernel that needs them.
+constexpr int kFinParts = 128;
+
+__global__ void __launch_bounds__(NT)
+bsr_partials_kernel(const DevState* st, const double* spart, const int* nnz_p, double* psum) {
   __shared__ double sm[32];
+  if (!st->iter_active) return;
+  const int nnz = *nnz_p, chunk = (nnz + kFinParts - 1) / kFinParts;
+  const int lo = blockIdx.x * chunk, hi = min(nnz, lo + chunk);
+  double a = 0.0, b = 0.0;
+  for (int q = lo + threadIdx.x; q < hi; q += NT) {
+    const double2 v = *reinterpret_cast<const double2*>(spart + 2 * (int64_t)q);
+    a += v.x;
+    b += v.y;
+  }
+  a = block_sum<NT>(a, sm);
+  b = block_sum<NT>(b, sm);
+  if (threadIdx.x == 0) {
+    psum[2 * blockIdx.x] = a;
+    psum[2 * blockIdx.x + 1] = b;
+  }
+}
+
+// per-round reduction and the stop test (stored-diagonal trace)
+__global__ void __launch_bounds__(kFinParts)
+bsr_finalize_kernel(DevState* st, const double* psum, const int* nnz_p, cudaGraphConditionalHandle cond,
+                    int use_cond) {
+  __shared__ double sm[96];
   if (!st->iter_active) {
     if (use_cond && threadIdx.x == 0) cudaGraphSetConditional(cond, 0);
     return;
   }
+  touch_state(st, st->k);
   const int nnz = *nnz_p;
-  double a = 0.0, b = 0.0;
-  for (int t = threadIdx.x; t < nnz; t += 1024) { a += spart[2 * (int64_t)t]; b += spart[2 * (int64_t)t + 1]; }
-  a = block_sum<1024>(a, sm);
-  b = block_sum<1024>(b, sm);
+  double a = psum[2 * threadIdx.x], b = psum[2 * threadIdx.x + 1], c = 0.0;
+  block_sum3<kFinParts>(a, b, c, kFinParts, sm);
   if (threadIdx.x != 0) return;
   const int k = st->k + 1;
   double ca, cb, cc;
@@ -878,24 +1032,28 @@ __device__ __forceinline__ bool tile_active(const uint32_t* sbits, int nb, int W
   return act;
 }
 
+// The list runs through bands of TBAND tile rows, column by column: the tiles in flight at once (one per SM) then
+// share their block rows, about 8 x 19 of them instead of 2 x 76, and more of the operands come from L2.
+constexpr int TBAND = 8;
+
 __global__ void tile_count_kernel(const DevState* st, const uint32_t* sbits, int nb, int W, int ncg, int* counts) {
   if (!st->iter_active) return;
-  const int g = blockIdx.x;
+  const int lane = threadIdx.x, g = blockIdx.x * TBAND + lane % TBAND;
   int n = 0;
-  for (int c = threadIdx.x; c < ncg; c += 32) n += tile_active(sbits, nb, W, g, c) ? 1 : 0;
+  for (int c = lane / TBAND; c < ncg; c += 32 / TBAND) n += g * TTR < nb && tile_active(sbits, nb, W, g, c) ? 1 : 0;
   #pragma unroll
   for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
-  if (threadIdx.x == 0) counts[g] = n;
+  if (lane == 0) counts[blockIdx.x] = n;
 }
 
 __global__ void tile_fill_kernel(const DevState* st, const uint32_t* sbits, int nb, int W, int ncg, const int* tptr,
                                  int* tiles) {
   if (!st->iter_active) return;
-  const int g = blockIdx.x, lane = threadIdx.x;
-  int pos = tptr[g];
-  for (int c0 = 0; c0 < ncg; c0 += 32) {
-    const int c = c0 + lane;
-    const bool act = c < ncg && tile_active(sbits, nb, W, g, c);
+  const int lane = threadIdx.x, g = blockIdx.x * TBAND + lane % TBAND;
+  int pos = tptr[blockIdx.x];
+  for (int c0 = 0; c0 < ncg; c0 += 32 / TBAND) {
+    const int c = c0 + lane / TBAND;
+    const bool act = c < ncg && g * TTR < nb && tile_active(sbits, nb, W, g, c);
     const uint32_t m = __ballot_sync(0xffffffffu, act);
     if (act) tiles[pos + __popc(m & ((1u << lane) - 1u))] = g * ncg + c;
     pos += __popc(m);
@@ -960,10 +1118,10 @@ static int meta_sms() {
 
 cudaError_t tc_tiles_launch(const DevState* st, const Mat& X, const Pairs& P, const uint32_t* sbits, int nb, int W,
                             int* counts, int* tptr, int* tnnz, int* tiles, int* meta, cudaStream_t s) {
-  const int ng = (nb + TTR - 1) / TTR, ncg = (nb + TTC - 1) / TTC;
-  tile_count_kernel<<<ng, 32, 0, s>>>(st, sbits, nb, W, ncg, counts);
-  scan_kernel<<<1, 1024, 0, s>>>(counts, ng, tptr, tnnz, st);
-  tile_fill_kernel<<<ng, 32, 0, s>>>(st, sbits, nb, W, ncg, tptr, tiles);
+  const int ncg = (nb + TTC - 1) / TTC, bands = (nb + TTR * TBAND - 1) / (TTR * TBAND);
+  tile_count_kernel<<<bands, 32, 0, s>>>(st, sbits, nb, W, ncg, counts);
+  scan_kernel<<<1, 1024, 0, s>>>(counts, bands, tptr, tnnz, st);
+  tile_fill_kernel<<<bands, 32, 0, s>>>(st, sbits, nb, W, ncg, tptr, tiles);
   tile_meta_kernel<<<4 * meta_sms(), 256, 0, s>>>(st, X, P, sbits, nb, W, ncg, tiles, tnnz, meta);
   return cudaGetLastError();
 }
@@ -1013,8 +1171,10 @@ struct sp2_bsr_ctx {
   float* svals = nullptr;
   uint8_t* skeep = nullptr;
   double* spart = nullptr;       // per-pair partials; also the candidate scratch of rule 1
+  double* psum = nullptr;        // kFinParts sums of them
   double* sn2 = nullptr;         // per-pair ||X_IJ||_F^2 of the newest blocks
-  void* mixscr = nullptr;        // rule 2: per-row overflow keys and the cut
+  void* mixscr = nullptr;        // rule 1: histograms and tie counts; rule 2: per-row overflow keys and the cut
+  int ec_grid = 1;               // rule 1: CTAs of a pass
   void* lz = nullptr;            // norm = 1: Lanczos scratch for the mixed norm (nb x nb)
   int lzld = 0;
   int* counts = nullptr;
@@ -1065,7 +1225,7 @@ static void bsr_free(sp2_bsr_ctx* h) {
   cudaFree(h->tiles); cudaFree(h->tptr); cudaFree(h->tnnz); cudaFree(h->meta);
   cudaFree(h->S.ptr); cudaFree(h->S.col); cudaFree(h->S.row); cudaFree(h->S.nnz);
   cudaFree(h->FP.ptr); cudaFree(h->FP.col); cudaFree(h->FP.row); cudaFree(h->FP.nnz);
-  cudaFree(h->sbits); cudaFree(h->svals); cudaFree(h->skeep); cudaFree(h->spart); cudaFree(h->sn2);
+  cudaFree(h->sbits); cudaFree(h->svals); cudaFree(h->skeep); cudaFree(h->spart); cudaFree(h->psum); cudaFree(h->sn2);
   cudaFree(h->mixscr); cudaFree(h->lz);
   cudaFree(h->counts);
   cudaFree(h->fbits); cudaFree(h->frank); cudaFree(h->glo); cudaFree(h->ghi); cudaFree(h->gbad);
@@ -1154,11 +1314,13 @@ static cudaError_t add_round(sp2_bsr_ctx* h, cudaGraph_t g, cudaStream_t s, int 
                                                                     h->spart, h->sn2, tau2);
   }
   if (timed) cudaEventRecord(h->nev[2 * h->nrounds++ + 1], s);
-  if (h->lz) launch_lanczos_pairs(st, h->S.row, h->S.col, sn, h->spart, h->lz, nb, h->lzld, s);
-  bsr_finalize_kernel<<<1, 1024, 0, s>>>(st, h->spart, sn, h->cond, use_cond);
+  bsr_partials_kernel<<<kFinParts, NT, 0, s>>>(st, h->spart, sn, h->psum);
+  if (h->lz)
+    launch_lanczos_pairs(st, h->S.row, h->S.col, sn, h->spart, h->psum, kFinParts, h->lz, nb, h->lzld, s);
+  bsr_finalize_kernel<<<1, kFinParts, 0, s>>>(st, h->psum, sn, h->cond, use_cond);
   if (h->rule == SP2_TRUNC_ERROR)
-    bsr_errctl_kernel<<<1, kEC, 0, s>>>(st, h->sn2, h->S.row, h->S.col, sn, reinterpret_cast<uint64_t*>(h->spart),
-                                        h->skeep, tau2);
+    launch_errctl(st, h->sn2, h->S.row, h->S.col, sn, reinterpret_cast<uint64_t*>(h->spart), h->skeep, tau2, h->mixscr,
+                  h->ec_grid, s);
   else if (h->rule == SP2_TRUNC_MIXED)
     launch_mixctl(st, h->sn2, h->S.ptr, h->S.row, h->S.col, sn, nb, h->tau, h->mixscr, h->skeep, grid_persistent(), s);
   // 4. truncation -> next iterate
@@ -1251,6 +1413,7 @@ extern "C" sp2_status sp2_create_bsr_ex(int64_t N, int64_t n_occ, double tau, in
        cudaMalloc(&h->svals, sizeof(float) * BE * h->cap_s) == cudaSuccess &&
        cudaMalloc(&h->skeep, h->cap_s) == cudaSuccess &&
        cudaMalloc(&h->spart, sizeof(double) * 2 * h->cap_s) == cudaSuccess &&
+       cudaMalloc(&h->psum, sizeof(double) * 2 * kFinParts) == cudaSuccess &&
        cudaMalloc(&h->sn2, sizeof(double) * h->cap_s) == cudaSuccess &&
        cudaMalloc(&h->counts, sizeof(int) * nb) == cudaSuccess &&
        cudaMalloc(&h->fbits, sizeof(uint32_t) * nb * W) == cudaSuccess &&
@@ -1275,6 +1438,8 @@ extern "C" sp2_status sp2_create_bsr_ex(int64_t N, int64_t n_occ, double tau, in
          cudaMalloc(&h->meta, sizeof(int) * TMETA * (size_t)ng * ncg) == cudaSuccess;
   }
   if (ok && rule == SP2_TRUNC_MIXED) ok = cudaMalloc(&h->mixscr, mixctl_scratch_bytes(nb)) == cudaSuccess;
+  h->ec_grid = (int)std::min<int64_t>((h->cap_s + 1023) / 1024, grid_persistent() / 2);
+  if (ok && rule == SP2_TRUNC_ERROR) ok = cudaMalloc(&h->mixscr, errctl_scratch_bytes(h->ec_grid)) == cudaSuccess;
   if (ok && o.norm == 1) {
     h->lzld = (nb + 63) / 64 * 64;
     ok = cudaMalloc(&h->lz, lanczos_scratch_bytes(h->lzld)) == cudaSuccess;
@@ -1366,8 +1531,8 @@ extern "C" sp2_status sp2_run_bsr(sp2_bsr h, const int32_t* row_ptr_dev, const i
   bsr_scale_pairs_kernel<<<grid_persistent(), NT, 0, s>>>(st, row_ptr_dev, h->fbits, h->frank, vals_dev, W, h->FP,
                                                            h->svals, h->skeep, h->sn2, tau2);
   if (h->rule == SP2_TRUNC_ERROR)
-    bsr_errctl_kernel<<<1, kEC, 0, s>>>(nullptr, h->sn2, h->FP.row, h->FP.col, h->FP.nnz,
-                                        reinterpret_cast<uint64_t*>(h->spart), h->skeep, tau2);
+    launch_errctl(nullptr, h->sn2, h->FP.row, h->FP.col, h->FP.nnz, reinterpret_cast<uint64_t*>(h->spart), h->skeep, tau2,
+                  h->mixscr, h->ec_grid, s);
   else if (h->rule == SP2_TRUNC_MIXED)
     launch_mixctl(nullptr, h->sn2, h->FP.ptr, h->FP.row, h->FP.col, h->FP.nnz, nb, h->tau, h->mixscr, h->skeep,
                   grid_persistent(), s);
@@ -1479,6 +1644,7 @@ extern "C" int32_t sp2_test_bsr_keep(const float* dense_dev, int64_t N, double t
   const int nb = (int)(N / B);
   cudaStream_t s = (cudaStream_t)stream;
   const int npairs = nb * (nb + 1) / 2;
+  const int ec_grid = std::min((npairs + 1023) / 1024, grid_persistent() / 2);
   std::vector<int> row(npairs), col(npairs);
   for (int I = 0, q = 0; I < nb; ++I)
     for (int J = I; J < nb; ++J, ++q) { row[q] = I; col[q] = J; }
@@ -1492,7 +1658,8 @@ extern "C" int32_t sp2_test_bsr_keep(const float* dense_dev, int64_t N, double t
             cudaMalloc(&scratch, sizeof(uint64_t) * npairs) == cudaSuccess &&
             cudaMalloc(&drow, sizeof(int) * npairs) == cudaSuccess &&
             cudaMalloc(&dcol, sizeof(int) * npairs) == cudaSuccess && cudaMalloc(&dnp, sizeof(int)) == cudaSuccess &&
-            cudaMalloc(&keepp, npairs) == cudaSuccess && cudaMalloc(&mscr, mixctl_scratch_bytes(nb)) == cudaSuccess &&
+            cudaMalloc(&keepp, npairs) == cudaSuccess &&
+            cudaMalloc(&mscr, std::max(mixctl_scratch_bytes(nb), errctl_scratch_bytes(ec_grid))) == cudaSuccess &&
             cudaMalloc(&dptr, sizeof(int) * (nb + 1)) == cudaSuccess;
   std::vector<int> ptr(nb + 1, 0);
   for (int I = 0; I < nb; ++I) ptr[I + 1] = ptr[I] + (nb - I);
@@ -1508,7 +1675,7 @@ extern "C" int32_t sp2_test_bsr_keep(const float* dense_dev, int64_t N, double t
     if (ok) {
       test_pairs_gather_kernel<<<256, 256, 0, s>>>(n2_full, nb, drow, dcol, npairs, n2p);
       if (rule == SP2_TRUNC_ERROR)
-        bsr_errctl_kernel<<<1, kEC, 0, s>>>(nullptr, n2p, drow, dcol, dnp, scratch, keepp, tau * tau);
+        launch_errctl(nullptr, n2p, drow, dcol, dnp, scratch, keepp, tau * tau, mscr, ec_grid, s);
       else
         launch_mixctl(nullptr, n2p, dptr, drow, dcol, dnp, nb, tau, mscr, keepp, 256, s);
       test_pairs_scatter_kernel<<<256, 256, 0, s>>>(keepp, nb, drow, dcol, npairs, keep_dev);

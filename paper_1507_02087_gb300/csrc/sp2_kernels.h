@@ -76,10 +76,11 @@ cudaError_t launch_lanczos(DevState* st, const double* buf0, const double* buf1,
                            const double* part, int ntiles, void* lz, int N, int ld, cudaStream_t s);
 // The same estimate for the mixed norm of the block-sparse path: the spectral norm of the nb x nb
 // matrix of block norms of X - X^2, built from the square's upper-pair records (row[q], col[q],
-// part[2q] = ||(X - X^2)_IJ||_F^2, doubled off the diagonal; *nnz_p pairs); ld = nb rounded up
+// part[2q] = ||(X - X^2)_IJ||_F^2, doubled off the diagonal; *nnz_p pairs; their sums
+// in nsums records, v^2 first); ld = nb rounded up
 // to a multiple of 64 for lanczos_scratch_bytes.
 cudaError_t launch_lanczos_pairs(DevState* st, const int* row, const int* col, const int* nnz_p, const double* part,
-                                 void* lz, int nb, int ld, cudaStream_t s);
+                                 const double* sums, int nsums, void* lz, int nb, int ld, cudaStream_t s);
 // The estimate on the tensor-core path, one problem: X_{k-1} and X_k from the instance's piece
 // arena (inst: its device record), part / nparts the forward square's records of 4 doubles.
 cudaError_t add_lanczos_tc_nodes(cudaGraph_t g, cudaGraphNode_t dep, DevState* st, const tc::Instance* inst,

@@ -93,15 +93,13 @@ __device__ __forceinline__ void lz_operands(const DevState* st, const double* bu
 }
 
 // n x n operator stored with leading dimension ld; the square's partial records (v^2 first, `rec`
-// doubles each), ntiles of them (or *ntiles_dev when given), set the scale.
+// doubles each), ntiles of them, set the scale.
 __global__ void __launch_bounds__(kLzThreads)
-lz_start_kernel(const DevState* st, const double* __restrict__ part, int ntiles, const int* ntiles_dev, int rec,
-                LzScratch* lz, int N, int ld) {
+lz_start_kernel(const DevState* st, const double* __restrict__ part, int ntiles, int rec, LzScratch* lz, int N, int ld) {
   __shared__ double sm[96];
   if (st->done) return;
-  const int cnt = ntiles_dev ? *ntiles_dev : ntiles;
   double v2 = 0.0, ss = 0.0, none = 0.0;         // v_{k-1}^2 from the square's partials
-  for (int t = threadIdx.x; t < cnt; t += kLzThreads) v2 += part[rec * (int64_t)t];
+  for (int t = threadIdx.x; t < ntiles; t += kLzThreads) v2 += part[rec * (int64_t)t];
   for (int i = threadIdx.x; i < N; i += kLzThreads) {
     const double u = start_entry(i);
     ss = fma(u, u, ss);
@@ -433,14 +431,14 @@ size_t lanczos_scratch_bytes(int ld) {
 }
 
 // start, form (the caller's kernel and arguments), the steps and eig, on a stream or as a chain of graph nodes.
-static cudaError_t emit(f64tc::Sink& sink, DevState* st, const double* part, int ntiles, const int* ntiles_dev, int rec,
-                        LzScratch* lz, int N, int ld, const void* form, void** form_args, const void* fill = nullptr,
+static cudaError_t emit(f64tc::Sink& sink, DevState* st, const double* part, int ntiles, int rec, LzScratch* lz,
+                        int N, int ld, const void* form, void** form_args, const void* fill = nullptr,
                         void** fill_args = nullptr) {
   cudaError_t e = lanczos_prepare();
   if (e != cudaSuccess) return e;
   const DevState* cst = st;
   const LzScratch* clz = lz;
-  void* a0[] = {&cst, &part, &ntiles, &ntiles_dev, &rec, &lz, &N, &ld};
+  void* a0[] = {&cst, &part, &ntiles, &rec, &lz, &N, &ld};
   if ((e = sink.put((const void*)lz_start_kernel, dim3(1), dim3(kLzThreads), 0, a0)) != cudaSuccess) return e;
   if (fill && (e = sink.put(fill, dim3(form_blocks(ld)), dim3(256), 0, fill_args)) != cudaSuccess) return e;
   if ((e = sink.put(form, dim3(form_blocks(ld)), dim3(256), 0, form_args)) != cudaSuccess) return e;
@@ -459,7 +457,7 @@ static cudaError_t emit_f64(f64tc::Sink& sink, DevState* st, const double* buf0,
   LzScratch* lz = static_cast<LzScratch*>(scratch);
   const DevState* cst = st;
   void* form[] = {&cst, &buf0, &buf1, &S, &lz};
-  return emit(sink, st, part, ntiles, nullptr, 2, lz, N, ld, (const void*)lz_form_kernel, form);
+  return emit(sink, st, part, ntiles, 2, lz, N, ld, (const void*)lz_form_kernel, form);
 }
 
 static cudaError_t emit_tc(f64tc::Sink& sink, DevState* st, const tc::Instance* inst, const double* part, int nparts,
@@ -467,7 +465,7 @@ static cudaError_t emit_tc(f64tc::Sink& sink, DevState* st, const tc::Instance* 
   LzScratch* lz = static_cast<LzScratch*>(scratch);
   const DevState* cst = st;
   void* form[] = {&cst, &inst, &lz};
-  return emit(sink, st, part, nparts, nullptr, 4, lz, N, ld, (const void*)lz_form_tc_kernel, form);
+  return emit(sink, st, part, nparts, 4, lz, N, ld, (const void*)lz_form_tc_kernel, form);
 }
 
 cudaError_t add_lanczos_nodes(cudaGraph_t g, cudaGraphNode_t dep, DevState* st, const double* buf0,
@@ -509,14 +507,14 @@ cudaError_t launch_lanczos_tc(DevState* st, const tc::Instance* inst, const doub
 }
 
 cudaError_t launch_lanczos_pairs(DevState* st, const int* row, const int* col, const int* nnz_p, const double* part,
-                                 void* scratch, int nb, int ld, cudaStream_t s) {
+                                 const double* sums, int nsums, void* scratch, int nb, int ld, cudaStream_t s) {
   LzScratch* lz = static_cast<LzScratch*>(scratch);
   const DevState* cst = st;
   f64tc::Sink sink;
   sink.s = s;
   void* fill[] = {&cst, &lz, &ld};
   void* form[] = {&cst, &row, &col, &nnz_p, &part, &lz, &ld};
-  return emit(sink, st, part, 0, nnz_p, 2, lz, nb, ld, (const void*)lz_form_pairs_kernel, form,
+  return emit(sink, st, sums, nsums, 2, lz, nb, ld, (const void*)lz_form_pairs_kernel, form,
               (const void*)lz_zero_kernel, fill);
 }
 
