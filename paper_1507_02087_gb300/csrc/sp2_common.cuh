@@ -364,6 +364,19 @@ __device__ __forceinline__ void touch_state(const DevState* st, int k) {
   }
 }
 
+// a / w for a divisor shared by many quotients, given iw = 1.0 / w (correctly rounded): the quotient's estimate
+// a iw, its remainder by a fused multiply-add, and one correction give the correctly rounded quotient (P. Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34, 1990), in 3 FP64
+// operations; where the exactness conditions may fail (tiny, huge or special values) the plain division is used.
+__device__ __forceinline__ double divide_shared(double a, double w, double iw) {
+  const int ea = (__double2hiint(a) >> 20) & 0x7ff, ew = (__double2hiint(w) >> 20) & 0x7ff;
+  if (a == 0.0) return a / w;
+  // exponents away from the ends, so that neither the quotient nor the remainder leaves the normal range
+  if (ea < 200 || ea > 1846 || ew < 200 || ew > 1846 || ea - ew > 800 || ew - ea > 800) return a / w;
+  const double q = a * iw;
+  return fma(fma(-q, w, a), iw, q);
+}
+
 // Index of upper tile (I, J), I <= J, in a T x T grid whose upper tiles are numbered by rows.
 __host__ __device__ __forceinline__ int64_t upper_index(int I, int J, int T) {
   return (int64_t)I * T - (int64_t)I * (I - 1) / 2 + (J - I);
@@ -403,7 +416,9 @@ __device__ double mixed_norm_cta(int nb, double* scr, double* sm, BlockN2 block_
     block_sum3<NT>(ss, xy, none, nb, sm);
     lam = xy;                                  // x has unit norm: Rayleigh quotient
     if (!(ss > 0.0)) { lam = 0.0; break; }
-    const double inv = 1.0 / sqrt(ss);
+    if (tid == 0) sm[0] = 1.0 / sqrt(ss);      // one thread: a thousand of them keep the FP64 units busy for 10 us
+    __syncthreads();
+    const double inv = sm[0];
     bool same = true;
     for (int i = tid; i < nb; i += NT) {
       const double xn = y[i] * inv;

@@ -134,12 +134,16 @@ __global__ void scale_kernel(const DevState* st, const double* __restrict__ F, i
   if (st->done) return;
   const int N = st->N;
   const double lmax = st->scale_a, w = st->scale_w;   // (lmax, lmax - lmin) for SP2
+  __shared__ double s_iw;
+  if (threadIdx.x == 0) s_iw = 1.0 / w;
+  __syncthreads();
+  const double iw = s_iw;
   const int64_t total = (int64_t)N * N;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(e / N), j = (int)(e % N);
     const double f = F[(int64_t)i * ldf + j];
-    X0[(int64_t)i * ld + j] = ((i == j ? lmax : 0.0) - f) / w;
+    X0[(int64_t)i * ld + j] = divide_shared((i == j ? lmax : 0.0) - f, w, iw);
   }
 }
 
@@ -402,8 +406,9 @@ finalize_kernel(DevState* st, const double* __restrict__ part, int nparts, int s
     if (stride > 2) c += part[(int64_t)stride * t + 2];
   }
   block_sum3<kFinThreads>(a, b, c, nparts, sm);
-  double vk = sqrt(a);                           // v_{k-1} = ||X_{k-1} - X_{k-1}^2||_F
-  if (st->norm == 2) vk = st->spec_e;            // or e_{k-1}, the Lanczos estimate of the 2-norm
+  double vk = 0.0;                               // v_{k-1} = ||X_{k-1} - X_{k-1}^2||_F; one thread takes the root: FP64
+  if (threadIdx.x == 0) vk = st->norm == 2 ? st->spec_e : sqrt(a);   // operations run at 2 a clock and SM, so in all
+                                                 // 1024 threads it took 5 us (or e_{k-1}, the Lanczos estimate)
   if (st->norm == 1 && mscr) {                   // or m_{k-1}, the mixed norm over 64 x 64 tiles
     const int T = st->ld / kTile;
     vk = mixed_norm_cta<kFinThreads>(T, mscr, sm, [&](int I, int J) {
@@ -461,8 +466,8 @@ finalize_plain_kernel(DevState* st, const double* __restrict__ part, int nparts,
     b += part[2 * (int64_t)t + 1];
   }
   block_sum3<kFinThreads>(a, b, c, nparts, sm);
-  double vk = sqrt(a);
-  if (st->norm == 2) vk = st->spec_e;
+  double vk = 0.0;
+  if (threadIdx.x == 0) vk = st->norm == 2 ? st->spec_e : sqrt(a);
   if (st->norm == 1 && mscr) {
     const int T = st->ld / kTile;
     vk = mixed_norm_cta<kFinThreads>(T, mscr, sm, [&](int I, int J) {

@@ -115,7 +115,9 @@ lz_start_kernel(const DevState* st, const double* __restrict__ part, int ntiles,
     lz->beta[0] = 0.0;
   }
   double* q = lz_vec(lz, ld, 0);
-  const double inv = 1.0 / sqrt(ss);
+  if (threadIdx.x == 0) sm[0] = 1.0 / sqrt(ss);
+  __syncthreads();
+  const double inv = sm[0];
   for (int i = threadIdx.x; i < N; i += kLzThreads) q[i] = start_entry(i) * inv;
 }
 
@@ -199,9 +201,19 @@ __global__ void __launch_bounds__(kLzMvThreads)
 lz_step_kernel(const DevState* st, LzScratch* lz, int j, int N, int ld) {
   extern __shared__ __align__(16) float lz_smem[];
   __shared__ double sm[2][33];
-  __shared__ double s_alpha;
+  __shared__ double s_alpha, s_b, s_ib;
   if (st->done || !lz->live) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  // the warp's first row of A (up to 1024 columns of it), which does not wait for q_j
+  constexpr int PRE = 8;
+  const float4* __restrict__ A = reinterpret_cast<const float4*>(lz_a32(lz, ld));
+  const int h = ld / 4, row0 = blockIdx.x * nw + warp;
+  float4 pre[PRE];
+  if (row0 < N) {
+    #pragma unroll
+    for (int n = 0; n < PRE; ++n)
+      if (lane + 32 * n < h) pre[n] = A[(int64_t)row0 * h + lane + 32 * n];
+  }
   float* q32 = N <= kLzSmemN ? lz_smem : lz_q32(lz, ld);   // past it every CTA writes the same values
   double* q = lz_vec(lz, ld, j % 3);
   const int per = nw;                                       // rows of a CTA per sweep: one per warp
@@ -235,7 +247,12 @@ lz_step_kernel(const DevState* st, LzScratch* lz, int j, int N, int ld) {
       ss = fma(r, r, ss);
     }
     ss = cta_sum(ss, sm[0]);
-    const double b = sqrt(ss);
+    if (threadIdx.x == 0) {                                 // one thread: FP64 operations run at 2 a clock and SM
+      s_b = sqrt(ss);
+      s_ib = 1.0 / s_b;
+    }
+    __syncthreads();
+    const double b = s_b;
     const bool finite = isfinite(a) && isfinite(b);
     const bool more = finite && b > 1e-300;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -245,7 +262,7 @@ lz_step_kernel(const DevState* st, LzScratch* lz, int j, int N, int ld) {
       if (!more) lz->live = 0;
     }
     if (!more) return;
-    const double ib = 1.0 / b;
+    const double ib = s_ib;
     auto put = [&](int i, double u) {
       q32[i] = (float)u;
       if (i < N && mine(i)) q[i] = u;
@@ -258,24 +275,31 @@ lz_step_kernel(const DevState* st, LzScratch* lz, int j, int N, int ld) {
     for (int i = threadIdx.x + 4 * blockDim.x; i < ld; i += blockDim.x) put(i, i < N ? residual(i) * ib : 0.0);
   }
   __syncthreads();
-  const float4* __restrict__ A = reinterpret_cast<const float4*>(lz_a32(lz, ld));
   const float4* q4 = reinterpret_cast<const float4*>(q32);
   double* w = lz_vec(lz, ld, 3 + (j & 1));
-  const int h = ld / 4;
   double pa = 0.0;
-  for (int r = blockIdx.x * per + warp; r < N; r += gridDim.x * per) {
+  auto dot4 = [](const float4& x, const float4& v, float s) {
+    s = fmaf(x.x, v.x, s); s = fmaf(x.y, v.y, s); s = fmaf(x.z, v.z, s);
+    return fmaf(x.w, v.w, s);
+  };
+  for (int r = row0; r < N; r += gridDim.x * per) {
     const float4* ar = A + (int64_t)r * h;
     float s0 = 0.f, s1 = 0.f;
     int i = lane;
+    if (r == row0) {
+      #pragma unroll
+      for (int n = 0; n < PRE; ++n) {
+        const int c = lane + 32 * n;
+        if (c < h) (n & 1 ? s1 : s0) = dot4(pre[n], q4[c], n & 1 ? s1 : s0);
+      }
+      i += 32 * PRE;
+    }
     for (; i + 32 < h; i += 64) {
       const float4 x0 = ar[i], v0 = q4[i], x1 = ar[i + 32], v1 = q4[i + 32];
-      s0 = fmaf(x0.x, v0.x, s0); s0 = fmaf(x0.y, v0.y, s0); s0 = fmaf(x0.z, v0.z, s0); s0 = fmaf(x0.w, v0.w, s0);
-      s1 = fmaf(x1.x, v1.x, s1); s1 = fmaf(x1.y, v1.y, s1); s1 = fmaf(x1.z, v1.z, s1); s1 = fmaf(x1.w, v1.w, s1);
+      s0 = dot4(x0, v0, s0);
+      s1 = dot4(x1, v1, s1);
     }
-    if (i < h) {
-      const float4 x0 = ar[i], v0 = q4[i];
-      s0 = fmaf(x0.x, v0.x, s0); s0 = fmaf(x0.y, v0.y, s0); s0 = fmaf(x0.z, v0.z, s0); s0 = fmaf(x0.w, v0.w, s0);
-    }
+    if (i < h) s0 = dot4(ar[i], q4[i], s0);
     double s = (double)s0 + (double)s1;
     #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);

@@ -146,6 +146,10 @@ __global__ void batch_scale_split_kernel(const Instance* inst, int count, int sb
   const double lmax = st->lmax, w = st->lmax - st->lmin;
   const int fmt = In.fmt;
   const double cmid = 0.5 * (st->lmax + st->lmin), hw = 0.5 * w;
+  __shared__ double s_iw[2];
+  if (threadIdx.x < 2) s_iw[threadIdx.x] = 1.0 / (threadIdx.x ? hw : w);
+  __syncthreads();
+  const double iw = s_iw[0], ihw = s_iw[1];
   const int64_t plane = (int64_t)ld * ld;
   __nv_bfloat16* X = In.arena + (int64_t)tc::xslot(In.lowmem, In.hist0, 0) * In.slot_elems;
   __nv_bfloat16* Fp = In.arena + (int64_t)In.f_slot * In.slot_elems;
@@ -154,10 +158,10 @@ __global__ void batch_scale_split_kernel(const Instance* inst, int count, int sb
   for (int64_t e = b * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)sb * blockDim.x) {
     const int r = (int)(e / N), c = (int)(e % N);
     const double f = F[e];
-    const float x = (float)(((r == c ? lmax : 0.0) - f) / w);
+    const float x = (float)divide_shared((r == c ? lmax : 0.0) - f, w, iw);
     const int64_t off = (int64_t)r * ld + c;
     piece_store(fmt, X, plane, off, x);
-    const float fv = fmt == tc::FMT_FP16X2 ? (float)((f - (r == c ? cmid : 0.0)) / hw) : (float)f;
+    const float fv = fmt == tc::FMT_FP16X2 ? (float)divide_shared(f - (r == c ? cmid : 0.0), hw, ihw) : (float)f;
     piece_store(fmt, Fp, plane, off, fv);
   }
 }
@@ -186,8 +190,8 @@ __global__ void __launch_bounds__(kFT) batch_finalize_kernel(const Instance* ins
     c += In.part[4 * (int64_t)t + 2];
   }
   block_sum3<kFT>(a, b, c, nparts, sm);
-  double vk = sqrt(a);
-  if (st->norm == 2) vk = st->spec_e;   // e_{k-1}, the Lanczos estimate of the 2-norm (one problem)
+  double vk = 0.0;   // v_{k-1}, or e_{k-1}, the Lanczos estimate of the 2-norm (one problem)
+  if (threadIdx.x == 0) vk = st->norm == 2 ? st->spec_e : sqrt(a);
   if (st->norm == 1 && In.mscr) {
     // mixed norm over 128 x 128 blocks: single-CTA tiles give rec_block records per block (one per
     // epilogue warp); a 256 x 256 pair tile holds 16, record 8 rank + 4 hc + q covering
