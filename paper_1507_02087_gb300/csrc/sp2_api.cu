@@ -614,6 +614,13 @@ struct sp2_ctx {
   MixedEngine* mixed = nullptr;
 };
 
+static void free_digits(sp2::f64tc::Digits& d) {
+  cudaFree(d.dig);
+  cudaFree(d.exp);
+  d.dig = nullptr;
+  d.exp = nullptr;
+}
+
 static void free_ctx(sp2_ctx* h) {
   if (!h) return;
   int cur = 0;
@@ -629,10 +636,8 @@ static void free_ctx(sp2_ctx* h) {
   cudaFree(h->mscr);
   cudaFree(h->lz);
   cudaFree(h->sbuf);
-  for (sp2::f64tc::Digits* d : {&h->tc.X, &h->tc.S}) {
-    cudaFree(d->dig);
-    cudaFree(d->exp);
-  }
+  free_digits(h->tc.X);
+  free_digits(h->tc.S);
   cudaFree(h->part_lo);
   cudaFree(h->part_hi);
   cudaFree(h->part_bad);
@@ -647,6 +652,15 @@ static void free_ctx(sp2_ctx* h) {
   delete h;
 }
 
+// Zeroed device memory, or false (and a null pointer).
+static bool alloc_zero(double** p, size_t bytes) {
+  if (cudaMalloc(p, bytes) == cudaSuccess && cudaMemset(*p, 0, bytes) == cudaSuccess) return true;
+  (void)cudaGetLastError();
+  cudaFree(*p);
+  *p = nullptr;
+  return false;
+}
+
 // Digit buffers of one ld x ld matrix, zeroed (the rows past N stay zero).
 // False (and nothing held) when the memory is not there: the CUDA-core products need none.
 static bool alloc_digits(sp2::f64tc::Digits& d, int ld) {
@@ -655,15 +669,12 @@ static bool alloc_digits(sp2::f64tc::Digits& d, int ld) {
       cudaMemset(d.dig, 0, digit_bytes(ld)) == cudaSuccess && cudaMemset(d.exp, 0, exp_bytes(ld)) == cudaSuccess)
     return true;
   (void)cudaGetLastError();
-  cudaFree(d.dig);
-  cudaFree(d.exp);
-  d.dig = nullptr;
-  d.exp = nullptr;
+  free_digits(d);
   return false;
 }
 
-// The plan of the McWeeny step: it needs the digits of the shifted square too.
-static const sp2::f64tc::Plan* mcw_plan(const sp2_ctx* h) { return h->tc.on && h->tc.S.dig ? &h->tc : nullptr; }
+// The products' plan, or null: the CUDA-core kernels.  (With McWeeny it has the shifted square's digits too.)
+static const sp2::f64tc::Plan* plan_of(const sp2_ctx* h) { return h->tc.on ? &h->tc : nullptr; }
 
 // The FP64 path's loop graph: a WHILE node around {square, stop test} (SP2) or {shifted
 // square, stop test, product} (McWeeny).
@@ -676,11 +687,11 @@ static sp2_status build_f64_graph(sp2_ctx* h) {
   sp2_status s = add_while(h->graph, nullptr, 0, &h->cond, &node, &body);
   if (s != SP2_OK) return s;
   if (h->mcw)
-    SP2_TRY(sp2::add_mcw_loop_body(body, h->st_dev, h->buf[0], h->buf[1], h->sbuf, h->part, h->T, h->cond, mcw_plan(h),
+    SP2_TRY(sp2::add_mcw_loop_body(body, h->st_dev, h->buf[0], h->buf[1], h->sbuf, h->part, h->T, h->cond, plan_of(h),
                                    h->mscr, h->lz, (int)h->N));
   else
     SP2_TRY(sp2::add_f64_loop_body(body, h->st_dev, h->buf[0], h->buf[1], h->part, h->T, h->cond,
-                                   h->tc.on ? &h->tc : nullptr, h->mscr, h->lz, (int)h->N, h->pert, h->pert_count));
+                                   plan_of(h), h->mscr, h->lz, (int)h->N, h->pert, h->pert_count));
   SP2_TRY(cudaGraphInstantiate(&h->exec, h->graph, 0));
   return SP2_OK;
 }
@@ -752,7 +763,7 @@ static sp2_status enqueue_f64(sp2_ctx* h, const double* F, double* D, cudaStream
   SP2_TRY(sp2::launch_bounds_and_init(h->st_dev, F, N, N, h->part_lo, h->part_hi, h->part_bad, h->nparts, s));
   SP2_TRY(sp2::launch_scale_f64(h->st_dev, F, N, N, h->buf[0], h->ld, s));
   if (h->pert) SP2_TRY(sp2::launch_perturb(h->st_dev, h->buf[0], h->buf[1], h->pert, h->pert_count, N, 1, s));
-  if (h->mcw ? mcw_plan(h) != nullptr : h->tc.on)
+  if (h->tc.on)
     SP2_TRY(sp2::launch_f64_digits(h->st_dev, h->buf[0], h->buf[1], h->tc, N, s));
   SP2_TRY(cudaEventRecord(h->ev_loop[0], s));
   if (h->opts.launch_mode == 0) {
@@ -760,11 +771,11 @@ static sp2_status enqueue_f64(sp2_ctx* h, const double* F, double* D, cudaStream
   } else {
     for (int it = 0; it <= h->opts.max_iter; ++it)
       if (h->mcw)
-        SP2_TRY(sp2::launch_mcw_step_plain(h->st_dev, h->buf[0], h->buf[1], h->sbuf, h->part, h->T, s, mcw_plan(h),
+        SP2_TRY(sp2::launch_mcw_step_plain(h->st_dev, h->buf[0], h->buf[1], h->sbuf, h->part, h->T, s, plan_of(h),
                                            h->mscr, h->lz, N));
       else
         SP2_TRY(sp2::launch_f64_step_plain(h->st_dev, h->buf[0], h->buf[1], h->part, h->T, s,
-                                           h->tc.on ? &h->tc : nullptr, h->mscr, h->lz, N, h->pert, h->pert_count));
+                                           plan_of(h), h->mscr, h->lz, N, h->pert, h->pert_count));
   }
   SP2_TRY(cudaEventRecord(h->ev_loop[1], s));
   SP2_TRY(sp2::launch_copy_out(h->st_dev, h->buf[0], h->buf[1], h->ld, N, D, N, s));
@@ -923,10 +934,17 @@ extern "C" int32_t sp2_set_mcweeny(sp2_handle h, int32_t mode, double mu, double
   cudaSetDevice(h->device);
   sp2_status r = SP2_OK;
   if (cudaDeviceSynchronize() != cudaSuccess) r = SP2_ERR_CUDA;
+  bool dropped = false;
   if (r == SP2_OK && mode > 0 && !h->sbuf) {
     const size_t bytes = (size_t)h->ld * h->ld * sizeof(double);
-    if (cudaMalloc(&h->sbuf, bytes) != cudaSuccess || cudaMemset(h->sbuf, 0, bytes) != cudaSuccess) r = SP2_ERR_NOMEM;
-    else if (h->tc.on && !h->tc.S.dig) (void)alloc_digits(h->tc.S, h->ld);
+    bool ok = alloc_zero(&h->sbuf, bytes);
+    if (h->tc.on && !(ok && alloc_digits(h->tc.S, h->ld))) {   // the square comes before the digits
+      free_digits(h->tc.X);
+      h->tc.on = false;
+      dropped = true;
+      if (!ok) ok = alloc_zero(&h->sbuf, bytes);
+    }
+    if (!ok) r = SP2_ERR_NOMEM;
   }
   if (r == SP2_OK) {
     const int32_t m = mode;
@@ -940,7 +958,10 @@ extern "C" int32_t sp2_set_mcweeny(sp2_handle h, int32_t mode, double mu, double
   if (r == SP2_OK) {
     h->st_host->mcw = mode;
     h->mcw = mode;
-    if (h->opts.launch_mode == 0) r = build_f64_graph(h);
+  }
+  if ((r == SP2_OK || dropped) && h->opts.launch_mode == 0) {   // no graph may hold buffers that are gone
+    const sp2_status g = build_f64_graph(h);
+    if (r == SP2_OK) r = g;
   }
   (void)cudaGetLastError();
   cudaSetDevice(cur);

@@ -5,7 +5,23 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace sp2 {
+
+// A positive number of the current device, found by `find` (0: not found) and kept for the next call.  Kernel
+// attributes hold for one device, and several threads may come here at once: both then find the same.
+struct PerDevice {
+  std::atomic<int> v[64];
+  template <class Find>
+  int get(Find find) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return find(dev);
+    int n = v[dev].load(std::memory_order_acquire);
+    if (n <= 0) v[dev].store(n = find(dev), std::memory_order_release);
+    return n;
+  }
+};
 
 struct DevState;
 namespace f64tc {

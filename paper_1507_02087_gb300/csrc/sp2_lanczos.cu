@@ -442,11 +442,12 @@ int form_blocks(int ld) {
 }  // namespace
 
 cudaError_t lanczos_prepare() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  const cudaError_t e =
-      cudaFuncSetAttribute(lz_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kLzSmemN + 4096);
-  done = e == cudaSuccess;
+  static PerDevice done;
+  cudaError_t e = cudaSuccess;
+  done.get([&](int) {
+    e = cudaFuncSetAttribute(lz_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kLzSmemN + 4096);
+    return e == cudaSuccess ? 1 : 0;
+  });
   return e;
 }
 

@@ -69,16 +69,6 @@ __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* m
       : "memory");
 }
 
-// 3-D tiled TMA load (coordinates innermost first) completing on `bar`.
-__device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* map, int c0, int c1, int c2,
-                                            uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(smem_dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
-      : "memory");
-}
-
 // Contiguous copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) completing on `bar`.
 __device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile(
@@ -86,10 +76,6 @@ __device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint3
           smem_u32(smem_dst)),
       "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
-}
-
-__device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
 // True for one lane of a converged warp, the same one each time.  Written this way (and not as lane == 0)
@@ -200,19 +186,8 @@ __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Shared-memory matrix descriptor for a K-major bf16 tile stored with 64-byte swizzle:
-// rows of 64 B (32 bf16), 8-row core groups 512 B apart.
-__device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);      // start address, bits 0-13
-  d |= (uint64_t)1 << 16;                       // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(512 >> 4) << 32;              // stride byte offset: 8 rows x 64 B
-  d |= (uint64_t)1 << 46;                       // descriptor version for sm_100
-  d |= (uint64_t)4 << 61;                       // swizzle mode: 64-byte
-  return d;
-}
-
-// The same with the 8-row core groups `stride` bytes apart (a multiple of 512).
+// Shared-memory matrix descriptor for a K-major 16-bit tile stored with 64-byte swizzle: rows of 64 B, 8-row core
+// groups `stride` bytes apart (a multiple of 512).
 __device__ __forceinline__ uint64_t smem_desc_sw64_stride(uint32_t saddr, uint32_t stride) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
@@ -302,10 +277,6 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t saddr, uint32_t rank) {
   uint32_t d;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(saddr), "r"(rank));
   return d;
-}
-
-__device__ __forceinline__ void mbar_arrive_expect_tx_u32(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
 // Arrive on a barrier of either CTA of the pair (`cluster_addr` from mapa_shared), with relaxed
@@ -403,11 +374,6 @@ __device__ __forceinline__ void setmaxnreg_dec() {
 template <int N>
 __device__ __forceinline__ void setmaxnreg_inc() {
   asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
-}
-
-// Named barrier among `count` threads (id 1..15; id 0 is __syncthreads).
-__device__ __forceinline__ void named_bar(int id, int count) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
 }  // namespace ptx

@@ -109,3 +109,41 @@ def test_mcweeny_products_at_tile_edges(N, mode, xi):
                      bounds=(info["lambda_min"], info["lambda_max"]))
     assert info["status"] == 0 and abs(info["n_iter"] - ref.n) <= 1
     assert o.rel_error(D, ref.D, N // 2) <= 1e-12
+
+
+@pytest.mark.parametrize("left,mcw,used", [(90, False, 67), (150, False, 126), (150, True, 101), (250, True, 218)])
+def test_a_handle_without_room_for_the_digits_uses_the_fp64_units(left, mcw, used):
+    # MB left on the device at create: two iterates take 67, the digits 59 each, the McWeeny square 34.
+    # At 90 the digits fail; at 150 the square takes their place.
+    from paper_1507_02087_gb300 import sp2
+    N, MB = 2048, 1 << 20
+    case = inputs.dense_gapped(N, N // 2, gap=0.05, seed=1)
+    F, D = case.F.cuda(), torch.empty(N, N, dtype=torch.float64, device="cuda")
+    free = lambda: torch.cuda.mem_get_info()[0]
+
+    def solve():
+        before = free()
+        with sp2.Purifier(N, N // 2, "fp64") as P:
+            if mcw:
+                P.set_mcweeny("mcw-acc", 0.0, 0.05)
+            took = (before - free()) / 1e6
+            P.run(F, D)
+            return D.cpu(), P.info(), took
+
+    want, winfo, _ = solve()                                 # with room; loads the kernels too
+    torch.cuda.empty_cache()
+    hog = []
+    try:
+        for size in (1 << 30, 64 * MB, 16 * MB, 2 * MB):
+            while free() > left * 10**6 + size:
+                hog.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+        got, info, took = solve()
+    except torch.cuda.OutOfMemoryError:
+        pytest.skip("the device's free memory moved")
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    assert used - 5 <= took <= used + 8, took
+    # (where the runs stop may differ: the units' rounding floor is higher)
+    assert info["status"] == winfo["status"] == 0
+    assert float(torch.linalg.norm(got - want)) <= 1e-11 * (N / 2) ** 0.5
