@@ -20,15 +20,17 @@
 // alpha_{j-1}, forms r = w - alpha q_{j-1} - beta q_{j-2}, ||r|| and q_j = r / ||r|| for all N entries by itself
 // (FP64; 2 N clocks of the SM's FP64 units), then multiplies its rows: w = A q_j, one warp per row, FP32 products
 // summed in FP32 per lane and FP64 across lanes.  The steps thus have one launch between them and no CTA that
-// the others wait for: with the last CTA to finish doing the update alone, a step took 15 us at N = 1001, most of
-// it in that CTA's serial FP64 sums.  The FP32 rounding of A and
-// of the products perturbs A by about 1e-7 of its norm, far below the Lanczos truncation error.
+// the others wait for; up to N = kLzClusterN one cluster does them all in one launch (lz_cluster_kernel).  With the
+// last CTA to finish doing the update alone, a step took 15 us at N = 1001, most of it in that CTA's serial FP64
+// sums.  The FP32 rounding of A and of the products perturbs A by about 1e-7 of its norm, far below the Lanczos
+// truncation error.
 #include <math.h>
 
 #include "sp2_common.cuh"
 #include "sp2_f64_tc.cuh"
 #include "sp2_kernels.h"
 #include "sp2_tc.cuh"
+#include "tc_ptx.cuh"
 
 namespace sp2 {
 namespace {
@@ -38,6 +40,13 @@ constexpr int kLzThreads = 1024;      // start: one CTA
 constexpr int kLzMvBlocks = 152;      // step grid cap (one CTA per SM) = number of partial sums
 constexpr int kLzMvThreads = 1024;    // threads of a step: 512 while the grid cap is not reached, else 1024
 constexpr int kLzSmemN = 16384;       // q_j in shared memory up to this size
+constexpr int kLzCtas = 16;           // CTAs of the cluster that does all steps
+constexpr int kLzClThreads = 512;
+// Largest N it takes.  Time of one FP64 purification with 32 step launches and with the cluster (both with the
+// spectral stop): N = 130 13.5 -> 7.7 ms, 400 16.3 -> 10.0, 700 18.8 -> 13.0, 1001 21.7 -> 17.9, 1300 26.0 -> 25.5,
+// 1600 33.1 -> 33.4, 2000 39.1 -> 44.0: past the line 16 SMs read the matrix more slowly than 152.
+constexpr int kLzClusterN = 1280;
+constexpr int kLzClSmem = 222 * 1024; // dynamic shared memory it may have
 constexpr int kSturmThreads = 1024;   // 512 points per side
 constexpr int kSturmRounds = 3;       // 513^3 > 2^27: below FP32 resolution of the interval
 
@@ -312,6 +321,143 @@ lz_step_kernel(const DevState* st, LzScratch* lz, int j, int N, int ld) {
   if (threadIdx.x == 0) lz->part[j & 1][blockIdx.x] = pa;
 }
 
+// All steps in one launch, for N <= kLzClusterN: one cluster of kLzCtas CTAs, each with the entries and rows
+// c S .. c S + S - 1 (S = ceil(N / kLzCtas)), one entry of q_j and q_{j-1} in a register of its first S threads.
+// A step has two exchanges through distributed shared memory, each closed by a cluster barrier: the warps'
+// partials of alpha_j go to every CTA; then those of ||r||^2 and the entries of r, from which every CTA rounds
+// its own FP32 copy of q_{j+1}.  Every CTA adds the same partials in the same order, so all take the same
+// decisions.  A CTA keeps the first R of its rows of A in shared memory and reads the others from L2 in each step;
+// a warp multiplies four rows at a time, so that the loads of q and the FP64 sums across the lanes (16 clocks an
+// instruction and SM) are shared.  A step takes 5.5 us at N = 130, the chain of FP64 sums, root and barriers, and
+// 10.6 at N = 1001, where the rows from shared memory and L2 add to it; a step launch took 10 and 13.1.
+__device__ __forceinline__ double warp_sum(double x) {
+  #pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+__global__ void __cluster_dims__(kLzCtas, 1, 1) __launch_bounds__(kLzClThreads, 1)
+lz_cluster_kernel(const DevState* st, LzScratch* lz, int N, int ld, int R) {
+  extern __shared__ __align__(16) float lz_smem[];
+  constexpr int kParts = kLzCtas * ((kLzClusterN / kLzCtas + 31) / 32);
+  __shared__ double p_alpha[kParts], p_ss[kParts], s_w[kLzClusterN / kLzCtas];
+  __shared__ double s_b, s_ib;
+  if (st->done || !lz->live) return;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = kLzClThreads / 32;
+  const int c = blockIdx.x, S = (N + kLzCtas - 1) / kLzCtas, ew = (S + 31) / 32;   // ew: warps with entries
+  const int i0 = c * S, rows = N - i0 < S ? (N - i0 > 0 ? N - i0 : 0) : S;
+  double* r64 = reinterpret_cast<double*>(lz_smem);                                 // r of all entries
+  float* q32 = reinterpret_cast<float*>(r64 + kLzCtas * S);
+  float4* own = reinterpret_cast<float4*>(q32 + ld);                                // rows 0 .. R - 1
+  const double* q0 = lz_vec(lz, ld, 0);
+  const int h = ld / 4, G = (rows + 3) / 4;
+  const float4* A = reinterpret_cast<const float4*>(lz_a32(lz, ld)) + (int64_t)i0 * h;
+  for (int i = tid; i < (rows < R ? rows : R) * h; i += kLzClThreads) own[i] = A[i];
+  double q = tid < rows ? q0[i0 + tid] : 0.0, qp = 0.0, bj = 0.0;
+  for (int i = tid; i < ld; i += kLzClThreads) q32[i] = i < N ? (float)q0[i] : 0.f;
+  const uint32_t a_pa = ptx::smem_u32(p_alpha), a_ps = ptx::smem_u32(p_ss), a_r = ptx::smem_u32(r64);
+  // lane l < kLzCtas of a warp stores the warp's sum into the array of CTA l
+  auto share = [&](uint32_t arr, double x) {
+    if (lane < kLzCtas) ptx::st_cluster_f64(ptx::mapa_shared(arr + 8 * (c * ew + warp), lane), x);
+  };
+  auto total = [&](const double* p) {
+    double t = 0.0;
+    for (int n = lane; n < kLzCtas * ew; n += 32) t += p[n];
+    return warp_sum(t);
+  };
+  ptx::cluster_sync();                                     // every CTA runs before the first remote store
+  for (int j = 0; j < kLzSteps; ++j) {
+    const float4* q4 = reinterpret_cast<const float4*>(q32);
+    auto dot4 = [](const float4& x, const float4& v, float s) {
+      s = fmaf(x.x, v.x, s); s = fmaf(x.y, v.y, s); s = fmaf(x.z, v.z, s);
+      return fmaf(x.w, v.w, s);
+    };
+    for (int g = warp; g < G; g += nw) {                   // rows g, g + G, g + 2 G, g + 3 G
+      const float4* x[4];
+      #pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int r = g + k * G < rows ? g + k * G : g;
+        x[k] = r < R ? own + r * h : A + (int64_t)r * h;
+      }
+      float s0[4] = {}, s1[4] = {};
+      for (int i = lane; i < h; i += 64) {
+        const bool more = i + 32 < h;
+        const int i1 = more ? i + 32 : i;
+        float4 a0[4], a1[4];
+        #pragma unroll
+        for (int k = 3; k >= 0; --k) { a0[k] = x[k][i]; a1[k] = x[k][i1]; }
+        const float4 v0 = q4[i], v1 = q4[i1];
+        #pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          s0[k] = dot4(a0[k], v0, s0[k]);
+          if (more) s1[k] = dot4(a1[k], v1, s1[k]);
+        }
+      }
+      // the sums of four rows across the lanes: halves, then quarters, of the warp take a row each
+      double t[4];
+      #pragma unroll
+      for (int k = 0; k < 4; ++k) t[k] = (double)s0[k] + (double)s1[k];
+      const bool up = lane & 16, odd = lane & 8;
+      double u0 = up ? t[2] : t[0], u1 = up ? t[3] : t[1];
+      u0 += __shfl_xor_sync(0xffffffffu, up ? t[0] : t[2], 16);
+      u1 += __shfl_xor_sync(0xffffffffu, up ? t[1] : t[3], 16);
+      double v = odd ? u1 : u0;
+      v += __shfl_xor_sync(0xffffffffu, odd ? u0 : u1, 8);
+      #pragma unroll
+      for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      const int r = g + (lane >> 3) * G;
+      if ((lane & 7) == 0 && r < rows) s_w[r] = v;
+    }
+    __syncthreads();
+    const double w = tid < rows ? s_w[tid] : 0.0;
+    if (warp < ew) share(a_pa, warp_sum(q * w));
+    ptx::cluster_sync();
+    double a = 0.0, r = 0.0;
+    if (warp < ew) {
+      a = total(p_alpha);
+      if (j + 1 < kLzSteps) {
+        r = w - a * q - (j > 0 ? bj * qp : 0.0);
+        if (tid < S)
+          for (int o = 0; o < kLzCtas; ++o) ptx::st_cluster_f64(ptx::mapa_shared(a_r + 8 * (c * S + tid), o), r);
+        share(a_ps, warp_sum(r * r));
+      }
+    }
+    if (j + 1 == kLzSteps) {                               // the last alpha closes the tridiagonal matrix
+      if (c == 0 && tid == 0) {
+        lz->alpha[j] = a;
+        lz->m = kLzSteps;
+        lz->live = 0;
+      }
+      break;
+    }
+    ptx::cluster_sync();
+    if (warp == 0) {
+      const double ss = total(p_ss);
+      if (lane == 0) {                                     // one thread: FP64 operations run at 2 a clock and SM
+        const double b = sqrt(ss);
+        const bool finite = isfinite(a) && isfinite(b), more = finite && b > 1e-300;
+        s_b = more ? b : -1.0;
+        s_ib = 1.0 / b;
+        if (c == 0) {
+          lz->alpha[j] = finite ? a : __longlong_as_double(0x7ff8000000000000ll);
+          lz->m = j + 1;
+          lz->beta[j + 1] = b;
+          if (!more) lz->live = 0;
+        }
+      }
+    }
+    __syncthreads();
+    if (s_b < 0.0) break;                                  // the same in every CTA
+    bj = s_b;
+    const double ib = s_ib;
+    qp = q;
+    q = r * ib;
+    for (int i = tid; i < N; i += kLzClThreads) q32[i] = (float)(r64[i] * ib);
+    __syncthreads();
+  }
+  ptx::cluster_sync();                                     // no CTA leaves while another still writes to it
+}
+
 // Number of eigenvalues of the m x m tridiagonal (alpha, beta) below x: the count of negative
 // pivots of the LDL^T factorisation of T - x I (Sturm sequence), tiny pivots pushed to -pivmin.
 __device__ __forceinline__ int sturm_count(const float* al, const float* be2, int m, float x) {
@@ -434,6 +580,39 @@ int step_blocks(int N) {
 }
 int step_smem(int N, int ld) { return N <= kLzSmemN ? 4 * ld : 0; }
 
+// Shared memory of the cluster's CTAs without rows of A, and how many rows fit beside it.
+int cluster_base(int N, int ld) { return 8 * kLzCtas * ((N + kLzCtas - 1) / kLzCtas) + 4 * ld; }
+int cluster_rows(int N, int ld) {
+  const int S = (N + kLzCtas - 1) / kLzCtas, fit = (kLzClSmem - cluster_base(N, ld)) / (4 * ld);
+  return fit < S ? fit : S;
+}
+
+// Whether the device can hold the cluster (its size is above the portable eight).
+bool cluster_fits() {
+  static PerDevice fits;
+  return fits.get([](int) {
+    const void* k = (const void*)lz_cluster_kernel;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kLzCtas);
+    cfg.blockDim = dim3(kLzClThreads);
+    cfg.dynamicSmemBytes = kLzClSmem;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kLzCtas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kLzClSmem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess || n < 1) {
+      (void)cudaGetLastError();
+      return 1;
+    }
+    return 2;
+  }) == 2;
+}
+
 int form_blocks(int ld) {
   const int64_t b = ((int64_t)ld * (ld / 2) + 255) / 256;
   return (int)(b < 152 * 16 ? b : 152 * 16);
@@ -442,6 +621,7 @@ int form_blocks(int ld) {
 }  // namespace
 
 cudaError_t lanczos_prepare() {
+  (void)cluster_fits();                          // asks the device once, before any capture
   static PerDevice done;
   cudaError_t e = cudaSuccess;
   done.get([&](int) {
@@ -467,10 +647,17 @@ static cudaError_t emit(f64tc::Sink& sink, DevState* st, const double* part, int
   if ((e = sink.put((const void*)lz_start_kernel, dim3(1), dim3(kLzThreads), 0, a0)) != cudaSuccess) return e;
   if (fill && (e = sink.put(fill, dim3(form_blocks(ld)), dim3(256), 0, fill_args)) != cudaSuccess) return e;
   if ((e = sink.put(form, dim3(form_blocks(ld)), dim3(256), 0, form_args)) != cudaSuccess) return e;
-  for (int j = 0; j < kLzSteps; ++j) {
-    void* a[] = {&cst, &lz, &j, &N, &ld};
-    e = sink.put((const void*)lz_step_kernel, dim3(step_blocks(N)), dim3(step_threads(N)), step_smem(N, ld), a);
+  if (N <= kLzClusterN && cluster_fits()) {
+    int R = cluster_rows(N, ld);
+    void* a[] = {&cst, &lz, &N, &ld, &R};
+    e = sink.put((const void*)lz_cluster_kernel, dim3(kLzCtas), dim3(kLzClThreads), cluster_base(N, ld) + 4 * ld * R, a);
     if (e != cudaSuccess) return e;
+  } else {
+    for (int j = 0; j < kLzSteps; ++j) {
+      void* a[] = {&cst, &lz, &j, &N, &ld};
+      e = sink.put((const void*)lz_step_kernel, dim3(step_blocks(N)), dim3(step_threads(N)), step_smem(N, ld), a);
+      if (e != cudaSuccess) return e;
+    }
   }
   int blocks = step_blocks(N);
   void* a1[] = {&st, &clz, &blocks};

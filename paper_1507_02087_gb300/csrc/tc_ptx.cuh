@@ -279,6 +279,11 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t saddr, uint32_t rank) {
   return d;
 }
 
+// A double into the shared memory of a CTA of the cluster (`cluster_addr` from mapa_shared).
+__device__ __forceinline__ void st_cluster_f64(uint32_t cluster_addr, double x) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr), "d"(x) : "memory");
+}
+
 // Arrive on a barrier of either CTA of the pair (`cluster_addr` from mapa_shared), with relaxed
 // semantics: for an arrive that only hands back tensor memory whose tcgen05.ld reads have
 // already completed (tcgen05.wait::ld), so nothing in memory needs a release fence.
