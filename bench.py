@@ -35,8 +35,11 @@ sys.path.insert(0, ROOT)
 METRIC = "time-to-D & TFLOP/s, mixed vs FP64 SP2 on 1 GB300 at ||D-D_ref||_F/sqrt(nocc)<=1e-6"
 N_DEFAULT, GAP_DEFAULT = 8192, 0.01
 TOL = 1e-6
-# FP64 runs on the SMs' FP64 pipes: the nominal 1.25 TFLOP/s over 152 SMs at the
-# 2070 MHz maximum clock is 4 flop per clock per SM; taken at the measured clock.
+# FP64 products: from F64_TC_MIN_N on, exact sums of digit products on the tensor cores; below, the SMs' FP64
+# pipes (the nominal 1.25 TFLOP/s over 152 SMs at the 2070 MHz maximum clock is 4 flop per clock per SM; taken
+# at the measured clock).
+F64_TC_MIN_N, F64_DIGIT_PRODUCTS = 129, 34
+LZ_CLUSTER_N = 1280   # all Lanczos steps in one launch up to this size
 SMS, FP64_FLOP_PER_CLK_SM, SM_MAX_MHZ = 152, 4.0, 2070.0
 # 16-bit piece products per square on the tensor cores, per precision mode
 PRODUCTS = {"mixed": 6, "bf16x6": 6, "bf16x3": 3, "fp16x3": 3, "tf32x3": 3}
@@ -365,13 +368,13 @@ def run_batch(a, ws, rank, local):
 
 
 def bsr_launches(squares, rule):
-    """Kernels of one block-sparse run (dense output off): 14 set-up kernels, 12 per loop
-    round (+1 each with the error-controlled rule, +3 with the mixed-norm rule, +35 Lanczos
-    launches per round for the mixed-norm stop that goes with it), rounds launched in pairs."""
-    extra = {"error": 1, "mixed": 3}.get(rule, 0)
-    lz = 35 if rule == "mixed" else 0
+    """Kernels of one block-sparse run (dense output off): 13 set-up kernels, 17 per loop
+    round (+9 each with the error-controlled rule, +3 with the mixed-norm rule, +5 Lanczos launches
+    (up to LZ_CLUSTER_N block rows) per round for the mixed-norm stop that goes with it), rounds launched in pairs."""
+    extra = {"error": 9, "mixed": 3}.get(rule, 0)
+    lz = 5 if rule == "mixed" else 0
     rounds = squares + (squares & 1)
-    return 14 + extra + (12 + extra + lz) * rounds
+    return 13 + extra + (17 + extra + lz) * rounds
 
 
 def bsr_error_bound(tb, D):
@@ -646,13 +649,15 @@ def main():
     n_iter = info["n_iter"]
     flops = useful_flops(N, squares, n_iter, mixed, 2 if mixed else 0) if mixed else N * N * (N + 1) * squares
     tflops = flops / (ms * 1e-3) / 1e12
-    # FP64 path per square: square (+ McWeeny product) + finalize (+ 35 Lanczos launches for the
-    # spectral stop); bounds, init, scaling and the output copy once
-    per_square = 2 + (1 if a.mcweeny else 0) + (35 if a.norm == "spectral" else 0)
+    # FP64 path per square: square (+ McWeeny product), each with the digits of what it wrote on the
+    # tensor cores, + finalize (+ the Lanczos launches for the spectral stop); bounds, init, scaling (and
+    # its digits) and the output copy once
+    digits = 1 if N >= F64_TC_MIN_N else 0
+    per_square = (1 + digits) * (2 if a.mcweeny else 1) + 1 + ((4 if N <= LZ_CLUSTER_N else 35) if a.norm == "spectral" else 0)
     # tensor-core path: bounds, init, scaling; {square, finalize, loop check} per forward round; two
     # correction products; {derivative step, advance} per derivative round; refinement input and pair;
     # the output assembly
-    launches_per_step = (3 + per_square * squares + 1) if not mixed else (3 + 3 * squares + 2 + 2 * n_iter + 3 + 1)
+    launches_per_step = (3 + digits + per_square * squares + 1) if not mixed else (3 + 3 * squares + 2 + 2 * n_iter + 3 + 1)
 
     # roofline of the dominant kernel, timed on its own inside the same device loop:
     # a forward-only handle runs the square + stop-test loop; loop time / squares is
@@ -689,16 +694,23 @@ def main():
                     "traffic": FWD_TRAFFIC_BYTES.get((N, tile_used, a.precision))}
     else:
         kern_ms = statistics.mean(l / s for l, s in zip(loop_ms, [i["hist_len"] for i in infos]))
-        mhz = clk.get("sm_mhz") or SM_MAX_MHZ
-        peak = SMS * FP64_FLOP_PER_CLK_SM * mhz * 1e6 / 1e12
-        alg = N * N * (N + 1) * (2 if a.mcweeny else 1)     # McWeeny: two products per step
+        useful = N * N * (N + 1) * (2 if a.mcweeny else 1)     # McWeeny: two products per step
+        step = ", one McWeeny step of two products" if a.mcweeny else ""
+        if digits:
+            peak, peak_src = tensor_peak("fp16x3")
+            alg, bound, kname = F64_DIGIT_PRODUCTS * useful, "tensor", "f64_product_kernel (+digits, finalize)" + step
+            basis = "N^2 (N+1) useful flops per product x %d exact digit products" % F64_DIGIT_PRODUCTS
+        else:
+            mhz = clk.get("sm_mhz") or SM_MAX_MHZ
+            peak = SMS * FP64_FLOP_PER_CLK_SM * mhz * 1e6 / 1e12
+            peak_src = f"152 SMs x 4 FP64 flop/clk x {mhz:.0f} MHz (median SM clock under load)"
+            alg, bound, kname = useful, "alu", "small_product_kernel (+finalize)" + step
+            basis = "N^2 (N+1) useful flops per product"
         achieved = alg / (kern_ms * 1e-3) / 1e12
-        kname = ("mcw_square_kernel + mcw_prod_kernel (+finalize), one McWeeny step" if a.mcweeny
-                 else "syrk_f64_kernel (+finalize)")
-        roofline = {"bound": "alu", "kernel": kname, "achieved": achieved, "peak": peak,
+        roofline = {"bound": bound, "kernel": kname, "achieved": achieved, "peak": peak,
                     "unit": "TFLOP/s", "frac": achieved / peak, "ms_per_launch": kern_ms,
-                    "peak_source": f"152 SMs x 4 FP64 flop/clk x {mhz:.0f} MHz (median SM clock under load)",
-                    "algorithmic_flops_per_launch": alg, "traffic": None}
+                    "basis": basis, "useful_tflops": useful / (kern_ms * 1e-3) / 1e12,
+                    "peak_source": peak_src, "algorithmic_flops_per_launch": alg, "traffic": None}
 
     # end to end through the public API with host buffers (copies inside the timed region), right
     # after the device-timed steps and before the long FP64 comparison run
