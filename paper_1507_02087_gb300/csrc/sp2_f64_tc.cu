@@ -506,6 +506,7 @@ f64_product_kernel(const Args a) {
         int go = ok;
         if (lane == 0) go = ok && !abort_s && mbar_wait_cluster(&xempty_bar[ew], xphase ^ 1, until);
         go = __shfl_sync(0xffffffffu, go, 0);
+        __syncwarp();                    // orders the lanes' stores after lane 0's wait (a shuffle orders no memory)
         if (go) {
           #pragma unroll 1
           for (int j = 0; j < G; j += 4) {
@@ -526,6 +527,7 @@ f64_product_kernel(const Args a) {
             go = mbar_wait_cluster(&xfull_bar[ew], xphase, until);
           }
           go = __shfl_sync(0xffffffffu, go, 0);
+          __syncwarp();                  // and their loads of the others' sums
         }
         if (!go) ok = false;
       }
