@@ -52,6 +52,18 @@ int32_t sp2_test_tc_gemm_ex(const void* arena_dev, int32_t ld, int32_t nslots, i
  * involved: the kernel returns normally and the context stays usable. */
 int32_t sp2_test_tc_timeout(const void* arena_dev, int32_t ld, int32_t wait_ms, float* out_dev, void* stream);
 
+/* The FP64 product S = X X^T on the tensor cores (the digit sums of SP2_PREC_FP64) on its own: X_dev, out_dev N x N
+ * FP64 row-major device matrices, 1 <= N <= 8192; only j >= i is computed, and mirrored.  Tiles of 128 x bn whose k
+ * range ks CTAs of a cluster share: (bn, ks) = (32, 1), (64, 1), (64, 2), (64, 4) or (64, 8).  exp_dev: NULL, or N
+ * int32 that receive the rows' exponents e_i (||x_i|| < 2^e_i, |x_ik| <= 2^(e_i - 1)).
+ * hook 0: none.  1: CTA 0 leaves its first stage uncopied, so that waits, limited to wait_ms (0: 2000), run out and
+ * the call returns SP2_ERR_TIMEOUT.  2 (3): in each cluster of ks > 1 CTAs, all but the first (only the first) find
+ * the run over when they start, as after a wait that ran out elsewhere; the first decides for its cluster: with 2 the
+ * product is complete, with 3 out_dev receives zeros.  Every CTA stays until its cluster is done, so neither
+ * touches memory of a CTA that has left.  Synchronises `stream`; returns an sp2_status. */
+int32_t sp2_test_f64_product(const double* X_dev, int64_t N, int32_t bn, int32_t ks, int32_t hook, int32_t wait_ms,
+                             double* out_dev, int32_t* exp_dev, void* stream);
+
 /* 1 if this library was built with device-side bounds checks (libsp2_debug.so, built with
  * SP2_DEVICE_CHECKS=1), 0 for the release library. */
 int32_t sp2_build_device_checks(void);

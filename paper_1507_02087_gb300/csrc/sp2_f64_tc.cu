@@ -33,6 +33,7 @@
 
 #include <cstring>
 
+#include "../../include/sp2_testing.h"
 #include "sp2_common.cuh"
 #include "sp2_f64_tc.cuh"
 #include "sp2_kernels.h"
@@ -152,7 +153,11 @@ __device__ __forceinline__ long long fixed56(double x, int e) {
 __global__ void __launch_bounds__(DT)
 digits_kernel(const DevState* st, const double* buf0, const double* buf1, const double* S, int ld, int N, __half* dig,
               int32_t* exps) {
-  if (st->done) return;
+  // the stop test beside it may set st->done: one reading per warp, whose lanes stay together (the digits of a run
+  // that is over are not used)
+  int over = 0;
+  if ((threadIdx.x & 31) == 0) over = *static_cast<const volatile int32_t*>(&st->done);
+  if (__shfl_sync(0xffffffffu, over, 0)) return;
   const double* X = S ? S : (st->wrote ? buf1 : buf0);
   const int rr = threadIdx.x >> 5, r = blockIdx.x * 8 + rr, lane = threadIdx.x & 31;
   if (r >= N) return;
@@ -222,7 +227,15 @@ struct Args {
   double* part;
   const uint8_t *digA, *digB;            // digits of the A and the B operand
   const int32_t *ea, *eb;                // row exponents of the A and the B operand
+  uint64_t wait_ns;                      // limit of every wait
   int32_t ld, tiles, op;
+  int32_t hook;                          // 0, or a Hook of the testing entry
+};
+
+enum Hook : int32_t {
+  HOOK_SKIP_COPY = 1,   // CTA 0 leaves its first stage uncopied: waits run out
+  HOOK_OTHERS_OVER = 2, // the CTAs of a cluster but its first read the run as over
+  HOOK_FIRST_OVER = 3   // only the first does
 };
 
 // What the epilogue writes: out = pk ? s : 2 x - s, or ca s + cb x + cc I with gen set.
@@ -333,17 +346,21 @@ f64_product_kernel(const Args a) {
   __shared__ __align__(8) uint64_t xempty_bar[8];    // and the others have taken this CTA's
   __shared__ uint32_t tmem_base_s;
   __shared__ volatile int abort_s;
+  __shared__ volatile int over_s;        // st->done as thread 0 read it
 
   DevState* st = a.st;
-  if (st->done) return;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int ld = a.ld, cols = (ld + BN - 1) / BN;
   const int rank = KS > 1 ? (int)cluster_ctarank() : 0;
   const int unit = blockIdx.x / KS, units = gridDim.x / KS;       // clusters
   const int kb0 = (ld / KB) * rank / KS, nkb = (ld / KB) * (rank + 1) / KS - kb0;   // this CTA's k-blocks
-  if (blockIdx.x == 0 && threadIdx.x == 0 && a.op != OP_MCW_SQ) st->wrote = (st->k + (a.op == OP_SP2 ? 1 : 0)) & 1;
+  const uint64_t wait_ns = a.wait_ns;
   if (threadIdx.x == 0) {
+    int over = st->done;
+    if (KS > 1 && a.hook >= HOOK_OTHERS_OVER) over |= (a.hook == HOOK_FIRST_OVER) == (rank == 0) ? 1 : 0;
+    over_s = over;
+    if (blockIdx.x == 0 && !over && a.op != OP_MCW_SQ) st->wrote = (st->k + (a.op == OP_SP2 ? 1 : 0)) & 1;
     for (int w = 0; w < 8; ++w) { mbar_init(&xfull_bar[w], KS > 1 ? KS - 1 : 1); mbar_init(&xempty_bar[w], KS > 1 ? KS - 1 : 1); }
     for (int s = 0; s < STG; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
     for (int b = 0; b < NS; ++b) { mbar_init(&accf_bar[b], 1); mbar_init(&acce_bar[b], 8); }
@@ -357,8 +374,12 @@ f64_product_kernel(const Args a) {
   else __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
+  // One reading of st->done decides for the whole cluster, its first CTA's: a wait that gives up elsewhere sets it
+  // during the launch, and a CTA that left on it alone would be written to by the others.
+  const bool over = (KS > 1 ? ld_cluster_u32(mapa_shared(smem_u32(const_cast<int*>(&over_s)), 0)) : (uint32_t)over_s) != 0;
 
-  if (warp < 4) {
+  if (over) {
+  } else if (warp < 4) {
     if (warp == 0) {
       if (elect_one()) {
         int stage = 0;
@@ -372,7 +393,11 @@ f64_product_kernel(const Args a) {
           int I, J;
           locate(t, cols, BM / BN, I, J);
           for (int kb = 0; kb < nkb; ++kb) {
-            if (abort_s || !mbar_wait(&empty_bar[stage], phase ^ 1, globaltimer_ns() + kWaitNs)) { ok = false; break; }
+            if (abort_s || !mbar_wait(&empty_bar[stage], phase ^ 1, globaltimer_ns() + wait_ns)) { ok = false; break; }
+            if (a.hook == HOOK_SKIP_COPY && blockIdx.x == 0 && t == unit && kb == 0) {
+              if (++stage == STG) { stage = 0; phase ^= 1; }
+              continue;
+            }
             uint8_t* sA = smem + stage * SBYTES;
             mbar_arrive_expect_tx(&full_bar[stage], SBYTES);
             bulk_load(sA, a.digA + (kb0 + kb) * kstride + (int64_t)I * A_BYTES, A_BYTES, &full_bar[stage]);
@@ -384,7 +409,7 @@ f64_product_kernel(const Args a) {
         }
         if (!ok) give_up(st, &abort_s);
         for (int s = 0; s < STG; ++s)    // wait (bounded) until every copy issued here has landed
-          if (armed[s]) mbar_wait(&full_bar[s], armed_par[s], globaltimer_ns() + kWaitNs);
+          if (armed[s]) mbar_wait(&full_bar[s], armed_par[s], globaltimer_ns() + wait_ns);
       }
     } else if (warp == 1) {
       if (elect_one()) {
@@ -394,7 +419,7 @@ f64_product_kernel(const Args a) {
         bool ok = true;
         for (int t = unit; t < a.tiles && ok; t += units) {
           for (int kb = 0; kb < nkb && ok; ++kb) {
-            if (abort_s || !mbar_wait(&full_bar[stage], phase, globaltimer_ns() + kWaitNs)) { ok = false; break; }
+            if (abort_s || !mbar_wait(&full_bar[stage], phase, globaltimer_ns() + wait_ns)) { ok = false; break; }
             tc_fence_after();
             const uint32_t sA = smem_u32(smem + stage * SBYTES);
             const uint32_t sB = sA + A_BYTES;
@@ -403,7 +428,7 @@ f64_product_kernel(const Args a) {
               const uint32_t dt = tmem_base + (uint32_t)(s * BN);
               uint32_t accumulate = 1;
               if (kb == 0 || closes(kb - 1, s)) {
-                if (abort_s || !mbar_wait(&acce_bar[s], ((phases >> s) & 1u) ^ 1u, globaltimer_ns() + kWaitNs)) {
+                if (abort_s || !mbar_wait(&acce_bar[s], ((phases >> s) & 1u) ^ 1u, globaltimer_ns() + wait_ns)) {
                   ok = false;
                   break;
                 }
@@ -431,7 +456,7 @@ f64_product_kernel(const Args a) {
         }
         if (!ok) give_up(st, &abort_s);
         mma_commit(&drain_bar);
-        mbar_wait(&drain_bar, 0, globaltimer_ns() + kWaitNs);
+        mbar_wait(&drain_bar, 0, globaltimer_ns() + wait_ns);
       }
     }
   } else {
@@ -460,7 +485,7 @@ f64_product_kernel(const Args a) {
           const int s = __ffs(todo) - 1;
           todo &= todo - 1u;
           int got = 0;
-          if (lane == 0) got = !abort_s && mbar_wait(&accf_bar[s], (phases >> s) & 1u, globaltimer_ns() + kWaitNs);
+          if (lane == 0) got = !abort_s && mbar_wait(&accf_bar[s], (phases >> s) & 1u, globaltimer_ns() + wait_ns);
           got = __shfl_sync(0xffffffffu, got, 0);
           if (!got) {
             ok = false;
@@ -502,7 +527,7 @@ f64_product_kernel(const Args a) {
         // to every other CTA its columns, from every other CTA this one's; the slot of sender p is p, less
         // one past the receiver
         const uint32_t slots = smem_u32(smem + STG * SBYTES);
-        const uint64_t until = globaltimer_ns() + kWaitNs;
+        const uint64_t until = globaltimer_ns() + wait_ns;
         int go = ok;
         if (lane == 0) go = ok && !abort_s && mbar_wait_cluster(&xempty_bar[ew], xphase ^ 1, until);
         go = __shfl_sync(0xffffffffu, go, 0);
@@ -669,6 +694,13 @@ static int slots_of(int bn, int ks) {
   return slots[bn == 64][ks == 8 ? 3 : ks / 2].get([&](int dev) { return find_slots(dev, bn, ks); });
 }
 
+static void set_tiles(Plan& P, int ld, int bn, int ks) {
+  P.ld = ld;
+  P.bn = bn;
+  P.ks = ks;
+  P.recs = 2 * 64 / (bn / 2 / ks);
+}
+
 // The shape with the least time in this model: rounds of tiles, each its k-blocks (68 products of 48 clocks, 44 at
 // width 32: reading A bounds them) and about 12 k clocks for filling the pipe, the last drains and the epilogue,
 // less with fewer columns to finish.  One iteration of a run, unsplit and split: N = 400 54 -> 37 us (16 tiles, 152 SMs),
@@ -686,9 +718,7 @@ void choose_tiles(Plan& P, int ld) {
     const double t = (double)((n + slots - 1) / slots) * tile;
     if (t < best) {
       best = t;
-      P.bn = bn;
-      P.ks = ks;
-      P.recs = 2 * 64 / (bn / 2 / ks);
+      set_tiles(P, ld, bn, ks);
     }
   }
 }
@@ -718,7 +748,7 @@ cudaError_t emit_digits(Sink& sink, const DevState* st, const double* buf0, cons
 }
 
 cudaError_t emit_product(Sink& sink, DevState* st, double* buf0, double* buf1, double* S, double* part,
-                         const Plan& P, Op op) {
+                         const Plan& P, Op op, int hook, int wait_ms) {
   const Digits& A = op == OP_MCW_PROD ? P.S : P.X;
   Args a;
   std::memset(&a, 0, sizeof(a));
@@ -734,6 +764,8 @@ cudaError_t emit_product(Sink& sink, DevState* st, double* buf0, double* buf1, d
   a.ld = P.ld;
   a.tiles = tiles_of(P.ld, P.bn);
   a.op = op;
+  a.hook = hook;
+  a.wait_ns = wait_ms > 0 ? (uint64_t)wait_ms * 1000000ull : kWaitNs;
   const int slots = slots_of(P.bn, P.ks);
   if (slots < 1) return cudaErrorNotSupported;
   void* args[] = {&a};
@@ -743,3 +775,51 @@ cudaError_t emit_product(Sink& sink, DevState* st, double* buf0, double* buf1, d
 
 }  // namespace f64tc
 }  // namespace sp2
+
+extern "C" int32_t sp2_test_f64_product(const double* X_dev, int64_t N, int32_t bn, int32_t ks, int32_t hook,
+                                        int32_t wait_ms, double* out_dev, int32_t* exp_dev, void* stream) {
+  using namespace sp2::f64tc;
+  const bool shape = (bn == 32 && ks == 1) || (bn == 64 && (ks == 1 || ks == 2 || ks == 4 || ks == 8));
+  if (!X_dev || !out_dev || N < 1 || N > 8192 || !shape || hook < 0 || hook > 3 || wait_ms < 0 || wait_ms > 2000)
+    return SP2_ERR_INVALID_ARG;
+  const cudaStream_t s = (cudaStream_t)stream;
+  const int ld = (int)(N + 63) / 64 * 64, T = ld / 64;
+  const size_t bytes = sizeof(double) * (size_t)ld * ld, row = sizeof(double) * (size_t)N;
+  const size_t pbytes = part_bytes(kMinN, T, MAX_RECS);
+  Plan P;
+  set_tiles(P, ld, bn, ks);
+  sp2::DevState h;
+  std::memset(&h, 0, sizeof(h));
+  h.N = (int)N;
+  h.ld = ld;
+  h.tr[0] = 1.0;                         // above nocc = 0: X_1 = X_0^2
+  sp2::DevState* st = nullptr;
+  double *buf = nullptr, *part = nullptr;
+  Sink sink;
+  sink.s = s;
+  bool ok = cudaMalloc(&st, sizeof(h)) == cudaSuccess && cudaMalloc(&buf, 2 * bytes) == cudaSuccess &&
+            cudaMalloc(&part, pbytes) == cudaSuccess && cudaMalloc(&P.X.dig, digit_bytes(ld)) == cudaSuccess &&
+            cudaMalloc(&P.X.exp, exp_bytes(ld)) == cudaSuccess;
+  ok = ok && cudaMemcpyAsync(st, &h, sizeof(h), cudaMemcpyHostToDevice, s) == cudaSuccess &&
+       cudaMemsetAsync(buf, 0, 2 * bytes, s) == cudaSuccess &&
+       cudaMemsetAsync(P.X.dig, 0, digit_bytes(ld), s) == cudaSuccess &&
+       cudaMemsetAsync(P.X.exp, 0, exp_bytes(ld), s) == cudaSuccess &&
+       cudaMemcpy2DAsync(buf, sizeof(double) * ld, X_dev, row, row, N, cudaMemcpyDeviceToDevice, s) == cudaSuccess;
+  double* buf1 = buf + (size_t)ld * ld;
+  ok = ok && emit_digits(sink, st, buf, buf1, nullptr, P, (int)N) == cudaSuccess &&
+       emit_product(sink, st, buf, buf1, nullptr, part, P, OP_SP2, hook, wait_ms) == cudaSuccess &&
+       cudaMemcpy2DAsync(out_dev, row, buf1, sizeof(double) * ld, row, N, cudaMemcpyDeviceToDevice, s) == cudaSuccess &&
+       (!exp_dev || cudaMemcpyAsync(exp_dev, P.X.exp, sizeof(int32_t) * N, cudaMemcpyDeviceToDevice, s) == cudaSuccess) &&
+       cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s) == cudaSuccess;
+  ok = cudaStreamSynchronize(s) == cudaSuccess && ok;
+  cudaFree(st);
+  cudaFree(buf);
+  cudaFree(part);
+  cudaFree(P.X.dig);
+  cudaFree(P.X.exp);
+  if (!ok) {
+    (void)cudaGetLastError();
+    return SP2_ERR_CUDA;
+  }
+  return h.status;
+}

@@ -64,9 +64,10 @@ struct Sink {
 // Digits of the newest iterate (buf0 or buf1, st->wrote), or of S when `S` is given.
 cudaError_t emit_digits(Sink& sink, const DevState* st, const double* buf0, const double* buf1, const double* S,
                         const Plan& P, int N);
-// The product `op` over the upper tiles, with the partial records of the stop test.
+// The product `op` over the upper tiles, with the partial records of the stop test.  hook, wait_ms: of the testing
+// entry (0: none, waits of 2 s).
 cudaError_t emit_product(Sink& sink, DevState* st, double* buf0, double* buf1, double* S, double* part,
-                         const Plan& P, Op op);
+                         const Plan& P, Op op, int hook = 0, int wait_ms = 0);
 
 }  // namespace f64tc
 }  // namespace sp2

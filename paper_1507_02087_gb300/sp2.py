@@ -81,6 +81,8 @@ def lib() -> ctypes.CDLL:
         L.sp2_test_tc_gemm_ex.restype = i32
         L.sp2_test_tc_timeout.argtypes = [vp, i32, i32, vp, vp]
         L.sp2_test_tc_timeout.restype = i32
+        L.sp2_test_f64_product.argtypes = [vp, i64, i32, i32, i32, i32, vp, vp, vp]
+        L.sp2_test_f64_product.restype = i32
         L.sp2_build_device_checks.argtypes = []
         L.sp2_build_device_checks.restype = i32
         L.sp2_test_tc_bounds.argtypes = [vp, i32, i32, i32, vp, vp]
