@@ -1105,24 +1105,13 @@ __global__ void tile_meta_kernel(const DevState* st, Mat X, Pairs P, const uint3
   }
 }
 
-// SMs of the current device (queried once, before any stream capture; see build_graph)
-static int meta_sms() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 1;
-  }
-  return sms;
-}
-
 cudaError_t tc_tiles_launch(const DevState* st, const Mat& X, const Pairs& P, const uint32_t* sbits, int nb, int W,
                             int* counts, int* tptr, int* tnnz, int* tiles, int* meta, cudaStream_t s) {
   const int ncg = (nb + TTC - 1) / TTC, bands = (nb + TTR * TBAND - 1) / (TTR * TBAND);
   tile_count_kernel<<<bands, 32, 0, s>>>(st, sbits, nb, W, ncg, counts);
   scan_kernel<<<1, 1024, 0, s>>>(counts, bands, tptr, tnnz, st);
   tile_fill_kernel<<<bands, 32, 0, s>>>(st, sbits, nb, W, ncg, tptr, tiles);
-  tile_meta_kernel<<<4 * meta_sms(), 256, 0, s>>>(st, X, P, sbits, nb, W, ncg, tiles, tnnz, meta);
+  tile_meta_kernel<<<4 * sm_count(), 256, 0, s>>>(st, X, P, sbits, nb, W, ncg, tiles, tnnz, meta);
   return cudaGetLastError();
 }
 
@@ -1246,11 +1235,9 @@ static void bsr_free(sp2_bsr_ctx* h) {
 
 // Persistent grid of the numeric square: the resident CTAs of the whole GPU.
 static int numeric_grid() {
-  static int n = 0;
-  if (!n) {
-    int dev = 0, sms = 1, per = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  static PerDevice grid;
+  return grid.get([](int) {
+    int per = 1;
     if (cudaFuncSetAttribute(bsr_numeric_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, NUM_SMEM) !=
             cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, bsr_numeric_kernel, NUM_THREADS, NUM_SMEM) !=
@@ -1259,21 +1246,11 @@ static int numeric_grid() {
       (void)cudaGetLastError();
       per = 1;
     }
-    n = std::max(1, sms) * per;
-  }
-  return n;
+    return sm_count() * per;
+  });
 }
 
-static int grid_persistent() {
-  static int n = 0;
-  if (!n) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (n <= 0) n = 1;
-  }
-  return n * 4;
-}
+static int grid_persistent() { return sm_count() * 4; }
 
 // One loop round (the body of the WHILE node, or one unrolled round in launch mode 1).
 // The buffers alternate by round: round k reads X[(k-1)&1] and writes X[k&1]; a graph
@@ -1347,7 +1324,6 @@ static sp2_status build_graph(sp2_bsr_ctx* h) {
   cudaGraph_t body = np.conditional.phGraph_out[0];
   (void)grid_persistent();   // device queries before capture
   (void)numeric_grid();
-  (void)meta_sms();
   tc_prepare();
   if (h->lz) BSR_TRY(lanczos_prepare());
   cudaStream_t cs;

@@ -24,6 +24,7 @@
 
 #include "../../include/sp2.h"
 #include "sp2_bsr.cuh"
+#include "sp2_kernels.h"
 #include "sp2_tc.cuh"
 #include "tc_ptx.cuh"
 
@@ -364,17 +365,14 @@ __global__ void __launch_bounds__(TTHREADS, 1) bsr_tc_kernel(const TcArgs a) {
   }
 }
 
+// One CTA per SM; sets the kernel's attribute on the current device first.
 static int tc_grid() {
-  static int n = 0;
-  if (!n) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (n <= 0) n = 1;
+  static PerDevice grid;
+  return grid.get([](int) {
     if (cudaFuncSetAttribute(bsr_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TSMEM) != cudaSuccess)
       (void)cudaGetLastError();
-  }
-  return n;
+    return sm_count();
+  });
 }
 
 void tc_prepare() { (void)tc_grid(); }

@@ -23,6 +23,16 @@ struct PerDevice {
   }
 };
 
+// SMs of the current device.
+inline int sm_count() {
+  static PerDevice sms;
+  const int n = sms.get([](int dev) {
+    int v = 0;
+    return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? v : 0;
+  });
+  return n > 0 ? n : 1;
+}
+
 struct DevState;
 namespace f64tc {
 struct Plan;

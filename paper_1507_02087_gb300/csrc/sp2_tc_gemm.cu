@@ -949,17 +949,6 @@ cudaError_t tc_make_maps(void* arena, int ld, int nslots, int fmt, tc::Instance*
   return cudaSuccess;
 }
 
-static int sm_count() {
-  static int n = 0;
-  if (!n) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (n <= 0) n = 1;
-  }
-  return n;
-}
-
 // The kernel instance for a job: tile kind (and width) x piece format.
 template <int FMT>
 static void* kernel_of_fmt(int pair, int tn) {
@@ -975,21 +964,22 @@ static void* kernel_of(int pair, int tn, int fmt) {
 }
 
 static cudaError_t tc_prepare() {
-  static bool done = false;
-  if (done) return cudaSuccess;
+  static PerDevice done;
   cudaError_t e = cudaSuccess;
-  for (int kind = 0; kind < 4 && e == cudaSuccess; ++kind)   // pair, then the single widths
-    for (int fmt = 0; fmt < 3 && e == cudaSuccess; ++fmt)
-      e = cudaFuncSetAttribute(kernel_of(kind == 0, 16 << kind, fmt), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kind == 0 ? tc::P_SMEM_BYTES : tc::SMEM_BYTES);
-  if (e == cudaSuccess) done = true;
+  done.get([&](int) {
+    for (int kind = 0; kind < 4 && e == cudaSuccess; ++kind)   // pair, then the single widths
+      for (int fmt = 0; fmt < 3 && e == cudaSuccess; ++fmt)
+        e = cudaFuncSetAttribute(kernel_of(kind == 0, 16 << kind, fmt), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kind == 0 ? tc::P_SMEM_BYTES : tc::SMEM_BYTES);
+    return e == cudaSuccess ? 1 : 0;
+  });
   return e;
 }
 
 // Clusters of two that fit on the GPU at once (one CTA per SM); 0 if the query fails.
 static int pair_slots() {
-  static int n = -1;
-  if (n < 0) {
+  static PerDevice slots;
+  return slots.get([](int) {
     if (tc_prepare() != cudaSuccess) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * sm_count());
@@ -1000,9 +990,8 @@ static int pair_slots() {
       (void)cudaGetLastError();
       c = sm_count() / 2;
     }
-    n = c;
-  }
-  return n;
+    return c;
+  });
 }
 
 // Persistent grid: one CTA (or one CTA pair) per tile up to what the GPU holds at once.
