@@ -73,11 +73,22 @@ typedef enum {
  * rounded up to a multiple of 128 (256 with CTA-pair tiles); see sp2_opts.history. */
 typedef enum {
   SP2_PREC_FP64 = 0,   /* FP64 products and FP64 everything (the plain method).  For N >= 129 the products
-                          are formed on the tensor cores as exact integer sums of 8-bit digit products,
-                          rounded to FP64 once (56 bits per value under a power-of-two scale per row):
-                          the error of a product is below that of a chain of FP64 multiply-adds.
-                          Workspace 14 ld^2 bytes beside the two iterates (twice that with McWeeny); a
-                          handle that cannot have it multiplies on the FP64 units */
+                          are formed on the tensor cores as integer sums of 8-bit digit products (56 bits
+                          per value under one power-of-two scale per row).  Their error is bounded by
+                          norms: at most (2^-54 sqrt(N) + 2^-59 N) ||x_i|| ||x_j|| + 2^-53 |s_ij| for the
+                          element s_ij = x_i . x_j of rows x_i, x_j (a chain of FP64 multiply-adds: N 2^-53
+                          sum_k |x_ik x_jk|).  It is not bounded element by element: elements far below
+                          their row's norm, such as the far off-diagonals of a local matrix, lose relative
+                          accuracy, and below about 2^-56 of it they are noise or zero.  The last bits
+                          depend on how a product is split over the SMs and can differ between devices.
+                          Where v_i falls on the rounding floor the run can stop some steps (up to four
+                          seen) from where multiply-adds would.  Workspace 14 ld^2 bytes beside the two
+                          iterates (twice that with McWeeny, which adds a third), taken at create if the
+                          device has it then: 30 (52) ld^2 bytes in all, so make other large allocations
+                          first.  A handle that cannot have it multiplies on the FP64 units, element by
+                          element accurate and some 25 times slower at N = 2048; sp2_set_mcweeny gives the
+                          workspace up, for all later runs of the handle, where its own buffer needs the
+                          room */
   SP2_PREC_MIXED = 1,  /* = SP2_PREC_BF16X6: each FP32 value stored exactly as three bf16
                           pieces (P = 3), products as the six piece products with a + b <= 2
                           (FP32-accurate) */

@@ -9,22 +9,30 @@
 // and the 34 digit products with s <= 7 are formed on the tensor cores.  The FP32 accumulators hold every
 // V_s exactly up to 2^24, and each is drained before it can pass that (period); the V_s are added in 64-bit
 // integer registers in units of 2^-62 (|sum| < 1 by Cauchy's inequality, so it fits) and the total is rounded
-// to FP64 once.  No other rounding happens, so the result does not depend on the order of the sums.
+// to FP64 once.  V_0 .. V_5 are whole numbers of units; V_6 2^-2 and V_7 2^-10 are rounded to the unit at each of
+// their drains, at most ld / 128 + ks times each in the ks CTAs that share a tile, so the last bits depend on the
+// split, and with it on the device's SMs and clusters.  (Digit splittings of this kind: K. Ozaki, T. Ogita, S. Oishi,
+// S. M. Rump, "Error-free transformations of matrix multiplication by using fast routines of matrix multiplication
+// and its applications", Numer. Algorithms 59, 2012.)
 //
-// Error against the exact product, in units of 2^(e_i + e_j): the digits' own rounding, at most 2^-57 per
-// value; the products with s >= 8 that are left out, about sqrt(5 K) 2^-67.6; the V_6 and V_7 rounded to the
-// unit.  An FMA chain rounds K times at 2^-53 of its partial sums.  ||D - D_exact||_F / ||D||_F against the
-// exact projector at N = 400 / 1001 / 1500 (McW-ACC) / 2048: 8.6e-15 / 2.1e-14 / 2.4e-14 / 4.4e-14, with FMA
-// chains 1.3e-14 / 3.0e-14 / 4.3e-14 / 6.1e-14.  The lower floor of ||X - X^2|| can move the stop by a few steps where
-// it falls on that floor (12 of 60 drawn problems), with the smaller error each time.
+// Error against the exact product, in units of 2^(e_i + e_j) <= 16 ||x_i|| ||x_j||: the digits' own rounding, at most
+// 2^-57 per value; the products with s >= 8 that are left out, at most 5.02 K 2^-66 and for random digits about
+// sqrt(5 K) 2^-67.6; at most ld / 128 + ks units of 2^-62 from the drains.  In all at most (2^-54 sqrt(K) + 2^-59 K)
+// ||x_i|| ||x_j|| and half a unit in the last place, against K 2^-53 |x_i| |x_j| for an FMA chain.  The bound holds for
+// norms only: an element far below its row's norm has fewer digits (56 - k bits at 2^-k of the scale), and where
+// |x_i| |x_j| is far below ||x_i|| ||x_j||, as far from the diagonal of a local matrix, the result loses the relative
+// accuracy that an FMA chain keeps (entries that decay by ten per eight off the diagonal, one square: 2e-11 of an
+// element of 6e-8, 2e-6 at 7e-13; below about 1e-17 noise or zero).
+// ||D - D_exact||_F / ||D||_F against the exact projector at N = 400 / 1001 / 1500 (McW-ACC) / 2048: 8.5e-15 / 2.0e-14 /
+// 2.3e-14 / 4.2e-14, with FMA chains 1.3e-14 / 2.9e-14 / 4.2e-14 / 6.1e-14.  The lower floor of ||X - X^2|| can move the
+// stop by a few steps where it falls on that floor (12 of 60 drawn problems), with the smaller error each time.
 //
 // Time of one purification against the FP64 units (64 x 64 tiles, 0.98 of their peak at large N): N = 400
 // 1.37 ms against 18.1, N = 1500 (McW-ACC) 5.38 against 77.4, N = 2048 16.5 against 418.
 //
 // Tiles are 128 x bn (bn = 32 or 64), over the upper triangle; where they are fewer than the SMs, or fill the
 // last round badly, a cluster of ks CTAs shares a tile's k range (choose_tiles): each sums its part, then gives
-// each of the others its columns through distributed shared memory, and every CTA finishes 64 / ks columns.  The
-// sums are integers, so the split changes no bit.  A stage holds
+// each of the others its columns through distributed shared memory, and every CTA finishes 64 / ks columns.  A stage holds
 // the 7 digits of 32 k-columns of both operands, so 14 digit planes feed 34 products.  What bounds the
 // products is the reading of A from shared memory: a 128 x 64 x 16 product takes 48 clocks for 32 of
 // arithmetic.  Warp roles as in the other tensor-core kernels: warp 0 copies, warp 1 issues the products,
