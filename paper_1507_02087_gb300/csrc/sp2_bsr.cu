@@ -516,7 +516,9 @@ bsr_numeric_kernel(DevState* st, Mat X, int W, Pairs P, float* svals, uint8_t* s
 // m = (budget - units below G) / u(G) of them in q order are dropped.  The pair list is
 // in (I, J) order, so q breaks ties as (I, J) does.  `cbits` (nnz entries of scratch)
 // caches each pair's candidate bits (~0 if none).  Nine launches of about 3 us; as one CTA with eight passes
-// it took 115 us for 5.9 k pairs, and its time grew with them.
+// it took 115 us for 5.9 k pairs, and its time grew with them.  Up to 1024 pairs (44 block rows) one CTA and one launch
+// for all passes: a run with 1 block row 0.87 -> 0.69 ms, with 16 1.71 -> 1.50, with 44 3.05 -> 2.72 against the nine
+// launches, which cost the smallest lattices more than the selection in one CTA did (1 block row 0.73, 2 0.92 then 1.03).
 constexpr int kEC = 256, kECBins = 2048, kECPasses = 6;
 
 struct EcStep { unsigned long long prefix, below; };
@@ -595,11 +597,11 @@ __device__ __forceinline__ uint64_t ec_budget(double tau2, int& e) {
   return (uint64_t)floor(ldexp(tau2, 40 - e));
 }
 
+// The passes, each by a grid of kEC threads a CTA: as a launch of its own, or one after the other in one CTA.
+
 // candidate bits and the total of their units (total zeroed before), the histograms cleared
-__global__ void __launch_bounds__(kEC)
-ec_candidates_kernel(const DevState* st, const double* n2, const int* row, const int* col, const int* nnz_p,
-                     uint64_t* cbits, double tau2, EcScratch* S) {
-  if (st && !st->iter_active) return;
+__device__ __forceinline__ void ec_candidates(const double* n2, const int* row, const int* col, const int* nnz_p,
+                                              uint64_t* cbits, double tau2, EcScratch* S) {
   const int nnz = *nnz_p, lane = threadIdx.x & 31;
   int e;
   (void)ec_budget(tau2, e);
@@ -618,11 +620,9 @@ ec_candidates_kernel(const DevState* st, const double* n2, const int* row, const
   if (lane == 0 && acc) atomicAdd(&S->total, (unsigned long long)acc);
 }
 
-__global__ void __launch_bounds__(kEC)
-ec_pass_kernel(const DevState* st, const int* nnz_p, const uint64_t* cbits, double tau2, EcScratch* S, int pass) {
+__device__ __forceinline__ void ec_pass(const int* nnz_p, const uint64_t* cbits, double tau2, EcScratch* S, int pass) {
   __shared__ unsigned long long hist[kECBins];
   __shared__ unsigned long long sm[kEC + 2];
-  if (st && !st->iter_active) return;
   int e;
   const uint64_t budget = ec_budget(tau2, e);
   if (S->total <= budget) return;                 // everything fits
@@ -659,11 +659,9 @@ ec_pass_kernel(const DevState* st, const int* nnz_p, const uint64_t* cbits, doub
 }
 
 // The key's bits G and how many pairs weigh them before each CTA's range of q.
-__global__ void __launch_bounds__(kEC)
-ec_ties_kernel(const DevState* st, const int* nnz_p, const uint64_t* cbits, double tau2, EcScratch* S) {
+__device__ __forceinline__ void ec_ties(const int* nnz_p, const uint64_t* cbits, double tau2, EcScratch* S) {
   __shared__ unsigned long long sm[kEC + 2];
   __shared__ int s_n;
-  if (st && !st->iter_active) return;
   int e;
   const uint64_t budget = ec_budget(tau2, e);
   if (S->total <= budget) return;
@@ -680,11 +678,10 @@ ec_ties_kernel(const DevState* st, const int* nnz_p, const uint64_t* cbits, doub
   if (threadIdx.x == 0) S->ties[blockIdx.x] = s_n;
 }
 
-__global__ void __launch_bounds__(kEC)
-ec_keep_kernel(const DevState* st, const int* nnz_p, const uint64_t* cbits, double tau2, EcScratch* S, uint8_t* keep) {
+__device__ __forceinline__ void ec_keep(const int* nnz_p, const uint64_t* cbits, double tau2, EcScratch* S,
+                                        uint8_t* keep) {
   __shared__ int s_warp[kEC / 32];
   __shared__ int s_before;
-  if (st && !st->iter_active) return;
   int e;
   const uint64_t budget = ec_budget(tau2, e);
   const int nnz = *nnz_p, chunk = (nnz + gridDim.x - 1) / gridDim.x, tid = threadIdx.x, lane = tid & 31;
@@ -727,6 +724,43 @@ ec_keep_kernel(const DevState* st, const int* nnz_p, const uint64_t* cbits, doub
   }
 }
 
+__global__ void __launch_bounds__(kEC)
+ec_candidates_kernel(const DevState* st, const double* n2, const int* row, const int* col, const int* nnz_p,
+                     uint64_t* cbits, double tau2, EcScratch* S) {
+  if (!st || st->iter_active) ec_candidates(n2, row, col, nnz_p, cbits, tau2, S);
+}
+__global__ void __launch_bounds__(kEC)
+ec_pass_kernel(const DevState* st, const int* nnz_p, const uint64_t* cbits, double tau2, EcScratch* S, int pass) {
+  if (!st || st->iter_active) ec_pass(nnz_p, cbits, tau2, S, pass);
+}
+__global__ void __launch_bounds__(kEC)
+ec_ties_kernel(const DevState* st, const int* nnz_p, const uint64_t* cbits, double tau2, EcScratch* S) {
+  if (!st || st->iter_active) ec_ties(nnz_p, cbits, tau2, S);
+}
+__global__ void __launch_bounds__(kEC)
+ec_keep_kernel(const DevState* st, const int* nnz_p, const uint64_t* cbits, double tau2, EcScratch* S, uint8_t* keep) {
+  if (!st || st->iter_active) ec_keep(nnz_p, cbits, tau2, S, keep);
+}
+
+// All passes in one CTA, for a grid of one.
+__global__ void __launch_bounds__(kEC)
+ec_small_kernel(const DevState* st, const double* n2, const int* row, const int* col, const int* nnz_p, uint64_t* cbits,
+                double tau2, EcScratch* S, uint8_t* keep) {
+  if (st && !st->iter_active) return;
+  if (threadIdx.x == 0) S->total = 0ull;
+  __syncthreads();
+  ec_candidates(n2, row, col, nnz_p, cbits, tau2, S);
+  __syncthreads();
+  #pragma unroll 1
+  for (int p = 0; p < kECPasses; ++p) {
+    ec_pass(nnz_p, cbits, tau2, S, p);
+    __syncthreads();
+  }
+  ec_ties(nnz_p, cbits, tau2, S);
+  __syncthreads();
+  ec_keep(nnz_p, cbits, tau2, S, keep);
+}
+
 __global__ void ec_all_kernel(const DevState* st, const int* nnz_p, uint8_t* keep) {   // tau = 0 drops nothing
   if (st && !st->iter_active) return;
   const int nnz = *nnz_p;
@@ -743,6 +777,10 @@ void launch_errctl(const DevState* st, const double* n2, const int* row, const i
     return;
   }
   EcScratch* S = static_cast<EcScratch*>(scratch);
+  if (grid == 1) {
+    ec_small_kernel<<<1, kEC, 0, s>>>(st, n2, row, col, nnz_p, cbits, tau2, S, keep);
+    return;
+  }
   cudaMemsetAsync(&S->total, 0, sizeof(S->total), s);
   ec_candidates_kernel<<<grid, kEC, 0, s>>>(st, n2, row, col, nnz_p, cbits, tau2, S);
   for (int p = 0; p < kECPasses; ++p) ec_pass_kernel<<<grid, kEC, 0, s>>>(st, nnz_p, cbits, tau2, S, p);

@@ -1,5 +1,7 @@
-"""Handles on two devices of one process, without a GPU: the library's host code linked against a stand-in for the
-CUDA runtime (fake_runtime.c).  Limits and numbers that CUDA keeps per device have to be set and found per device."""
+"""The library's host code linked against a stand-in for the CUDA runtime (fake_runtime.c), without a GPU.
+
+Handles on two devices of one process: limits and numbers that CUDA keeps per device have to be set and found per
+device.  Launches of a round: where they are the time of a small problem, there are no more of them than needed."""
 import glob
 import os
 import subprocess
@@ -78,3 +80,39 @@ def library(tmp_path_factory):
 def test_handles_on_a_second_device(library):
     r = subprocess.run([sys.executable, "-c", PROGRAM, library, ROOT], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+SELECTION = r"""
+import ctypes, sys
+sys.path.insert(0, sys.argv[2])
+import numpy as np
+from paper_1507_02087_gb300 import sp2
+sp2.LIB_PATH = sys.argv[1]
+L = sp2.lib()
+F, D = np.zeros(4 << 20), np.zeros(4 << 20)
+rp, ci = np.arange(65, dtype=np.int32), np.arange(64, dtype=np.int32)
+
+def launches(nb, rule):
+    o = sp2.sp2_opts()
+    L.sp2_default_opts(ctypes.byref(o))
+    o.max_iter, o.launch_mode = 7, 1                          # every round is launched, in pairs: ten of them
+    h = ctypes.c_void_p()
+    assert L.sp2_create_bsr_ex(32 * nb, 16 * nb, 1e-4, rule, ctypes.byref(o), ctypes.byref(h)) == 0
+    before = L.fake_launched(0)
+    assert L.sp2_run_bsr(h, rp.ctypes.data, ci.ctypes.data, F.ctypes.data, nb, D.ctypes.data, None) == 0
+    n = L.fake_launched(0) - before
+    L.sp2_destroy_bsr(h)
+    return n
+
+for nb in (1, 4, 44):
+    print(nb, launches(nb, 1) - launches(nb, 0))
+"""
+
+
+def test_the_selection_of_a_small_lattice_is_one_launch(library):
+    # the error-controlled rule against the rule per block, which needs no selection: one launch more for X_0 and for
+    # each of ten rounds
+    r = subprocess.run([sys.executable, "-c", SELECTION, library, ROOT], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
+    extra = dict(tuple(map(int, line.split())) for line in r.stdout.splitlines())
+    assert extra == {1: 11, 4: 11, 44: 11}, extra
