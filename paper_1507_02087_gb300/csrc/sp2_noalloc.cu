@@ -141,10 +141,9 @@ static sp2_status run_noalloc(const double* F_dev, double* D_dev, int64_t N, int
   }
   // as a handle of this size: the products on the tensor cores, or on the CUDA cores
   sp2::f64tc::Plan tc;
-  tc.on = sp2::f64tc::wanted(N);
+  if (sp2::f64tc::wanted(N)) sp2::f64tc::choose_tiles(tc, ld);
+  tc.on = tc.bn > 0;
   if (tc.on) {
-    sp2::f64tc::choose_tiles(tc, ld);
-    if (tc.bn <= 0) return SP2_ERR_CUDA;
     tc.X.dig = (__half*)(base + kOffDig);
     tc.X.exp = (int32_t*)(base + kOffExp);
     if (cudaMemsetAsync(tc.X.dig, 0, sp2::f64tc::digit_bytes(ld), s) != cudaSuccess ||

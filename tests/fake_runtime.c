@@ -8,9 +8,10 @@
 #define KERNELS 4096
 enum { DEVICES = 2 };
 static const int kSms[DEVICES] = {152, 100};
-static int device, refused, launched[DEVICES], nlimits;
+static int device, refused, launched[DEVICES], nlimits, no_limits;
 static struct { const void* func; int device, bytes; } limits[KERNELS];
 
+void fake_no_limits(int on) { no_limits = on; }   /* raising a kernel's limit fails from now on */
 int fake_refused(void) { return refused; }
 int fake_launched(int d) { return launched[d]; }
 
@@ -32,6 +33,7 @@ cudaError_t cudaDeviceGetAttribute(int* v, enum cudaDeviceAttr a, int d) {
 }
 cudaError_t cudaFuncSetAttribute(const void* func, enum cudaFuncAttribute a, int bytes) {
   if (a != cudaFuncAttributeMaxDynamicSharedMemorySize) return cudaSuccess;
+  if (no_limits) return cudaErrorInvalidValue;
   for (int i = 0; i < nlimits; ++i)
     if (limits[i].func == func && limits[i].device == device) { limits[i].bytes = bytes; return cudaSuccess; }
   limits[nlimits].func = func; limits[nlimits].device = device; limits[nlimits++].bytes = bytes;

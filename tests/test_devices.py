@@ -116,3 +116,25 @@ def test_the_selection_of_a_small_lattice_is_one_launch(library):
     assert r.returncode == 0, r.stderr[-2000:]
     extra = dict(tuple(map(int, line.split())) for line in r.stdout.splitlines())
     assert extra == {1: 11, 4: 11, 44: 11}, extra
+
+
+UNITS = r"""
+import ctypes, sys
+sys.path.insert(0, sys.argv[2])
+import numpy as np
+from paper_1507_02087_gb300 import sp2
+sp2.LIB_PATH = sys.argv[1]
+L = sp2.lib()
+L.fake_no_limits(1)
+F, D, info = np.zeros(300 * 300), np.zeros(300 * 300), np.zeros(4, dtype=np.int32)
+h = ctypes.c_void_p()
+print(L.sp2_create(300, 150, 0, None, ctypes.byref(h)), L.sp2_run(h, F.ctypes.data, D.ctypes.data, None))
+print(L.sp2_run_fp64_noalloc(F.ctypes.data, D.ctypes.data, 300, 150, info.ctypes.data, None), L.fake_refused())
+"""
+
+
+def test_fp64_runs_where_the_tensor_core_kernels_cannot(library):
+    # kernels that need a raised limit are left out; the FP64 units need none, in a handle and without one
+    r = subprocess.run([sys.executable, "-c", UNITS, library, ROOT], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert r.stdout.split() == ["0"] * 4, r.stdout
