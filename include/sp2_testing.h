@@ -58,9 +58,9 @@ int32_t sp2_test_tc_timeout(const void* arena_dev, int32_t ld, int32_t wait_ms, 
  * int32 that receive the rows' exponents e_i (||x_i|| < 2^e_i, |x_ik| <= 2^(e_i - 1)).
  * hook 0: none.  1: CTA 0 leaves its first stage uncopied, so that waits, limited to wait_ms (0: 2000), run out and
  * the call returns SP2_ERR_TIMEOUT.  2 (3): in each cluster of ks > 1 CTAs, all but the first (only the first) find
- * the run over when they start, as after a wait that ran out elsewhere; the first decides for its cluster: with 2 the
- * product is complete, with 3 out_dev receives zeros.  Every CTA stays until its cluster is done, so neither
- * touches memory of a CTA that has left.  Synchronises `stream`; returns an sp2_status. */
+ * the run over when they start, as after a wait that ran out elsewhere; the others wait for their sums in vain, and the
+ * call returns SP2_ERR_TIMEOUT.  Every CTA stays until its cluster is done, so no memory of a CTA that has left is
+ * touched.  Synchronises `stream`; returns an sp2_status. */
 int32_t sp2_test_f64_product(const double* X_dev, int64_t N, int32_t bn, int32_t ks, int32_t hook, int32_t wait_ms,
                              double* out_dev, int32_t* exp_dev, void* stream);
 

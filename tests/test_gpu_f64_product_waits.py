@@ -1,8 +1,8 @@
 """The waits of the FP64 product on the tensor cores (csrc/sp2_f64_tc.cu) where a run ends during the launch.
 
-A wait that gives up ends the run while other clusters are still starting.  The first CTA of each cluster decides
-whether it takes part, and every CTA stays until its cluster is done: the testing entry lets some CTAs of every
-cluster find the run over at their start, and lets waits run out, without a fault.
+A wait that gives up ends the run while other clusters are still starting, so that some CTAs of a cluster may find it
+over and others not.  Every CTA stays until its cluster is done: the testing entry lets some CTAs of every cluster
+find the run over at their start, and lets waits run out, without a fault.
 """
 import pytest
 import torch
@@ -27,13 +27,14 @@ def X():
 
 
 @pytest.mark.parametrize("ks", SPLITS)
-def test_the_first_cta_decides_for_its_cluster(X, ks):
+@pytest.mark.parametrize("hook", [2, 3])         # all but the first CTA of a cluster, or only the first
+def test_ctas_that_find_the_run_over_stay_in_their_cluster(X, ks, hook):
     want, status = product(X, ks, 0)
     assert status == 0 and torch.allclose(want, X @ X.T, rtol=0, atol=1e-10)
-    got, status = product(X, ks, 2)              # the others find the run over: the first does not
-    assert status == 0 and torch.equal(got, want)
-    got, status = product(X, ks, 3)              # the first finds it over: none takes part
-    assert status == 0 and not got.any()
+    _, status = product(X, ks, hook, wait_ms=50)
+    assert status == 4                           # SP2_ERR_TIMEOUT: the others wait for their sums in vain
+    again, status = product(X, ks, 0)            # the context stays usable
+    assert status == 0 and torch.equal(again, want)
 
 
 @pytest.mark.parametrize("ks", [1] + SPLITS)
