@@ -537,10 +537,9 @@ f64_product_kernel(const Args a) {
         // one past the receiver
         const uint32_t slots = smem_u32(smem + STG * SBYTES);
         const uint64_t until = globaltimer_ns() + wait_ns;
-        int go = ok;
-        if (lane == 0) go = ok && !abort_s && mbar_wait_cluster(&xempty_bar[ew], xphase ^ 1, until);
-        go = __shfl_sync(0xffffffffu, go, 0);
-        __syncwarp();                    // orders the lanes' stores after lane 0's wait (a shuffle orders no memory)
+        // every lane waits, since the wait orders the accesses of its own lane only (as lane 0's wait, a shuffle and a
+        // __syncwarp, the runs at N = 400 and 1500 took 3 % longer)
+        int go = __all_sync(0xffffffffu, ok && !abort_s && mbar_wait_cluster(&xempty_bar[ew], xphase ^ 1, until));
         if (go) {
           #pragma unroll 1
           for (int j = 0; j < G; j += 4) {
@@ -558,10 +557,8 @@ f64_product_kernel(const Args a) {
             #pragma unroll 1
             for (int o = 0; o < KS; ++o)
               if (o != rank) mbar_arrive_cluster(mapa_shared(smem_u32(&xfull_bar[ew]), o));
-            go = mbar_wait_cluster(&xfull_bar[ew], xphase, until);
           }
-          go = __shfl_sync(0xffffffffu, go, 0);
-          __syncwarp();                  // and their loads of the others' sums
+          go = __all_sync(0xffffffffu, mbar_wait_cluster(&xfull_bar[ew], xphase, until));
         }
         if (!go) ok = false;
       }
