@@ -545,8 +545,10 @@ cudaError_t launch_perturb(DevState* st, double* buf0, double* buf1, const doubl
 // ---- one product of the loop, by size ------------------------------------------------------------
 // The digits a tensor-core product needs are made before the loop (X_0, launch_f64_digits) and after each product:
 // of the new iterate, beside the stop test (which only that needs), and of the McWeeny step's square.
-// N <= 128: 8 x 8 tiles on the FP64 units (the tensor-core product has about 35 us of latency a square, against
-// some 10 there); else the tensor cores, or 64 x 64 tiles on the FP64 units where the digit buffers were not to be had.
+// N <= 128: 8 x 8 tiles on the FP64 units, which stage their rows whole in shared memory of that width; else the tensor
+// cores, or 64 x 64 tiles on the FP64 units where the digit buffers were not to be had.  A round takes 16 us at N = 128
+// and 28 us on the tensor cores at N = 129 (230 us in 64 x 64 tiles), so the line is the staging's limit; how far
+// past it the 8 x 8 tiles would still win was not measured.
 enum ProductOp { kSquare = 0, kMcwSquare = 1, kMcwProd = 2 };
 
 static int recs_of(const f64tc::Plan* tc, int N) { return tc ? tc->recs : (N <= kSmallN ? kSmallRecs : 1); }

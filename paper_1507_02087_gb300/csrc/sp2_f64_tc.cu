@@ -28,7 +28,7 @@
 // stop by a few steps where it falls on that floor (12 of 60 drawn problems), with the smaller error each time.
 //
 // Time of one purification against the FP64 units (64 x 64 tiles, 0.98 of their peak at large N): N = 400
-// 1.37 ms against 18.1, N = 1500 (McW-ACC) 5.38 against 77.4, N = 2048 16.5 against 418.
+// 1.34 ms against 18.4, N = 1500 (McW-ACC) 5.18 against 77.5, N = 2048 16.7 against 418.
 //
 // Tiles are 128 x bn (bn = 32 or 64), over the upper triangle; where they are fewer than the SMs, or fill the
 // last round badly, a cluster of ks CTAs shares a tile's k range (choose_tiles): each sums its part, then gives
@@ -709,8 +709,8 @@ static void set_tiles(Plan& P, int ld, int bn, int ks) {
 
 // The shape with the least time in this model: rounds of tiles, each its k-blocks (68 products of 48 clocks, 44 at
 // width 32: reading A bounds them) and about 12 k clocks for filling the pipe, the last drains and the epilogue,
-// less with fewer columns to finish.  One iteration of a run, unsplit and split: N = 400 54 -> 37 us (16 tiles, 152 SMs),
-// N = 700 76 -> 45, N = 1500 (156 tiles) 260 -> 213; N = 2048 stays unsplit.
+// less with fewer columns to finish.  One iteration of a run, unsplit and split: N = 400 54 -> 35 us (16 tiles, 152 SMs),
+// N = 700 76 -> 42, N = 1500 (156 tiles) 260 -> 205; N = 2048 stays unsplit.
 void choose_tiles(Plan& P, int ld) {
   P.ld = ld;
   double best = 1e300;

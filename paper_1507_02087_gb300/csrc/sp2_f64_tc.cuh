@@ -31,7 +31,7 @@ struct Plan {
   bool on = false;
 };
 
-// Sizes at which the tensor-core products are used (see sp2_f64_tc.cu).
+// Sizes at which the tensor-core products are used (see emit_product in sp2_dense_f64.cu).
 constexpr int kMinN = 129;
 // Bytes of the partial records of a problem with T x T tiles of 64 and `recs` records per upper tile (64 for
 // N < kMinN).

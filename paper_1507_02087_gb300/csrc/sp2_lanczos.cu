@@ -8,9 +8,9 @@
 // is available without forming X^2, and e_{k-1} = ||A||_2 = max |lambda(A)| is estimated by
 // kLzSteps steps of the symmetric Lanczos recurrence (three-term, no reorthogonalisation: lost
 // orthogonality only repeats converged extreme Ritz values) from a fixed start vector.  The
-// extreme eigenvalues of the tridiagonal matrix come from multisection with Sturm counts (one
-// warp, 32 points a round, in FP32: the tridiagonal of the scaled A is O(1) and the estimate only
-// needs a few digits).  The Ritz values are inside the spectrum, so the estimate is a lower
+// extreme eigenvalues of the tridiagonal matrix come from multisection with Sturm counts (512
+// points a side, three rounds, in FP32: the tridiagonal of the scaled A is O(1) and the estimate
+// only needs a few digits).  The Ritz values are inside the spectrum, so the estimate is a lower
 // bound of e that approaches it from below; the stop test only needs its logarithm.
 //
 // Per estimate: start (1 CTA: coefficients, start vector, a power-of-two scale 2^-s with 2^s near

@@ -1011,8 +1011,12 @@ int tc_tiles(int ld, int upper, int pair, int tn) {
 
 // The narrowest width whose upper tiles all run at once, or 128 (then 128 x 128 and pair tiles compete): a launch
 // that leaves SMs idle takes the time of one tile, and a narrower tile is shorter, in its epilogue above all
-// (16 columns of it take about 3 k clocks). fp16x3 at N = 400, 10 tiles of 128 columns against 40 of 32 on 152 SMs:
-// 2.50 -> 1.73 ms a purification.
+// (16 columns of it take about 3 k clocks).  A purification with 128 x 32 or 128 x 64, 128 x 128 and pair tiles, from
+// the smallest problems to the largest that fit (N = 1408 on 152 SMs), ms:
+//   fp16x3 N = 300 1.61 1.93 2.51, 700 2.13 2.50 2.96, 1001 2.57 2.85 3.28, 1400 3.30 3.50 4.02
+//   bf16x6         1.84 2.38 3.43,     2.53 3.21 4.25,      3.09 3.72 4.84,      4.09 4.64 6.30
+//   tf32x3         1.88 2.24 3.23,     2.72 3.16 3.96,      3.36 3.75 4.53,      4.43 4.71 5.74
+//   fp16x3 batches: 30 of N = 128 1.78 2.07 2.62, N = 300, 500, 700 and 900 2.65 2.86 3.27.
 int tc_tile_width(const int* ld, int count) {
   for (int tn : {32, 64}) {
     int64_t n = 0;
